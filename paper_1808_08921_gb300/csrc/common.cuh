@@ -89,6 +89,11 @@ __host__ __device__ constexpr int opp(int m) {
                      : 15;
 }
 
+// The nine pairs of opposite directions: pair k is (pair_m(k), opp(pair_m(k))).
+__host__ __device__ constexpr int pair_m(int k) {
+    return k == 0 ? 0 : k == 1 ? 2 : k == 2 ? 4 : k == 3 ? 6 : k == 4 ? 7 : k == 5 ? 8 : k == 6 ? 9 : k == 7 ? 14 : 15;
+}
+
 __host__ __device__ inline uint32_t pack_coord(int x, int y, int z) {
     return ((uint32_t)x << 20) | ((uint32_t)y << 10) | (uint32_t)z;
 }
@@ -195,6 +200,21 @@ __device__ __forceinline__ typename PopT<ST>::T* pop_loc(const Lat& L, bool afte
     if (s == NONE) return f + (size_t)m * L.nSpad + i;
     return f + (size_t)opp(m) * L.nSpad + s;
 }
+
+// A launch macro M(AFTER_EVEN, ST) for the state of lattice L (variables L and
+// after_even in scope).
+#define LBMDEM_BY_STATE(M)                    \
+    do {                                      \
+        if (after_even) {                     \
+            if (L.st == 0) M(true, 0);        \
+            else if (L.st == 1) M(true, 1);   \
+            else M(true, 2);                  \
+        } else {                              \
+            if (L.st == 0) M(false, 0);       \
+            else if (L.st == 1) M(false, 1);  \
+            else M(false, 2);                 \
+        }                                     \
+    } while (0)
 
 // Particles as seen by the lattice kernels (current time level).
 struct PartView {

@@ -641,22 +641,14 @@ void launch_inlet_outlet(const Lat& L, const BC& bc, bool after_even, cudaStream
     int n = 2 * L.ny * L.nz;
     int blocks = (n + 127) / 128;
 #define LBMDEM_IO(AE, ST) k_inlet_outlet<AE, ST><<<blocks, 128, 0, s>>>(L, bc)
-    if (after_even) {
-        if (L.st == 0) LBMDEM_IO(true, 0);
-        else if (L.st == 1) LBMDEM_IO(true, 1);
-        else LBMDEM_IO(true, 2);
-    } else {
-        if (L.st == 0) LBMDEM_IO(false, 0);
-        else if (L.st == 1) LBMDEM_IO(false, 1);
-        else LBMDEM_IO(false, 2);
-    }
+    LBMDEM_BY_STATE(LBMDEM_IO);
 #undef LBMDEM_IO
 }
 
 // ------------------------------------------------------------ read-out
 
-template <int ST>
-__global__ void k_read_fields(Lat L, bool after_even, double* rho, double* u, uint8_t* solid) {
+template <bool AFTER_EVEN, int ST>
+__global__ void k_read_fields(Lat L, double* rho, double* u, uint8_t* solid) {
     size_t N = (size_t)L.nx * L.ny * L.nz;
     size_t n = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (n >= N) return;
@@ -672,7 +664,7 @@ __global__ void k_read_fields(Lat L, bool after_even, double* rho, double* u, ui
     if (fl) {
 #pragma unroll
         for (int m = 0; m < Q; ++m) {
-            double g = (double)to_f<ST>(*pop_loc<ST>(L, after_even, x, y, z, i, m), L.fsi);
+            double g = (double)to_f<ST>(*pop_loc<ST>(L, AFTER_EVEN, x, y, z, i, m), L.fsi);
             d += g;
             jx += cx(m) * g;
             jy += cy(m) * g;
@@ -692,61 +684,84 @@ void launch_read_fields(const Lat& L, bool after_even, double* rho, double* u, u
                         cudaStream_t s) {
     size_t N = (size_t)L.nx * L.ny * L.nz;
     unsigned blocks = (unsigned)((N + 255) / 256);
-    if (L.st == 0) k_read_fields<0><<<blocks, 256, 0, s>>>(L, after_even, rho, u, solid);
-    else if (L.st == 1) k_read_fields<1><<<blocks, 256, 0, s>>>(L, after_even, rho, u, solid);
-    else k_read_fields<2><<<blocks, 256, 0, s>>>(L, after_even, rho, u, solid);
+#define LBMDEM_RF(AE, ST) k_read_fields<AE, ST><<<blocks, 256, 0, s>>>(L, rho, u, solid)
+    LBMDEM_BY_STATE(LBMDEM_RF);
+#undef LBMDEM_RF
 }
 
 // ------------------------------------------------------------ plane means
 
 // Sums over the fluid nodes of every x plane of the current state: out[3 x]
 // += sum (rho - rho_f), out[3 x + 1] += sum rho u_x, out[3 x + 2] += count.
-// Consecutive compact nodes share a plane, so each warp reduces runs of
-// equal x before one FP64 atomic per run head.
-template <int ST>
-__global__ void k_plane_sums(Lat L, bool after_even, double* out) {
-    uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    float d = 0.f, jx = 0.f, n = 0.f;
-    int x = -1;
-    if (i < L.nS && fluid_bit(L, i)) {
-        int y, z;
-        unpack_coord(L.coord[i], x, y, z);
+// A plane's nodes are one range of each region of the compact order (its
+// first words' bases); PLANE_SPLIT blocks share a plane, every thread adds
+// its nodes' FP32 terms in FP64, and each block adds its sums to the plane's
+// with one atomic per quantity.  FP64 adds run at 2 lanes per clock and SM
+// here, so the count of them decides: one per node and quantity, against 64
+// when every lane summed its whole warp (128 x 128 x 1024 column, 4.15 M
+// fluid nodes: 1568 -> 100 us; 160^3, all fluid: 1449 -> 81 us).  The parity is
+// a template parameter: as a run-time branch around every population it keeps
+// the 19 loads of a node one behind the other (252 us).
+constexpr int PLANE_SPLIT = 4, PLANE_THREADS = 256;
+
+template <bool AFTER_EVEN, int ST>
+__global__ void __launch_bounds__(PLANE_THREADS) k_plane_sums(Lat L, double* out) {
+    const int px = blockIdx.x / PLANE_SPLIT, part = blockIdx.x % PLANE_SPLIT;
+    const size_t w0 = (size_t)px * L.ny * L.nw;
+    const bool last = px + 1 == L.nx;
+    const uint4 r0 = L.rec[w0], r1 = last ? r0 : L.rec[w0 + (size_t)L.ny * L.nw];
+    double sd = 0.0, sj = 0.0;
+    uint32_t n = 0;
+    for (int region = 0; region < 2; ++region) {
+        const uint32_t lo = region ? r0.w : r0.z, hi = last ? (region ? L.nS : L.nA) : (region ? r1.w : r1.z);
+        for (uint32_t i = lo + part * PLANE_THREADS + threadIdx.x; i < hi; i += PLANE_SPLIT * PLANE_THREADS) {
+            if (!fluid_bit(L, i)) continue;
+            int x, y, z;
+            unpack_coord(L.coord[i], x, y, z);
+            float d = 0.f, jx = 0.f;
 #pragma unroll
-        for (int m = 0; m < Q; ++m) {
-            float g = to_f<ST>(*pop_loc<ST>(L, after_even, x, y, z, i, m), L.fsi);
-            d += g;
-            jx += cx(m) * g;
+            for (int m = 0; m < Q; ++m) {
+                const float g = to_f<ST>(*pop_loc<ST>(L, AFTER_EVEN, x, y, z, i, m), L.fsi);
+                d += g;
+                jx += cx(m) * g;
+            }
+            sd += (double)d;
+            sj += (double)jx;
+            ++n;
         }
-        n = 1.f;
     }
     const unsigned full = 0xffffffffu;
-    const int lane = threadIdx.x & 31;
-    // sums over the lanes of the warp that share this lane's plane; the
-    // lowest such lane adds them (compact order keeps most warps in one plane)
-    double sd = 0.0, sj = 0.0, sn = 0.0;
-    for (int l = 0; l < 32; ++l) {
-        float a = __shfl_sync(full, d, l), b = __shfl_sync(full, jx, l), c = __shfl_sync(full, n, l);
-        int xl = __shfl_sync(full, x, l);
-        if (xl == x) {
-            sd += a;
-            sj += b;
-            sn += c;
-        }
+    n = __reduce_add_sync(full, n);
+#pragma unroll
+    for (int o = 16; o; o >>= 1) {
+        sd += __shfl_xor_sync(full, sd, o);
+        sj += __shfl_xor_sync(full, sj, o);
     }
-    unsigned peers = __match_any_sync(full, x);
-    if (x >= 0 && lane == __ffs(peers) - 1) {
-        atomicAdd(&out[3 * x], sd);
-        atomicAdd(&out[3 * x + 1], sj);
-        atomicAdd(&out[3 * x + 2], sn);
+    __shared__ double sh[2][PLANE_THREADS / 32];
+    __shared__ uint32_t shn[PLANE_THREADS / 32];
+    if ((threadIdx.x & 31) == 0) {
+        sh[0][threadIdx.x >> 5] = sd;
+        sh[1][threadIdx.x >> 5] = sj;
+        shn[threadIdx.x >> 5] = n;
+    }
+    __syncthreads();
+    if (threadIdx.x < 2) {
+        double v = 0.0;
+        for (int w = 0; w < PLANE_THREADS / 32; ++w) v += sh[threadIdx.x][w];
+        if (v != 0.0) atomicAdd(&out[3 * px + threadIdx.x], v);
+    } else if (threadIdx.x == 2) {
+        uint32_t v = 0;
+        for (int w = 0; w < PLANE_THREADS / 32; ++w) v += shn[w];
+        if (v) atomicAdd(&out[3 * px + 2], (double)v);
     }
 }
 
 void launch_plane_sums(const Lat& L, bool after_even, double* out, cudaStream_t s) {
-    unsigned blocks = (L.nS + 255) / 256;
-    if (!blocks) return;
-    if (L.st == 0) k_plane_sums<0><<<blocks, 256, 0, s>>>(L, after_even, out);
-    else if (L.st == 1) k_plane_sums<1><<<blocks, 256, 0, s>>>(L, after_even, out);
-    else k_plane_sums<2><<<blocks, 256, 0, s>>>(L, after_even, out);
+    const unsigned blocks = (unsigned)L.nx * PLANE_SPLIT;
+    if (!L.nS) return;
+#define LBMDEM_PS(AE, ST) k_plane_sums<AE, ST><<<blocks, PLANE_THREADS, 0, s>>>(L, out)
+    LBMDEM_BY_STATE(LBMDEM_PS);
+#undef LBMDEM_PS
 }
 
 }  // namespace lbmdem
