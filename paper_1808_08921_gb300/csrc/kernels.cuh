@@ -213,22 +213,159 @@ void launch_adj_boundary(const AdjArgs& A, double shape, double* d_amp, cudaStre
 void launch_adj_step(const AdjArgs& A, const float* nat, float* out, float dl, double* d_omega, cudaStream_t s);
 
 // Parameter derivatives of the reverse kernels: each block sums its
-// threads' terms and adds them to one of GRAD_COPIES FP64 accumulators
-// (blockIdx % GRAD_COPIES: no long queue of atomics on one address); the
-// host adds the copies.
+// threads' FP32 terms in FP64 and adds the sum to one of GRAD_COPIES FP64
+// accumulators (blockIdx % GRAD_COPIES: no long queue of atomics on one
+// address); the host adds the copies.  FP64 adds run at 2 lanes per clock and
+// SM here, so the terms go through shared memory to one warp, which adds
+// blockDim / 32 of them per lane before its five shuffle steps (a tree in
+// every warp spends five warp-wide adds on 32 terms).
 constexpr int GRAD_COPIES = 64;
-__device__ __forceinline__ void block_sum_to(double v, double* dst) {
-    __shared__ double part[32];
-#pragma unroll
-    for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (lane == 0) part[wid] = v;
+constexpr int GRAD_THREADS = 256;  // largest block
+__device__ __forceinline__ void block_sum_to(float v, double* dst) {
+    __shared__ float part[GRAD_THREADS];
+    const unsigned tid = threadIdx.x + blockDim.x * threadIdx.y, nt = blockDim.x * blockDim.y;
+    part[tid] = v;
     __syncthreads();
-    if (wid == 0) {
-        v = lane < (int)(blockDim.x >> 5) ? part[lane] : 0.0;
+    if (tid < 32) {
+        double s = 0.0;
+        for (unsigned k = tid; k < nt; k += 32) s += (double)part[k];
 #pragma unroll
-        for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == 0 && v != 0.0) atomicAdd(dst, v);
+        for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (tid == 0 && s != 0.0) atomicAdd(dst, s);
+    }
+}
+
+// The collision's transpose, pair by pair.  Opposite directions share |c.u|,
+// so the equilibria of a pair are an even part plus or minus an odd one, and
+// the contractions A = sum_i v_i dn^eq_i/drho and B = sum_i v_i dn^eq_i/dJ
+// (dn^eq/dJ = w (3 c + 9 (c.u) c - 3 u)) need only the pair's sum p and
+// difference q of v: half the arithmetic of direction-by-direction sums.
+struct RevMoments {
+    float drho, rho, ux, uy, uz, uu15;
+};
+__device__ __forceinline__ RevMoments rev_moments(const float g[Q], float rho_f) {
+    float drho = 0.f, jx = 0.f, jy = 0.f, jz = 0.f;
+#pragma unroll
+    for (int m = 0; m < Q; ++m) {
+        drho += g[m];
+        jx += cx(m) * g[m];
+        jy += cy(m) * g[m];
+        jz += cz(m) * g[m];
+    }
+    RevMoments M;
+    M.drho = drho;
+    M.rho = rho_f + drho;
+    const float ir = 1.0f / M.rho;
+    M.ux = jx * ir;
+    M.uy = jy * ir;
+    M.uz = jz * ir;
+    M.uu15 = 1.5f * (M.ux * M.ux + M.uy * M.uy + M.uz * M.uz);
+    return M;
+}
+// c.u of direction m and the equilibrium deviations of m and opp(m)
+__device__ __forceinline__ void rev_eq(const RevMoments& M, int m, float& cu, float& em, float& eo) {
+    cu = (float)cx(m) * M.ux + (float)cy(m) * M.uy + (float)cz(m) * M.uz;
+    const float even = M.drho + M.rho * (4.5f * cu * cu - M.uu15), odd = 3.0f * M.rho * cu;
+    em = wt(m) * (even + odd);
+    eo = wt(m) * (even - odd);
+}
+// Sums with the integer weights 36 w (1, 2, 12), scaled by 1/36 at the end:
+// the FP32 weights add up to 1 + 1.5e-8, a bias that a recursion of hundreds
+// of steps turns into 1e-6 of the gradient; scaled() is unbiased.
+struct RevSums {
+    float A = 0.f, Bx = 0.f, By = 0.f, Bz = 0.f;
+    float s = 0.f, cc = 0.f;
+    static __device__ __forceinline__ float iw(int m) {
+        return m == 18 ? 12.f : (cx(m) * cx(m) + cy(m) * cy(m) + cz(m) * cz(m)) == 1 ? 2.f : 1.f;
+    }
+    // x / 36, the product corrected by its exact residual
+    static __device__ __forceinline__ float scaled(float x) {
+        const float q = x * (1.f / 36.f);
+        return fmaf(fmaf(-36.f, q, x), 1.f / 36.f, q);
+    }
+    // the pair (m, opp(m)): p = v_m + v_opp, q = v_m - v_opp
+    __device__ __forceinline__ void add(int m, float cu, float p, float q) {
+        const float wp = iw(m) * p, t = 9.0f * cu * wp + (3.0f * iw(m)) * q;
+        s += wp;
+        cc += cu * cu * wp;
+        Bx += cx(m) * t;
+        By += cy(m) * t;
+        Bz += cz(m) * t;
+    }
+    __device__ __forceinline__ void finish(const RevMoments& M, float v18) {
+        s += 12.f * v18;
+        A = scaled(s * (1.0f + M.uu15) - 4.5f * cc);
+        Bx = scaled(Bx - 3.0f * M.ux * s);
+        By = scaled(By - 3.0f * M.uy * s);
+        Bz = scaled(Bz - 3.0f * M.uz * s);
+    }
+    __device__ __forceinline__ float dot(int m) const { return Bx * cx(m) + By * cy(m) + Bz * cz(m); }
+};
+
+// Transposed pressure face (Section 2.4) on the adjoint of one boundary node,
+// element m at a[m P]: the adjoint of the five unknowns moves onto the knowns
+// (the forward formulas are linear in the knowns and in the boundary
+// density), the unknowns' adjoint becomes zero.  Side 0: inlet, 1: outlet.
+// Returns the derivative in the boundary density.  Every load is issued
+// before the first store: written as read-modify-writes the compiler has to
+// keep their order (the 19 planes may alias), and the kernel waited for 14
+// loads one after another (10.6 -> 4.0 us per launch at 64 x 64 lines).
+template <int SIDE>
+__device__ __forceinline__ float adj_face(float* a, size_t P) {
+    float v[Q];
+#pragma unroll
+    for (int m = 0; m < Q; ++m) v[m] = a[m * P];
+    // the unknowns 0, 6, 7, 8, 9 of the inlet are the knowns of the outlet
+    // and the other way round: pairs (unknown, known) share their index pair
+    constexpr int in[5] = {0, 6, 7, 8, 9}, out[5] = {1, 11, 10, 13, 12};
+    float ar, ay, az, two;
+    if (SIDE == 0) {
+        ar = v[0] * (1.f / 3.f) + (v[6] + v[7] + v[8] + v[9]) * (1.f / 6.f);
+        ay = 0.5f * (v[7] - v[6]);
+        az = 0.5f * (v[9] - v[8]);
+        two = -2.f * ar;
+    } else {
+        // forward: rux = rest + 2 (g0 + g6 + g7 + g8 + g9) - drho_b;
+        // g1 = g0 - rux/3, g11 = g6 - rux/6 + Ny, g10 = g7 - rux/6 - Ny,
+        // g13 = g8 - rux/6 + Nz, g12 = g9 - rux/6 - Nz
+        ar = -(v[1] * (1.f / 3.f) + (v[11] + v[10] + v[13] + v[12]) * (1.f / 6.f));
+        ay = 0.5f * (v[11] - v[10]);
+        az = 0.5f * (v[13] - v[12]);
+        two = 2.f * ar;
+    }
+    const float rest = SIDE == 0 ? -ar : ar;
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+        const int u = SIDE == 0 ? in[k] : out[k], w = SIDE == 0 ? out[k] : in[k];
+        a[w * P] = v[w] + (v[u] + two);
+        a[u * P] = 0.f;
+    }
+    a[18 * P] = v[18] + rest;
+    a[2 * P] = v[2] + (rest + ay);
+    a[3 * P] = v[3] + (rest - ay);
+    a[4 * P] = v[4] + (rest + az);
+    a[5 * P] = v[5] + (rest - az);
+    a[14 * P] = v[14] + (rest + ay + az);
+    a[15 * P] = v[15] + (rest + ay - az);
+    a[16 * P] = v[16] + (rest - ay + az);
+    a[17 * P] = v[17] + (rest - ay - az);
+    return ar;
+}
+
+// Transposed zero-gradient outlet: the unknowns' adjoint of outlet node o
+// goes to the upstream node u.
+__device__ __forceinline__ void adj_copy(float* a, size_t P, size_t u, size_t o) {
+    constexpr int um[5] = {1, 10, 11, 12, 13};
+    float s[5], t[5];
+#pragma unroll
+    for (int q = 0; q < 5; ++q) {
+        s[q] = a[um[q] * P + o];
+        t[q] = a[um[q] * P + u];
+    }
+#pragma unroll
+    for (int q = 0; q < 5; ++q) {
+        a[um[q] * P + u] = t[q] + s[q];
+        a[um[q] * P + o] = 0.f;
     }
 }
 

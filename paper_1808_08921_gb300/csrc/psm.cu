@@ -41,13 +41,13 @@ __device__ __forceinline__ size_t dense(const PsmArgs& A, int x, int y, int z) {
 
 // node of this thread in the 3-D launch of psm_grid: z along the block's
 // threads, y and x from the block indices (no integer division); false past
-// the end of a z line
+// the end of a z line or of a plane's lines
 __device__ __forceinline__ bool grid_node(const PsmArgs& A, int& x, int& y, int& z, size_t& k) {
     z = blockIdx.x * blockDim.x + threadIdx.x;
-    y = blockIdx.y;
+    y = blockIdx.y * blockDim.y + threadIdx.y;
     x = blockIdx.z;
     k = dense(A, x, y, z);
-    return z < A.nz;
+    return z < A.nz && y < A.ny;
 }
 
 __device__ __forceinline__ double smooth_step(double v) {
@@ -56,23 +56,68 @@ __device__ __forceinline__ double smooth_step(double v) {
     return v * v * (3.0 - 2.0 * v);
 }
 
-// node offset from a centre along one axis, nearest periodic image
-__device__ __forceinline__ double image(double d, double L, bool periodic) {
-    return periodic ? d - L * floor(d / L + 0.5) : d;
+// node offset from a centre along one axis, nearest periodic image; iL = 1/L
+// (the image count differs from that of d / L at most where both images are
+// equally far)
+__device__ __forceinline__ double image(double d, double L, double iL, bool periodic) {
+    return periodic ? d - L * floor(d * iL + 0.5) : d;
 }
 
+// One block per segment of a z line.  The block first collects, in index
+// order, the spheres that can reach the segment (their distance in the x, y
+// plane and to the z interval, with a margin of 0.01 lu over the exact test
+// below, far above the FP32 rounding of offsets within the box); its nodes then evaluate only those.  Evaluating every sphere at
+// every node is FP64 arithmetic at 2 lanes per clock and SM: 7.77 ms for
+// 128 spheres on 64 x 64 x 256, against 0.31 ms.  The kept spheres go through
+// the same test and product in the same order, so eps is the same bit for
+// bit.  A segment reached by more than EPS_LIST spheres walks them all.
+constexpr int EPS_LIST = 256;
 __global__ void k_psm_eps(PsmArgs A, const double* X, const double* R, int n, float* eps) {
+    __shared__ int s_list[EPS_LIST];
+    __shared__ int s_count[9];  // per warp, then the list's length
     int x, y, z;
     size_t k;
-    if (!grid_node(A, x, y, z, k)) return;
-    if (!A.px && (x == 0 || x == A.nx - 1)) {
-        eps[k] = 0.f;
+    const bool inside = grid_node(A, x, y, z, k);
+    const bool end = !A.px && (x == 0 || x == A.nx - 1);  // uniform over the block
+    if (end) {
+        if (inside) eps[k] = 0.f;
         return;
     }
+    const int z0 = blockIdx.x * blockDim.x, z1 = min(z0 + (int)blockDim.x, A.nz) - 1;
+    const double zc = 0.5 * (z0 + z1), iL[3] = {1.0 / A.nx, 1.0 / A.ny, 1.0 / A.nz};
+    const float zh = 0.5f * (float)(z1 - z0);
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    int total = 0;
+    for (int p0 = 0; p0 < n; p0 += blockDim.x) {
+        const int p = p0 + threadIdx.x;
+        bool near = false;
+        if (p < n) {
+            const float rx = (float)image(x - X[3 * p], A.nx, iL[0], A.px),
+                        ry = (float)image(y - X[3 * p + 1], A.ny, iL[1], true);
+            const float dz = fmaxf(fabsf((float)image(zc - X[3 * p + 2], A.nz, iL[2], true)) - zh, 0.f);
+            const float reach = (float)R[p] + 0.51f;
+            near = rx * rx + ry * ry + dz * dz < reach * reach;
+        }
+        const unsigned bal = __ballot_sync(0xffffffffu, near);
+        if (lane == 0) s_count[wid] = __popc(bal);
+        __syncthreads();
+        int at = total;
+        for (int w = 0; w < nw; ++w) {
+            if (w < wid) at += s_count[w];
+            total += s_count[w];
+        }
+        at += __popc(bal & ((1u << lane) - 1u));
+        if (near && at < EPS_LIST) s_list[at] = p;
+        __syncthreads();
+    }
+    if (!inside) return;
+    const bool all = total > EPS_LIST;
+    const int m = all ? n : total;
     double keep = 1.0;
-    for (int p = 0; p < n; ++p) {
-        const double rx = image(x - X[3 * p], A.nx, A.px), ry = image(y - X[3 * p + 1], A.ny, true),
-                     rz = image(z - X[3 * p + 2], A.nz, true);
+    for (int t = 0; t < m; ++t) {
+        const int p = all ? t : s_list[t];
+        const double rx = image(x - X[3 * p], A.nx, iL[0], A.px), ry = image(y - X[3 * p + 1], A.ny, iL[1], true),
+                     rz = image(z - X[3 * p + 2], A.nz, iL[2], true);
         const double d2 = rx * rx + ry * ry + rz * rz, reach = R[p] + 0.5;
         if (d2 >= reach * reach) continue;
         keep *= 1.0 - smooth_step(R[p] - sqrt(d2) + 0.5);
@@ -197,55 +242,14 @@ __global__ void k_psm_adj_boundary(PsmArgs A, float* a, double shape, double* d_
         const size_t P = A.N;
         if (A.inlet == 0) {
             const size_t i = dense(A, 0, y, z);
-            const float a0 = a[0 * P + i], a6 = a[6 * P + i], a7 = a[7 * P + i], a8 = a[8 * P + i],
-                        a9 = a[9 * P + i];
-            const float ar = a0 * (1.f / 3.f) + (a6 + a7 + a8 + a9) * (1.f / 6.f);
-            const float ay = 0.5f * (a7 - a6), az = 0.5f * (a9 - a8);
-            a[1 * P + i] += a0 - 2.f * ar;
-            a[11 * P + i] += a6 - 2.f * ar;
-            a[10 * P + i] += a7 - 2.f * ar;
-            a[13 * P + i] += a8 - 2.f * ar;
-            a[12 * P + i] += a9 - 2.f * ar;
-            a[18 * P + i] += -ar;
-            a[2 * P + i] += -ar + ay;
-            a[3 * P + i] += -ar - ay;
-            a[4 * P + i] += -ar + az;
-            a[5 * P + i] += -ar - az;
-            a[14 * P + i] += -ar + ay + az;
-            a[15 * P + i] += -ar + ay - az;
-            a[16 * P + i] += -ar - ay + az;
-            a[17 * P + i] += -ar - ay - az;
-            a[0 * P + i] = a[6 * P + i] = a[7 * P + i] = a[8 * P + i] = a[9 * P + i] = 0.f;
-            da = (double)ar * shape;
+            da = (double)adj_face<0>(a + i, P) * shape;
         }
         const size_t o = dense(A, A.nx - 1, y, z);
         if (A.outlet == 0) {
             const size_t u = dense(A, A.nx - 2, y, z);
-            const int um[5] = {1, 10, 11, 12, 13};
-            for (int q = 0; q < 5; ++q) {
-                a[um[q] * P + u] += a[um[q] * P + o];
-                a[um[q] * P + o] = 0.f;
-            }
+            adj_copy(a, P, u, o);
         } else if (A.outlet == 1) {
-            const float a1 = a[1 * P + o], a11 = a[11 * P + o], a10 = a[10 * P + o], a13 = a[13 * P + o],
-                        a12 = a[12 * P + o];
-            const float ar = -(a1 * (1.f / 3.f) + (a11 + a10 + a13 + a12) * (1.f / 6.f));
-            const float ay = 0.5f * (a11 - a10), az = 0.5f * (a13 - a12);
-            a[0 * P + o] += a1 + 2.f * ar;
-            a[6 * P + o] += a11 + 2.f * ar;
-            a[7 * P + o] += a10 + 2.f * ar;
-            a[8 * P + o] += a13 + 2.f * ar;
-            a[9 * P + o] += a12 + 2.f * ar;
-            a[18 * P + o] += ar;
-            a[2 * P + o] += ar + ay;
-            a[3 * P + o] += ar - ay;
-            a[4 * P + o] += ar + az;
-            a[5 * P + o] += ar - az;
-            a[14 * P + o] += ar + ay + az;
-            a[15 * P + o] += ar + ay - az;
-            a[16 * P + o] += ar - ay + az;
-            a[17 * P + o] += ar - ay - az;
-            a[1 * P + o] = a[11 * P + o] = a[10 * P + o] = a[13 * P + o] = a[12 * P + o] = 0.f;
+            adj_face<1>(a + o, P);
         }
     }
 #pragma unroll
@@ -253,12 +257,17 @@ __global__ void k_psm_adj_boundary(PsmArgs A, float* a, double shape, double* d_
     if ((threadIdx.x & 31) == 0 && da != 0.0) atomicAdd(d_amp, da);
 }
 
-// lam_k = J^T mu + dl_k / dg_k at every node, with the tau and eps derivatives
-__global__ void __launch_bounds__(256) k_psm_adj_step(PsmArgs A, const float* lin, const float* gt, float* lout,
+// lam_k = J^T mu + dl_k / dg_k at every node, with the tau and eps derivatives.
+// 248 B per node (39 us at the copy rate on 64 x 64 x 256), but bound by issue
+// and occupancy: 2600 instructions per warp at 140 registers took 147 us.  The
+// pairwise contractions, the derivatives as two sums with per-node factors
+// (no division per direction) and blocks of 256 threads at 80 registers (24
+// warps per SM; 119 registers and 16 warps: 83 us) bring it to 63 us.
+__global__ void __launch_bounds__(GRAD_THREADS, 3) k_psm_adj_step(PsmArgs A, const float* lin, const float* gt, float* lout,
                                                       const float* eps, float dl, double* d_tau, double* G) {
     int x, y, z;
     size_t k;
-    double dt = 0.0;
+    float dt = 0.f;
     if (grid_node(A, x, y, z, k)) {
         const int ym = y == 0 ? A.ny - 1 : y - 1, yp = y == A.ny - 1 ? 0 : y + 1;
         const int zm = z == 0 ? A.nz - 1 : z - 1, zp = z == A.nz - 1 ? 0 : z + 1;
@@ -272,40 +281,46 @@ __global__ void __launch_bounds__(256) k_psm_adj_step(PsmArgs A, const float* li
             const int ys = cy(m) > 0 ? yp : (cy(m) < 0 ? ym : y), zs = cz(m) > 0 ? zp : (cz(m) < 0 ? zm : z);
             mu[m] = out ? lin[(size_t)opp(m) * A.N + k] : lin[(size_t)m * A.N + dense(A, xs, ys, zs)];
         }
-        float g[Q], geq[Q];
+        float g[Q];
 #pragma unroll
         for (int m = 0; m < Q; ++m) g[m] = gt[(size_t)m * A.N + k];
-        float drho, ux, uy, uz;
-        psm_eq(g, A.rho_f, drho, ux, uy, uz, geq);
+        const RevMoments M = rev_moments(g, A.rho_f);
         const float e = eps[k], tau = A.tau, sh = tau - 0.5f, den = (1.0f - e) + sh;
         float B, a;
         psm_weights(e, tau, B, a);
-        const float dB_dtau = e * (1.0f - e) / (den * den), dB_de = sh * (1.0f + sh) / (den * den);
-        const float da_dtau = -dB_dtau / tau - (1.0f - B) / (tau * tau);
-        const float uu = ux * ux + uy * uy + uz * uz;
-        float Aa = 0.f, Bx = 0.f, By = 0.f, Bz = 0.f, wmu = 0.f, st = 0.f, se = 0.f;
-#pragma unroll
-        for (int m = 0; m < Q; ++m) {
-            const float om = g[opp(m)] - g[m] + wt(m) * drho - geq[opp(m)];
-            st += mu[m] * (-da_dtau * (g[m] - geq[m]) + dB_dtau * om);
-            se += mu[m] * (dB_de * ((g[m] - geq[m]) / tau + om));
-            wmu += wt(m) * mu[m];
-            const float nu = a * mu[m] - B * mu[opp(m)];
-            const float cu = cx(m) * ux + cy(m) * uy + cz(m) * uz;
-            const float wn = wt(m) * nu;
-            Aa += wn * (1.0f - 4.5f * cu * cu + 1.5f * uu);
-            const float kk = 3.0f + 9.0f * cu;
-            Bx += wn * (kk * cx(m) - 3.0f * ux);
-            By += wn * (kk * cy(m) - 3.0f * uy);
-            Bz += wn * (kk * cz(m) - 3.0f * uz);
+        // with d_m = g_m - g^eq_m:  Om_m = d_opp(m) - (g_m - w drho), and the
+        // tau and eps derivatives are two sums, mu.d and mu.Om, with per-node
+        // factors
+        RevSums S;
+        float sd, so, wmu;
+        {
+            const float e18 = wt(18) * (M.drho - M.rho * M.uu15);
+            sd = mu[18] * (g[18] - e18);
+            so = mu[18] * (wt(18) * M.drho - e18);
+            wmu = 12.f * mu[18];
         }
-        const float add = x == A.probe_x ? dl : 0.f;
 #pragma unroll
-        for (int m = 0; m < Q; ++m)
-            lout[(size_t)m * A.N + k] = (1.0f - a - B) * mu[m] + B * mu[opp(m)] + B * wmu + Aa + Bx * cx(m) +
-                                        By * cy(m) + Bz * cz(m) + add;
+        for (int q = 0; q < 9; ++q) {
+            const int m = pair_m(q), o = opp(m);
+            float cu, em, eo;
+            rev_eq(M, m, cu, em, eo);
+            const float dm = g[m] - em, d_o = g[o] - eo, wd = wt(m) * M.drho;
+            sd += mu[m] * dm + mu[o] * d_o;
+            so += mu[m] * (d_o - (g[m] - wd)) + mu[o] * (dm - (g[o] - wd));
+            const float p = mu[m] + mu[o], r = mu[m] - mu[o];
+            wmu += RevSums::iw(m) * p;
+            S.add(m, cu, (a - B) * p, (a + B) * r);  // nu = a mu - B mu_opp
+        }
+        S.finish(M, (a - B) * mu[18]);
+        const float id = 1.0f / (den * den), it = 1.0f / tau;
+        const float dB_dtau = e * (1.0f - e) * id, dB_de = sh * (1.0f + sh) * id;
+        const float da_dtau = -dB_dtau * it - (1.0f - B) * it * it;
+        const float st = dB_dtau * so - da_dtau * sd, se = dB_de * (sd * it + so);
+        const float base = B * RevSums::scaled(wmu) + S.A + (x == A.probe_x ? dl : 0.f), keep = 1.0f - a - B;
+#pragma unroll
+        for (int m = 0; m < Q; ++m) lout[(size_t)m * A.N + k] = keep * mu[m] + B * mu[opp(m)] + (base + S.dot(m));
         G[k] += (double)se;
-        dt = (double)st;
+        dt = st;
     }
     block_sum_to(dt, d_tau + (blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z)) % GRAD_COPIES);
 }
@@ -357,17 +372,19 @@ __global__ void k_psm_grad_x(PsmArgs A, const double* G, const float* eps, const
     }
 }
 
-// one thread per node: z lines in blocks of up to 256 threads, one block row
-// per (y, x)
-static void psm_grid(const PsmArgs& A, dim3& grid, dim3& block) {
+// one thread per node: segments of z lines of up to 256 threads and, where
+// the lines are shorter, several lines per block up to 256 threads in all
+// (lines: 1 for the kernel whose blocks work on one line)
+static void psm_grid(const PsmArgs& A, dim3& grid, dim3& block, int lines = 0) {
     const int tz = A.nz >= 256 ? 256 : ((A.nz + 31) / 32) * 32;
-    block = dim3(tz, 1, 1);
-    grid = dim3((A.nz + tz - 1) / tz, A.ny, A.nx);
+    const int ty = lines ? lines : GRAD_THREADS / tz;
+    block = dim3(tz, ty, 1);
+    grid = dim3((A.nz + tz - 1) / tz, (A.ny + ty - 1) / ty, A.nx);
 }
 
 void launch_psm_eps(const PsmArgs& A, const double* X, const double* R, int n, float* eps, cudaStream_t s) {
     dim3 g, b;
-    psm_grid(A, g, b);
+    psm_grid(A, g, b, 1);
     k_psm_eps<<<g, b, 0, s>>>(A, X, R, n, eps);
 }
 void launch_psm_step(const PsmArgs& A, const float* gin, float* gout, const float* eps, cudaStream_t s) {
