@@ -130,6 +130,10 @@ struct lbmdem_ctx {
     DBuf<int> nb_cnt, nb_j, nb_cnt2, nb_j2;
     DBuf<int8_t> nb_sh, nb_sh2;
     DBuf<float4> nb_dref, nb_ft, nb_dref2, nb_ft2;
+    DBuf<int> nb_slot, dem_foreign, dem_slots;  // exchange slots of the one-launch DEM
+    DBuf<float> nb_R;
+    DBuf<uint16_t> dem_push;
+    int* dem_slots_host = nullptr;  // pinned, valid once the stream is synchronised after build_neighbours
     CellGrid grid{};
     CellBufs cells;       // the DEM's cell list (cells 2 R + dem_skin wide)
     CellBufs band_cells;  // cells R + skin wide: a band node's candidates lie within R + skin
@@ -246,7 +250,6 @@ static Dem make_dem(lbmdem_ctx* c) {
     Dem D{};
     D.n = c->np;
     D.K = c->p.dem_substeps;
-    D.cluster = 8;
     D.dt = 1.0f / (float)c->p.dem_substeps;
     D.kn = (float)(2.0 * c->p.E_p / (3.0 * (1.0 - c->p.nu_p * c->p.nu_p)));
     D.kt = (float)(2.0 * c->p.E_p / ((1.0 + c->p.nu_p) * (2.0 - c->p.nu_p)));
@@ -278,6 +281,11 @@ static Dem make_dem(lbmdem_ctx* c) {
     D.nb_j = c->nb_j.p;
     D.nb_dref = c->nb_dref.p;
     D.nb_ft = c->nb_ft.p;
+    D.nb_slot = c->nb_slot.p;
+    D.push = c->dem_push.p;
+    D.nb_R = c->nb_R.p;
+    D.foreign = c->dem_foreign.p;
+    D.slots = *c->dem_slots_host;
     D.org = c->org.p;
     D.orgw = c->orgw.p;
     D.xf = c->xf.p;
@@ -289,6 +297,7 @@ static Dem make_dem(lbmdem_ctx* c) {
     D.max_vel_bits = &s->max_vel_bits;
     D.hard_disp = (float)c->hard;
     D.px = c->p.inlet == LBMDEM_X_PERIODIC;
+    D.dry = !c->lbm;
     D.Lx = c->p.nx;
     D.Ly = c->p.ny;
     D.Lz = c->p.nz;
@@ -367,6 +376,8 @@ static int build_neighbours(lbmdem_ctx* c, bool carry) {
     B.old_j = have_old ? c->nb_j.p : nullptr;
     B.old_sh = have_old ? c->nb_sh.p : nullptr;
     B.old_ft = have_old ? c->nb_ft.p : nullptr;
+    CK(c->nb_R.ensure(ne));
+    B.nR = c->nb_R.p;
     B.status = &c->st.p->status;
     launch_nb_build(B, c->stream);
     CK(cudaGetLastError());
@@ -375,6 +386,14 @@ static int build_neighbours(lbmdem_ctx* c, bool carry) {
     c->nb_sh.swap(c->nb_sh2);
     c->nb_dref.swap(c->nb_dref2);
     c->nb_ft.swap(c->nb_ft2);
+    // exchange slots; every caller synchronises the stream before it launches a step
+    CK(c->nb_slot.ensure(ne));
+    CK(c->dem_push.ensure((size_t)std::max(np, 1) * DEM_MAX_CTAS));
+    CK(c->dem_foreign.ensure(DEM_MAX_CTAS));
+    CK(c->dem_slots.ensure(1));
+    launch_dem_ghosts(make_dem(c), c->nb_slot.p, c->dem_push.p, c->dem_foreign.p, c->dem_slots.p, c->stream);
+    CK(cudaGetLastError());
+    CK(cudaMemcpyAsync(c->dem_slots_host, c->dem_slots.p, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     return 0;
 }
 
@@ -599,7 +618,7 @@ static void record_pair_end(lbmdem_ctx* c, size_t idx, cudaStream_t st = nullptr
 static bool links_in_collide(const lbmdem_ctx* c, int parity) { return c->fused_links && parity == 0; }
 
 static int64_t kernels_per_step(const lbmdem_ctx* c, int parity) {
-    int64_t k = 1;  // DEM
+    int64_t k = dem_launches(c->np, c->p.dem_substeps);
     if (c->lbm) {
         k += c->nband ? 4 : 1;
         k += c->nS ? 1 : 0;
@@ -670,7 +689,7 @@ static void enqueue_step(lbmdem_ctx* c, int parity, bool monitor) {
             cudaEventRecord(c->ev_join, c->side);
             Dem D = make_dem(c);
             if (tm) record_pair_begin(c, 4, e);
-            launch_dem_step(D, false, s);
+            launch_dem_step(D, s);
             if (tm) record_pair_end(c, e);
             cudaStreamWaitEvent(s, c->ev_join, 0);
             return;
@@ -678,7 +697,7 @@ static void enqueue_step(lbmdem_ctx* c, int parity, bool monitor) {
     }
     Dem D = make_dem(c);
     if (tm) record_pair_begin(c, 4, e);
-    launch_dem_step(D, false, s);
+    launch_dem_step(D, s);
     if (tm) record_pair_end(c, e);
 }
 
@@ -779,9 +798,9 @@ static int relayout(lbmdem_ctx* c) {
     if (c->lbm) {
         if (int r = build_layout(c, false)) return r;
     }
-    Dem D = make_dem(c);
-    launch_dem_step(D, true, s);
+    launch_dem_init(make_dem(c), s);
     CK(cudaGetLastError());
+    if (!c->lbm) CK(cudaStreamSynchronize(s));  // the exchange slots' count (build_layout synchronises)
     c->relayouts++;
     destroy_graph(c);
     return 0;
@@ -872,7 +891,10 @@ int lbm_dem_init(const lbmdem_params* pp, lbmdem_ctx** out) {
         cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming) != cudaSuccess)
         return bail(LBMDEM_ERR_CUDA);
     if (c->st.alloc(1) != cudaSuccess) return bail(LBMDEM_ERR_OOM);
-    if (cudaMallocHost((void**)&c->st_host, sizeof(DevStats)) != cudaSuccess) return bail(LBMDEM_ERR_OOM);
+    if (cudaMallocHost((void**)&c->st_host, sizeof(DevStats)) != cudaSuccess ||
+        cudaMallocHost((void**)&c->dem_slots_host, sizeof(int)) != cudaSuccess)
+        return bail(LBMDEM_ERR_OOM);
+    *c->dem_slots_host = 0;
     if (cudaMemset(c->st.p, 0, sizeof(DevStats)) != cudaSuccess) return bail(LBMDEM_ERR_CUDA);
     if (c->lbm) {
         if (c->owner.alloc(c->N) || c->deep.alloc(c->N) || c->band.alloc(c->N) || c->rec.alloc(c->W) ||
@@ -1028,8 +1050,7 @@ int lbm_dem_set_packing(lbmdem_ctx* c, int32_t n, const double* X, const double*
     c->probe_cap = 0;
     c->probe.release();
     if (int r = ensure_probe(c, 4096)) return r;
-    Dem D = make_dem(c);
-    launch_dem_step(D, true, s);
+    launch_dem_init(make_dem(c), s);
     CK(cudaGetLastError());
     CK(cudaMemcpyAsync(c->st_host, c->st.p, sizeof(DevStats), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
@@ -1909,6 +1930,7 @@ void lbm_dem_destroy(lbmdem_ctx* c) {
     destroy_graph(c);
     for (cudaEvent_t e : c->ev) cudaEventDestroy(e);
     if (c->st_host) cudaFreeHost(c->st_host);
+    if (c->dem_slots_host) cudaFreeHost(c->dem_slots_host);
     if (c->side) cudaStreamSynchronize(c->side);
     if (c->ev_fork) cudaEventDestroy(c->ev_fork);
     if (c->ev_join) cudaEventDestroy(c->ev_join);

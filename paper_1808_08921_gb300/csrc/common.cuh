@@ -236,9 +236,10 @@ struct PartView {
     double* Th;           // [NREP][n][3] hydrodynamic torque accumulators
 };
 
-// The link kernel spreads its atomics over NREP copies of each sphere's
-// force and torque accumulators (fewer same-address collisions); the DEM
-// kernel and the read-out sum the copies.
+// The link kernels spread their atomics over NREP copies of each sphere's
+// force and torque accumulators (fewer same-address collisions: with one copy
+// the even kernel with links takes 279 instead of 183 us on the 128 x 128 x
+// 1024 column); the DEM kernel and the read-out sum the copies.
 constexpr int NREP = 4;
 
 // Exact "inside" test shared by painting and the map update: |y - X|^2 < R^2

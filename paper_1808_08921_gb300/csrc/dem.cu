@@ -1,24 +1,23 @@
 // dem.cu -- the solid phase (Section 2.2, Eqs. 9-12).
 //
-//  * k_dem_step_dsm: one launch per LBM step, one thread-block cluster of up
-//    to 16 CTAs, a team of TEAM threads per sphere holding the sphere's
-//    state in registers; positions and half-step velocities are exchanged
-//    through distributed shared memory.  k_dem_step is the general form
-//    (state in global memory, several spheres per team) for packings too
-//    large for one cluster, and computes the initial contact forces.
-//  * Both: one thread-block cluster (co-scheduled), a team per sphere.  It runs the K velocity-
-//    Verlet substeps of length 1/K with the hydrodynamic force and torque of
-//    the step held fixed: kick + drift of the own sphere, one cluster barrier,
-//    then the contact forces of the own sphere from its neighbour list and
-//    the closing kick.  Positions and half-step velocities read by the
-//    neighbours are double-buffered by substep parity, so one barrier per
-//    substep suffices.  Each pair is evaluated by both spheres with mirror-
-//    exact arithmetic, so the two forces are exact negatives and no atomics
-//    are needed.  The hydrodynamic force and torque that drive a sphere are
-//    the mean of the exchange sums of this and the previous LBM step (the
-//    half-way bounce-back force alternates from step to step; the two-step
-//    mean of Ladd's momentum-exchange method keeps the explicit coupling of
-//    light spheres stable).
+//  * Every LBM step runs the K velocity-Verlet substeps of length 1/K with the
+//    hydrodynamic force and torque of the step held fixed: kick + drift of
+//    the own sphere, an exchange of positions and half-step velocities, then
+//    the contact forces of the own sphere from its neighbour list and the
+//    closing kick.  A team of TEAM threads works on each sphere.  The
+//    exchanged records are double-buffered by substep parity, so one
+//    synchronisation per substep suffices.  Each pair is evaluated by both
+//    spheres with mirror-exact arithmetic, so the two forces are exact
+//    negatives and no atomics are needed.  The hydrodynamic force and torque
+//    that drive a sphere are the mean of the exchange sums of this and the
+//    previous LBM step (the half-way bounce-back force alternates from step
+//    to step; the two-step mean of Ladd's momentum-exchange method keeps the
+//    explicit coupling of light spheres stable).
+//  * k_dem_step_dsm: packings of up to 2048 spheres, one launch per LBM step,
+//    one thread-block cluster (one CTA for up to 64 spheres), the spheres'
+//    state in registers, the exchange in shared memory.
+//  * k_dem_begin / k_dem_substep: larger packings, one launch per substep over
+//    the whole GPU, the state in global memory.
 //  * neighbour lists: uniform cells of size >= 2 R_max + skin over the
 //    periodic y, z box; every periodic image is a separate entry (a sphere in
 //    a narrow box can touch two images of the same neighbour).  Rebuilt only
@@ -26,15 +25,11 @@
 //
 // Positions are X = Xref (FP64, fixed between re-layouts) + dX (FP32 with a
 // Kahan compensation term), so the substep loop needs no FP64 arithmetic.
-#include <cooperative_groups.h>
-
 #include <algorithm>
 
 #include "common.cuh"
 #include "kernels.cuh"
 #include "layout.cuh"
-
-namespace cg = cooperative_groups;
 
 namespace lbmdem {
 
@@ -45,34 +40,36 @@ __device__ __forceinline__ float3 crossf(float3 a, float3 b) {
 
 constexpr int TEAM = 4;  // threads per sphere: they share its neighbour list
 
+// Reduced radius R_i R_j / (R_i + R_j) of a pair.
+__device__ __forceinline__ float reduced_radius(float Ri, float Rj) { return __fdividef(Ri * Rj, Ri + Rj); }
+
 // One contact of sphere i with neighbour entry (j, image) (Eqs. 11-12):
 // Hertz normal force, incremental Mindlin tangential force from the
 // half-step relative velocity at the contact point, previous tangential
 // force projected on the current tangent plane, Coulomb cap.  dl = dX_j -
-// dX_i; dr = the entry's reference separation (w: (R_i + R_j)^2 - |xyz|^2).
-// Updates the history h (force on i) and adds the force and torque on i.
+// dX_i; dr = the entry's reference separation (w: (R_i + R_j)^2 - |xyz|^2);
+// Rs the pair's reduced radius.  Updates the history h (force on i) and adds
+// the force and torque on i; a pair out of contact (and an unused entry,
+// dr.w < 0) adds nothing and clears h.  Without branches, so that the
+// contacts of a lane interleave: each is a chain of some 400 cycles.
 // The arithmetic is mirror-exact: sphere j, evaluating the same pair,
 // obtains exactly the negative force.  Square roots and divisions use the
 // hardware approximations (reciprocal square root, fast divide; a few ulp):
 // deterministic functions of symmetric operands, so exactness of the pair
 // is kept.
-__device__ __forceinline__ void pair_contact(const Dem& D, float Ri, float Rj, float3 dl, float4 dr, float3 vi,
-                                             float3 wi, float3 vj, float3 wj, float dt_inc, float4& h, float3& F,
-                                             float3& T) {
+__device__ __forceinline__ void pair_contact(const Dem& D, float Ri, float Rj, float Rs, float3 dl, float4 dr,
+                                             float3 vi, float3 wi, float3 vj, float3 wj, float dt_inc, float3& h,
+                                             float3& F, float3& T) {
     float3 d = make_float3(dr.x + dl.x, dr.y + dl.y, dr.z + dl.z);
     float cut = Ri + Rj;
     // cut^2 - |d|^2 without cancellation: e0 - 2 dref.dl - dl.dl
     float qd = dr.w - (2.f * (dr.x * dl.x + dr.y * dl.y + dr.z * dl.z) + (dl.x * dl.x + dl.y * dl.y + dl.z * dl.z));
-    if (!(qd > 0.f)) {
-        h = make_float4(0.f, 0.f, 0.f, 0.f);
-        return;
-    }
+    const bool touch = qd > 0.f;
     float d2 = d.x * d.x + d.y * d.y + d.z * d.z;
     float idist = rsqrtf(d2);
     float dist = d2 * idist;
     float delta = __fdividef(qd, cut + dist);
     float3 n = make_float3(d.x * idist, d.y * idist, d.z * idist);
-    float Rs = __fdividef(Ri * Rj, Ri + Rj);
     float rd = Rs * delta;
     float sq = rd * rsqrtf(rd);
     float fn = D.kn * sq * delta;
@@ -89,52 +86,26 @@ __device__ __forceinline__ void pair_contact(const Dem& D, float Ri, float Rj, f
     float3 ft = make_float3(h.x - hn * n.x + kdt * vt.x, h.y - hn * n.y + kdt * vt.y, h.z - hn * n.z + kdt * vt.z);
     float ftm2 = ft.x * ft.x + ft.y * ft.y + ft.z * ft.z;
     float cap = D.mu * fn;
-    if (ftm2 > cap * cap) {  // |F_t| > mu |F_n|, compared in squares
-        float sc = cap * rsqrtf(ftm2);
-        ft = make_float3(ft.x * sc, ft.y * sc, ft.z * sc);
-    }
-    h = make_float4(ft.x, ft.y, ft.z, 0.f);
+    // |F_t| > mu |F_n|, compared in squares
+    const float sc = ftm2 > cap * cap ? cap * rsqrtf(ftm2) : 1.0f;
+    // rounded products: with them, a force inside the cap and one on it take
+    // the same operations in the sums below
+    ft = make_float3(__fmul_rn(ft.x, sc), __fmul_rn(ft.y, sc), __fmul_rn(ft.z, sc));
     float3 Fk = make_float3(-fn * n.x + ft.x, -fn * n.y + ft.y, -fn * n.z + ft.z);
     float3 Tk = crossf(ri, Fk);
-    F.x += Fk.x;
-    F.y += Fk.y;
-    F.z += Fk.z;
-    T.x += Tk.x;
-    T.y += Tk.y;
-    T.z += Tk.z;
-}
-
-// Contact forces on sphere i from its neighbour list, positions and half-
-// step velocities of substep buffer b in global memory.  dt_inc = 0
-// evaluates without tangential increment.  Lane `tl` of the sphere's team
-// takes entries tl, tl + TEAM, ...; the caller reduces over the team.
-__device__ void contact_forces(const Dem& D, int i, int b, float dt_inc, int tl, float3& F, float3& T) {
-    F = make_float3(0.f, 0.f, 0.f);
-    T = make_float3(0.f, 0.f, 0.f);
-    float3 xi = f3(__ldcg(&D.dXb[b * D.n + i]));
-    float3 vi = f3(__ldcg(&D.Vhb[b * D.n + i])), wi = f3(__ldcg(&D.Whb[b * D.n + i]));
-    float Ri = D.R[i];
-    int cnt = D.nb_cnt[i];
-    for (int k = tl; k < cnt; k += TEAM) {
-        size_t e = (size_t)i * D.nbmax + k;
-        int j = D.nb_j[e];
-        float4 dr = D.nb_dref[e];
-        float3 xj = f3(__ldcg(&D.dXb[b * D.n + j]));
-        float3 vj = f3(__ldcg(&D.Vhb[b * D.n + j])), wj = f3(__ldcg(&D.Whb[b * D.n + j]));
-        float4 h = D.nb_ft[e];
-        pair_contact(D, Ri, D.R[j], make_float3(xj.x - xi.x, xj.y - xi.y, xj.z - xi.z), dr, vi, wi, vj, wj,
-                     dt_inc, h, F, T);
-        D.nb_ft[e] = h;
-    }
+    const float3 Fs = make_float3(F.x + Fk.x, F.y + Fk.y, F.z + Fk.z), Ts = make_float3(T.x + Tk.x, T.y + Tk.y, T.z + Tk.z);
+    h = touch ? ft : make_float3(0.f, 0.f, 0.f);
+    F = touch ? Fs : F;
+    T = touch ? Ts : T;
 }
 
 // First half kick of velocity Verlet and the drift of one substep:
 // half-step velocities vh, wh from the contact (fc, tc), hydrodynamic (fa,
 // ta) and body forces; the displacement dx advanced with Kahan-compensated
-// FP32 accumulation (compensation c); q <- normalize(q + dt/2 (0, wh) q).
+// FP32 accumulation (compensation c).
 __device__ __forceinline__ void kick_drift(const Dem& D, float3 fc, float3 tc, float3 fa, float3 ta, float im,
                                            float iI, float3 v, float3 w, float3& vh, float3& wh, float3& dx,
-                                           float3& c, float4& q) {
+                                           float3& c) {
     const float dt = D.dt;
     vh = make_float3(v.x + 0.5f * dt * (fc.x + fa.x + D.g.x) * im, v.y + 0.5f * dt * (fc.y + fa.y + D.g.y) * im,
                      v.z + 0.5f * dt * (fc.z + fa.z + D.g.z) * im);
@@ -144,6 +115,11 @@ __device__ __forceinline__ void kick_drift(const Dem& D, float3 fc, float3 tc, f
     float tx = dx.x + yx, ty = dx.y + yy, tz = dx.z + yz;
     c = make_float3((tx - dx.x) - yx, (ty - dx.y) - yy, (tz - dx.z) - yz);
     dx = make_float3(tx, ty, tz);
+}
+
+// Orientation over one substep: q <- normalize(q + dt/2 (0, wh) q).
+__device__ __forceinline__ void spin(const Dem& D, float3 wh, float4& q) {
+    const float dt = D.dt;
     float dq0 = -(wh.x * q.y + wh.y * q.z + wh.z * q.w);
     float3 wxv = crossf(wh, make_float3(q.y, q.z, q.w));
     float4 dq = make_float4(dq0, q.x * wh.x + wxv.x, q.x * wh.y + wxv.y, q.x * wh.z + wxv.z);
@@ -199,20 +175,19 @@ __device__ __forceinline__ void sphere_frame(const Dem& D, int i, float& dmax, f
     vmax = fmaxf(vmax, vv);
 }
 
-// The same outputs for the per-step kernel: the integer origins depend only
-// on Xref, which changes only at re-layouts (after which the general kernel
-// runs sphere_frame), so only the FP32 offset of the centre is renewed.
-// Lane `tl` < 3 of the sphere's team computes axis tl; lane 0 checks.
-__device__ __forceinline__ void sphere_offset(const Dem& D, int i, int tl, float& dmax, float& vmax, uint32_t& bad) {
+// The same outputs for the per-step kernels: the integer origins depend only
+// on Xref, which changes only at re-layouts (after which k_dem_init runs
+// sphere_frame), so only the FP32 offset of the centre is renewed, from the
+// state in registers (every lane of the team holds it).  Lane `tl` < 3 of the
+// sphere's team computes axis tl from its Xref and origin; lane 0 checks.
+__device__ __forceinline__ void sphere_offset(const Dem& D, int i, int tl, double Xref, int org, float3 dx, float3 c,
+                                              float3 v, float& dmax, float& vmax, uint32_t& bad) {
     if (tl < 3) {
-        const float* dx = reinterpret_cast<const float*>(&D.dX[i]);
-        const float* c = reinterpret_cast<const float*>(&D.dXc[i]);
-        const int* o = reinterpret_cast<const int*>(&D.org[i]);
-        double X = D.Xref[3 * i + tl] + (double)dx[tl] - (double)c[tl];
-        reinterpret_cast<float*>(&D.xf[i])[tl] = (float)(X - o[tl]);
+        const float d = tl == 0 ? dx.x : tl == 1 ? dx.y : dx.z, k = tl == 0 ? c.x : tl == 1 ? c.y : c.z;
+        double X = Xref + (double)d - (double)k;
+        reinterpret_cast<float*>(&D.xf[i])[tl] = (float)(X - org);
     }
     if (tl == 0) {
-        float4 dx = D.dX[i], v = D.V[i];
         float dd = sqrtf(dx.x * dx.x + dx.y * dx.y + dx.z * dx.z);
         float vv = sqrtf(v.x * v.x + v.y * v.y + v.z * v.z);
         if (!(dd == dd) || !(vv == vv) || isinf(dd) || isinf(vv)) bad |= ST_UNSTABLE;
@@ -242,144 +217,151 @@ __device__ __forceinline__ void flush_maxima(const Dem& D, float dmax, float vma
     }
 }
 
-__global__ void k_dem_step(Dem D, int init_only) {
-    cg::cluster_group cl = cg::this_cluster();
-    const int nth = gridDim.x * blockDim.x;
-    const int tid = blockIdx.x * blockDim.x + threadIdx.x;
-    const int team = tid / TEAM, tl = tid % TEAM, nteams = nth / TEAM;
-    const int iters = (D.n + nteams - 1) / nteams;  // uniform: shuffles stay converged
-    if (!init_only && tid == 0) *D.layout_fresh = 0u;  // this step's map update is done
-    if (init_only) {
-        for (int i = tid; i < D.n; i += nth) {
-            D.dXb[i] = D.dX[i];
-            D.Vhb[i] = D.V[i];
-            D.Whb[i] = D.W[i];
+// Hydrodynamic drive of sphere i: the mean of this and the previous step's
+// exchange sums.  Lane tl < 3 of the team takes component tl of both (FP64 adds
+// run at 2 lanes per clock and SM), then the team shares them.  Every lane
+// of the warp calls it; `lead` is the lane of the team's first thread.
+__device__ __forceinline__ void hydro_drive(const Dem& D, int i, int tl, bool have, int lead, float3& fa, float3& ta) {
+    const unsigned full = 0xffffffffu;
+    float hf = 0.f, ht = 0.f;
+    if (have && tl < 3) {
+        double f = D.Fh[3 * (size_t)i + tl], t = D.Th[3 * (size_t)i + tl];
+#pragma unroll
+        for (int r = 1; r < NREP; ++r) {
+            f += D.Fh[3 * ((size_t)r * D.n + i) + tl];
+            t += D.Th[3 * ((size_t)r * D.n + i) + tl];
         }
-        cl.sync();
-        for (int it = 0; it < iters; ++it) {
-            int i = team + it * nteams;
-            float3 F = make_float3(0.f, 0.f, 0.f), T = F;
-            if (i < D.n) contact_forces(D, i, 0, 0.f, tl, F, T);
-            team_sum(F, T);
-            if (i < D.n && tl == 0) {
-                D.Fc[i] = make_float4(F.x, F.y, F.z, 0.f);
-                D.Tc[i] = make_float4(T.x, T.y, T.z, 0.f);
-            }
-        }
-    } else {
-        for (int it = 0; it < iters; ++it) {
-            int i = team + it * nteams;
-            if (i >= D.n || tl != 0) continue;
-            double f[3] = {0.0, 0.0, 0.0}, t[3] = {0.0, 0.0, 0.0};
-            for (int r = 0; r < NREP; ++r)
-                for (int a = 0; a < 3; ++a) {
-                    f[a] += D.Fh[3 * ((size_t)r * D.n + i) + a];
-                    t[a] += D.Th[3 * ((size_t)r * D.n + i) + a];
-                }
-            D.Fa[i] = make_float4((float)(0.5 * (f[0] + D.Fh_prev[3 * i])), (float)(0.5 * (f[1] + D.Fh_prev[3 * i + 1])),
-                                  (float)(0.5 * (f[2] + D.Fh_prev[3 * i + 2])), 0.f);
-            D.Ta[i] = make_float4((float)(0.5 * (t[0] + D.Th_prev[3 * i])), (float)(0.5 * (t[1] + D.Th_prev[3 * i + 1])),
-                                  (float)(0.5 * (t[2] + D.Th_prev[3 * i + 2])), 0.f);
-            for (int a = 0; a < 3; ++a) {
-                D.Fh_prev[3 * i + a] = f[a];
-                D.Th_prev[3 * i + a] = t[a];
-            }
-        }
+        hf = 0.5f * (float)(f + D.Fh_prev[3 * (size_t)i + tl]);
+        ht = 0.5f * (float)(t + D.Th_prev[3 * (size_t)i + tl]);
+        D.Fh_prev[3 * (size_t)i + tl] = f;
+        D.Th_prev[3 * (size_t)i + tl] = t;
     }
-    for (int s = 0; s < (init_only ? 0 : D.K); ++s) {
-        const int b = s & 1;
-        // kick + drift of the own spheres (lane 0 of each sphere's team owns
-        // every per-sphere update, so no barrier is needed between substeps)
-        for (int it = 0; it < iters; ++it) {
-            int i = team + it * nteams;
-            if (i >= D.n || tl != 0) continue;
-            float4 dx = D.dX[i];
-            float4 vh, wh;
-            if (D.fixed[i]) {
-                vh = wh = make_float4(0.f, 0.f, 0.f, 0.f);
-            } else {
-                float3 v = f3(D.V[i]), w = f3(D.W[i]), dxx = f3(dx), c = f3(D.dXc[i]);
-                float4 q = D.q[i];
-                float3 vh3, wh3;
-                kick_drift(D, f3(D.Fc[i]), f3(D.Tc[i]), f3(D.Fa[i]), f3(D.Ta[i]), D.invm[i], D.invI[i], v, w, vh3,
-                           wh3, dxx, c, q);
-                vh = make_float4(vh3.x, vh3.y, vh3.z, 0.f);
-                wh = make_float4(wh3.x, wh3.y, wh3.z, 0.f);
-                dx = make_float4(dxx.x, dxx.y, dxx.z, 0.f);
-                D.dX[i] = dx;
-                D.dXc[i] = make_float4(c.x, c.y, c.z, 0.f);
-                D.q[i] = q;
-            }
-            D.dXb[b * D.n + i] = dx;
-            D.Vhb[b * D.n + i] = vh;
-            D.Whb[b * D.n + i] = wh;
-        }
-        cl.sync();
-        // contact forces (a team per sphere) and the closing kick
-        for (int it = 0; it < iters; ++it) {
-            int i = team + it * nteams;
-            bool act = i < D.n && !D.fixed[i];
-            float3 F = make_float3(0.f, 0.f, 0.f), T = F;
-            if (act) contact_forces(D, i, b, D.dt, tl, F, T);
-            team_sum(F, T);
-            if (i < D.n && tl == 0) {
-                if (!act) {
-                    D.V[i] = D.W[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-                    continue;
-                }
-                D.Fc[i] = make_float4(F.x, F.y, F.z, 0.f);
-                D.Tc[i] = make_float4(T.x, T.y, T.z, 0.f);
-                float3 v, w;
-                close_kick(D, f3(D.Vhb[b * D.n + i]), f3(D.Whb[b * D.n + i]), F, T, f3(D.Fa[i]), f3(D.Ta[i]),
-                           D.invm[i], D.invI[i], v, w);
-                D.V[i] = make_float4(v.x, v.y, v.z, 0.f);
-                D.W[i] = make_float4(w.x, w.y, w.z, 0.f);
-            }
-        }
-    }
-    // outputs of the step: lattice frame of every sphere, displacement and
-    // speed maxima for the re-layout decision, NaN / skin checks
-    float dmax = 0.f, vmax = 0.f;
-    uint32_t bad = 0;
-    for (int it = 0; it < iters; ++it) {
-        int i = team + it * nteams;
-        if (i >= D.n || tl != 0) continue;
-        sphere_frame(D, i, dmax, vmax, bad);
-    }
-    flush_maxima(D, dmax, vmax, bad);
-    cl.sync();
+    fa = make_float3(__shfl_sync(full, hf, lead), __shfl_sync(full, hf, lead + 1), __shfl_sync(full, hf, lead + 2));
+    ta = make_float3(__shfl_sync(full, ht, lead), __shfl_sync(full, ht, lead + 1), __shfl_sync(full, ht, lead + 2));
 }
 
-// The same K substeps with every sphere's state in registers of its team and
-// the per-substep exchange (displacement and half-step velocities) in the
-// distributed shared memory of the cluster: one cluster of up to 16 CTAs of
-// DSM_THREADS threads, spc = blockDim / TEAM spheres per CTA, sphere j in CTA
-// j / spc.  The first NBT neighbour entries of each team lane live in
-// registers (with their tangential history) for the whole launch; further
-// entries go through global memory.  Used when every sphere has a team.
-constexpr int DSM_THREADS = 512;
-constexpr int NBT = 3;
+// ------------------------------------------------------------ one launch
 
-__global__ void __launch_bounds__(DSM_THREADS, 1) k_dem_step_dsm(Dem D) {
-    extern __shared__ float4 xchg[];  // [2 substep parities][3: dX, Vh, Wh][spc]
-    // Launched with a programmatic dependency on the link kernel: the
+// The K substeps with every sphere's state in registers of its team.  One
+// cluster of C CTAs, spc = blockDim / TEAM spheres per CTA, sphere i in CTA
+// i / spc.  Each CTA's shared memory holds the exchanged record of its own
+// spheres (slots 0 .. spc - 1) and of the spheres of other CTAs that its own
+// neighbour lists name (slots from spc on, assigned by k_dem_ghosts); a sphere
+// pushes its record into every CTA that holds it, and all reads of a substep
+// are local.  Reading the neighbours through the cluster window instead
+// carries each record once per contact, and that window moves about 18 B per
+// clock and SM.  The pushes complete a transaction barrier of the receiving
+// CTA, which waits for the bytes of all its foreign records; nothing else
+// crosses CTAs (a cluster barrier that releases costs 380 to 480 cycles, more
+// with remote stores in flight).  The own spheres' records are ordered by
+// __syncthreads (30 to 45 cycles).  Three record buffers: a CTA pushes substep
+// s + 3 after it has received s + 2 from the CTAs it pushes to (neighbourhood
+// is mutual), which they sent after their __syncthreads of s + 1, so all their
+// threads are through with substep s.
+// 2048 spheres, K = 10: 29 us per step with reads through the cluster window
+// and cluster barriers, @@ us; one CTA of 32 spheres 19 us, @@ us.
+// The first NBT neighbour entries of each team lane live in registers (with
+// their tangential history) for the whole launch; further entries go through
+// global memory.
+constexpr int DSM_THREADS = 512;
+constexpr int DSM_SOLO = 256;  // largest launch of one CTA (twice the registers per thread)
+constexpr int DSM_BUFS = 3;
+constexpr int NBT = 3;
+static_assert(DEM_MAX_CTAS % TEAM == 0, "push targets are split over a team's lanes");
+
+__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ uint32_t cluster_addr(uint32_t a, uint32_t rank) {
+    uint32_t r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(rank));
+    return r;
+}
+// stores into another CTA's shared memory that count on its barrier
+__device__ __forceinline__ void push4(uint32_t a, float4 v, uint32_t bar) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(a),
+                 "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "r"(bar)
+                 : "memory");
+}
+__device__ __forceinline__ void push1(uint32_t a, float v, uint32_t bar) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.f32 [%0], %1, [%2];" ::"r"(a), "f"(v), "r"(bar)
+                 : "memory");
+}
+__device__ __forceinline__ bool bar_done(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{ .reg .pred p; mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2; selp.u32 %0, 1, 0, p; }"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0u;
+}
+// tries before a wait gives up (each suspends for up to some microseconds):
+// the status latches a timeout and the step ends with what it has
+constexpr int DSM_TRIES = 1 << 16;
+constexpr uint32_t RECORD_BYTES = 36;
+
+// The lane's register entries 0 .. U - 1 (warp-uniform U).
+template <int U, class Contact>
+__device__ __forceinline__ void contacts_n(Contact contact) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) contact(u);
+}
+
+template <bool MULTI>
+__global__ void __launch_bounds__(MULTI ? DSM_THREADS : DSM_SOLO, 1) k_dem_step_dsm(Dem D) {
+    // exchanged records, [DSM_BUFS][slots]: {dX, Vh.x}, {Vh.yz, Wh.xy}, Wh.z
+    extern __shared__ float4 smem[];
+    __shared__ __align__(8) unsigned long long bars[DSM_BUFS];
+    float4* xa = smem;
+    float4* xb = smem + DSM_BUFS * D.slots;
+    float* xc = reinterpret_cast<float*>(smem + 2 * DSM_BUFS * D.slots);
+    // Launched with a programmatic dependency on the previous kernel: the
     // sphere state and neighbour entries (last written by the previous
     // step's DEM, long complete) are read before waiting for it; the
     // exchange sums it writes, and every write of this kernel, come after.
-    cg::cluster_group cl = cg::this_cluster();
+    // All loads of the state are independent of one another.  With the fluid
+    // off the previous kernel is the previous step's DEM itself.
+    if (D.dry) pdl_wait();
+    const unsigned full = 0xffffffffu;
     const int spc = blockDim.x / TEAM;
     const int tl = threadIdx.x % TEAM, ls = threadIdx.x / TEAM;
     const int i = blockIdx.x * spc + ls;
     const bool have = i < D.n;
-    const unsigned full = 0xffffffffu;
     const int lead = (threadIdx.x & 31) & ~(TEAM - 1);  // lane of the team's first thread
     const float3 zero = make_float3(0.f, 0.f, 0.f);
     float3 dx = zero, dxc = zero, v = zero, w = zero, fc = zero, tc = zero;
     float4 q = make_float4(1.f, 0.f, 0.f, 0.f);
+    double Xr = 0.0;
+    int org = 0;
     float im = 0.f, iI = 0.f, Ri = 1.f;
     bool fixed = true;
     int cnt = 0;
+    // slots of this sphere in the CTAs tl, tl + TEAM, ... (16 bits each)
+    uint32_t push[DEM_MAX_CTAS / TEAM / 2];
+#pragma unroll
+    for (int d = 0; d < DEM_MAX_CTAS / TEAM / 2; ++d) push[d] = 0xffffffffu;
+    // this lane's neighbour entries tl + u TEAM, u < NBT: slot, radius,
+    // reference separation (w < 0: unused) and history
+    int nj[NBT];
+    float nR[NBT], nRs[NBT];
+    float4 ndr[NBT];
+    float3 nh[NBT];
+#pragma unroll
+    for (int u = 0; u < NBT; ++u) {
+        nj[u] = 0;
+        nR[u] = 1.f;
+        ndr[u] = make_float4(0.f, 0.f, 0.f, -1.f);
+        nh[u] = zero;
+    }
     if (have) {
+        cnt = D.nb_cnt[i];
+#pragma unroll
+        for (int u = 0; u < NBT; ++u) {  // every list holds more than NBT TEAM entries, used or not
+            const size_t e = (size_t)i * D.nbmax + tl + u * TEAM;
+            nj[u] = D.nb_slot[e];
+            nR[u] = D.nb_R[e];
+            ndr[u] = D.nb_dref[e];
+            nh[u] = f3(D.nb_ft[e]);
+        }
         dx = f3(D.dX[i]);
         dxc = f3(D.dXc[i]);
         v = f3(D.V[i]);
@@ -391,86 +373,103 @@ __global__ void __launch_bounds__(DSM_THREADS, 1) k_dem_step_dsm(Dem D) {
         iI = D.invI[i];
         Ri = D.R[i];
         fixed = D.fixed[i] != 0;
-        cnt = D.nb_cnt[i];
+        if (tl < 3) {
+            Xr = D.Xref[3 * i + tl];
+            org = reinterpret_cast<const int*>(&D.org[i])[tl];
+        }
+        if (MULTI) {
+#pragma unroll
+            for (int d = 0; d < DEM_MAX_CTAS / TEAM; d += 2) {
+                const uint32_t lo = D.push[(size_t)i * DEM_MAX_CTAS + tl + d * TEAM],
+                               hi = D.push[(size_t)i * DEM_MAX_CTAS + tl + (d + 1) * TEAM];
+                push[d / 2] = lo | (hi << 16);
+            }
+        }
     }
-    // this lane's neighbour entries tl + u TEAM, u < NBT; the neighbour's CTA
-    // rank and slot are packed as (rank << 16) | slot once, so the substeps
-    // need no division by the spheres per CTA
-    int nj[NBT];
-    float4 ndr[NBT];
-    float3 nh[NBT];
 #pragma unroll
     for (int u = 0; u < NBT; ++u) {
-        int k = tl + u * TEAM;
-        nj[u] = -1;
-        if (k < cnt) {
-            size_t e = (size_t)i * D.nbmax + k;
-            const int j = D.nb_j[e], rk = j / spc;
-            nj[u] = (rk << 16) | (j - rk * spc);
-            ndr[u] = D.nb_dref[e];
-            nh[u] = f3(D.nb_ft[e]);
+        if (tl + u * TEAM >= cnt || fixed) {
+            nj[u] = 0;
+            nR[u] = 1.f;
+            ndr[u] = make_float4(0.f, 0.f, 0.f, -1.f);
+            nh[u] = zero;
         }
+        nRs[u] = reduced_radius(Ri, nR[u]);
+    }
+    const int used = fixed ? 0 : min((cnt - tl + TEAM - 1) / TEAM, NBT);
+    const int most = __reduce_max_sync(full, used > 0 ? used : 0);
+    uint32_t foreign = 0;  // bytes this CTA receives per substep
+    if (MULTI) {  // the barriers exist before a record is pushed at them
+        if (threadIdx.x == 0) {
+            for (int k = 0; k < DSM_BUFS; ++k)
+                asm volatile("mbarrier.init.shared.b64 [%0], 1;" ::"r"(smem_addr(&bars[k])) : "memory");
+            asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        }
+        foreign = RECORD_BYTES * (uint32_t)D.foreign[blockIdx.x];
+        asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
     }
     pdl_wait();
+    pdl_trigger();
     if (blockIdx.x == 0 && threadIdx.x == 0) *D.layout_fresh = 0u;  // this step's map update is done
-    // hydrodynamic drive: the mean of this and the previous step's exchange
-    // sums.  The FP64 replica sums are split over the team: lane tl < 3
-    // sums force and torque component tl (same operations and order as one
-    // lane would), then the team shares them.
-    float hf = 0.f, ht = 0.f;
-    if (have && tl < 3) {
-        double f = 0.0, t = 0.0;
-        for (int r = 0; r < NREP; ++r) {
-            f += D.Fh[3 * ((size_t)r * D.n + i) + tl];
-            t += D.Th[3 * ((size_t)r * D.n + i) + tl];
-        }
-        hf = (float)(0.5 * (f + D.Fh_prev[3 * i + tl]));
-        ht = (float)(0.5 * (t + D.Th_prev[3 * i + tl]));
-        D.Fh_prev[3 * i + tl] = f;
-        D.Th_prev[3 * i + tl] = t;
-        reinterpret_cast<float*>(&D.Fa[i])[tl] = hf;
-        reinterpret_cast<float*>(&D.Ta[i])[tl] = ht;
-    }
-    const float3 fa = make_float3(__shfl_sync(full, hf, lead), __shfl_sync(full, hf, lead + 1),
-                                  __shfl_sync(full, hf, lead + 2));
-    const float3 ta = make_float3(__shfl_sync(full, ht, lead), __shfl_sync(full, ht, lead + 1),
-                                  __shfl_sync(full, ht, lead + 2));
+    float3 fa, ta;
+    hydro_drive(D, i, tl, have, lead, fa, ta);
+    float dmax = 0.f, vmax = 0.f;
+    uint32_t bad = 0;
     for (int s = 0; s < D.K; ++s) {
-        const int b = s & 1;
+        const int buf = s % DSM_BUFS, b = buf * D.slots;
         float3 vh = zero, wh = zero;
-        if (!fixed) kick_drift(D, fc, tc, fa, ta, im, iI, v, w, vh, wh, dx, dxc, q);
-        if (have && tl == 0) {
-            xchg[(b * 3 + 0) * spc + ls] = make_float4(dx.x, dx.y, dx.z, 0.f);
-            xchg[(b * 3 + 1) * spc + ls] = make_float4(vh.x, vh.y, vh.z, 0.f);
-            xchg[(b * 3 + 2) * spc + ls] = make_float4(wh.x, wh.y, wh.z, 0.f);
-        }
-        cl.sync();
-        float3 F = zero, T = zero;
-        if (have && !fixed) {
+        if (!fixed) kick_drift(D, fc, tc, fa, ta, im, iI, v, w, vh, wh, dx, dxc);
+        const float4 ra = make_float4(dx.x, dx.y, dx.z, vh.x), rb = make_float4(vh.y, vh.z, wh.x, wh.y);
+        if (MULTI) {
+            const uint32_t bar = smem_addr(&bars[buf]);
+            if (threadIdx.x == 0)
+                asm volatile("mbarrier.arrive.expect_tx.shared.b64 _, [%0], %1;" ::"r"(bar), "r"(foreign) : "memory");
 #pragma unroll
-            for (int u = 0; u < NBT; ++u) {
-                if (nj[u] < 0) continue;
-                const int rk = nj[u] >> 16, lj = nj[u] & 0xffff;
-                const float4* rx = cl.map_shared_rank(xchg, rk);
-                float4 xj = rx[(b * 3 + 0) * spc + lj], vj = rx[(b * 3 + 1) * spc + lj],
-                       wj = rx[(b * 3 + 2) * spc + lj];
-                float4 h = make_float4(nh[u].x, nh[u].y, nh[u].z, 0.f);
-                pair_contact(D, Ri, __ldg(&D.R[rk * spc + lj]), make_float3(xj.x - dx.x, xj.y - dx.y, xj.z - dx.z), ndr[u],
-                             vh, wh, f3(vj), f3(wj), D.dt, h, F, T);
-                nh[u] = f3(h);
-            }
-            for (int k = tl + NBT * TEAM; k < cnt; k += TEAM) {  // entries beyond the registers
-                size_t e = (size_t)i * D.nbmax + k;
-                int j = D.nb_j[e];
-                int rk = j / spc, lj = j - rk * spc;
-                const float4* rx = cl.map_shared_rank(xchg, rk);
-                float4 h = D.nb_ft[e];
-                float4 xjj = rx[(b * 3 + 0) * spc + lj];
-                pair_contact(D, Ri, D.R[j], make_float3(xjj.x - dx.x, xjj.y - dx.y, xjj.z - dx.z), D.nb_dref[e], vh,
-                             wh, f3(rx[(b * 3 + 1) * spc + lj]), f3(rx[(b * 3 + 2) * spc + lj]), D.dt, h, F, T);
-                D.nb_ft[e] = h;
+            for (int d = 0; d < DEM_MAX_CTAS / TEAM; ++d) {
+                const uint32_t slot = (push[d / 2] >> (16 * (d & 1))) & 0xffffu;
+                if (slot == 0xffffu) continue;
+                const uint32_t rank = tl + d * TEAM, rbar = cluster_addr(bar, rank);
+                push4(cluster_addr(smem_addr(&xa[b + slot]), rank), ra, rbar);
+                push4(cluster_addr(smem_addr(&xb[b + slot]), rank), rb, rbar);
+                push1(cluster_addr(smem_addr(&xc[b + slot]), rank), wh.z, rbar);
             }
         }
+        if (have) {
+            if (tl == 0) xa[b + ls] = ra;
+            if (tl == 1) xb[b + ls] = rb;
+            if (tl == 2) xc[b + ls] = wh.z;
+        }
+        if (!fixed) spin(D, wh, q);
+        __syncthreads();
+        if (MULTI) {
+            const uint32_t bar = smem_addr(&bars[buf]), parity = (uint32_t)(s / DSM_BUFS) & 1u;
+            int tries = 0;
+            while (!bar_done(bar, parity))
+                if (++tries > DSM_TRIES) {
+                    bad |= ST_TIMEOUT;
+                    break;
+                }
+        }
+        float3 F = zero, T = zero;
+        auto contact = [&](int slot, float Rj, float Rs, float4 dr, float3& h) {
+            const float4 a = xa[b + slot], c = xb[b + slot];
+            const float wz = xc[b + slot];
+            pair_contact(D, Ri, Rj, Rs, make_float3(a.x - dx.x, a.y - dx.y, a.z - dx.z), dr, vh, wh,
+                         make_float3(a.w, c.x, c.y), make_float3(c.z, c.w, wz), D.dt, h, F, T);
+        };
+        auto entry = [&](int u) { contact(nj[u], nR[u], nRs[u], ndr[u], nh[u]); };
+        if (most == 3) contacts_n<3>(entry);
+        else if (most == 2) contacts_n<2>(entry);
+        else if (most == 1) contacts_n<1>(entry);
+        if (!fixed)
+            for (int k = tl + NBT * TEAM; k < cnt; k += TEAM) {  // entries beyond the registers
+                const size_t e = (size_t)i * D.nbmax + k;
+                float3 h = f3(D.nb_ft[e]);
+                contact(D.nb_slot[e], D.nb_R[e], reduced_radius(Ri, D.nb_R[e]), D.nb_dref[e], h);
+                D.nb_ft[e] = make_float4(h.x, h.y, h.z, 0.f);
+            }
+        __syncwarp();
         team_sum(F, T);
         if (fixed) {
             v = w = zero;
@@ -480,47 +479,282 @@ __global__ void __launch_bounds__(DSM_THREADS, 1) k_dem_step_dsm(Dem D) {
             close_kick(D, vh, wh, F, T, fa, ta, im, iI, v, w);
         }
     }
-    cl.sync();  // no CTA leaves while another may still read its shared memory
     if (have) {
 #pragma unroll
         for (int u = 0; u < NBT; ++u)
-            if (nj[u] >= 0) D.nb_ft[(size_t)i * D.nbmax + tl + u * TEAM] = make_float4(nh[u].x, nh[u].y, nh[u].z, 0.f);
+            if (u < used) D.nb_ft[(size_t)i * D.nbmax + tl + u * TEAM] = make_float4(nh[u].x, nh[u].y, nh[u].z, 0.f);
         if (tl == 0) {
             D.dX[i] = make_float4(dx.x, dx.y, dx.z, 0.f);
             D.dXc[i] = make_float4(dxc.x, dxc.y, dxc.z, 0.f);
+        } else if (tl == 1) {
             D.V[i] = make_float4(v.x, v.y, v.z, 0.f);
             D.W[i] = make_float4(w.x, w.y, w.z, 0.f);
+        } else if (tl == 2) {
             D.q[i] = q;
+        } else {
             D.Fc[i] = make_float4(fc.x, fc.y, fc.z, 0.f);
             D.Tc[i] = make_float4(tc.x, tc.y, tc.z, 0.f);
         }
+        sphere_offset(D, i, tl, Xr, org, dx, dxc, v, dmax, vmax, bad);
     }
+    flush_maxima(D, dmax, vmax, bad);
+    if (MULTI) {  // no CTA leaves while another may still push into it (after a wait that gave up)
+        asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+        asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    }
+}
+
+// Slots of the exchange for k_dem_step_dsm, one block per CTA of that launch
+// (shared memory: a flag per sphere): the spheres of other CTAs that are
+// neighbours of this CTA's spheres get the slots from spc on in index order,
+// each entry its neighbour's slot, each named sphere its slot in this CTA
+// (push, 0xffff elsewhere).  foreign[c] receives the number of those spheres,
+// *slots the largest slot count.
+__global__ void k_dem_ghosts(Dem D, int spc, int* nb_slot, uint16_t* push, int* foreign, int* slots) {
+    extern __shared__ uint8_t need[];
+    __shared__ uint32_t part[33];
+    const int c = blockIdx.x, i0 = c * spc, i1 = min(i0 + spc, D.n);
+    for (int j = threadIdx.x; j < D.n; j += blockDim.x) need[j] = 0;
+    __syncthreads();
+    for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x)
+        for (int k = 0; k < D.nb_cnt[i]; ++k) {
+            const int j = D.nb_j[(size_t)i * D.nbmax + k];
+            if (j < i0 || j >= i1) need[j] = 1;
+        }
+    // and those whose lists name this CTA's spheres: at a distance that rounds
+    // to the edge of the skin only one of a pair may list the other, and the
+    // record buffers count on pushes going both ways between two CTAs
+    for (int j = threadIdx.x; j < D.n; j += blockDim.x) {
+        if (j >= i0 && j < i1) continue;
+        for (int k = 0; k < D.nb_cnt[j]; ++k) {
+            const int i = D.nb_j[(size_t)j * D.nbmax + k];
+            if (i >= i0 && i < i1) need[j] = 1;
+        }
+    }
+    __syncthreads();
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    int base = spc;
+    for (int j0 = 0; j0 < D.n; j0 += blockDim.x) {
+        const int j = j0 + threadIdx.x;
+        const bool g = j < D.n && need[j];
+        const unsigned bal = __ballot_sync(0xffffffffu, g);
+        if (lane == 0) part[wid] = __popc(bal);
+        __syncthreads();
+        int at = base + __popc(bal & ((1u << lane) - 1u));
+        for (int k = 0; k < nw; ++k) {
+            if (k < wid) at += part[k];
+            base += part[k];
+        }
+        if (j < D.n) push[(size_t)j * DEM_MAX_CTAS + c] = g ? (uint16_t)at : (uint16_t)0xffffu;
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) {
+        foreign[c] = base - spc;
+        atomicMax(slots, base);
+    }
+    for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x)
+        for (int k = 0; k < D.nb_cnt[i]; ++k) {
+            const size_t e = (size_t)i * D.nbmax + k;
+            const int j = D.nb_j[e];
+            nb_slot[e] = j >= i0 && j < i1 ? j - i0 : (int)push[(size_t)j * DEM_MAX_CTAS + c];
+        }
+}
+
+// ------------------------------------------------------------ one launch per substep
+
+// Larger packings: k_dem_begin takes the hydrodynamic drive, the first half
+// kick and the drift; k_dem_substep evaluates the contacts of substep s and
+// closes it, then opens substep s + 1 or, after the last, writes the step's
+// outputs.  Chained by programmatic dependent launch, one team per sphere over
+// the whole GPU; the records are exchanged through the L2.  About 2 us per
+// substep whatever the count (launch hand-over and one round of loads),
+// against 18 us for one cluster of 8 CTAs taking several spheres per team with
+// the state in global memory (4096 spheres, K = 10: 180 -> @@ us per step).
+constexpr int SUB_THREADS = 128;
+
+// q: the lane TEAM - 1 carries the orientation
+__device__ __forceinline__ void open_substep(const Dem& D, int i, int tl, int b, float3 dx, float3 c, float4 q,
+                                             float3 fc, float3 tc, float3 fa, float3 ta, float3 v, float3 w,
+                                             bool fixed, float im, float iI) {
+    float3 vh = make_float3(0.f, 0.f, 0.f), wh = vh;
+    if (!fixed) kick_drift(D, fc, tc, fa, ta, im, iI, v, w, vh, wh, dx, c);
+    if (tl == 0) {
+        D.dX[i] = make_float4(dx.x, dx.y, dx.z, 0.f);
+        D.dXb[b * D.n + i] = make_float4(dx.x, dx.y, dx.z, vh.x);
+    } else if (tl == 1) {
+        D.dXc[i] = make_float4(c.x, c.y, c.z, 0.f);
+        D.Vhb[b * D.n + i] = make_float4(vh.y, vh.z, wh.x, wh.y);
+    } else if (tl == 2) {
+        D.Whb[b * D.n + i] = make_float4(wh.z, 0.f, 0.f, 0.f);
+    } else if (!fixed) {
+        spin(D, wh, q);
+        D.q[i] = q;
+    }
+}
+static_assert(TEAM == 4, "open_substep splits its stores over four lanes");
+
+__global__ void __launch_bounds__(SUB_THREADS) k_dem_begin(Dem D) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x, tl = t % TEAM, i = t / TEAM;
+    const bool have = i < D.n;
+    pdl_wait();
+    pdl_trigger();
+    if (t == 0) *D.layout_fresh = 0u;  // this step's map update is done
+    float3 fa, ta;
+    hydro_drive(D, i, tl, have, (threadIdx.x & 31) & ~(TEAM - 1), fa, ta);
+    if (!have) return;
+    if (tl == 0) D.Fa[i] = make_float4(fa.x, fa.y, fa.z, 0.f);
+    if (tl == 1) D.Ta[i] = make_float4(ta.x, ta.y, ta.z, 0.f);
+    open_substep(D, i, tl, 0, f3(D.dX[i]), f3(D.dXc[i]), D.q[i], f3(D.Fc[i]), f3(D.Tc[i]), fa, ta, f3(D.V[i]), f3(D.W[i]), D.fixed[i] != 0, D.invm[i],
+                 D.invI[i]);
+}
+
+__global__ void __launch_bounds__(SUB_THREADS) k_dem_substep(Dem D, int s) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x, tl = t % TEAM, i = t / TEAM;
+    const bool have = i < D.n;
+    const int b = s & 1;
+    // the lists and constants change only at re-layouts: read ahead of the wait
+    int cnt = 0;
+    bool fixed = true;
+    float Ri = 1.f, im = 0.f, iI = 0.f;
+    int nj[NBT];
+    float nR[NBT];
+    float4 ndr[NBT];
+    if (have) {
+        fixed = D.fixed[i] != 0;
+        cnt = fixed ? 0 : D.nb_cnt[i];
+        Ri = D.R[i];
+        im = D.invm[i];
+        iI = D.invI[i];
+    }
+#pragma unroll
+    for (int u = 0; u < NBT; ++u) {
+        const int k = tl + u * TEAM;
+        nj[u] = -1;
+        if (k < cnt) {
+            const size_t e = (size_t)i * D.nbmax + k;
+            nj[u] = D.nb_j[e];
+            nR[u] = D.nb_R[e];
+            ndr[u] = D.nb_dref[e];
+        }
+    }
+    const double Xr = have && tl < 3 ? D.Xref[3 * i + tl] : 0.0;
+    const int org = have && tl < 3 ? reinterpret_cast<const int*>(&D.org[i])[tl] : 0;
+    pdl_wait();
+    pdl_trigger();
+    const float3 zero = make_float3(0.f, 0.f, 0.f);
+    float3 F = zero, T = zero, dx = zero, vh = zero, wh = zero, c = zero, fa = zero, ta = zero;
+    float4 q = make_float4(1.f, 0.f, 0.f, 0.f);
+    // every load of the substep is issued before any is used
+    float4 xa[NBT], xb[NBT], nh[NBT];
+    float xc[NBT];
+    if (have) {
+        const float4 a = D.dXb[b * D.n + i], e = D.Vhb[b * D.n + i];
+        const float z = D.Whb[b * D.n + i].x;
+#pragma unroll
+        for (int u = 0; u < NBT; ++u) {
+            if (tl + u * TEAM >= cnt) continue;
+            xa[u] = D.dXb[b * D.n + nj[u]];
+            xb[u] = D.Vhb[b * D.n + nj[u]];
+            xc[u] = D.Whb[b * D.n + nj[u]].x;
+            nh[u] = D.nb_ft[(size_t)i * D.nbmax + tl + u * TEAM];
+        }
+        c = f3(D.dXc[i]);
+        fa = f3(D.Fa[i]);
+        ta = f3(D.Ta[i]);
+        if (tl == TEAM - 1) q = D.q[i];
+        dx = f3(a);
+        vh = make_float3(a.w, e.x, e.y);
+        wh = make_float3(e.z, e.w, z);
+    }
+    auto contact = [&](int k, float4 a, float4 e, float z, float3 h, float Rj, float4 dr) {
+        pair_contact(D, Ri, Rj, reduced_radius(Ri, Rj), make_float3(a.x - dx.x, a.y - dx.y, a.z - dx.z), dr, vh, wh,
+                     make_float3(a.w, e.x, e.y), make_float3(e.z, e.w, z), D.dt, h, F, T);
+        D.nb_ft[(size_t)i * D.nbmax + k] = make_float4(h.x, h.y, h.z, 0.f);
+    };
+#pragma unroll
+    for (int u = 0; u < NBT; ++u)
+        if (tl + u * TEAM < cnt) contact(tl + u * TEAM, xa[u], xb[u], xc[u], f3(nh[u]), nR[u], ndr[u]);
+    for (int k = tl + NBT * TEAM; k < cnt; k += TEAM) {
+        const size_t e = (size_t)i * D.nbmax + k;
+        const size_t j = b * (size_t)D.n + D.nb_j[e];
+        contact(k, D.dXb[j], D.Vhb[j], D.Whb[j].x, f3(D.nb_ft[e]), D.nb_R[e], D.nb_dref[e]);
+    }
+    __syncwarp();
+    team_sum(F, T);
     float dmax = 0.f, vmax = 0.f;
     uint32_t bad = 0;
-    __syncwarp();
-    if (have) sphere_offset(D, i, tl, dmax, vmax, bad);
+    if (have) {
+        float3 v = zero, w = zero;
+        if (!fixed) close_kick(D, vh, wh, F, T, fa, ta, im, iI, v, w);
+        if (s + 1 < D.K) {
+            open_substep(D, i, tl, b ^ 1, dx, c, q, F, T, fa, ta, v, w, fixed, im, iI);
+        } else {
+            if (tl == 0) D.V[i] = make_float4(v.x, v.y, v.z, 0.f);
+            if (tl == 1) D.W[i] = make_float4(w.x, w.y, w.z, 0.f);
+            if (tl == 2 && !fixed) D.Fc[i] = make_float4(F.x, F.y, F.z, 0.f);
+            if (tl == 3 && !fixed) D.Tc[i] = make_float4(T.x, T.y, T.z, 0.f);
+            sphere_offset(D, i, tl, Xr, org, dx, c, v, dmax, vmax, bad);
+        }
+    }
+    if (s + 1 == D.K) flush_maxima(D, dmax, vmax, bad);
+}
+
+// Initial contact forces (no tangential increment) and the spheres' lattice
+// frame, after set_packing and after every re-layout.
+__global__ void __launch_bounds__(SUB_THREADS) k_dem_init(Dem D) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x, tl = t % TEAM, i = t / TEAM;
+    const bool have = i < D.n;
+    float3 F = make_float3(0.f, 0.f, 0.f), T = F;
+    if (have) {
+        const float3 xi = f3(D.dX[i]), vi = f3(D.V[i]), wi = f3(D.W[i]);
+        const int cnt = D.nb_cnt[i];
+        for (int k = tl; k < cnt; k += TEAM) {
+            const size_t e = (size_t)i * D.nbmax + k;
+            const int j = D.nb_j[e];
+            const float3 xj = f3(D.dX[j]);
+            float3 h = f3(D.nb_ft[e]);
+            pair_contact(D, D.R[i], D.R[j], reduced_radius(D.R[i], D.R[j]),
+                         make_float3(xj.x - xi.x, xj.y - xi.y, xj.z - xi.z), D.nb_dref[e], vi, wi, f3(D.V[j]),
+                         f3(D.W[j]), 0.f, h, F, T);
+            D.nb_ft[e] = make_float4(h.x, h.y, h.z, 0.f);
+        }
+    }
+    team_sum(F, T);
+    float dmax = 0.f, vmax = 0.f;
+    uint32_t bad = 0;
+    if (have && tl == 0) {
+        D.Fc[i] = make_float4(F.x, F.y, F.z, 0.f);
+        D.Tc[i] = make_float4(T.x, T.y, T.z, 0.f);
+        sphere_frame(D, i, dmax, vmax, bad);
+    }
     flush_maxima(D, dmax, vmax, bad);
 }
 
-// Largest cluster (CTAs of DSM_THREADS threads) the DSM kernel can run with
+// ------------------------------------------------------------ launches
+
+// Largest cluster (CTAs of DSM_THREADS threads) k_dem_step_dsm can run with
 // on each device, found on the first initialisation launch (outside any
-// stream capture); 0 = not found (the general kernel serves).
+// stream capture); 0 = not found (the launches per substep serve).
 static int g_dsm_cluster[64];
 static bool g_dsm_probed[64];
+constexpr size_t dsm_smem(int slots) { return (size_t)slots * DSM_BUFS * RECORD_BYTES; }
 
 static void probe_dsm(int dev) {
     if (dev < 0 || dev >= 64 || g_dsm_probed[dev]) return;
     g_dsm_probed[dev] = true;
     g_dsm_cluster[dev] = 0;
-    if (cudaFuncSetAttribute(k_dem_step_dsm, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+    const size_t most = dsm_smem(DEM_MAX_CTAS * DSM_THREADS / TEAM);  // every sphere in every CTA
+    if (cudaFuncSetAttribute(k_dem_step_dsm<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+        cudaFuncSetAttribute(k_dem_step_dsm<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most) !=
+            cudaSuccess) {
         cudaGetLastError();
         return;
     }
-    for (int C : {16, 8}) {
+    for (int C : {DEM_MAX_CTAS, 8}) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(C, 1, 1);
         cfg.blockDim = dim3(DSM_THREADS, 1, 1);
-        cfg.dynamicSmemBytes = 6 * (DSM_THREADS / TEAM) * sizeof(float4);
+        cfg.dynamicSmemBytes = most;
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeClusterDimension;
         attr[0].val.clusterDim.x = C;
@@ -529,7 +763,7 @@ static void probe_dsm(int dev) {
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         int ncl = 0;
-        if (cudaOccupancyMaxActiveClusters(&ncl, k_dem_step_dsm, &cfg) == cudaSuccess && ncl > 0) {
+        if (cudaOccupancyMaxActiveClusters(&ncl, k_dem_step_dsm<true>, &cfg) == cudaSuccess && ncl > 0) {
             g_dsm_cluster[dev] = C;
             break;
         }
@@ -537,54 +771,66 @@ static void probe_dsm(int dev) {
     }
 }
 
-void launch_dem_step(const Dem& D, bool init_only, cudaStream_t s) {
+// CTAs and threads per CTA of the one-launch form for n spheres; false where
+// they do not fit one cluster.  The smallest CTAs that fit: a CTA holds half
+// an SM's registers at 256 threads, so DEM clusters of concurrent columns
+// (batches) find room next to the lattice kernels.
+static bool dsm_shape(int n, int& C, int& T) {
     int dev = 0;
     cudaGetDevice(&dev);
-    if (init_only) probe_dsm(dev);
-    long long need = (long long)TEAM * (D.n > 0 ? D.n : 1);
+    const int cmax = dev >= 0 && dev < 64 ? g_dsm_cluster[dev] : 0;
+    const long long need = (long long)TEAM * (n > 0 ? n : 1);
+    if (cmax <= 0 || need > (long long)cmax * DSM_THREADS) return false;
+    T = need <= (long long)cmax * (DSM_THREADS / 2) ? DSM_THREADS / 2 : DSM_THREADS;
+    C = (int)((need + T - 1) / T);
+    if (C == 1) T = (int)(((need + 31) / 32) * 32);
+    return true;
+}
+
+void launch_dem_ghosts(const Dem& D, int* nb_slot, uint16_t* push, int* foreign, int* slots, cudaStream_t s) {
+    int dev = 0, C, T;
+    cudaGetDevice(&dev);
+    probe_dsm(dev);
+    cudaMemsetAsync(slots, 0, sizeof(int), s);
+    if (D.n <= 0 || !dsm_shape(D.n, C, T)) return;
+    if (C < DEM_MAX_CTAS) cudaMemsetAsync(push, 0xff, sizeof(uint16_t) * (size_t)D.n * DEM_MAX_CTAS, s);
+    k_dem_ghosts<<<C, 256, D.n, s>>>(D, T / TEAM, nb_slot, push, foreign, slots);
+}
+
+int dem_launches(int n, int K) {
+    int C, T;
+    return dsm_shape(n, C, T) ? 1 : K + 1;
+}
+
+void launch_dem_init(const Dem& D, cudaStream_t s) {
+    const unsigned blocks = (unsigned)(((long long)TEAM * D.n + SUB_THREADS - 1) / SUB_THREADS);
+    if (D.n > 0) k_dem_init<<<blocks, SUB_THREADS, 0, s>>>(D);
+}
+
+void launch_dem_step(const Dem& D, cudaStream_t s) {
+    int C, T;
+    if (!dsm_shape(D.n, C, T)) {
+        const unsigned blocks = (unsigned)(((long long)TEAM * D.n + SUB_THREADS - 1) / SUB_THREADS);
+        launch_pdl(k_dem_begin, blocks, SUB_THREADS, s, D);
+        for (int k = 0; k < D.K; ++k) launch_pdl(k_dem_substep, blocks, SUB_THREADS, s, D, k);
+        return;
+    }
     cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // pdl_wait before the sums are read
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = C;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
     cudaLaunchConfig_t cfg = {};
     cfg.stream = s;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    int cmax = dev >= 0 && dev < 64 ? g_dsm_cluster[dev] : 0;
-    if (!init_only && cmax > 0 && need <= (long long)cmax * DSM_THREADS) {
-        // the smallest CTAs that fit the cluster: a CTA holds half an SM's
-        // registers at 256 threads, so DEM clusters of concurrent columns
-        // (batches) find room next to the lattice kernels
-        int T = need <= (long long)cmax * (DSM_THREADS / 2) ? DSM_THREADS / 2 : DSM_THREADS;
-        int C = 1;
-        if (need > T) C = (int)((need + T - 1) / T);
-        else T = (int)(((need + 31) / 32) * 32);
-        cfg.gridDim = dim3(C, 1, 1);
-        cfg.blockDim = dim3(T, 1, 1);
-        cfg.dynamicSmemBytes = 6 * (T / TEAM) * sizeof(float4);
-        attr[0].val.clusterDim.x = C;
-        // programmatic dependency on the link kernel (pdl_wait first)
-        attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[1].val.programmaticStreamSerializationAllowed = 1;
-        cfg.numAttrs = 2;
-        cudaLaunchKernelEx(&cfg, k_dem_step_dsm, D);
-        return;
-    }
-    // general kernel: TEAM threads per sphere, up to 8 CTAs of up to 1024
-    // threads, several spheres per team when needed
-    int C = 1;
-    int T = (int)(((need + 31) / 32) * 32);
-    if (T > 256) {
-        C = (int)std::min<long long>(D.cluster, (need + 255) / 256);
-        T = (int)((need + C - 1) / C);
-        T = ((T + 31) / 32) * 32;
-        if (T > 1024) T = 1024;
-    }
+    cfg.numAttrs = C > 1 ? 2 : 1;
     cfg.gridDim = dim3(C, 1, 1);
     cfg.blockDim = dim3(T, 1, 1);
-    cfg.dynamicSmemBytes = 0;
-    attr[0].val.clusterDim.x = C;
-    cudaLaunchKernelEx(&cfg, k_dem_step, D, init_only ? 1 : 0);
+    cfg.dynamicSmemBytes = dsm_smem(D.slots);
+    if (C > 1) cudaLaunchKernelEx(&cfg, k_dem_step_dsm<true>, D);
+    else cudaLaunchKernelEx(&cfg, k_dem_step_dsm<false>, D);
 }
 
 // ------------------------------------------------------------ neighbour lists
@@ -729,6 +975,7 @@ __global__ void k_nb_build(NbBuild B) {
             }
         }
         B.ft[e] = h;
+        B.nR[e] = (float)B.R[B.nj[e]];
     }
     B.cnt[i] = cnt;
 }

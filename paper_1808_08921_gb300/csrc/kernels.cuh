@@ -134,9 +134,12 @@ struct FlipBuf {
     uint32_t cap;
 };
 
+// CTAs of the largest cluster the one-launch DEM takes.
+constexpr int DEM_MAX_CTAS = 16;
+
 // DEM state (Section 2.2).
 struct Dem {
-    int n, K, cluster;
+    int n, K;
     float dt;                // 1 / K
     float kn, kt, mu;        // Eqs. 11-12 prefactors
     float3 g;                // body force
@@ -145,12 +148,14 @@ struct Dem {
     const double* Xref;
     float4* dX;              // canonical displacement since re-layout
     float4* dXc;             // Kahan compensation
-    float4* dXb;             // [2][n] double buffer read by the force phase
+    // records of the launches per substep, [2][n] by substep parity:
+    // {dX, Vh.x}, {Vh.yz, Wh.xy}, {Wh.z}
+    float4* dXb;
     float4* V;
     float4* W;
     float4* q;
-    float4* Vhb;             // [2][n]
-    float4* Whb;             // [2][n]
+    float4* Vhb;
+    float4* Whb;
     float4* Fc;              // contact force (persistent across steps)
     float4* Tc;
     const double* Fh;        // hydrodynamic force/torque sums of this step (Eqs. 18-19)
@@ -168,6 +173,12 @@ struct Dem {
     const int* nb_j;
     const float4* nb_dref;   // xyz: X_ref_j + shift - X_ref_i, w: (R_i+R_j)^2 - |xyz|^2
     float4* nb_ft;           // tangential history (force on i)
+    const float* nb_R;       // radius of j
+    // one-launch form: slots of the exchange (k_dem_ghosts)
+    const int* nb_slot;      // [n * nbmax] slot of the neighbour in the sphere's CTA
+    const uint16_t* push;    // [n][DEM_MAX_CTAS] slot of the sphere in each CTA, 0xffff where it has none
+    const int* foreign;      // [DEM_MAX_CTAS] spheres of other CTAs a CTA holds
+    int slots;               // slots per CTA and record buffer
     // outputs for the lattice kernels
     int4* org;
     int4* orgw;
@@ -179,6 +190,7 @@ struct Dem {
     uint32_t* max_vel_bits;
     float hard_disp;             // displacement at which the layout is invalid
     int px;
+    int dry;                 // the fluid is off: DEM steps follow one another directly
     double Lx, Ly, Lz;
 };
 
@@ -199,7 +211,10 @@ void launch_map_update(const Lat& L, const PartView& P, const Band& band, const 
 void launch_link_words(const Lat& L, uint2* lw, cudaStream_t s);
 
 // dem.cu
-void launch_dem_step(const Dem& D, bool init_only, cudaStream_t s);
+void launch_dem_ghosts(const Dem& D, int* nb_slot, uint16_t* push, int* foreign, int* slots, cudaStream_t s);
+void launch_dem_init(const Dem& D, cudaStream_t s);
+void launch_dem_step(const Dem& D, cudaStream_t s);
+int dem_launches(int n, int K);  // kernels of one launch_dem_step
 // adjoint.cu: reverse-mode kernels of the lattice step for a fixed packing
 struct AdjArgs {
     Lat L;

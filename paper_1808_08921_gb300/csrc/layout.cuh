@@ -65,6 +65,7 @@ struct NbBuild {
     int8_t* nsh;     // [n*nbmax*4] image shift in box lengths
     float4* dref;    // xyz: X_ref_j + shift - X_ref_i; w: (R_i + R_j)^2 - |xyz|^2 (FP64-exact)
     float4* ft;
+    float* nR;       // [n*nbmax] radius of the neighbour
     const int* old_cnt;
     const int* old_j;
     const int8_t* old_sh;
