@@ -93,6 +93,7 @@ struct lbmdem_ctx {
     DBuf<uint8_t> deep, band;
     DBuf<uint4> rec, rec2;
     DBuf<uint32_t> maskB, maskB2, cntA, cntB, scan_tmp;
+    DBuf<uint32_t> flip;  // [2][W] map changes of the last two steps
     DBuf<uint8_t> f, f2;  // populations, 4 or 2 bytes each
     DBuf<uint32_t> coord, fbits;
     uint32_t nA = 0, nS = 0, nSpad = 0;
@@ -218,6 +219,7 @@ static Lat make_lat(lbmdem_ctx* c) {
     L.fsi = 1.0f / L.fs;
     L.rec = c->rec.p;
     L.maskB = c->maskB.p;
+    L.flip = c->flip.p;
     L.coord = c->coord.p;
     L.fbits = c->fbits.p;
     L.owner = c->owner.p;
@@ -506,6 +508,9 @@ static int build_layout(lbmdem_ctx* c, bool fresh) {
     // exceeds the largest displacement since the layout
     CK(cudaMemsetAsync(&c->st.p->disp_layout_bits, 0, sizeof(uint32_t), s));
     CK(cudaMemsetAsync(&c->st.p->layout_fresh, 1, sizeof(uint32_t), s));
+    // the queues and masks of earlier steps' changes belong to the old layout
+    CK(cudaMemsetAsync(c->st.p->nflip, 0, sizeof(c->st.p->nflip), s));
+    CK(cudaMemsetAsync(c->flip.p, 0, sizeof(uint32_t) * 2 * c->W, s));
     // link lists, grouped by sphere (direction-major inside a sphere)
     int np = c->np;
     size_t ng = (size_t)std::max(np, 1) * LINK_GROUPS;
@@ -561,7 +566,7 @@ static int build_layout(lbmdem_ctx* c, bool fresh) {
     uint32_t cap = c->p.max_flips > 0 ? (uint32_t)c->p.max_flips
                                       : std::min<uint32_t>(1u << 20, std::max<uint32_t>(4096u, nband / 8));
     if (cap != c->flip_cap) {
-        CK(c->flip_rec.alloc(cap));
+        CK(c->flip_rec.alloc(2 * (size_t)cap));
         CK(c->flip_scratch.alloc((size_t)cap * Q * Q));
         CK(c->flip_valid.alloc((size_t)cap * Q));
         c->flip_cap = cap;
@@ -612,48 +617,61 @@ static void record_pair_end(lbmdem_ctx* c, size_t idx, cudaStream_t st = nullptr
         cudaEventRecord(c->ev[2 * idx + 1], st);
 }
 
-// kernels one step issues: map update (4 when there is a band, else 1),
-// collide, links (if any surface entries and the step's links are not in the
-// collide kernel), inlet/outlet (if any), DEM
 static bool links_in_collide(const lbmdem_ctx* c, int parity) { return c->fused_links && parity == 0; }
-
-static int64_t kernels_per_step(const lbmdem_ctx* c, int parity) {
-    int64_t k = dem_launches(c->np, c->p.dem_substeps);
-    if (c->lbm) {
-        k += c->nband ? 4 : 1;
-        k += c->nS ? 1 : 0;
-        k += c->nwarps && !links_in_collide(c, parity) ? 1 : 0;
-        bool px = c->p.inlet == LBMDEM_X_PERIODIC;
-        k += (!px && !(c->p.inlet != 0 && c->p.outlet > 1)) ? 1 : 0;
-    }
-    return k;
-}
 
 static bool inlet_outlet_active(const lbmdem_ctx* c) {
     return c->p.inlet != LBMDEM_X_PERIODIC && !(c->p.inlet != 0 && c->p.outlet > 1);
 }
 
-static void enqueue_step(lbmdem_ctx* c, int parity, bool monitor) {
+// band nodes whose owner can change: none while every sphere is fixed (the
+// layout paints the owners by the same rule from the same positions)
+static uint32_t tested_band(const lbmdem_ctx* c) { return c->any_mobile ? c->nband : 0u; }
+
+// Where the inlet / outlet of a step runs: as a kernel of its own beside the
+// DEM (the step leaves a complete state), or inside the next step's first
+// kernel (only where the next step follows at once).
+enum { INLET_NOW = 0, INLET_NEXT = 1 };
+
+// kernels one step issues: map update, collide, links (if any surface entries
+// and the step's links are not in the collide kernel), inlet/outlet (if any
+// and not left to the next step), DEM
+static int64_t kernels_per_step(const lbmdem_ctx* c, int parity, int inlet = INLET_NOW) {
+    int64_t k = dem_launches(c->np, c->p.dem_substeps);
+    if (c->lbm) {
+        k += map_update_launches(tested_band(c), parity);
+        k += c->nS ? 1 : 0;
+        k += c->nwarps && !links_in_collide(c, parity) ? 1 : 0;
+        k += inlet_outlet_active(c) && inlet == INLET_NOW ? 1 : 0;
+    }
+    return k;
+}
+
+// inlet: where this step's inlet / outlet runs; follows: the step continues a
+// run whose previous step ended with its DEM and left its inlet / outlet, if
+// there is one, to this step
+static void enqueue_step(lbmdem_ctx* c, int parity, bool monitor, int inlet = INLET_NOW, bool follows = false) {
     cudaStream_t s = c->stream;
     bool tm = c->timing;
     size_t e = 0;
-    c->launches += kernels_per_step(c, parity);
+    c->launches += kernels_per_step(c, parity, inlet);
     if (c->lbm) {
         Lat L = make_lat(c);
         PartView P = make_part(c);
-        Band B{c->band_coord.p, c->band_cand.p, c->band_slack.p, c->nband};
+        Band B{c->band_coord.p, c->band_cand.p, c->band_slack.p, tested_band(c)};
         FlipBuf F{c->flip_rec.p, c->flip_scratch.p, c->flip_valid.p, c->flip_cap};
+        DevStats* sd = c->st.p;
+        BC bc{c->p.inlet, c->p.outlet, c->src, &sd->t_inlet};
         if (tm) record_pair_begin(c, 2, e);
-        launch_map_update(L, P, B, F, c->st.p, parity == 1, parity, c->fused_links ? c->linkw.p : nullptr, c->batched,
-                          s);
+        launch_map_update(L, P, B, F, sd, parity, c->fused_links ? c->linkw.p : nullptr,
+                          follows && inlet_outlet_active(c) ? &bc : nullptr, follows, c->batched, s);
         if (tm) record_pair_end(c, e);
         Mon mon{};
-        DevStats* sd = c->st.p;
         mon.acc = sd->mon;
         mon.umax_bits = &sd->max_u_bits;
         mon.status = &sd->status;
         mon.probe_sum = c->p.probe_x >= 0 && !c->suppress_probe ? c->probe.p : nullptr;
         mon.t_dev = &sd->t;
+        mon.t_inlet = &sd->t_inlet;
         mon.pA0 = c->pA0;
         mon.pA1 = c->pA1;
         mon.pB0 = c->pB0;
@@ -678,8 +696,7 @@ static void enqueue_step(lbmdem_ctx* c, int parity, bool monitor) {
         // the inlet/outlet only needs this step's populations and the DEM only
         // this step's link sums: they run side by side, the boundary on a
         // side stream joined before the next step
-        BC bc{c->p.inlet, c->p.outlet, c->src, &sd->t};
-        if (inlet_outlet_active(c)) {
+        if (inlet_outlet_active(c) && inlet == INLET_NOW) {
             cudaEventRecord(c->ev_fork, s);
             cudaStreamWaitEvent(c->side, c->ev_fork, 0);
             size_t e2 = 0;
@@ -699,6 +716,19 @@ static void enqueue_step(lbmdem_ctx* c, int parity, bool monitor) {
     if (tm) record_pair_begin(c, 4, e);
     launch_dem_step(D, s);
     if (tm) record_pair_end(c, e);
+}
+
+// n consecutive steps from parity p0 on the stream (or into a graph that is
+// being captured): only the last one's inlet / outlet runs as a kernel of its
+// own, and each step's first kernel starts early behind the DEM before it.
+// monitored(k): whether step k accumulates the totals.  With per-group timing
+// every step ends complete, so that the groups stay apart.
+template <class Monitored>
+static void enqueue_run(lbmdem_ctx* c, int n, int p0, Monitored monitored) {
+    for (int k = 0; k < n; ++k) {
+        const bool last = k == n - 1;
+        enqueue_step(c, (p0 + k) & 1, monitored(k), last || c->timing ? INLET_NOW : INLET_NEXT, k > 0 && !c->timing);
+    }
 }
 
 static int collect_timing(lbmdem_ctx* c) {
@@ -738,7 +768,7 @@ static int capture_graph(lbmdem_ctx* c) {
     int64_t l0 = c->launches;
     CK(cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
     c->capturing = true;
-    for (int k = 0; k < c->glen; ++k) enqueue_step(c, k & 1, mon && k == c->glen - 1);
+    enqueue_run(c, c->glen, 0, [&](int k) { return mon && k == c->glen - 1; });
     c->capturing = false;
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaStreamEndCapture(c->stream, &g);
@@ -899,7 +929,7 @@ int lbm_dem_init(const lbmdem_params* pp, lbmdem_ctx** out) {
     if (c->lbm) {
         if (c->owner.alloc(c->N) || c->deep.alloc(c->N) || c->band.alloc(c->N) || c->rec.alloc(c->W) ||
             c->rec2.alloc(c->W) || c->maskB.alloc(c->W) || c->maskB2.alloc(c->W) ||
-            c->cntA.alloc(c->W + 1) || c->cntB.alloc(c->W + 1) ||
+            c->cntA.alloc(c->W + 1) || c->cntB.alloc(c->W + 1) || c->flip.alloc(2 * c->W) ||
             c->scan_tmp.alloc(scan_tmp_size(std::max(c->W + 1, (size_t)1 << 24))) ||
             c->band_count.alloc(1))
             return bail(LBMDEM_ERR_OOM);
@@ -1112,14 +1142,19 @@ int lbm_dem_step(lbmdem_ctx* c, int64_t n) {
                 if (int r = collect_timing(c)) return r;
             }
         } else {
-            bool mon = c->p.monitor_every > 0 && ((c->t + 1) % c->p.monitor_every == 0);
+            // up to the next graph, the next check or the end
+            const int64_t me = c->p.monitor_every, t = c->t;
+            const int m = c->timing ? 1 : (int)std::min<int64_t>({n, std::max<int64_t>(room, 1), t % 2 ? 1 : c->glen});
             size_t pairs0 = c->ev_pairs;
-            enqueue_step(c, (int)(c->t & 1), mon);
+            enqueue_run(c, m, (int)(t & 1), [&](int k) {
+                const bool mon = me > 0 && (t + k + 1) % me == 0;
+                if (mon) c->mon_step = t + k;
+                return mon;
+            });
             CK(cudaGetLastError());
-            if (mon) c->mon_step = c->t;
-            c->t += 1;
-            n -= 1;
-            c->steps_until_check -= 1;
+            c->t += m;
+            n -= m;
+            c->steps_until_check -= m;
             if (c->timing && c->ev_pairs > pairs0) {
                 if (int r = collect_timing(c)) return r;
             }
@@ -1253,7 +1288,7 @@ int capture_body(lbmdem_batch* b, lbmdem_ctx* c, cudaGraph_t body, int nsteps, v
     BCK(cudaStreamBeginCaptureToGraph(c->stream, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
     const bool mon = c->p.monitor_every > 0;
     c->batched = true;
-    for (int k = 0; k < nsteps; ++k) enqueue_step(c, k & 1, mon && k == nsteps - 1);
+    enqueue_run(c, nsteps, 0, [&](int k) { return mon && k == nsteps - 1; });
     c->batched = false;
     if (ctl_kernel) ctl_kernel<<<1, 32, 0, c->stream>>>(ctl, i, &c->st.p->status, h);
     cudaGraph_t g = body;
@@ -1422,7 +1457,8 @@ int lbm_dem_batch_step(lbmdem_batch* b, const int64_t* steps) {
         lbmdem_ctx* c = b->cols[i];
         BCK(cudaStreamWaitEvent(c->stream, b->done, 0));
         if (rem[i] <= 0) continue;
-        for (int64_t k = 0; k < rem[i]; ++k) c->launches += kernels_per_step(c, (int)((c->t + k) & 1));
+        for (int64_t k = 0; k < rem[i]; ++k)  // a pair's even step leaves its inlet to the odd one
+            c->launches += kernels_per_step(c, (int)(k & 1), k % 2 == 0 && k + 1 < rem[i] ? INLET_NEXT : INLET_NOW);
         c->launches += (rem[i] + 1) / 2;  // loop control
         if (c->p.monitor_every > 0) c->mon_step = c->t + rem[i] - 1;
         c->t += rem[i];  // corrected from the device count by lbm_dem_batch_sync if a loop stopped early

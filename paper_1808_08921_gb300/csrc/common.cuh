@@ -113,6 +113,7 @@ struct Lat {
     float fs, fsi;        // storage scale and its inverse (powers of two)
     uint4* rec;           // [nx*ny*nw] {maskF, maskA, baseA, baseB}
     uint32_t* maskB;      // [nx*ny*nw]
+    uint32_t* flip;       // [2][nx*ny*nw] nodes the map update of a step made fluid or solid, by step parity
     uint32_t* coord;      // [nSpad]
     uint32_t* fbits;      // [nSpad / 32]
     int32_t* owner;       // [nx*ny*nz]
@@ -188,6 +189,27 @@ template <int ST> __device__ __forceinline__ typename PopT<ST>::T* pops(const La
     return static_cast<typename PopT<ST>::T*>(L.f);
 }
 
+// The map before this step's map update, from the committed map and the
+// nodes that update changed (flip: the masks of the step's parity).
+__device__ __forceinline__ uint32_t old_fluid_index(const Lat& L, const uint32_t* flip, int x, int y, int z, int dx,
+                                                    int dy, int dz) {
+    int xs = x + dx;
+    if (L.px) {
+        xs = wrap1(xs, L.nx);
+    } else if (xs < 0 || xs >= L.nx) {
+        return NONE;
+    }
+    int ys = wrap1(y + dy, L.ny), zs = wrap1(z + dz, L.nz);
+    uint32_t wi = ((uint32_t)xs * L.ny + ys) * L.nw + (zs >> 5);
+    uint4 r = L.rec[wi];
+    const uint32_t fl = r.x ^ flip[wi];
+    uint32_t bit = 1u << (zs & 31);
+    if (!(fl & bit)) return NONE;
+    uint32_t low = bit - 1u;
+    if (r.y & bit) return r.z + __popc(r.y & low);
+    return r.w + __popc(L.maskB[wi] & low);
+}
+
 // Location of population m of fluid node (x,y,z) with compact index i, in the
 // state between steps.  after_even = true: the state after an even step
 // (natural populations sit in the neighbours' reversed slots).
@@ -215,6 +237,17 @@ __device__ __forceinline__ typename PopT<ST>::T* pop_loc(const Lat& L, bool afte
             else M(false, 2);                 \
         }                                     \
     } while (0)
+
+// The same by the map before this step's map update.
+template <int ST>
+__device__ __forceinline__ typename PopT<ST>::T* old_pop_loc(const Lat& L, const uint32_t* flip, bool after_even, int x,
+                                                             int y, int z, uint32_t i, int m) {
+    typename PopT<ST>::T* f = pops<ST>(L);
+    if (!after_even || m == 18) return f + (size_t)m * L.nSpad + i;
+    uint32_t s = old_fluid_index(L, flip, x, y, z, -cx(m), -cy(m), -cz(m));
+    if (s == NONE) return f + (size_t)m * L.nSpad + i;
+    return f + (size_t)opp(m) * L.nSpad + s;
+}
 
 // Particles as seen by the lattice kernels (current time level).
 struct PartView {
@@ -289,6 +322,7 @@ struct DevStats {
     double mon[6];           // sum rho, sum rho u, max|u|, step
     uint32_t max_u_bits;
     uint32_t layout_fresh;   // 1 from a layout build until the first step's DEM
+    unsigned long long t_inlet;  // steps completed when the last collided step ends: the source time of its inlet
 };
 
 // Programmatic dependent launch.  The kernels of a step are launched with

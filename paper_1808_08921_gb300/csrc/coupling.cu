@@ -18,14 +18,16 @@
 //    largest displacement since the layout -- (where spheres overlap, the one
 //    with the smallest |x - X|^2 / R^2 owns the node, the lowest index on a
 //    tie; the inlet/outlet planes stay fluid).  Changed nodes are
-//    queued; for each, the natural populations of the node and its 18
-//    neighbours are gathered with the old map, the conversion is applied
+//    queued and committed to the map; for each, the natural populations of
+//    the node and its 18 neighbours are gathered with the map as it was
+//    (committed map and the step's changes), and the conversion is applied
 //    (covered node: its momentum goes to the sphere, Eq. 16; uncovered node:
 //    equilibrium at the mean density of its fluid neighbours and the surface
-//    velocity, the sphere loses that momentum, Eq. 17), the map is committed,
-//    and the populations are scattered back with the new map (in the AA
-//    layout the slot of a population depends on whether its upstream
-//    neighbour is fluid).
+//    velocity, the sphere loses that momentum, Eq. 17).  Before an even step
+//    the populations sit in their nodes' own slots, so the uncovered node's
+//    are written there at once; before an odd step the slot of a population
+//    depends on whether its upstream neighbour is fluid, and a third kernel
+//    scatters the gathered populations back with the new map.
 #include "common.cuh"
 #include "kernels.cuh"
 
@@ -248,9 +250,10 @@ struct MapArgs {
     Band band;
     FlipBuf F;
     DevStats* st;
-    int par;        // parity of the step (selects the flip counter)
-    int after_even; // layout of the state the step starts from
+    int par;        // parity of the step (selects the queue, its counter and the flip masks)
     uint2* lw;      // link words renewed around converted nodes (null: not kept)
+    BC bc;          // the previous step's inlet / outlet,
+    int io_blocks;  // applied by the first io_blocks blocks of the band kernel
 };
 
 // Link word of the stored node (x, y, z) from the owner map (see LW_MASK):
@@ -304,12 +307,45 @@ void launch_link_words(const Lat& L, uint2* lw, cudaStream_t s) {
     if (L.nS) k_link_words<<<(L.nS + 255) / 256, 256, 0, s>>>(L, lw);
 }
 
-__global__ void k_map_band(MapArgs A) {
-    pdl_trigger();  // launched normally: its predecessors are the DEM and the boundary branch
-    uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k == 0) {
-        A.st->nflip[A.par ^ 1] = 0;
-        A.st->t += 1ull;  // the step starts: t counts it from here on
+// Masks and queue of a step's changes.
+__device__ __forceinline__ uint32_t* flip_masks(const Lat& L, int par) {
+    return L.flip + (size_t)par * L.nx * L.ny * L.nw;
+}
+
+// First kernel of a step: counts it, applies the previous step's inlet /
+// outlet (its blocks come first: the source density is evaluated in FP64
+// before the wait for the previous kernel), resets the spheres' sums, and
+// re-tests the band.  A changed node is queued and committed here, so that
+// the conversions need no kernel between their gather and their link words:
+// the gather reconstructs the map as it was from the step's flip masks.  Those
+// of the previous step (other parity) are cleared here from its queue.
+// Launched with a programmatic dependency on the DEM, which hides its launch
+// behind the substeps (2.2 us per step as an ordinary successor of the DEM and
+// of a boundary kernel on a second stream).
+template <bool AFTER_EVEN, int ST>
+__global__ void __launch_bounds__(256) k_map_band(MapArgs A) {
+    const Lat& L = A.L;
+    if ((int)blockIdx.x < A.io_blocks) {
+        __shared__ float s_drho;
+        if (threadIdx.x == 0) s_drho = (float)source_drho(A.bc.src, A.st->t_inlet);
+        __syncthreads();
+        pdl_wait();
+        pdl_trigger();
+        inlet_outlet_node<AFTER_EVEN, ST>(L, A.bc, s_drho, blockIdx.x * blockDim.x + threadIdx.x);
+        return;
+    }
+    const uint32_t k = (blockIdx.x - A.io_blocks) * blockDim.x + threadIdx.x;
+    const float slack = k < A.band.n ? A.band.slack[k] : 0.f;
+    pdl_wait();
+    pdl_trigger();
+    if (k == 0) A.st->t += 1ull;  // the step starts: t counts it from here on
+    {
+        const uint32_t prev = min(A.st->nflip[A.par ^ 1], A.F.cap), stride = (gridDim.x - A.io_blocks) * blockDim.x;
+        for (uint32_t w = k; w < prev; w += stride) {
+            int x, y, z;
+            unpack_coord(A.F.rec[(size_t)(A.par ^ 1) * A.F.cap + w].coord, x, y, z);
+            flip_masks(L, A.par ^ 1)[((uint32_t)x * L.ny + y) * L.nw + (z >> 5)] = 0u;
+        }
     }
     if (k < (uint32_t)A.P.n) {
         for (int r = 0; r < NREP; ++r)
@@ -343,9 +379,8 @@ __global__ void k_map_band(MapArgs A) {
     // sphere has moved since keeps its owner
     if (!A.st->layout_fresh) {
         const float moved = __uint_as_float(A.st->disp_layout_bits);
-        if (A.band.slack[k] > moved + 1e-5f * (1.f + moved)) return;
+        if (slack > moved + 1e-5f * (1.f + moved)) return;
     }
-    const Lat& L = A.L;
     int x, y, z;
     unpack_coord(A.band.coord[k], x, y, z);
     const size_t li = ((size_t)x * L.ny + y) * L.nz + z;
@@ -408,39 +443,79 @@ __global__ void k_map_band(MapArgs A) {
         }
     }
     if (old != best) {
+        bool fl;
+        const uint32_t ci = stored_index(L, x, y, z, fl);
+        if (best == OWNER_FLUID && ci == NONE) {  // would need a node outside the stored set
+            atomicOr(&A.st->status, ST_SKIN);
+            return;
+        }
         uint32_t slot = atomicAdd(&A.st->nflip[A.par], 1u);
-        if (slot < A.F.cap) {
-            Flip f;
-            f.coord = A.band.coord[k];
-            f.old_owner = old;
-            f.new_owner = best;
-            f.pad = 0;
-            A.F.rec[slot] = f;
-        } else {
+        if (slot >= A.F.cap) {
             atomicOr(&A.st->status, ST_CAPACITY);
+            return;
+        }
+        Flip f;
+        f.coord = A.band.coord[k];
+        f.old_owner = old;
+        f.new_owner = best;
+        f.pad = 0;
+        A.F.rec[(size_t)A.par * A.F.cap + slot] = f;
+        L.owner[li] = best;
+        if (old == OWNER_FLUID || best == OWNER_FLUID) {
+            const uint32_t wi = ((uint32_t)x * L.ny + y) * L.nw + (z >> 5), bit = 1u << (z & 31);
+            atomicXor(&L.rec[wi].x, bit);
+            atomicOr(&flip_masks(L, A.par)[wi], bit);
+            if (ci != NONE) atomicXor(&L.fbits[ci >> 5], 1u << (ci & 31));
         }
     }
 }
 
 // One block per queued node (grid-stride over the queue): thread t < 361
-// gathers population m = t % 19 of node j = t / 19 with the old map, where
-// j < 18 is the neighbour x + c_j and j = 18 the node itself; thread 361,
-// idle during the gather, loads the sphere's state and the node's offset
-// from its centre meanwhile and then applies the conversion.
+// gathers population m = t % 19 of node j = t / 19 with the map as it was,
+// where j < 18 is the neighbour x + c_j and j = 18 the node itself; thread
+// 361, idle during the gather, loads the sphere's state and the node's offset
+// from its centre meanwhile and then applies the conversion.  The 19 first
+// threads of the last warp (of its own, so neither path waits for the other)
+// renew the link words of the node and its 18 neighbours from the committed
+// owner map (neighbours shared by two queued nodes get the same word twice).
 constexpr int MAP_THREADS = 384;  // >= 19 * 19
-template <int ST>
-__global__ void __launch_bounds__(MAP_THREADS) k_map_gather_convert(MapArgs A) {
+constexpr int LW_THREADS = 32;    // the link words' warp
+template <bool AFTER_EVEN, int ST>
+__global__ void __launch_bounds__(MAP_THREADS + LW_THREADS) k_map_gather_convert(MapArgs A) {
     pdl_wait();
     pdl_trigger();
     const Lat& L = A.L;
+    const uint32_t* flip = flip_masks(L, A.par);
+    const Flip* queue = A.F.rec + (size_t)A.par * A.F.cap;
     __shared__ float sg[Q * Q];
     __shared__ float srho[Q];
     __shared__ int sv[Q];
     const uint32_t nf = min(A.st->nflip[A.par], A.F.cap);
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        A.st->nflip[A.par ^ 1] = 0;  // cleared by the band kernel: free for the next step
+        if (nf) A.st->flips_total += (unsigned long long)nf;
+    }
+    if (threadIdx.x >= MAP_THREADS) {
+        const int jn = threadIdx.x - MAP_THREADS;  // 0 ... 17: neighbour x + c_jn, 18: the node
+        if (jn >= Q) return;
+        for (uint32_t w = blockIdx.x; w < nf; w += gridDim.x) {
+            int x, y, z;
+            unpack_coord(queue[w].coord, x, y, z);
+            int xs = x + cx(jn);
+            if (L.px) xs = wrap1(xs, L.nx);
+            else if (xs < 0 || xs >= L.nx) continue;
+            const int ys = wrap1(y + cy(jn), L.ny), zs = wrap1(z + cz(jn), L.nz);
+            bool fl;
+            const uint32_t ci = stored_index(L, xs, ys, zs, fl);
+            if (ci != NONE) A.lw[ci] = link_word(L, xs, ys, zs);
+        }
+        return;
+    }
+    auto sync = [] { asm volatile("bar.sync 1, %0;" ::"n"(MAP_THREADS) : "memory"); };
     const int t = threadIdx.x, j = t / Q, m = t % Q;
     constexpr int CT = Q * Q;  // the converting thread
     for (uint32_t w = blockIdx.x; w < nf; w += gridDim.x) {
-        const Flip f = A.F.rec[w];
+        const Flip f = queue[w];
         int x, y, z;
         unpack_coord(f.coord, x, y, z);
         float* sc = A.F.scratch + (size_t)w * Q * Q;
@@ -465,24 +540,23 @@ __global__ void __launch_bounds__(MAP_THREADS) k_map_gather_convert(MapArgs A) {
             if (L.px) xs = wrap1(xs, L.nx);
             else in = xs >= 0 && xs < L.nx;
             if (in) {
-                bool fl;
-                uint32_t ci = stored_index(L, xs, ys, zs, fl);
-                if (fl && ci != NONE) {
-                    g = to_f<ST>(*pop_loc<ST>(L, A.after_even, xs, ys, zs, ci, m), L.fsi);
+                const uint32_t ci = old_fluid_index(L, flip, xs, ys, zs, 0, 0, 0);
+                if (ci != NONE) {
+                    g = to_f<ST>(*old_pop_loc<ST>(L, flip, AFTER_EVEN, xs, ys, zs, ci, m), L.fsi);
                     valid = true;
                 }
             }
             sg[t] = g;
-            if (valid) sc[t] = g;
+            if (AFTER_EVEN && valid) sc[t] = g;
             if (m == 0) sv[j] = valid ? 1 : 0;
         }
-        __syncthreads();
+        sync();
         if (t < Q) {  // density of each gathered node
             float d = 0.f;
             for (int mm = 0; mm < Q; ++mm) d += sg[t * Q + mm];
             srho[t] = L.rho_f + d;
         }
-        __syncthreads();
+        sync();
         if (t == CT) {
             // mean density of the fluid neighbours (not the node itself)
             float rs = 0.f, rc = 0.f;
@@ -517,10 +591,16 @@ __global__ void __launch_bounds__(MAP_THREADS) k_map_gather_convert(MapArgs A) {
                             uz = V.z + (W.x * r1 - W.y * r0);
                 const double vb[3] = {ux, uy, uz};
                 float uu15 = 1.5f * (ux * ux + uy * uy + uz * uz);
-                float* g = sc + 18 * Q;
+                // into the scratch, or at once into the node's own slots (no
+                // other node's gather reads a slot of a node that was solid)
+                bool fl;
+                const uint32_t ci = stored_index(L, x, y, z, fl);
+                auto* own = pops<ST>(L) + ci;
                 for (int mm = 0; mm < Q; ++mm) {
                     float cu = cx(mm) * ux + cy(mm) * uy + cz(mm) * uz;
-                    g[mm] = wt(mm) * ((rbf - L.rho_f) + rbf * (3.f * cu + 4.5f * cu * cu - uu15));
+                    const float geq = wt(mm) * ((rbf - L.rho_f) + rbf * (3.f * cu + 4.5f * cu * cu - uu15));
+                    if (AFTER_EVEN) sc[18 * Q + mm] = geq;
+                    else own[(size_t)mm * L.nSpad] = from_f<ST>(geq, L.fs);
                 }
                 sv[18] = 1;
                 double mom[3] = {rb * vb[0], rb * vb[1], rb * vb[2]};
@@ -532,80 +612,25 @@ __global__ void __launch_bounds__(MAP_THREADS) k_map_gather_convert(MapArgs A) {
                 atomicAdd(&A.P.Th[3 * o + 2], -(r[0] * mom[1] - r[1] * mom[0]));
             }
         }
-        __syncthreads();
-        if (t < Q) A.F.valid[(size_t)w * Q + t] = (uint8_t)sv[t];
-        __syncthreads();  // shared arrays are reused by the next queued node
+        sync();
+        if (AFTER_EVEN && t < Q) A.F.valid[(size_t)w * Q + t] = (uint8_t)sv[t];
+        sync();  // shared arrays are reused by the next queued node
     }
-}
-
-__device__ void map_commit_one(const MapArgs& A, uint32_t k);
-
-__global__ void k_map_commit(MapArgs A) {
-    pdl_wait();
-    pdl_trigger();
-    uint32_t nf = min(A.st->nflip[A.par], A.F.cap);
-    uint32_t t0 = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t0 == 0) atomicAdd(&A.st->flips_total, (unsigned long long)nf);
-    for (uint32_t k = t0; k < nf; k += gridDim.x * blockDim.x) map_commit_one(A, k);
-}
-
-__device__ void map_commit_one(const MapArgs& A, uint32_t k) {
-    const Lat& L = A.L;
-    Flip f = A.F.rec[k];
-    int x, y, z;
-    unpack_coord(f.coord, x, y, z);
-    size_t li = ((size_t)x * L.ny + y) * L.nz + z;
-    bool fl;
-    uint32_t ci = stored_index(L, x, y, z, fl);
-    uint32_t wi = ((uint32_t)x * L.ny + y) * L.nw + (z >> 5);
-    uint32_t bit = 1u << (z & 31);
-    if (f.new_owner == OWNER_FLUID) {
-        if (ci == NONE) {  // would need a node outside the stored set
-            atomicOr(&A.st->status, ST_SKIN);
-            return;
-        }
-        atomicOr(&L.rec[wi].x, bit);
-        atomicOr(&L.fbits[ci >> 5], 1u << (ci & 31));
-    } else if (f.old_owner == OWNER_FLUID) {
-        atomicAnd(&L.rec[wi].x, ~bit);
-        if (ci != NONE) atomicAnd(&L.fbits[ci >> 5], ~(1u << (ci & 31)));
-    }
-    L.owner[li] = f.new_owner;
 }
 
 // One block per queued node: thread t < 361 writes population m = t % 19 of
-// node j = t / 19 back with the new map; the 19 first threads of the warp
-// after those (a warp of its own, so neither path waits for the other)
-// renew the link words of the node and its 18 neighbours from the committed
-// owner map (neighbours shared by two queued nodes get the same word twice).
-constexpr int SCATTER_THREADS = MAP_THREADS + 32;
+// node j = t / 19 back with the new map (before an odd step only).
 template <int ST>
-__global__ void __launch_bounds__(SCATTER_THREADS) k_map_scatter(MapArgs A) {
+__global__ void __launch_bounds__(MAP_THREADS) k_map_scatter(MapArgs A) {
     pdl_wait();
     pdl_trigger();
     const Lat L = A.L;
     const uint32_t nf = min(A.st->nflip[A.par], A.F.cap);
     const int t = threadIdx.x, j = t / Q, m = t % Q;
-    if (t >= Q * Q) {
-        const int jn = t - MAP_THREADS;  // 0 ... 17: neighbour x + c_jn, 18: the node
-        if (jn < 0) return;
-        if (A.lw == nullptr || jn >= Q) return;
-        for (uint32_t w = blockIdx.x; w < nf; w += gridDim.x) {
-            int x, y, z;
-            unpack_coord(A.F.rec[w].coord, x, y, z);
-            int xs = x + cx(jn);
-            if (L.px) xs = wrap1(xs, L.nx);
-            else if (xs < 0 || xs >= L.nx) continue;
-            const int ys = wrap1(y + cy(jn), L.ny), zs = wrap1(z + cz(jn), L.nz);
-            bool fl;
-            const uint32_t ci = stored_index(L, xs, ys, zs, fl);
-            if (ci != NONE) A.lw[ci] = link_word(L, xs, ys, zs);
-        }
-        return;
-    }
+    if (t >= Q * Q) return;
     for (uint32_t w = blockIdx.x; w < nf; w += gridDim.x) {
         if (!A.F.valid[(size_t)w * Q + j]) continue;
-        const Flip f = A.F.rec[w];
+        const Flip f = A.F.rec[(size_t)A.par * A.F.cap + w];
         int x, y, z;
         unpack_coord(f.coord, x, y, z);
         int xs = x + cx(j), ys = wrap1(y + cy(j), L.ny), zs = wrap1(z + cz(j), L.nz);
@@ -613,7 +638,7 @@ __global__ void __launch_bounds__(SCATTER_THREADS) k_map_scatter(MapArgs A) {
         bool fl;
         uint32_t ci = stored_index(L, xs, ys, zs, fl);
         if (!fl || ci == NONE) continue;
-        *pop_loc<ST>(L, A.after_even, xs, ys, zs, ci, m) = from_f<ST>(A.F.scratch[(size_t)w * Q * Q + t], L.fs);
+        *pop_loc<ST>(L, true, xs, ys, zs, ci, m) = from_f<ST>(A.F.scratch[(size_t)w * Q * Q + t], L.fs);
     }
 }
 
@@ -623,25 +648,32 @@ __global__ void __launch_bounds__(SCATTER_THREADS) k_map_scatter(MapArgs A) {
 // (a settling packing converts a few hundred nodes per step); columns of a
 // batch, which share the GPU with each other, take 256-thread band blocks
 // and 152 conversion blocks, fewer blocks to schedule beside the other
-// columns' kernels.
+// columns' kernels, and the band kernel without the early launch, whose
+// waiting blocks would keep room from the other columns.
 void launch_map_update(const Lat& L, const PartView& P, const Band& band, const FlipBuf& F,
-                       DevStats* st, bool after_even, int step_parity, uint2* lw, bool shared_gpu, cudaStream_t s) {
-    MapArgs A{L, P, band, F, st, step_parity, after_even ? 1 : 0, lw};
+                       DevStats* st, int step_parity, uint2* lw, const BC* inlet, bool early, bool shared_gpu,
+                       cudaStream_t s) {
+    const unsigned bb = shared_gpu ? 256 : 64;
+    const unsigned io = inlet ? (unsigned)((2 * L.ny * L.nz + bb - 1) / bb) : 0u;
+    MapArgs A{L, P, band, F, st, step_parity, lw, inlet ? *inlet : BC{}, (int)io};
+    const bool after_even = step_parity == 1;
     uint32_t nb = band.n > (uint32_t)P.n ? band.n : (uint32_t)P.n;
     if (nb == 0) nb = 1;
-    const unsigned bb = shared_gpu ? 256 : 64;
-    k_map_band<<<(nb + bb - 1) / bb, bb, 0, s>>>(A);
-    if (band.n == 0) return;
+    const unsigned blocks = io + (nb + bb - 1) / bb;
     // the queued count is read on the device: fixed grids stride over it
     const unsigned grid = shared_gpu ? 152 : 4 * 152;
-    if (L.st == 0) launch_pdl(k_map_gather_convert<0>, grid, MAP_THREADS, s, A);
-    else if (L.st == 1) launch_pdl(k_map_gather_convert<1>, grid, MAP_THREADS, s, A);
-    else launch_pdl(k_map_gather_convert<2>, grid, MAP_THREADS, s, A);
-    launch_pdl(k_map_commit, grid, 256, s, A);
-    const unsigned sthreads = lw ? SCATTER_THREADS : MAP_THREADS;
-    if (L.st == 0) launch_pdl(k_map_scatter<0>, grid, sthreads, s, A);
-    else if (L.st == 1) launch_pdl(k_map_scatter<1>, grid, sthreads, s, A);
-    else launch_pdl(k_map_scatter<2>, grid, sthreads, s, A);
+    const unsigned gthreads = MAP_THREADS + (lw ? LW_THREADS : 0);
+#define LBMDEM_MB(AE, ST)                                                              \
+    do {                                                                               \
+        if (early && !shared_gpu) launch_pdl(k_map_band<AE, ST>, blocks, bb, s, A);    \
+        else k_map_band<AE, ST><<<blocks, bb, 0, s>>>(A);                              \
+        if (band.n) launch_pdl(k_map_gather_convert<AE, ST>, grid, gthreads, s, A);    \
+        if (band.n && AE) launch_pdl(k_map_scatter<ST>, grid, MAP_THREADS, s, A);      \
+    } while (0)
+    LBMDEM_BY_STATE(LBMDEM_MB);
+#undef LBMDEM_MB
 }
+
+int map_update_launches(uint32_t nband, int step_parity) { return nband ? (step_parity == 1 ? 3 : 2) : 1; }
 
 }  // namespace lbmdem

@@ -13,6 +13,7 @@ struct Mon {
     uint32_t* status;
     double* probe_sum;              // [2 * capacity] (sum drho, count) per step, or null
     const unsigned long long* t_dev;
+    unsigned long long* t_inlet;
     uint32_t pA0, pA1, pB0, pB1;    // compact index ranges of the probe plane
 };
 
@@ -66,6 +67,50 @@ __device__ __forceinline__ void pressure_face(float g[Q], float drho_b, int side
         g[10] = g[7] - rux * (1.f / 6.f) - Ny;
         g[13] = g[8] - rux * (1.f / 6.f) + Nz;
         g[12] = g[9] - rux * (1.f / 6.f) - Nz;
+    }
+}
+
+// The inlet / outlet of the step that ended, one thread per boundary node:
+// k < ny nz the inlet plane, then the outlet plane.  drho: the source's
+// density deviation at the new time.
+template <bool AFTER_EVEN, int ST>
+__device__ __forceinline__ void inlet_outlet_node(const Lat& L, const BC& bc, float drho, int k) {
+    auto* f = pops<ST>(L);
+    const int plane = L.ny * L.nz;
+    if (k >= 2 * plane) return;
+    int side = k >= plane;
+    int yz = side ? k - plane : k;
+    int y = yz / L.nz, z = yz - y * L.nz;
+    int x = side ? L.nx - 1 : 0;
+    bool fl;
+    uint32_t i = stored_index(L, x, y, z, fl);
+    if (!fl || i == NONE) return;
+    if (side == 0) {
+        if (bc.inlet != 0) return;
+        float g[Q];
+#pragma unroll
+        for (int m = 0; m < Q; ++m)
+            if (cx(m) <= 0) g[m] = to_f<ST>(*pop_loc<ST>(L, AFTER_EVEN, x, y, z, i, m), L.fsi);
+        pressure_face(g, drho, 0);
+#pragma unroll
+        for (int m = 0; m < Q; ++m)
+            if (cx(m) > 0) f[(size_t)m * L.nSpad + i] = from_f<ST>(g[m], L.fs);  // source outside: own slot
+    } else if (bc.outlet == 0) {
+        bool ufl;
+        uint32_t u = stored_index(L, x - 1, y, z, ufl);
+        if (!ufl || u == NONE) return;
+#pragma unroll
+        for (int m = 0; m < Q; ++m)
+            if (cx(m) < 0) f[(size_t)m * L.nSpad + i] = *pop_loc<ST>(L, AFTER_EVEN, x - 1, y, z, u, m);
+    } else if (bc.outlet == 1) {
+        float g[Q];
+#pragma unroll
+        for (int m = 0; m < Q; ++m)
+            if (cx(m) >= 0) g[m] = to_f<ST>(*pop_loc<ST>(L, AFTER_EVEN, x, y, z, i, m), L.fsi);
+        pressure_face(g, 0.f, 1);
+#pragma unroll
+        for (int m = 0; m < Q; ++m)
+            if (cx(m) < 0) f[(size_t)m * L.nSpad + i] = from_f<ST>(g[m], L.fs);
     }
 }
 
@@ -128,7 +173,7 @@ struct Flip {
 };
 
 struct FlipBuf {
-    Flip* rec;
+    Flip* rec;        // [2][cap] by step parity
     float* scratch;   // [cap][19][19]
     uint8_t* valid;   // [cap][19]
     uint32_t cap;
@@ -205,9 +250,12 @@ void launch_read_fields(const Lat& L, bool after_even, double* rho, double* u, u
 
 // coupling.cu
 void launch_links(const Lat& L, const PartView& P, const LinkLists& B, cudaStream_t s);
+// inlet: null, or the boundary of the previous step, applied on the way;
+// early: the previous step's DEM is the only predecessor on the stream
 void launch_map_update(const Lat& L, const PartView& P, const Band& band, const FlipBuf& F,
-                       DevStats* st, bool after_even, int step_parity, uint2* lw, bool shared_gpu,
+                       DevStats* st, int step_parity, uint2* lw, const BC* inlet, bool early, bool shared_gpu,
                        cudaStream_t s);
+int map_update_launches(uint32_t nband, int step_parity);
 void launch_link_words(const Lat& L, uint2* lw, cudaStream_t s);
 
 // dem.cu

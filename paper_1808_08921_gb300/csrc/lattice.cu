@@ -157,6 +157,7 @@ template <bool MON, int ST>
 __global__ void __launch_bounds__(256) k_collide_even(Lat L, Mon mon) {
     pdl_wait();
     pdl_trigger();
+    if (blockIdx.x == 0 && threadIdx.x == 0) *mon.t_inlet = *mon.t_dev;
     auto* f = pops<ST>(L);
     uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
     uint32_t i0 = t * 4u;
@@ -306,6 +307,7 @@ template <bool MON, int ST>
 __global__ void __maxnreg__(72) k_collide_even_links(Lat L, Mon mon, PartView P, const uint2* __restrict__ lwp) {
     pdl_wait();
     pdl_trigger();
+    if (blockIdx.x == 0 && threadIdx.x == 0) *mon.t_inlet = *mon.t_dev;
     auto* f = pops<ST>(L);
     const uint32_t gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const uint32_t rep = gw % NREP;
@@ -472,6 +474,7 @@ template <bool MON, int ST>
 __global__ void __launch_bounds__(256, 4) k_collide_odd(Lat L, Mon mon) {
     pdl_wait();
     pdl_trigger();
+    if (blockIdx.x == 0 && threadIdx.x == 0) *mon.t_inlet = *mon.t_dev;
     auto* f = pops<ST>(L);
     uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     MonAcc a = {0, 0, 0, 0, 0, 0, 0, 0, 0};
@@ -591,48 +594,10 @@ void launch_collide(const Lat& L, const Mon& mon, bool odd, bool monitor, int ti
 
 template <bool AFTER_EVEN, int ST>
 __global__ void k_inlet_outlet(Lat L, BC bc) {
-    auto* f = pops<ST>(L);
     __shared__ float s_drho;
-    // the density the step ends with: t + 1, counted by the map update
     if (threadIdx.x == 0) s_drho = (float)source_drho(bc.src, *bc.t_dev);
     __syncthreads();
-    int plane = L.ny * L.nz;
-    int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= 2 * plane) return;
-    int side = k >= plane;
-    int yz = side ? k - plane : k;
-    int y = yz / L.nz, z = yz - y * L.nz;
-    int x = side ? L.nx - 1 : 0;
-    bool fl;
-    uint32_t i = stored_index(L, x, y, z, fl);
-    if (!fl || i == NONE) return;
-    if (side == 0) {
-        if (bc.inlet != 0) return;
-        float g[Q];
-#pragma unroll
-        for (int m = 0; m < Q; ++m)
-            if (cx(m) <= 0) g[m] = to_f<ST>(*pop_loc<ST>(L, AFTER_EVEN, x, y, z, i, m), L.fsi);
-        pressure_face(g, s_drho, 0);
-#pragma unroll
-        for (int m = 0; m < Q; ++m)
-            if (cx(m) > 0) f[(size_t)m * L.nSpad + i] = from_f<ST>(g[m], L.fs);  // source outside: own slot
-    } else if (bc.outlet == 0) {
-        bool ufl;
-        uint32_t u = stored_index(L, x - 1, y, z, ufl);
-        if (!ufl || u == NONE) return;
-#pragma unroll
-        for (int m = 0; m < Q; ++m)
-            if (cx(m) < 0) f[(size_t)m * L.nSpad + i] = *pop_loc<ST>(L, AFTER_EVEN, x - 1, y, z, u, m);
-    } else if (bc.outlet == 1) {
-        float g[Q];
-#pragma unroll
-        for (int m = 0; m < Q; ++m)
-            if (cx(m) >= 0) g[m] = to_f<ST>(*pop_loc<ST>(L, AFTER_EVEN, x, y, z, i, m), L.fsi);
-        pressure_face(g, 0.f, 1);
-#pragma unroll
-        for (int m = 0; m < Q; ++m)
-            if (cx(m) < 0) f[(size_t)m * L.nSpad + i] = from_f<ST>(g[m], L.fs);
-    }
+    inlet_outlet_node<AFTER_EVEN, ST>(L, bc, s_drho, blockIdx.x * blockDim.x + threadIdx.x);
 }
 
 void launch_inlet_outlet(const Lat& L, const BC& bc, bool after_even, cudaStream_t s) {
