@@ -22,32 +22,12 @@
 //     knowns through the transposed Zou-He formulas; at a zero-gradient
 //     outlet it adds the unknowns' adjoint to the upstream node.
 // Populations are deviations g = n - w rho_f throughout (the derivatives are
-// the same).  The forward states come from the product path itself: the
-// snapshot kernel reads the natural populations out of the AA layout.
+// the same).  The forward states come from the product path itself: its
+// collide kernels write out the natural populations they read.
 #include "common.cuh"
 #include "kernels.cuh"
 
 namespace lbmdem {
-
-// natural populations of every fluid stored node, [19][nSpad] FP32
-template <bool AFTER_EVEN, int ST>
-__global__ void k_adj_snapshot(Lat L, float* nat) {
-    uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= L.nS || !fluid_bit(L, i)) return;
-    int x, y, z;
-    unpack_coord(L.coord[i], x, y, z);
-#pragma unroll
-    for (int m = 0; m < Q; ++m)
-        nat[(size_t)m * L.nSpad + i] = to_f<ST>(*pop_loc<ST>(L, AFTER_EVEN, x, y, z, i, m), L.fsi);
-}
-
-void launch_adj_snapshot(const Lat& L, bool after_even, float* nat, cudaStream_t s) {
-    unsigned blocks = (L.nS + 255) / 256;
-    if (!blocks) return;
-#define LBMDEM_SN(AE, ST) k_adj_snapshot<AE, ST><<<blocks, 256, 0, s>>>(L, nat)
-    LBMDEM_BY_STATE(LBMDEM_SN);
-#undef LBMDEM_SN
-}
 
 // neighbour table: nbr[m][i] = compact index of x_i + c_m if fluid, else NONE
 __global__ void k_adj_nbr(Lat L, uint32_t* nbr) {

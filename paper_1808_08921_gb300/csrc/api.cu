@@ -627,6 +627,16 @@ static bool inlet_outlet_active(const lbmdem_ctx* c) {
 // layout paints the owners by the same rule from the same positions)
 static uint32_t tested_band(const lbmdem_ctx* c) { return c->any_mobile ? c->nband : 0u; }
 
+// The spheres' motion: nothing to do beside a fluid whose spheres are all fixed.
+static bool dem_active(const lbmdem_ctx* c) { return c->any_mobile || !c->lbm; }
+
+// Whether a step takes its links.  They drive free spheres; fixed ones
+// bounce every link with a zero wall velocity, which leaves the populations as
+// they are, so only the force and torque sums are left, and of those only
+// the last step's can ever be read (64 x 64 x 512 column of fixed spheres,
+// R 11.4: 28 us of 95 per step).
+static bool links_taken(const lbmdem_ctx* c, bool last) { return c->nwarps && (c->any_mobile || last); }
+
 // Where the inlet / outlet of a step runs: as a kernel of its own beside the
 // DEM (the step leaves a complete state), or inside the next step's first
 // kernel (only where the next step follows at once).
@@ -635,35 +645,45 @@ enum { INLET_NOW = 0, INLET_NEXT = 1 };
 // kernels one step issues: map update, collide, links (if any surface entries
 // and the step's links are not in the collide kernel), inlet/outlet (if any
 // and not left to the next step), DEM
-static int64_t kernels_per_step(const lbmdem_ctx* c, int parity, int inlet = INLET_NOW) {
-    int64_t k = dem_launches(c->np, c->p.dem_substeps);
+static int64_t kernels_per_step(const lbmdem_ctx* c, int parity, int inlet = INLET_NOW, bool last = true) {
+    int64_t k = dem_active(c) ? dem_launches(c->np, c->p.dem_substeps) : 0;
     if (c->lbm) {
         k += map_update_launches(tested_band(c), parity);
         k += c->nS ? 1 : 0;
-        k += c->nwarps && !links_in_collide(c, parity) ? 1 : 0;
+        k += links_taken(c, last) && !links_in_collide(c, parity) ? 1 : 0;
         k += inlet_outlet_active(c) && inlet == INLET_NOW ? 1 : 0;
     }
     return k;
 }
 
 // inlet: where this step's inlet / outlet runs; follows: the step continues a
-// run whose previous step ended with its DEM and left its inlet / outlet, if
-// there is one, to this step
-static void enqueue_step(lbmdem_ctx* c, int parity, bool monitor, int inlet = INLET_NOW, bool follows = false) {
+// run whose previous step left its inlet / outlet, if there is one, to this
+// step; last: the step's forces can be read; snap: where the state before the
+// step goes (null: nowhere)
+static void enqueue_step(lbmdem_ctx* c, int parity, bool monitor, int inlet, bool follows, bool last,
+                         float* snap = nullptr) {
     cudaStream_t s = c->stream;
     bool tm = c->timing;
     size_t e = 0;
-    c->launches += kernels_per_step(c, parity, inlet);
+    c->launches += kernels_per_step(c, parity, inlet, last);
     if (c->lbm) {
         Lat L = make_lat(c);
         PartView P = make_part(c);
         Band B{c->band_coord.p, c->band_cand.p, c->band_slack.p, tested_band(c)};
         FlipBuf F{c->flip_rec.p, c->flip_scratch.p, c->flip_valid.p, c->flip_cap};
         DevStats* sd = c->st.p;
-        BC bc{c->p.inlet, c->p.outlet, c->src, &sd->t_inlet};
+        const BC bc{c->p.inlet, c->p.outlet, c->src, &sd->t_end[parity]};
+        const BC bc_prev{c->p.inlet, c->p.outlet, c->src, &sd->t_end[parity ^ 1]};
+        const bool links = links_taken(c, last);
+        bool fused = links && links_in_collide(c, parity);
+        if (fused && snap) {  // the kernel with links writes no snapshot
+            fused = false;
+            c->launches += 1;
+        }
+        if (!links) P.n = 0;  // nor the spheres' tables
         if (tm) record_pair_begin(c, 2, e);
         launch_map_update(L, P, B, F, sd, parity, c->fused_links ? c->linkw.p : nullptr,
-                          follows && inlet_outlet_active(c) ? &bc : nullptr, follows, c->batched, s);
+                          follows && inlet_outlet_active(c) ? &bc_prev : nullptr, follows, c->batched, s);
         if (tm) record_pair_end(c, e);
         Mon mon{};
         mon.acc = sd->mon;
@@ -671,7 +691,6 @@ static void enqueue_step(lbmdem_ctx* c, int parity, bool monitor, int inlet = IN
         mon.status = &sd->status;
         mon.probe_sum = c->p.probe_x >= 0 && !c->suppress_probe ? c->probe.p : nullptr;
         mon.t_dev = &sd->t;
-        mon.t_inlet = &sd->t_inlet;
         mon.pA0 = c->pA0;
         mon.pA1 = c->pA1;
         mon.pB0 = c->pB0;
@@ -680,14 +699,13 @@ static void enqueue_step(lbmdem_ctx* c, int parity, bool monitor, int inlet = IN
             cudaMemsetAsync(sd->mon, 0, sizeof(double) * 6, s);
             cudaMemsetAsync(&sd->max_u_bits, 0, sizeof(uint32_t), s);
         }
-        const bool fused = links_in_collide(c, parity);
         if (tm) record_pair_begin(c, parity == 1 ? 0 : 5, e);
         if (fused)
             launch_collide_even_links(L, mon, P, c->linkw.p, monitor, c->p.tile > 0 ? c->p.tile : 64, s);
         else
-            launch_collide(L, mon, parity == 1, monitor, c->p.tile > 0 ? c->p.tile : 64, s);
+            launch_collide(L, mon, parity == 1, monitor, snap, c->p.tile > 0 ? c->p.tile : 64, s);
         if (tm) record_pair_end(c, e);
-        if (!fused) {
+        if (links && !fused) {
             LinkLists LL{c->surf_link.p, c->warp_p.p, c->chunk_dir.p, c->nwarps};
             if (tm) record_pair_begin(c, 1, e);
             launch_links(L, P, LL, s);
@@ -696,7 +714,11 @@ static void enqueue_step(lbmdem_ctx* c, int parity, bool monitor, int inlet = IN
         // the inlet/outlet only needs this step's populations and the DEM only
         // this step's link sums: they run side by side, the boundary on a
         // side stream joined before the next step
-        if (inlet_outlet_active(c) && inlet == INLET_NOW) {
+        if (inlet_outlet_active(c) && inlet == INLET_NOW && !dem_active(c)) {
+            if (tm) record_pair_begin(c, 3, e);
+            launch_inlet_outlet(L, bc, parity == 0, s);
+            if (tm) record_pair_end(c, e);
+        } else if (inlet_outlet_active(c) && inlet == INLET_NOW) {
             cudaEventRecord(c->ev_fork, s);
             cudaStreamWaitEvent(c->side, c->ev_fork, 0);
             size_t e2 = 0;
@@ -712,6 +734,7 @@ static void enqueue_step(lbmdem_ctx* c, int parity, bool monitor, int inlet = IN
             return;
         }
     }
+    if (!dem_active(c)) return;
     Dem D = make_dem(c);
     if (tm) record_pair_begin(c, 4, e);
     launch_dem_step(D, s);
@@ -727,7 +750,8 @@ template <class Monitored>
 static void enqueue_run(lbmdem_ctx* c, int n, int p0, Monitored monitored) {
     for (int k = 0; k < n; ++k) {
         const bool last = k == n - 1;
-        enqueue_step(c, (p0 + k) & 1, monitored(k), last || c->timing ? INLET_NOW : INLET_NEXT, k > 0 && !c->timing);
+        enqueue_step(c, (p0 + k) & 1, monitored(k), last || c->timing ? INLET_NOW : INLET_NEXT, k > 0 && !c->timing,
+                     last || c->timing);
     }
 }
 
@@ -1458,7 +1482,10 @@ int lbm_dem_batch_step(lbmdem_batch* b, const int64_t* steps) {
         BCK(cudaStreamWaitEvent(c->stream, b->done, 0));
         if (rem[i] <= 0) continue;
         for (int64_t k = 0; k < rem[i]; ++k)  // a pair's even step leaves its inlet to the odd one
-            c->launches += kernels_per_step(c, (int)(k & 1), k % 2 == 0 && k + 1 < rem[i] ? INLET_NEXT : INLET_NOW);
+        {
+            const bool last = k % 2 == 1 || k + 1 == rem[i];
+            c->launches += kernels_per_step(c, (int)(k & 1), last ? INLET_NOW : INLET_NEXT, last);
+        }
         c->launches += (rem[i] + 1) / 2;  // loop control
         if (c->p.monitor_every > 0) c->mon_step = c->t + rem[i] - 1;
         c->t += rem[i];  // corrected from the device count by lbm_dem_batch_sync if a loop stopped early
@@ -1548,6 +1575,16 @@ int lbm_dem_adjoint(lbmdem_ctx* c, int64_t steps, int32_t every, const double* t
         int64_t n = std::min<int64_t>(every, steps - g * every);
         if (int r = lbm_dem_step(c, n)) return r;
     }
+    // the reverse sweep's memory, mapped while the forward run is on the GPU
+    const size_t nbytes = (size_t)Q * c->nSpad * sizeof(float);
+    DBuf<float> nat, adj, adj2;
+    DBuf<uint32_t> nbr;
+    DBuf<double> grads;
+    CK(nat.alloc((size_t)Q * c->nSpad * (size_t)every));
+    CK(adj.alloc((size_t)Q * c->nSpad));
+    CK(adj2.alloc((size_t)Q * c->nSpad));
+    CK(nbr.alloc((size_t)(Q - 1) * c->nSpad));
+    CK(grads.alloc(GRAD_COPIES + 1));  // omega derivative copies, then the amplitude's
     std::vector<double> trace((size_t)(t0 + steps));
     int64_t len = 0;
     if (int r = lbm_dem_read_probe(c, trace.data(), t0 + steps, &len)) return r;
@@ -1561,27 +1598,13 @@ int lbm_dem_adjoint(lbmdem_ctx* c, int64_t steps, int32_t every, const double* t
         dl[(size_t)k] = 2.0 * e;
         if (trace_out) trace_out[k] = p;
     }
-    // probe-plane fluid nodes (static: every sphere is fixed)
-    int64_t np_plane = 0;
-    {
-        std::vector<uint32_t> fb(c->nSpad / 32), coord(c->nSpad);
-        CK(cudaMemcpy(fb.data(), c->fbits.p, sizeof(uint32_t) * fb.size(), cudaMemcpyDeviceToHost));
-        CK(cudaMemcpy(coord.data(), c->coord.p, sizeof(uint32_t) * coord.size(), cudaMemcpyDeviceToHost));
-        for (uint32_t i = 0; i < c->nS; ++i)
-            if ((fb[i >> 5] >> (i & 31) & 1u) && (int)(coord[i] >> 20) == c->p.probe_x) ++np_plane;
-    }
+    // probe-plane fluid nodes (static: every sphere is fixed), counted by the probe
+    double np_plane = 0.0;
+    CK(cudaMemcpyAsync(&np_plane, c->probe.p + 2 * t0 + 1, sizeof(double), cudaMemcpyDeviceToHost, s));
+    CK(cudaStreamSynchronize(s));
     if (np_plane == 0) return fail(c, LBMDEM_ERR_STATE, "adjoint: probe plane without fluid");
     // backward: recompute each segment from its checkpoint, keeping the
     // natural populations of every step, then walk the adjoint back
-    const size_t nbytes = (size_t)Q * c->nSpad * sizeof(float);
-    DBuf<float> nat, adj, adj2;
-    DBuf<uint32_t> nbr;
-    DBuf<double> grads;
-    CK(nat.alloc((size_t)Q * c->nSpad * (size_t)every));
-    CK(adj.alloc((size_t)Q * c->nSpad));
-    CK(adj2.alloc((size_t)Q * c->nSpad));
-    CK(nbr.alloc((size_t)(Q - 1) * c->nSpad));
-    CK(grads.alloc(GRAD_COPIES + 1));  // omega derivative copies, then the amplitude's
     CK(cudaMemsetAsync(adj.p, 0, nbytes, s));
     CK(cudaMemsetAsync(grads.p, 0, (GRAD_COPIES + 1) * sizeof(double), s));
     launch_adj_nbr(make_lat(c), nbr.p, s);
@@ -1595,20 +1618,23 @@ int lbm_dem_adjoint(lbmdem_ctx* c, int64_t steps, int32_t every, const double* t
         CK(cudaMemcpyAsync(&c->st.p->t, &tdev, sizeof(tdev), cudaMemcpyHostToDevice, s));
         c->t = tg;
         Lat L = make_lat(c);
+        // the trace is already complete; the forces are those of the last step
+        // recomputed
+        c->suppress_probe = true;
         for (int64_t k = 0; k < n; ++k) {
-            launch_adj_snapshot(L, (c->t & 1) == 1, nat.p + (size_t)Q * c->nSpad * k, s);
-            c->suppress_probe = true;  // the trace is already complete
-            enqueue_step(c, (int)(c->t & 1), false);
-            c->suppress_probe = false;
+            const bool last = k == n - 1;
+            enqueue_step(c, (int)(c->t & 1), false, last ? INLET_NOW : INLET_NEXT, k > 0, last && g == 0,
+                         nat.p + (size_t)Q * c->nSpad * k);
             c->t += 1;
         }
+        c->suppress_probe = false;
         CK(cudaGetLastError());
         AdjArgs A{L, nbr.p, adj.p, c->p.inlet, c->p.outlet, c->p.probe_x};
         for (int64_t k = n - 1; k >= 0; --k) {
             int64_t t = tg + k;  // step t -> t + 1
             A.adj = adj.p;
             launch_adj_boundary(A, source_shape(c->src, t + 1), grads.p + GRAD_COPIES, s);
-            float dlt = (float)(dl[(size_t)(t - t0)] * cs2 / (double)np_plane);
+            float dlt = (float)(dl[(size_t)(t - t0)] * cs2 / np_plane);
             launch_adj_step(A, nat.p + (size_t)Q * c->nSpad * k, adj2.p, dlt, grads.p, s);
             adj.swap(adj2);
         }

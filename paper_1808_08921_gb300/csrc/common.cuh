@@ -322,7 +322,7 @@ struct DevStats {
     double mon[6];           // sum rho, sum rho u, max|u|, step
     uint32_t max_u_bits;
     uint32_t layout_fresh;   // 1 from a layout build until the first step's DEM
-    unsigned long long t_inlet;  // steps completed when the last collided step ends: the source time of its inlet
+    unsigned long long t_end[2];  // by step parity: t at the end of the last such step, the source time of its inlet
 };
 
 // Programmatic dependent launch.  The kernels of a step are launched with

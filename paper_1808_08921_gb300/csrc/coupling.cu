@@ -327,7 +327,7 @@ __global__ void __launch_bounds__(256) k_map_band(MapArgs A) {
     const Lat& L = A.L;
     if ((int)blockIdx.x < A.io_blocks) {
         __shared__ float s_drho;
-        if (threadIdx.x == 0) s_drho = (float)source_drho(A.bc.src, A.st->t_inlet);
+        if (threadIdx.x == 0) s_drho = (float)source_drho(A.bc.src, *A.bc.t_dev);
         __syncthreads();
         pdl_wait();
         pdl_trigger();
@@ -338,7 +338,7 @@ __global__ void __launch_bounds__(256) k_map_band(MapArgs A) {
     const float slack = k < A.band.n ? A.band.slack[k] : 0.f;
     pdl_wait();
     pdl_trigger();
-    if (k == 0) A.st->t += 1ull;  // the step starts: t counts it from here on
+    if (k == 0) A.st->t_end[A.par] = A.st->t += 1ull;  // the step starts: t counts it from here on
     {
         const uint32_t prev = min(A.st->nflip[A.par ^ 1], A.F.cap), stride = (gridDim.x - A.io_blocks) * blockDim.x;
         for (uint32_t w = k; w < prev; w += stride) {

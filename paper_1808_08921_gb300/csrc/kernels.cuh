@@ -13,7 +13,6 @@ struct Mon {
     uint32_t* status;
     double* probe_sum;              // [2 * capacity] (sum drho, count) per step, or null
     const unsigned long long* t_dev;
-    unsigned long long* t_inlet;
     uint32_t pA0, pA1, pB0, pB1;    // compact index ranges of the probe plane
 };
 
@@ -240,7 +239,7 @@ struct Dem {
 };
 
 // lattice.cu
-void launch_collide(const Lat& L, const Mon& mon, bool odd, bool monitor, int tile, cudaStream_t s);
+void launch_collide(const Lat& L, const Mon& mon, bool odd, bool monitor, float* snap, int tile, cudaStream_t s);
 void launch_collide_even_links(const Lat& L, const Mon& mon, const PartView& P, const uint2* lw, bool monitor,
                                int tile, cudaStream_t s);
 void launch_inlet_outlet(const Lat& L, const BC& bc, bool after_even, cudaStream_t s);
@@ -251,7 +250,7 @@ void launch_read_fields(const Lat& L, bool after_even, double* rho, double* u, u
 // coupling.cu
 void launch_links(const Lat& L, const PartView& P, const LinkLists& B, cudaStream_t s);
 // inlet: null, or the boundary of the previous step, applied on the way;
-// early: the previous step's DEM is the only predecessor on the stream
+// early: the previous step's last kernel is the only predecessor on the stream
 void launch_map_update(const Lat& L, const PartView& P, const Band& band, const FlipBuf& F,
                        DevStats* st, int step_parity, uint2* lw, const BC* inlet, bool early, bool shared_gpu,
                        cudaStream_t s);
@@ -270,7 +269,6 @@ struct AdjArgs {
     float* adj;           // [19][nSpad] adjoint of the natural populations
     int inlet, outlet, probe_x;
 };
-void launch_adj_snapshot(const Lat& L, bool after_even, float* nat, cudaStream_t s);
 void launch_adj_nbr(const Lat& L, uint32_t* nbr, cudaStream_t s);
 void launch_adj_boundary(const AdjArgs& A, double shape, double* d_amp, cudaStream_t s);
 void launch_adj_step(const AdjArgs& A, const float* nat, float* out, float dl, double* d_omega, cudaStream_t s);

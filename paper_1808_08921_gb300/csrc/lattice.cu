@@ -153,11 +153,13 @@ __device__ __forceinline__ void mon_flush(const MonAcc& a, const Mon& mon, bool 
 // Even step: node-local.  Each thread owns 4 consecutive compact nodes and
 // moves them with 128-bit loads and stores; solid nodes inside a quad are
 // processed harmlessly (their slots are never read while they are solid).
-template <bool MON, int ST>
-__global__ void __launch_bounds__(256) k_collide_even(Lat L, Mon mon) {
+// SNAP: the natural populations the step starts from also go to snap
+// ([19][nSpad] FP32) for the reverse sweep, from the registers they are
+// collided in.
+template <bool MON, int ST, bool SNAP>
+__global__ void __launch_bounds__(256) k_collide_even(Lat L, Mon mon, float* snap) {
     pdl_wait();
     pdl_trigger();
-    if (blockIdx.x == 0 && threadIdx.x == 0) *mon.t_inlet = *mon.t_dev;
     auto* f = pops<ST>(L);
     uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
     uint32_t i0 = t * 4u;
@@ -173,6 +175,10 @@ __global__ void __launch_bounds__(256) k_collide_even(Lat L, Mon mon) {
 #pragma unroll
         for (int m = 0; m < Q; ++m)
             v[m] = ld4<ST>(f + (size_t)m * L.nSpad + i0, L.fsi);
+        if (SNAP) {
+#pragma unroll
+            for (int m = 0; m < Q; ++m) __stcs(reinterpret_cast<float4*>(snap + (size_t)m * L.nSpad + i0), v[m]);
+        }
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             float g[Q];
@@ -307,7 +313,6 @@ template <bool MON, int ST>
 __global__ void __maxnreg__(72) k_collide_even_links(Lat L, Mon mon, PartView P, const uint2* __restrict__ lwp) {
     pdl_wait();
     pdl_trigger();
-    if (blockIdx.x == 0 && threadIdx.x == 0) *mon.t_inlet = *mon.t_dev;
     auto* f = pops<ST>(L);
     const uint32_t gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const uint32_t rep = gw % NREP;
@@ -470,11 +475,10 @@ struct LineProbe {
 // its own slot m when x - c_m is solid or outside), collides, and scatters
 // direction m to slot m of x + c_m (or its own slot opp(m)).  Each thread
 // reads and writes the same 19 locations, so the update is in place.
-template <bool MON, int ST>
-__global__ void __launch_bounds__(256, 4) k_collide_odd(Lat L, Mon mon) {
+template <bool MON, int ST, bool SNAP>
+__global__ void __launch_bounds__(256, 4) k_collide_odd(Lat L, Mon mon, float* snap) {
     pdl_wait();
     pdl_trigger();
-    if (blockIdx.x == 0 && threadIdx.x == 0) *mon.t_inlet = *mon.t_dev;
     auto* f = pops<ST>(L);
     uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     MonAcc a = {0, 0, 0, 0, 0, 0, 0, 0, 0};
@@ -544,6 +548,10 @@ __global__ void __launch_bounds__(256, 4) k_collide_odd(Lat L, Mon mon) {
             g[m] = to_f<ST>(f[off], L.fsi);
         }
         g[18] = to_f<ST>(f[18u * L.nSpad + i], L.fsi);
+        if (SNAP) {
+#pragma unroll
+            for (int m = 0; m < Q; ++m) __stcs(snap + (uint32_t)m * L.nSpad + i, g[m]);
+        }
         float drho, jx, jy, jz;
         bgk(g, L.tau_inv, L.rho_f, drho, jx, jy, jz);
 #pragma unroll
@@ -563,30 +571,28 @@ __global__ void __launch_bounds__(256, 4) k_collide_odd(Lat L, Mon mon) {
 }
 
 template <int ST>
-static void launch_collide_st(const Lat& L, const Mon& mon, bool odd, bool monitor, int tile, cudaStream_t s) {
-    if (!odd) {
-        uint32_t threads = (L.nS + 3) / 4;
-        uint32_t blocks = (threads + tile - 1) / tile;
-        if (monitor)
-            launch_pdl(k_collide_even<true, ST>, blocks, tile, s, L, mon);
-        else
-            launch_pdl(k_collide_even<false, ST>, blocks, tile, s, L, mon);
+static void launch_collide_st(const Lat& L, const Mon& mon, bool odd, bool monitor, float* snap, int tile,
+                              cudaStream_t s) {
+    const uint32_t threads = odd ? L.nS : (L.nS + 3) / 4, blocks = (threads + tile - 1) / tile;
+    if (odd) {
+        if (snap) launch_pdl(k_collide_odd<false, ST, true>, blocks, tile, s, L, mon, snap);
+        else if (monitor) launch_pdl(k_collide_odd<true, ST, false>, blocks, tile, s, L, mon, snap);
+        else launch_pdl(k_collide_odd<false, ST, false>, blocks, tile, s, L, mon, snap);
     } else {
-        uint32_t blocks = (L.nS + tile - 1) / tile;
-        if (monitor)
-            launch_pdl(k_collide_odd<true, ST>, blocks, tile, s, L, mon);
-        else
-            launch_pdl(k_collide_odd<false, ST>, blocks, tile, s, L, mon);
+        if (snap) launch_pdl(k_collide_even<false, ST, true>, blocks, tile, s, L, mon, snap);
+        else if (monitor) launch_pdl(k_collide_even<true, ST, false>, blocks, tile, s, L, mon, snap);
+        else launch_pdl(k_collide_even<false, ST, false>, blocks, tile, s, L, mon, snap);
     }
 }
 
-// tile: threads per block (64, 128 or 256; the kernels are bounded for 256)
-void launch_collide(const Lat& L, const Mon& mon, bool odd, bool monitor, int tile, cudaStream_t s) {
+// tile: threads per block (64, 128 or 256; the kernels are bounded for 256);
+// snap: null, or where the state before the step goes (not with monitor)
+void launch_collide(const Lat& L, const Mon& mon, bool odd, bool monitor, float* snap, int tile, cudaStream_t s) {
     if (L.nS == 0) return;
     switch (L.st) {
-        case 0: launch_collide_st<0>(L, mon, odd, monitor, tile, s); break;
-        case 1: launch_collide_st<1>(L, mon, odd, monitor, tile, s); break;
-        default: launch_collide_st<2>(L, mon, odd, monitor, tile, s); break;
+        case 0: launch_collide_st<0>(L, mon, odd, monitor, snap, tile, s); break;
+        case 1: launch_collide_st<1>(L, mon, odd, monitor, snap, tile, s); break;
+        default: launch_collide_st<2>(L, mon, odd, monitor, snap, tile, s); break;
     }
 }
 

@@ -68,3 +68,27 @@ def test_solid_fraction_where_a_segment_meets_many_spheres():
     ref = o.probe()[:STEPS] / 3.0
     o.close()
     assert np.abs(tr - ref).max() <= 1e-3 * np.abs(ref - ref[0]).max()
+
+
+@pytest.mark.parametrize("storage", [lbmdem.F32, lbmdem.BF16_DEV])
+@pytest.mark.parametrize("R", [3.2, 8.5])
+def test_snapshots_of_short_and_odd_runs(storage, R):
+    """The reverse sweep's states from the collide kernels: checkpoints every
+    2 steps, a run shorter than the interval and an odd last segment give the
+    gradient of one segment (FP32 rounding of the same sums); spheres on both
+    sides of the radius at which the even steps take their links themselves."""
+    n = 4 if R < 5 else 2
+    w = workloads.random_small(3, nx=48, ny=24, nz=24, n=n, R=R, tau=0.7, mobile=False)
+    assert len(w.R) == n
+    w.amplitude, w.omega, w.probe_x = 1e-3, 0.2, 5
+    for steps in (7, 24):
+        target = np.full(steps, 1.0 / 3.0)
+        out = []
+        for every in (2, 10, 60):
+            g = lbmdem.Sim.from_workload(w, storage=storage, skin=0.1)
+            out.append(g.adjoint(steps, every, target))
+            g.close()
+        for o in out[1:]:
+            assert np.array_equal(o[3], out[0][3])
+            assert abs(o[1] - out[0][1]) <= 1e-6 * abs(out[0][1])
+            assert abs(o[2] - out[0][2]) <= 1e-6 * abs(out[0][2])
