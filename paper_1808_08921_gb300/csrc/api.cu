@@ -19,6 +19,7 @@
 #include <mutex>
 #include <cuda.h>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/lbmdem.h"
@@ -34,6 +35,7 @@ template <class T>
 struct DBuf {
     T* p = nullptr;
     size_t n = 0;
+    bool own = true;  // false: a part of a Slab
     DBuf() = default;
     DBuf(const DBuf&) = delete;
     DBuf& operator=(const DBuf&) = delete;
@@ -52,13 +54,49 @@ struct DBuf {
     }
     cudaError_t ensure(size_t count) { return count <= n && p ? cudaSuccess : alloc(count + count / 8); }
     void release() {
-        if (p) cudaFree(p);
+        if (p && own) cudaFree(p);
         p = nullptr;
         n = 0;
+        own = true;
+    }
+    void view(T* q, size_t count) {
+        release();
+        p = q;
+        n = count;
+        own = false;
     }
     void swap(DBuf& o) {
         std::swap(p, o.p);
         std::swap(n, o.n);
+        std::swap(own, o.own);
+    }
+};
+
+// Several arrays in one device allocation: an allocation and its release take
+// 65 us here whatever its size up to some 100 MB, and a context holds some
+// sixty arrays.  take() is called in two passes over the same arrays: a first
+// one that measures, then, after reserve(), one that hands the parts out.
+struct Slab {
+    DBuf<uint8_t> mem;
+    size_t off = 0;
+    bool measuring = true;
+    void measure() {
+        off = 0;
+        measuring = true;
+    }
+    // keeps a block that is large enough; the parts of an earlier one are gone
+    cudaError_t reserve() {
+        cudaError_t e = off <= mem.n ? cudaSuccess : mem.alloc(off);
+        off = 0;
+        measuring = false;
+        return e;
+    }
+    template <class T>
+    void take(DBuf<T>& b, size_t count) {
+        count = std::max<size_t>(count, 1);
+        off = (off + 255) / 256 * 256;
+        if (!measuring) b.view(reinterpret_cast<T*>(mem.p + off), count);
+        off += sizeof(T) * count;
     }
 };
 
@@ -69,7 +107,23 @@ constexpr int NGROUP = 6;  // collide odd, links, map update, inlet/outlet, DEM,
 // cell-list buffers (per-sphere cell, per-cell counts, starts, fill cursors
 // and the spheres in cell order)
 struct CellBufs {
+    Slab slab;
     DBuf<int> of, count, start, fill, order;
+    cudaError_t ensure(size_t np, size_t ncell) {
+        if (of.n >= np && fill.n >= ncell && of.p) return cudaSuccess;
+        auto parts = [&] {
+            slab.take(of, np);
+            slab.take(order, np);
+            slab.take(count, ncell + 1);
+            slab.take(start, ncell + 1);
+            slab.take(fill, ncell);
+        };
+        slab.measure();
+        parts();
+        cudaError_t e = slab.reserve();
+        if (e == cudaSuccess) parts();
+        return e;
+    }
 };
 
 struct lbmdem_ctx {
@@ -88,6 +142,7 @@ struct lbmdem_ctx {
     Source src{};
     double skin = 0.25, dem_skin = 0.5, trigger = 0.0, hard = 0.0;
     // lattice
+    Slab lat_slab;
     DBuf<int32_t> owner;
     DBuf<unsigned long long> paint_best;
     DBuf<uint8_t> deep, band;
@@ -116,6 +171,7 @@ struct lbmdem_ctx {
     uint32_t flip_cap = 0;
     uint32_t pA0 = 0, pA1 = 0, pB0 = 0, pB1 = 0;
     // particles
+    Slab part_slab;
     int np = 0;
     bool any_mobile = false;
     double Rmax = 0;
@@ -131,6 +187,7 @@ struct lbmdem_ctx {
     DBuf<int> nb_cnt, nb_j, nb_cnt2, nb_j2;
     DBuf<int8_t> nb_sh, nb_sh2;
     DBuf<float4> nb_dref, nb_ft, nb_dref2, nb_ft2;
+    Slab nb_slab;
     DBuf<int> nb_slot, dem_foreign, dem_slots;  // exchange slots of the one-launch DEM
     DBuf<float> nb_R;
     DBuf<uint16_t> dem_push;
@@ -139,6 +196,7 @@ struct lbmdem_ctx {
     CellBufs cells;       // the DEM's cell list (cells 2 R + dem_skin wide)
     CellBufs band_cells;  // cells R + skin wide: a band node's candidates lie within R + skin
     // stats, probe
+    DBuf<uint8_t> stage;  // read-outs
     DBuf<DevStats> st;
     DevStats* st_host = nullptr;
     DBuf<double> probe;
@@ -336,12 +394,8 @@ static int build_cell_grid(lbmdem_ctx* c, CellGrid& G, double h, CellBufs& B) {
     G.h.z = (double)c->p.nz / G.nc.z;
     G.lo.y = G.lo.z = 0;
     int ncell = G.nc.x * G.nc.y * G.nc.z;
-    CK(B.of.ensure(np));
-    CK(B.count.ensure(ncell + 1));
+    CK(B.ensure(np, ncell));
     CK(c->scan_tmp.ensure(scan_tmp_size((size_t)ncell + 1)));  // allocated at init with a lattice
-    CK(B.start.ensure(ncell + 1));
-    CK(B.fill.ensure(ncell));
-    CK(B.order.ensure(np));
     launch_cells(c->Xref.p, np, G, B.of.p, B.count.p, B.start.p, B.fill.p, B.order.p, c->scan_tmp.p, c->stream);
     CK(cudaGetLastError());
     return 0;
@@ -354,11 +408,23 @@ static int build_cells(lbmdem_ctx* c) { return build_cell_grid(c, c->grid, 2.0 *
 static int build_neighbours(lbmdem_ctx* c, bool carry) {
     int np = c->np;
     size_t ne = (size_t)std::max(np, 1) * c->nbmax;
-    CK(c->nb_cnt2.ensure(np));
-    CK(c->nb_j2.ensure(ne));
-    CK(c->nb_sh2.ensure(4 * ne));
-    CK(c->nb_dref2.ensure(ne));
-    CK(c->nb_ft2.ensure(ne));
+    if (c->nb_R.n < ne || !c->nb_R.p) {  // a larger packing than before (nothing to carry over)
+        auto parts = [&] {
+            for (DBuf<int>* b : {&c->nb_cnt, &c->nb_cnt2}) c->nb_slab.take(*b, np);
+            for (DBuf<int>* b : {&c->nb_j, &c->nb_j2, &c->nb_slot}) c->nb_slab.take(*b, ne);
+            for (DBuf<int8_t>* b : {&c->nb_sh, &c->nb_sh2}) c->nb_slab.take(*b, 4 * ne);
+            for (DBuf<float4>* b : {&c->nb_dref, &c->nb_dref2, &c->nb_ft, &c->nb_ft2}) c->nb_slab.take(*b, ne);
+            c->nb_slab.take(c->nb_R, ne);
+            c->nb_slab.take(c->dem_push, (size_t)std::max(np, 1) * DEM_MAX_CTAS);
+            c->nb_slab.take(c->dem_foreign, DEM_MAX_CTAS);
+            c->nb_slab.take(c->dem_slots, 1);
+        };
+        c->nb_slab.measure();
+        parts();
+        CK(c->nb_slab.reserve());
+        parts();
+        carry = false;
+    }
     NbBuild B{};
     B.X = c->Xref.p;
     B.R = c->Rd.p;
@@ -378,7 +444,6 @@ static int build_neighbours(lbmdem_ctx* c, bool carry) {
     B.old_j = have_old ? c->nb_j.p : nullptr;
     B.old_sh = have_old ? c->nb_sh.p : nullptr;
     B.old_ft = have_old ? c->nb_ft.p : nullptr;
-    CK(c->nb_R.ensure(ne));
     B.nR = c->nb_R.p;
     B.status = &c->st.p->status;
     launch_nb_build(B, c->stream);
@@ -389,10 +454,6 @@ static int build_neighbours(lbmdem_ctx* c, bool carry) {
     c->nb_dref.swap(c->nb_dref2);
     c->nb_ft.swap(c->nb_ft2);
     // exchange slots; every caller synchronises the stream before it launches a step
-    CK(c->nb_slot.ensure(ne));
-    CK(c->dem_push.ensure((size_t)std::max(np, 1) * DEM_MAX_CTAS));
-    CK(c->dem_foreign.ensure(DEM_MAX_CTAS));
-    CK(c->dem_slots.ensure(1));
     launch_dem_ghosts(make_dem(c), c->nb_slot.p, c->dem_push.p, c->dem_foreign.p, c->dem_slots.p, c->stream);
     CK(cudaGetLastError());
     CK(cudaMemcpyAsync(c->dem_slots_host, c->dem_slots.p, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
@@ -414,7 +475,12 @@ static int build_layout(lbmdem_ctx* c, bool fresh) {
     if (fresh) fill_i32(c->owner.p, OWNER_FLUID, c->N, s);
     CK(cudaMemsetAsync(c->deep.p, 0, c->N, s));
     CK(cudaMemsetAsync(c->band.p, 0, c->N, s));
-    if (fresh) CK(c->paint_best.alloc(c->N));
+    if (fresh) {  // the old populations are dead: their memory serves where it is large enough
+        if (c->f.n >= sizeof(unsigned long long) * c->N)
+            c->paint_best.view(reinterpret_cast<unsigned long long*>(c->f.p), c->N);
+        else
+            CK(c->paint_best.alloc(c->N));
+    }
     PaintArgs PA{c->Xref.p, c->Rd.p, nx, ny, nz, px, c->skin, fresh ? c->owner.p : nullptr,
                  fresh ? c->paint_best.p : nullptr, c->deep.p, c->band.p};
     launch_paint(PA, c->np, c->N, s);
@@ -449,8 +515,10 @@ static int build_layout(lbmdem_ctx* c, bool fresh) {
     CK(cudaGetLastError());
     // populations
     const size_t esz = c->p.storage == LBMDEM_F32 ? 4 : 2;
-    CK(c->f2.alloc((size_t)Q * nSpad * esz));
-    CK(cudaMemsetAsync(c->f2.p, 0, esz * Q * nSpad, s));  // zero deviations: rest at rho_f
+    const size_t fbytes = (size_t)Q * nSpad * esz;
+    if (fresh && c->f.n >= fbytes && c->f.n <= 2 * fbytes) c->f.swap(c->f2);  // a new packing reuses the memory
+    else CK(c->f2.alloc(fbytes));
+    CK(cudaMemsetAsync(c->f2.p, 0, fbytes, s));  // zero deviations: rest at rho_f
     Lat Lnew = make_lat(c);
     Lnew.nA = nA;
     Lnew.nS = nS;
@@ -588,6 +656,23 @@ static int build_layout(lbmdem_ctx* c, bool fresh) {
     }
     CK(cudaStreamSynchronize(s));
     destroy_graph(c);
+    return 0;
+}
+
+// ------------------------------------------------------------ read-out staging
+
+// Device memory for a read-out of `bytes`: up to STAGE_KEEP bytes stay with
+// the context from one read-out to the next (three allocations and releases
+// took 0.2 ms of a read of the fields), larger ones are `own`'s and end with it.
+constexpr size_t STAGE_KEEP = (size_t)64 << 20;
+static int stage(lbmdem_ctx* c, size_t bytes, DBuf<uint8_t>& own, uint8_t** p) {
+    if (bytes <= STAGE_KEEP) {
+        CK(c->stage.ensure(bytes));
+        *p = c->stage.p;
+    } else {
+        CK(own.alloc(bytes));
+        *p = own.p;
+    }
     return 0;
 }
 
@@ -951,11 +1036,22 @@ int lbm_dem_init(const lbmdem_params* pp, lbmdem_ctx** out) {
     *c->dem_slots_host = 0;
     if (cudaMemset(c->st.p, 0, sizeof(DevStats)) != cudaSuccess) return bail(LBMDEM_ERR_CUDA);
     if (c->lbm) {
-        if (c->owner.alloc(c->N) || c->deep.alloc(c->N) || c->band.alloc(c->N) || c->rec.alloc(c->W) ||
-            c->rec2.alloc(c->W) || c->maskB.alloc(c->W) || c->maskB2.alloc(c->W) ||
-            c->cntA.alloc(c->W + 1) || c->cntB.alloc(c->W + 1) || c->flip.alloc(2 * c->W) ||
-            c->scan_tmp.alloc(scan_tmp_size(std::max(c->W + 1, (size_t)1 << 24))) ||
-            c->band_count.alloc(1))
+        auto parts = [&] {
+            Slab& m = c->lat_slab;
+            m.take(c->owner, c->N);
+            m.take(c->deep, c->N);
+            m.take(c->band, c->N);
+            for (DBuf<uint4>* b : {&c->rec, &c->rec2}) m.take(*b, c->W);
+            for (DBuf<uint32_t>* b : {&c->maskB, &c->maskB2}) m.take(*b, c->W);
+            for (DBuf<uint32_t>* b : {&c->cntA, &c->cntB}) m.take(*b, c->W + 1);
+            m.take(c->flip, 2 * c->W);
+            m.take(c->scan_tmp, scan_tmp_size(std::max(c->W + 1, (size_t)1 << 24)));
+            m.take(c->band_count, 1);
+        };
+        c->lat_slab.measure();
+        parts();
+        if (c->lat_slab.reserve() == cudaSuccess) parts();
+        else
             return bail(LBMDEM_ERR_OOM);
     }
     c->src.waveform = LBMDEM_SINE;
@@ -1021,39 +1117,46 @@ int lbm_dem_set_packing(lbmdem_ctx* c, int32_t n, const double* X, const double*
     c->have_packing = false;
     destroy_graph(c);
     size_t nn = std::max(n, 1);
-    CK(c->Xref.alloc(3 * nn));
-    CK(c->Fh.alloc(3 * NREP * nn));
-    CK(c->Th.alloc(3 * NREP * nn));
-    CK(c->Fh_prev.alloc(3 * nn));
-    CK(c->Th_prev.alloc(3 * nn));
-    CK(c->Fa.alloc(nn));
-    CK(c->Ta.alloc(nn));
-    CK(c->dX.alloc(nn));
-    CK(c->dXc.alloc(nn));
-    CK(c->dXb.alloc(2 * nn));
-    CK(c->V.alloc(nn));
-    CK(c->Om.alloc(nn));
-    CK(c->q.alloc(nn));
-    CK(c->Vhb.alloc(2 * nn));
-    CK(c->Whb.alloc(2 * nn));
-    CK(c->Fc.alloc(nn));
-    CK(c->Tc.alloc(nn));
-    CK(c->xf.alloc(nn));
-    CK(c->ab.alloc((Q - 1) * nn));
-    CK(c->pk.alloc(3 * nn));
-    CK(c->org.alloc(nn));
-    CK(c->orgw.alloc(nn));
-    CK(c->R.alloc(nn));
-    CK(c->Rd.alloc(nn));
-    CK(c->invm.alloc(nn));
-    CK(c->invI.alloc(nn));
-    CK(c->fixed.alloc(nn));
+    // one block: what the host fills, what starts at zero, work arrays
+    size_t filled = 0, zeroed = 0;
+    auto parts = [&] {
+        Slab& m = c->part_slab;
+        m.take(c->Xref, 3 * nn);
+        m.take(c->V, nn);
+        m.take(c->Om, nn);
+        m.take(c->q, nn);
+        m.take(c->Rd, nn);
+        m.take(c->R, nn);
+        m.take(c->invm, nn);
+        m.take(c->invI, nn);
+        m.take(c->fixed, nn);
+        filled = m.off;
+        for (DBuf<float4>* b : {&c->dX, &c->dXc}) m.take(*b, nn);
+        for (DBuf<double>* b : {&c->Fh, &c->Th}) m.take(*b, 3 * NREP * nn);
+        for (DBuf<double>* b : {&c->Fh_prev, &c->Th_prev}) m.take(*b, 3 * nn);
+        zeroed = m.off;
+        for (DBuf<float4>* b : {&c->Fa, &c->Ta, &c->Fc, &c->Tc, &c->xf}) m.take(*b, nn);
+        for (DBuf<float4>* b : {&c->dXb, &c->Vhb, &c->Whb}) m.take(*b, 2 * nn);
+        m.take(c->ab, (Q - 1) * nn);
+        m.take(c->pk, 3 * nn);
+        for (DBuf<int4>* b : {&c->org, &c->orgw}) m.take(*b, nn);
+    };
+    c->part_slab.measure();
+    parts();
+    CK(c->part_slab.reserve());
+    parts();
     // host staging of the per-sphere constants (marshalling only)
-    std::vector<double> Xv(3 * nn, 0.0);
-    std::vector<float4> Vv(nn), Wv(nn), qv(nn), zero4(nn);
-    std::vector<float> Rv(nn, 1.f), imv(nn, 0.f), iIv(nn, 0.f);
-    std::vector<double> Rdv(nn, 1.0);
-    std::vector<uint8_t> fx(nn, 0);
+    std::vector<uint8_t> host(filled, 0);
+    uint8_t* base = c->part_slab.mem.p;
+    auto at = [&](auto& b) { return reinterpret_cast<std::remove_reference_t<decltype(b.p)>>(host.data() + ((uint8_t*)b.p - base)); };
+    double *Xv = at(c->Xref), *Rdv = at(c->Rd);
+    float4 *Vv = at(c->V), *Wv = at(c->Om), *qv = at(c->q);
+    float *Rv = at(c->R), *imv = at(c->invm), *iIv = at(c->invI);
+    uint8_t* fx = at(c->fixed);
+    for (size_t i = 0; i < nn; ++i) {
+        Rv[i] = 1.f;
+        Rdv[i] = 1.0;
+    }
     bool mobile = false;
     for (int i = 0; i < n; ++i) {
         for (int a = 0; a < 3; ++a) Xv[3 * i + a] = X[3 * i + a];
@@ -1075,24 +1178,10 @@ int lbm_dem_set_packing(lbmdem_ctx* c, int32_t n, const double* X, const double*
         imv[i] = (float)(1.0 / m);
         iIv[i] = (float)(1.0 / (0.4 * m * Rh[i] * Rh[i]));
     }
-    for (size_t i = 0; i < nn; ++i) zero4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     c->any_mobile = mobile;
     cudaStream_t s = c->stream;
-    CK(cudaMemcpyAsync(c->Xref.p, Xv.data(), sizeof(double) * 3 * nn, cudaMemcpyHostToDevice, s));
-    CK(cudaMemcpyAsync(c->V.p, Vv.data(), sizeof(float4) * nn, cudaMemcpyHostToDevice, s));
-    CK(cudaMemcpyAsync(c->Om.p, Wv.data(), sizeof(float4) * nn, cudaMemcpyHostToDevice, s));
-    CK(cudaMemcpyAsync(c->q.p, qv.data(), sizeof(float4) * nn, cudaMemcpyHostToDevice, s));
-    CK(cudaMemcpyAsync(c->dX.p, zero4.data(), sizeof(float4) * nn, cudaMemcpyHostToDevice, s));
-    CK(cudaMemcpyAsync(c->dXc.p, zero4.data(), sizeof(float4) * nn, cudaMemcpyHostToDevice, s));
-    CK(cudaMemcpyAsync(c->R.p, Rv.data(), sizeof(float) * nn, cudaMemcpyHostToDevice, s));
-    CK(cudaMemcpyAsync(c->Rd.p, Rdv.data(), sizeof(double) * nn, cudaMemcpyHostToDevice, s));
-    CK(cudaMemcpyAsync(c->invm.p, imv.data(), sizeof(float) * nn, cudaMemcpyHostToDevice, s));
-    CK(cudaMemcpyAsync(c->invI.p, iIv.data(), sizeof(float) * nn, cudaMemcpyHostToDevice, s));
-    CK(cudaMemcpyAsync(c->fixed.p, fx.data(), nn, cudaMemcpyHostToDevice, s));
-    CK(cudaMemsetAsync(c->Fh.p, 0, sizeof(double) * 3 * NREP * nn, s));
-    CK(cudaMemsetAsync(c->Th.p, 0, sizeof(double) * 3 * NREP * nn, s));
-    CK(cudaMemsetAsync(c->Fh_prev.p, 0, sizeof(double) * 3 * nn, s));
-    CK(cudaMemsetAsync(c->Th_prev.p, 0, sizeof(double) * 3 * nn, s));
+    CK(cudaMemcpyAsync(base, host.data(), filled, cudaMemcpyHostToDevice, s));
+    CK(cudaMemsetAsync(base + filled, 0, zeroed - filled, s));
     CK(cudaMemsetAsync(c->st.p, 0, sizeof(DevStats), s));
     if (int r = build_cells(c)) return r;
     if (int r = build_neighbours(c, false)) return r;
@@ -1689,7 +1778,6 @@ int lbm_dem_adjoint_psm(lbmdem_ctx* c, int64_t steps, int32_t every, const doubl
     CK(eps.alloc(N));
     const bool grads_wanted = dL_dtau || dL_damp || dL_dX;
     CK(ck.alloc(grads_wanted ? QN * (size_t)nseg : 1));
-    CK(snap.alloc(grads_wanted ? QN * (size_t)every : 1));
     CK(X.alloc(3 * (size_t)std::max(n, 1)));
     CK(trace.alloc((size_t)steps));
     CK(grads.alloc(GRAD_COPIES + 1));  // tau derivative copies, then the amplitude's
@@ -1716,6 +1804,11 @@ int lbm_dem_adjoint_psm(lbmdem_ctx* c, int64_t steps, int32_t every, const doubl
         g0.swap(g1);
     }
     CK(cudaGetLastError());
+    if (grads_wanted) {  // the reverse sweep's memory, mapped while the forward run is on the GPU
+        CK(snap.alloc(QN * (size_t)every));
+        CK(lam0.alloc(QN));
+        CK(lam1.alloc(QN));
+    }
     std::vector<double> tr((size_t)steps);
     CK(cudaMemcpyAsync(tr.data(), trace.p, sizeof(double) * steps, cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
@@ -1731,8 +1824,6 @@ int lbm_dem_adjoint_psm(lbmdem_ctx* c, int64_t steps, int32_t every, const doubl
     if (loss) *loss = L;
     if (!dL_dtau && !dL_damp && !dL_dX) return lbm_dem_status(c);  // the forward loss alone
     // backward: recompute each segment from its checkpoint, then the adjoint
-    CK(lam0.alloc(QN));
-    CK(lam1.alloc(QN));
     CK(cudaMemsetAsync(lam0.p, 0, sizeof(float) * QN, s));
     for (int64_t seg = nseg - 1; seg >= 0; --seg) {
         const int64_t tg = seg * every, m = std::min<int64_t>(every, steps - tg);
@@ -1822,9 +1913,10 @@ int lbm_dem_read_particles(lbmdem_ctx* c, double* X, double* V, double* Om, doub
     if (c->np == 0) return 0;
     CK(cudaSetDevice(c->p.device));
     size_t n = c->np;
-    DBuf<double> buf;
-    CK(buf.alloc(19 * n));
-    double* d = buf.p;
+    DBuf<uint8_t> own;
+    uint8_t* sp = nullptr;
+    if (int r = stage(c, sizeof(double) * 19 * n, own, &sp)) return r;
+    double* d = reinterpret_cast<double*>(sp);
     Dem D = make_dem(c);
     k_particles_out<<<(unsigned)((n + 127) / 128), 128, 0, c->stream>>>(D, c->Fh.p, c->Th.p, d, d + 3 * n,
                                                                       d + 6 * n, d + 9 * n, d + 13 * n,
@@ -1848,18 +1940,19 @@ int lbm_dem_read_fields(lbmdem_ctx* c, double* rho, double* u, uint8_t* solid) {
     if (!c->lbm) return fail(c, LBMDEM_ERR_STATE, "fluid is off");
     CK(cudaSetDevice(c->p.device));
     size_t N = c->N;
-    DBuf<double> dr, du;
-    DBuf<uint8_t> ds;
-    if (rho) CK(dr.alloc(N));
-    if (u) CK(du.alloc(3 * N));
-    if (solid) CK(ds.alloc(N));
+    DBuf<uint8_t> own;
+    uint8_t* sp = nullptr;
+    const size_t br = rho ? sizeof(double) * N : 0, bu = u ? 3 * sizeof(double) * N : 0;
+    if (int r = stage(c, std::max<size_t>(br + bu + (solid ? N : 0), 1), own, &sp)) return r;
+    double* dr = reinterpret_cast<double*>(sp);
+    double* du = reinterpret_cast<double*>(sp + br);
+    uint8_t* ds = sp + br + bu;
     Lat L = make_lat(c);
-    launch_read_fields(L, (c->t & 1) == 1, rho ? dr.p : nullptr, u ? du.p : nullptr, solid ? ds.p : nullptr,
-                       c->stream);
+    launch_read_fields(L, (c->t & 1) == 1, rho ? dr : nullptr, u ? du : nullptr, solid ? ds : nullptr, c->stream);
     CK(cudaGetLastError());
-    if (rho) CK(cudaMemcpyAsync(rho, dr.p, sizeof(double) * N, cudaMemcpyDeviceToHost, c->stream));
-    if (u) CK(cudaMemcpyAsync(u, du.p, sizeof(double) * 3 * N, cudaMemcpyDeviceToHost, c->stream));
-    if (solid) CK(cudaMemcpyAsync(solid, ds.p, N, cudaMemcpyDeviceToHost, c->stream));
+    if (rho) CK(cudaMemcpyAsync(rho, dr, br, cudaMemcpyDeviceToHost, c->stream));
+    if (u) CK(cudaMemcpyAsync(u, du, bu, cudaMemcpyDeviceToHost, c->stream));
+    if (solid) CK(cudaMemcpyAsync(solid, ds, N, cudaMemcpyDeviceToHost, c->stream));
     CK(cudaStreamSynchronize(c->stream));
     return lbm_dem_status(c);
 }
@@ -1870,13 +1963,15 @@ int lbm_dem_read_plane_means(lbmdem_ctx* c, double* rho, double* jx) {
     if (!c->lbm) return fail(c, LBMDEM_ERR_STATE, "fluid is off");
     CK(cudaSetDevice(c->p.device));
     const int nx = c->p.nx;
-    DBuf<double> d;
-    CK(d.alloc(3 * (size_t)nx));
-    CK(cudaMemsetAsync(d.p, 0, sizeof(double) * 3 * nx, c->stream));
-    launch_plane_sums(make_lat(c), (c->t & 1) == 1, d.p, c->stream);
+    DBuf<uint8_t> own;
+    uint8_t* sp = nullptr;
+    if (int r = stage(c, sizeof(double) * 3 * nx, own, &sp)) return r;
+    double* d = reinterpret_cast<double*>(sp);
+    CK(cudaMemsetAsync(d, 0, sizeof(double) * 3 * nx, c->stream));
+    launch_plane_sums(make_lat(c), (c->t & 1) == 1, d, c->stream);
     CK(cudaGetLastError());
     std::vector<double> h(3 * (size_t)nx);
-    CK(cudaMemcpyAsync(h.data(), d.p, sizeof(double) * 3 * nx, cudaMemcpyDeviceToHost, c->stream));
+    CK(cudaMemcpyAsync(h.data(), d, sizeof(double) * 3 * nx, cudaMemcpyDeviceToHost, c->stream));
     CK(cudaStreamSynchronize(c->stream));
     for (int x = 0; x < nx; ++x) {
         double n = h[3 * x + 2];
@@ -1899,11 +1994,13 @@ int lbm_dem_read_probe(lbmdem_ctx* c, double* trace, int64_t max_len, int64_t* l
     if (c->p.probe_x < 0 || !c->lbm || c->t == 0 || !trace || max_len <= 0) return lbm_dem_status(c);
     CK(cudaSetDevice(c->p.device));
     int64_t n = std::min<int64_t>(max_len, c->t);
-    DBuf<double> d;
-    CK(d.alloc(n));
-    k_probe_out<<<(unsigned)((n + 255) / 256), 256, 0, c->stream>>>(c->probe.p, n, c->p.rho_f, d.p);
+    DBuf<uint8_t> own;
+    uint8_t* sp = nullptr;
+    if (int r = stage(c, sizeof(double) * n, own, &sp)) return r;
+    double* d = reinterpret_cast<double*>(sp);
+    k_probe_out<<<(unsigned)((n + 255) / 256), 256, 0, c->stream>>>(c->probe.p, n, c->p.rho_f, d);
     CK(cudaGetLastError());
-    CK(cudaMemcpyAsync(trace, d.p, sizeof(double) * n, cudaMemcpyDeviceToHost, c->stream));
+    CK(cudaMemcpyAsync(trace, d, sizeof(double) * n, cudaMemcpyDeviceToHost, c->stream));
     CK(cudaStreamSynchronize(c->stream));
     return lbm_dem_status(c);
 }
@@ -1920,10 +2017,12 @@ __global__ void k_monitors_out(const DevStats* s, double rho_f, double* out) {
 int lbm_dem_read_monitors(lbmdem_ctx* c, double out[6]) {
     if (!c || !out) return LBMDEM_ERR_INVALID_ARG;
     if (!c->lbm) return fail(c, LBMDEM_ERR_STATE, "fluid is off");
-    DBuf<double> d;
-    CK(d.alloc(6));
-    k_monitors_out<<<1, 1, 0, c->stream>>>(c->st.p, c->p.rho_f, d.p);
-    CK(cudaMemcpyAsync(out, d.p, sizeof(double) * 5, cudaMemcpyDeviceToHost, c->stream));
+    DBuf<uint8_t> own;
+    uint8_t* sp = nullptr;
+    if (int r = stage(c, sizeof(double) * 6, own, &sp)) return r;
+    double* d = reinterpret_cast<double*>(sp);
+    k_monitors_out<<<1, 1, 0, c->stream>>>(c->st.p, c->p.rho_f, d);
+    CK(cudaMemcpyAsync(out, d, sizeof(double) * 5, cudaMemcpyDeviceToHost, c->stream));
     CK(cudaStreamSynchronize(c->stream));
     out[5] = (double)c->mon_step;
     return lbm_dem_status(c);
