@@ -93,8 +93,12 @@ __global__ void __launch_bounds__(256) k_adj_step(AdjArgs A, const float* nat, f
     const Lat& L = A.L;
     uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     float dw = 0.f;
-    if (i < L.nS && fluid_bit(L, i)) {
+    if (i < L.nS) {
+        // fluid: a packing of fixed spheres stores no other node
         const size_t P = L.nSpad;
+        float g[Q];
+#pragma unroll
+        for (int m = 0; m < Q; ++m) g[m] = __ldcs(nat + (size_t)m * P + i);
         float s[Q];
 #pragma unroll
         for (int j = 0; j < Q - 1; ++j) {
@@ -102,9 +106,6 @@ __global__ void __launch_bounds__(256) k_adj_step(AdjArgs A, const float* nat, f
             s[j] = d != NONE ? A.adj[(size_t)j * P + d] : A.adj[(size_t)opp(j) * P + i];
         }
         s[18] = A.adj[(size_t)18 * P + i];
-        float g[Q];
-#pragma unroll
-        for (int m = 0; m < Q; ++m) g[m] = nat[(size_t)m * P + i];
         const RevMoments M = rev_moments(g, L.rho_f);
         RevSums R;
         float sw = s[18] * (g[18] - wt(18) * (M.drho - M.rho * M.uu15));

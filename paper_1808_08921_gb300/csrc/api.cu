@@ -147,11 +147,11 @@ struct lbmdem_ctx {
     DBuf<unsigned long long> paint_best;
     DBuf<uint8_t> deep, band;
     DBuf<uint4> rec, rec2;
-    DBuf<uint32_t> maskB, maskB2, cntA, cntB, scan_tmp;
+    DBuf<uint32_t> fluid, fluid2, cnt, scan_tmp;
     DBuf<uint32_t> flip;  // [2][W] map changes of the last two steps
     DBuf<uint8_t> f, f2;  // populations, 4 or 2 bytes each
     DBuf<uint32_t> coord, fbits;
-    uint32_t nA = 0, nS = 0, nSpad = 0;
+    uint32_t nS = 0, nSpad = 0;
     DBuf<uint32_t> band_coord, band_count, band_coord2, slack_hist;
     DBuf<int4> band_cand, band_cand2;
     DBuf<float> band_slack, band_slack2;
@@ -162,14 +162,14 @@ struct lbmdem_ctx {
     DBuf<uint8_t> chunk_dir;  // direction (| flag) of every 32-record chunk
     uint32_t nwarps = 0;
     uint32_t nlink_raw = 0;  // link records before padding
-    DBuf<uint2> linkw;       // link word of every stored node (even steps' links in the collide kernel)
+    DBuf<uint2> linkw;       // link word of every stored node
     bool fused_links = false;
     bool batched = false;  // steps being captured into a batch graph (columns share the GPU)
     DBuf<Flip> flip_rec;
     DBuf<float> flip_scratch;
     DBuf<uint8_t> flip_valid;
     uint32_t flip_cap = 0;
-    uint32_t pA0 = 0, pA1 = 0, pB0 = 0, pB1 = 0;
+    uint32_t probe0 = 0, probe1 = 0;
     // particles
     Slab part_slab;
     int np = 0;
@@ -268,7 +268,6 @@ static Lat make_lat(lbmdem_ctx* c) {
     L.nz = c->p.nz;
     L.nw = c->nw;
     L.px = c->p.inlet == LBMDEM_X_PERIODIC;
-    L.nA = c->nA;
     L.nS = c->nS;
     L.nSpad = c->nSpad;
     L.f = c->f.p;
@@ -276,7 +275,7 @@ static Lat make_lat(lbmdem_ctx* c) {
     L.fs = L.st == 2 ? 4096.0f : 1.0f;  // FP16: deviations 1e-8 .. 16 stay normal
     L.fsi = 1.0f / L.fs;
     L.rec = c->rec.p;
-    L.maskB = c->maskB.p;
+    L.fluid = c->fluid.p;
     L.flip = c->flip.p;
     L.coord = c->coord.p;
     L.fbits = c->fbits.p;
@@ -490,28 +489,22 @@ static int build_layout(lbmdem_ctx* c, bool fresh) {
         c->paint_best.release();
     }
     // words into the spare record set (the current one is needed for the copy)
-    LayoutArgs LA{nx, ny, nz, c->nw, c->owner.p, c->deep.p, c->band.p, c->rec2.p, c->maskB2.p,
-                  c->cntA.p, c->cntB.p, nullptr};
-    CK(cudaMemsetAsync(c->cntA.p, 0, sizeof(uint32_t) * (c->W + 1), s));
-    CK(cudaMemsetAsync(c->cntB.p, 0, sizeof(uint32_t) * (c->W + 1), s));
+    LayoutArgs LA{nx, ny, nz, c->nw, c->owner.p, c->any_mobile ? c->deep.p : nullptr, c->band.p, c->rec2.p, c->fluid2.p, c->cnt.p, nullptr};
+    CK(cudaMemsetAsync(c->cnt.p, 0, sizeof(uint32_t) * (c->W + 1), s));
     launch_words(LA, s);
-    exclusive_scan(c->cntA.p, c->cntA.p, c->W + 1, c->scan_tmp.p, s);
-    exclusive_scan(c->cntB.p, c->cntB.p, c->W + 1, c->scan_tmp.p, s);
+    exclusive_scan(c->cnt.p, c->cnt.p, c->W + 1, c->scan_tmp.p, s);
     CK(cudaGetLastError());
-    uint32_t nA = 0, nB = 0;
-    if (int r = read_u32(c, c->cntA.p + c->W, &nA)) return r;
-    if (int r = read_u32(c, c->cntB.p + c->W, &nB)) return r;
-    uint64_t nS64 = (uint64_t)nA + nB;
-    if (nS64 >= 0xffffffe0ull) return fail(c, LBMDEM_ERR_INVALID_ARG, "lattice too large");
-    uint32_t nS = (uint32_t)nS64;
+    uint32_t nS = 0;
+    if (int r = read_u32(c, c->cnt.p + c->W, &nS)) return r;
+    if (nS >= 0xffffffe0u) return fail(c, LBMDEM_ERR_INVALID_ARG, "lattice too large");
     uint32_t nSpad = std::max<uint32_t>(32u, (nS + 31u) & ~31u);
     if ((uint64_t)Q * nSpad >= (1ull << 32))  // the kernels address populations with 32-bit offsets
         return fail(c, LBMDEM_ERR_INVALID_ARG, "lattice too large: %u stored nodes", nS);
-    launch_words_bases(LA, nA, s);
+    launch_words_bases(LA, s);
     CK(c->coord.ensure(nSpad));
     CK(c->fbits.ensure(nSpad / 32));
     LA.coord = c->coord.p;
-    launch_coords(LA, nA, nSpad, c->fbits.p, s);
+    launch_coords(LA, nSpad, c->fbits.p, s);
     CK(cudaGetLastError());
     // populations
     const size_t esz = c->p.storage == LBMDEM_F32 ? 4 : 2;
@@ -520,12 +513,13 @@ static int build_layout(lbmdem_ctx* c, bool fresh) {
     else CK(c->f2.alloc(fbytes));
     CK(cudaMemsetAsync(c->f2.p, 0, fbytes, s));  // zero deviations: rest at rho_f
     Lat Lnew = make_lat(c);
-    Lnew.nA = nA;
     Lnew.nS = nS;
     Lnew.nSpad = nSpad;
     Lnew.f = c->f2.p;
     Lnew.rec = c->rec2.p;
-    Lnew.maskB = c->maskB2.p;
+    Lnew.fluid = c->fluid2.p;
+    Lnew.coord = c->coord.p;
+    Lnew.fbits = c->fbits.p;
     if (!fresh && c->f.p) {
         Lat Lold = make_lat(c);
         launch_gather_old(Lnew, Lold, s);
@@ -534,8 +528,7 @@ static int build_layout(lbmdem_ctx* c, bool fresh) {
     c->f.swap(c->f2);
     c->f2.release();
     c->rec.swap(c->rec2);
-    c->maskB.swap(c->maskB2);
-    c->nA = nA;
+    c->fluid.swap(c->fluid2);
     c->nS = nS;
     c->nSpad = nSpad;
     // band list and its candidate spheres
@@ -625,11 +618,9 @@ static int build_layout(lbmdem_ctx* c, bool fresh) {
     const bool want = c->p.link_mode == 2 ||
                       (c->p.link_mode == 0 && c->p.storage == LBMDEM_F32 && c->Rmax >= 8.0);
     c->fused_links = want && c->nwarps > 0 && np <= LW_MAX_SPHERES && wide;
-    if (c->fused_links) {
-        CK(c->linkw.ensure(nSpad));
-        launch_link_words(make_lat(c), c->linkw.p, s);
-        CK(cudaGetLastError());
-    }
+    CK(c->linkw.ensure(nSpad));
+    launch_link_words(make_lat(c), c->linkw.p, s);
+    CK(cudaGetLastError());
     // conversion scratch
     uint32_t cap = c->p.max_flips > 0 ? (uint32_t)c->p.max_flips
                                       : std::min<uint32_t>(1u << 20, std::max<uint32_t>(4096u, nband / 8));
@@ -639,20 +630,18 @@ static int build_layout(lbmdem_ctx* c, bool fresh) {
         CK(c->flip_valid.alloc((size_t)cap * Q));
         c->flip_cap = cap;
     }
-    // probe plane ranges in compact order
-    c->pA0 = c->pA1 = c->pB0 = c->pB1 = 0;
+    // probe plane's range in compact order
+    c->probe0 = c->probe1 = 0;
     int xp = c->p.probe_x;
     if (xp >= 0 && xp < nx) {
         uint4 r0, r1;
-        CK(cudaMemcpyAsync(&r0, c->rec.p + (size_t)xp * ny * c->nw, sizeof(uint4), cudaMemcpyDeviceToHost, s));
+        const size_t wp = (size_t)ny * c->nw;
+        CK(cudaMemcpyAsync(&r0, c->rec.p + xp * wp, sizeof(uint4), cudaMemcpyDeviceToHost, s));
         if (xp + 1 < nx)
-            CK(cudaMemcpyAsync(&r1, c->rec.p + (size_t)(xp + 1) * ny * c->nw, sizeof(uint4),
-                               cudaMemcpyDeviceToHost, s));
+            CK(cudaMemcpyAsync(&r1, c->rec.p + (xp + 1) * wp, sizeof(uint4), cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
-        c->pA0 = r0.z;
-        c->pA1 = xp + 1 < nx ? r1.z : nA;
-        c->pB0 = r0.w;
-        c->pB1 = xp + 1 < nx ? r1.w : nS;
+        c->probe0 = r0.y;
+        c->probe1 = xp + 1 < nx ? r1.y : nS;
     }
     CK(cudaStreamSynchronize(s));
     destroy_graph(c);
@@ -767,7 +756,7 @@ static void enqueue_step(lbmdem_ctx* c, int parity, bool monitor, int inlet, boo
         }
         if (!links) P.n = 0;  // nor the spheres' tables
         if (tm) record_pair_begin(c, 2, e);
-        launch_map_update(L, P, B, F, sd, parity, c->fused_links ? c->linkw.p : nullptr,
+        launch_map_update(L, P, B, F, sd, parity, c->linkw.p,
                           follows && inlet_outlet_active(c) ? &bc_prev : nullptr, follows, c->batched, s);
         if (tm) record_pair_end(c, e);
         Mon mon{};
@@ -776,10 +765,8 @@ static void enqueue_step(lbmdem_ctx* c, int parity, bool monitor, int inlet, boo
         mon.status = &sd->status;
         mon.probe_sum = c->p.probe_x >= 0 && !c->suppress_probe ? c->probe.p : nullptr;
         mon.t_dev = &sd->t;
-        mon.pA0 = c->pA0;
-        mon.pA1 = c->pA1;
-        mon.pB0 = c->pB0;
-        mon.pB1 = c->pB1;
+        mon.p0 = c->probe0;
+        mon.p1 = c->probe1;
         if (monitor) {
             cudaMemsetAsync(sd->mon, 0, sizeof(double) * 6, s);
             cudaMemsetAsync(&sd->max_u_bits, 0, sizeof(uint32_t), s);
@@ -788,7 +775,7 @@ static void enqueue_step(lbmdem_ctx* c, int parity, bool monitor, int inlet, boo
         if (fused)
             launch_collide_even_links(L, mon, P, c->linkw.p, monitor, c->p.tile > 0 ? c->p.tile : 64, s);
         else
-            launch_collide(L, mon, parity == 1, monitor, snap, c->p.tile > 0 ? c->p.tile : 64, s);
+            launch_collide(L, mon, parity == 1, monitor, c->linkw.p, snap, c->p.tile > 0 ? c->p.tile : 64, s);
         if (tm) record_pair_end(c, e);
         if (links && !fused) {
             LinkLists LL{c->surf_link.p, c->warp_p.p, c->chunk_dir.p, c->nwarps};
@@ -1042,8 +1029,8 @@ int lbm_dem_init(const lbmdem_params* pp, lbmdem_ctx** out) {
             m.take(c->deep, c->N);
             m.take(c->band, c->N);
             for (DBuf<uint4>* b : {&c->rec, &c->rec2}) m.take(*b, c->W);
-            for (DBuf<uint32_t>* b : {&c->maskB, &c->maskB2}) m.take(*b, c->W);
-            for (DBuf<uint32_t>* b : {&c->cntA, &c->cntB}) m.take(*b, c->W + 1);
+            for (DBuf<uint32_t>* b : {&c->fluid, &c->fluid2}) m.take(*b, c->W);
+            m.take(c->cnt, c->W + 1);
             m.take(c->flip, 2 * c->W);
             m.take(c->scan_tmp, scan_tmp_size(std::max(c->W + 1, (size_t)1 << 24)));
             m.take(c->band_count, 1);

@@ -5,20 +5,24 @@
 // partially used 32-byte sectors):
 //   * S  = stored nodes = every node that is fluid now or within `skin` of a
 //          sphere surface on the solid side (it may become fluid before the
-//          next re-layout).  S = A + B, where A = nodes fluid at re-layout
-//          time (lexicographic x, y, z order, indices [0, nA)) and B = the
-//          remaining stored nodes (indices [nA, nS)), so the streamed region A
-//          is dense in fluid and B is only touched where a node converted.
+//          next re-layout; in a packing of fixed spheres none does, and
+//          only the fluid nodes are stored).  Order: x, then 32-node words along z, then y, then
+//          z inside the word: a warp's 32 consecutive nodes come from a few
+//          neighbouring lines of one word (about 4 x 32 lattice nodes at 25%
+//          fluid), and the nodes of the neighbouring lines in x and y are as
+//          contiguous as its own.
 //   * f  = populations as deviations g_i = f_i - w_i rho_f, structure of
 //          arrays [19][nSpad], in place with the AA access pattern; stored as
 //          FP32, or as BF16 / FP16 scaled by a power of two (FP16: 2^12, so
 //          that deviations of 1e-8 .. 16 stay normal numbers), always
 //          collided in FP32.
-//   * rec[w] = {maskF, maskA, baseA, baseB} for every 32-node word of a
-//          z-line: fluid-now bits, region-A bits and the compact indices of the
-//          first A and B node of the word; maskB[w] holds the B bits.  The
-//          compact index of a stored node is base + popc(mask & lower bits).
-//          The word table (16 B per 32 nodes) stays resident in L2.
+//   * rec[w] = {stored bits, base, prev, next} for every 32-node word of a
+//          z-line (fixed until the next re-layout): a stored node's compact
+//          index is base + popc(stored bits & lower bits); prev and next are
+//          the indices of the nodes before the word's first and after its
+//          last one (periodic in z), so that z +- 1 needs no other record.
+//          fluid[w] holds the fluid-now bits.  The word tables (20 B per 32
+//          nodes) stay resident in L2.
 //   * coord[i] = x << 20 | y << 10 | z of compact node i.
 //   * fbits[i / 32] = fluid-now bit of compact node i.
 //   * owner[lattice index] = index of the sphere a node belongs to, or FLUID.
@@ -107,13 +111,13 @@ __host__ __device__ inline void unpack_coord(uint32_t c, int& x, int& y, int& z)
 struct Lat {
     int nx, ny, nz, nw;   // nw = 32-node words per z-line
     int px;               // x periodic
-    uint32_t nA, nS, nSpad;
+    uint32_t nS, nSpad;
     void* f;              // [19][nSpad] deviations, element type by `st`
     int st;               // storage: 0 FP32, 1 BF16, 2 FP16 (scaled by fs)
     float fs, fsi;        // storage scale and its inverse (powers of two)
-    uint4* rec;           // [nx*ny*nw] {maskF, maskA, baseA, baseB}
-    uint32_t* maskB;      // [nx*ny*nw]
-    uint32_t* flip;       // [2][nx*ny*nw] nodes the map update of a step made fluid or solid, by step parity
+    uint4* rec;           // [nx*nw*ny] {stored bits, base, prev, next}
+    uint32_t* fluid;      // [nx*nw*ny] fluid-now bits
+    uint32_t* flip;       // [2][nx*nw*ny] nodes the map update of a step made fluid or solid, by step parity
     uint32_t* coord;      // [nSpad]
     uint32_t* fbits;      // [nSpad / 32]
     int32_t* owner;       // [nx*ny*nz]
@@ -130,6 +134,12 @@ __device__ __forceinline__ int imin_small(int d, int L) {
     return d;
 }
 
+// Word of node (x, y, z).
+__device__ __forceinline__ uint32_t word_of(const Lat& L, int x, int y, int z) {
+    return ((uint32_t)x * L.nw + (uint32_t)(z >> 5)) * L.ny + y;
+}
+__device__ __forceinline__ uint32_t rec_index(const uint4& r, uint32_t bit) { return r.y + __popc(r.x & (bit - 1u)); }
+
 // Compact index of node (x+dx, y+dy, z+dz) if it is fluid now, else NONE.
 // dx, dy, dz in {-1, 0, 1}.  Out-of-range x (non-periodic) returns NONE.
 __device__ __forceinline__ uint32_t fluid_index(const Lat& L, int x, int y, int z, int dx, int dy,
@@ -141,27 +151,21 @@ __device__ __forceinline__ uint32_t fluid_index(const Lat& L, int x, int y, int 
         return NONE;
     }
     int ys = wrap1(y + dy, L.ny), zs = wrap1(z + dz, L.nz);
-    uint32_t wi = ((uint32_t)xs * L.ny + ys) * L.nw + (zs >> 5);
-    uint4 r = __ldg(&L.rec[wi]);
-    uint32_t bit = 1u << (zs & 31);
-    if (!(r.x & bit)) return NONE;
-    uint32_t low = bit - 1u;
-    if (r.y & bit) return r.z + __popc(r.y & low);
-    return r.w + __popc(__ldg(&L.maskB[wi]) & low);
+    const uint32_t wi = word_of(L, xs, ys, zs);
+    const uint4 r = __ldg(&L.rec[wi]);
+    const uint32_t bit = 1u << (zs & 31);
+    return __ldg(&L.fluid[wi]) & bit ? rec_index(r, bit) : NONE;
 }
 
-// Same for a node given directly (used outside the hot kernel; reads the
-// record with a coherent load because the map-update kernels modify it).
+// Compact index of a stored node given directly, NONE if it is not stored
+// (used outside the hot kernel; reads the fluid bits with a coherent load
+// because the map-update kernels modify them).
 __device__ __forceinline__ uint32_t stored_index(const Lat& L, int x, int y, int z, bool& fluid) {
-    uint32_t wi = ((uint32_t)x * L.ny + y) * L.nw + (z >> 5);
-    uint4 r = L.rec[wi];
-    uint32_t bit = 1u << (z & 31);
-    fluid = (r.x & bit) != 0;
-    uint32_t low = bit - 1u;
-    if (r.y & bit) return r.z + __popc(r.y & low);
-    uint32_t mb = L.maskB[wi];
-    if (mb & bit) return r.w + __popc(mb & low);
-    return NONE;
+    const uint32_t wi = word_of(L, x, y, z);
+    const uint4 r = L.rec[wi];
+    const uint32_t bit = 1u << (z & 31);
+    fluid = (L.fluid[wi] & bit) != 0;
+    return r.x & bit ? rec_index(r, bit) : NONE;
 }
 
 __device__ __forceinline__ bool fluid_bit(const Lat& L, uint32_t i) {
@@ -200,14 +204,10 @@ __device__ __forceinline__ uint32_t old_fluid_index(const Lat& L, const uint32_t
         return NONE;
     }
     int ys = wrap1(y + dy, L.ny), zs = wrap1(z + dz, L.nz);
-    uint32_t wi = ((uint32_t)xs * L.ny + ys) * L.nw + (zs >> 5);
-    uint4 r = L.rec[wi];
-    const uint32_t fl = r.x ^ flip[wi];
-    uint32_t bit = 1u << (zs & 31);
-    if (!(fl & bit)) return NONE;
-    uint32_t low = bit - 1u;
-    if (r.y & bit) return r.z + __popc(r.y & low);
-    return r.w + __popc(L.maskB[wi] & low);
+    const uint32_t wi = word_of(L, xs, ys, zs);
+    const uint4 r = L.rec[wi];
+    const uint32_t bit = 1u << (zs & 31);
+    return (L.fluid[wi] ^ flip[wi]) & bit ? rec_index(r, bit) : NONE;
 }
 
 // Location of population m of fluid node (x,y,z) with compact index i, in the

@@ -251,7 +251,7 @@ struct MapArgs {
     FlipBuf F;
     DevStats* st;
     int par;        // parity of the step (selects the queue, its counter and the flip masks)
-    uint2* lw;      // link words renewed around converted nodes (null: not kept)
+    uint2* lw;      // link words, renewed around converted nodes
     BC bc;          // the previous step's inlet / outlet,
     int io_blocks;  // applied by the first io_blocks blocks of the band kernel
 };
@@ -344,7 +344,7 @@ __global__ void __launch_bounds__(256) k_map_band(MapArgs A) {
         for (uint32_t w = k; w < prev; w += stride) {
             int x, y, z;
             unpack_coord(A.F.rec[(size_t)(A.par ^ 1) * A.F.cap + w].coord, x, y, z);
-            flip_masks(L, A.par ^ 1)[((uint32_t)x * L.ny + y) * L.nw + (z >> 5)] = 0u;
+            flip_masks(L, A.par ^ 1)[word_of(L, x, y, z)] = 0u;
         }
     }
     if (k < (uint32_t)A.P.n) {
@@ -462,8 +462,8 @@ __global__ void __launch_bounds__(256) k_map_band(MapArgs A) {
         A.F.rec[(size_t)A.par * A.F.cap + slot] = f;
         L.owner[li] = best;
         if (old == OWNER_FLUID || best == OWNER_FLUID) {
-            const uint32_t wi = ((uint32_t)x * L.ny + y) * L.nw + (z >> 5), bit = 1u << (z & 31);
-            atomicXor(&L.rec[wi].x, bit);
+            const uint32_t wi = word_of(L, x, y, z), bit = 1u << (z & 31);
+            atomicXor(&L.fluid[wi], bit);
             atomicOr(&flip_masks(L, A.par)[wi], bit);
             if (ci != NONE) atomicXor(&L.fbits[ci >> 5], 1u << (ci & 31));
         }
@@ -662,12 +662,11 @@ void launch_map_update(const Lat& L, const PartView& P, const Band& band, const 
     const unsigned blocks = io + (nb + bb - 1) / bb;
     // the queued count is read on the device: fixed grids stride over it
     const unsigned grid = shared_gpu ? 152 : 4 * 152;
-    const unsigned gthreads = MAP_THREADS + (lw ? LW_THREADS : 0);
 #define LBMDEM_MB(AE, ST)                                                              \
     do {                                                                               \
         if (early && !shared_gpu) launch_pdl(k_map_band<AE, ST>, blocks, bb, s, A);    \
         else k_map_band<AE, ST><<<blocks, bb, 0, s>>>(A);                              \
-        if (band.n) launch_pdl(k_map_gather_convert<AE, ST>, grid, gthreads, s, A);    \
+        if (band.n) launch_pdl(k_map_gather_convert<AE, ST>, grid, MAP_THREADS + LW_THREADS, s, A);    \
         if (band.n && AE) launch_pdl(k_map_scatter<ST>, grid, MAP_THREADS, s, A);      \
     } while (0)
     LBMDEM_BY_STATE(LBMDEM_MB);

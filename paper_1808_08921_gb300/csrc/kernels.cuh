@@ -13,7 +13,7 @@ struct Mon {
     uint32_t* status;
     double* probe_sum;              // [2 * capacity] (sum drho, count) per step, or null
     const unsigned long long* t_dev;
-    uint32_t pA0, pA1, pB0, pB1;    // compact index ranges of the probe plane
+    uint32_t p0, p1;                // compact index range of the probe plane
 };
 
 struct Source {
@@ -145,13 +145,15 @@ struct LinkLists {
     uint32_t nwarps;
 };
 
-// Link word of a stored node, for the even steps' links inside the collide
-// kernel (one 8-byte word per node):
+// Link word of a stored node (one 8-byte word per node), for the odd collide
+// kernel's fluid neighbours (.x) and the even steps' links inside the collide
+// kernel:
 //   .x = link mask (bit m, m < 18: the neighbour x + c_m is solid) | sphere A << 18
 //   .y = B mask (bit m: that link's neighbour belongs to sphere B) | sphere B << 18
 // Sphere indices take 14 bits; LW_NONE stands for no sphere B, and as sphere
 // A for a node whose solid neighbours belong to more than two spheres (its
-// links then read the owner map).  Built at the layout from the owner map
+// links then read the owner map).  With more spheres than LW_MAX_SPHERES the
+// indices are cut off and only the mask is used.  Built at the layout from the owner map
 // and renewed for every converted node and its 18 neighbours.
 constexpr uint32_t LW_MASK = (1u << 18) - 1u;
 constexpr uint32_t LW_NONE = 0x3fffu;
@@ -239,7 +241,8 @@ struct Dem {
 };
 
 // lattice.cu
-void launch_collide(const Lat& L, const Mon& mon, bool odd, bool monitor, float* snap, int tile, cudaStream_t s);
+void launch_collide(const Lat& L, const Mon& mon, bool odd, bool monitor, const uint2* lw, float* snap, int tile,
+                    cudaStream_t s);
 void launch_collide_even_links(const Lat& L, const Mon& mon, const PartView& P, const uint2* lw, bool monitor,
                                int tile, cudaStream_t s);
 void launch_inlet_outlet(const Lat& L, const BC& bc, bool after_even, cudaStream_t s);

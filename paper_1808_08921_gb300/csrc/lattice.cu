@@ -191,7 +191,7 @@ __global__ void __launch_bounds__(256) k_collide_even(Lat L, Mon mon, float* sna
             if ((bits >> k) & 1u) {
                 if (MON) mon_add(a, drho, jx, jy, jz, L.rho_f);
                 uint32_t i = i0 + k;
-                if ((i >= mon.pA0 && i < mon.pA1) || (i >= mon.pB0 && i < mon.pB1)) {
+                if (i >= mon.p0 && i < mon.p1) {
                     a.pdrho += drho;
                     a.pcnt += 1.f;
                 }
@@ -332,7 +332,7 @@ __global__ void __maxnreg__(72) k_collide_even_links(Lat L, Mon mon, PartView P,
         float drho, jx, jy, jz;
         bgk(g, L.tau_inv, L.rho_f, drho, jx, jy, jz);
         if (MON) mon_add(a, drho, jx, jy, jz, L.rho_f);
-        if ((i >= mon.pA0 && i < mon.pA1) || (i >= mon.pB0 && i < mon.pB1)) {
+        if (i >= mon.p0 && i < mon.p1) {
             a.pdrho += drho;
             a.pcnt += 1.f;
         }
@@ -444,140 +444,133 @@ void launch_collide_even_links(const Lat& L, const Mon& mon, const PartView& P, 
     }
 }
 
-// compact index of bit `bit` of a word record if that node is fluid now
-__device__ __forceinline__ uint32_t word_index(const uint4& r, const uint32_t* mBp, uint32_t bit) {
-    if (!(r.x & bit)) return NONE;
-    uint32_t low = bit - 1u;
-    if (r.y & bit) return r.z + __popc(r.y & low);
-    return r.w + __popc(__ldg(mBp) & low);
-}
-
-// Neighbours x + c_m of node (x, y, z) on the z-line (xs, ys): the record of
-// the word holding z serves dz = -1, 0, +1 unless z +- 1 crosses a word.
-struct LineProbe {
-    const Lat& L;
-    size_t wl;
-    int w0;
-    uint4 r0;
-    __device__ __forceinline__ LineProbe(const Lat& L_, int xs, int ys, int z) : L(L_) {
-        wl = ((size_t)xs * L.ny + ys) * L.nw;
-        w0 = z >> 5;
-        r0 = __ldg(&L.rec[wl + w0]);
-    }
-    __device__ __forceinline__ uint32_t at(int zs) const {
-        int wz = zs >> 5;
-        uint4 r = wz == w0 ? r0 : __ldg(&L.rec[wl + wz]);
-        return word_index(r, &L.maskB[wl + wz], 1u << (zs & 31));
+// Compact indices of the stored nodes at z, z + 1 and z - 1 of one z-line
+// from one population count: b = z & 31, low the bits below it; the word's
+// prev and next serve the line's neighbours outside the word.
+struct LineIndex {
+    uint32_t c, p, m;
+    __device__ __forceinline__ LineIndex(const uint4& r, uint32_t b, uint32_t low, bool top) {
+        c = r.y + __popc(r.x & low);
+        p = top ? r.w : c + ((r.x >> b) & 1u);
+        m = b == 0u ? r.z : c - ((r.x >> ((b - 1u) & 31u)) & 1u);
     }
 };
 
 // Odd step: node x gathers direction m from slot opp(m) of x - c_m (or from
 // its own slot m when x - c_m is solid or outside), collides, and scatters
-// direction m to slot m of x + c_m (or its own slot opp(m)).  Each thread
-// reads and writes the same 19 locations, so the update is in place.
+// direction m to slot m of x + c_m (or its own slot opp(m)): the population
+// leaving along m and the one arriving against it share one location, so the
+// 18 element offsets are formed once and the update is in place.  Which
+// neighbours are fluid is read from the node's link word (a solid neighbour is
+// a link), where they are stored from nine word records: five lines that give
+// three neighbours each and four that give one.  Testing each neighbour's
+// fluid bit in its record, with two index regions per record and a second
+// record past a word's end, took 174 us on the 128 x 128 x 1024 column and 157
+// on 160^3 (all fluid), this form 160 and 138.  152 B per fluid node plus its
+// 8 B link word: 98 us and 97 us at the copy rate; it waits for its chain of
+// three dependent loads at 64 registers (80 leave fewer warps: 164 and 144;
+// 48 spill: 225 and 172).
 template <bool MON, int ST, bool SNAP>
-__global__ void __launch_bounds__(256, 4) k_collide_odd(Lat L, Mon mon, float* snap) {
+__global__ void __launch_bounds__(256, 4) k_collide_odd(Lat L, Mon mon, const uint2* __restrict__ lw, float* snap) {
     pdl_wait();
     pdl_trigger();
     auto* f = pops<ST>(L);
     uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     MonAcc a = {0, 0, 0, 0, 0, 0, 0, 0, 0};
-    bool active = i < L.nS && fluid_bit(L, i);
-    if (active) {
+    // three independent loads: then the word records, then the populations
+    const bool in = i < L.nS;
+    const uint32_t cw = in ? __ldcs(&L.coord[i]) : 0u, lwx = in ? __ldg(&lw[i].x) : 0u;
+    if (in && fluid_bit(L, i)) {
+        uint32_t wall = lwx & LW_MASK;  // directions without a fluid neighbour
         int x, y, z;
-        unpack_coord(__ldcs(&L.coord[i]), x, y, z);
-        const int zm = z == 0 ? L.nz - 1 : z - 1, zp = z == L.nz - 1 ? 0 : z + 1;
+        unpack_coord(cw, x, y, z);
+        const uint32_t b = z & 31, low = (1u << b) - 1u;
+        const bool top = b == 31u || z == L.nz - 1;
         const int ym = y == 0 ? L.ny - 1 : y - 1, yp = y == L.ny - 1 ? 0 : y + 1;
         int xm = x - 1, xp = x + 1;
-        bool hasm = true, hasp = true;
-        if (L.px) {
-            xm = x == 0 ? L.nx - 1 : xm;
-            xp = x == L.nx - 1 ? 0 : xp;
-        } else {
-            hasm = x > 0;
-            hasp = x < L.nx - 1;
+        if (x == 0) {
+            xm = L.px ? L.nx - 1 : 0;
+            if (!L.px) wall |= 1u << 1 | 1u << 10 | 1u << 11 | 1u << 12 | 1u << 13;  // c_x = -1
         }
-        uint32_t nb[Q - 1];  // compact index of x + c_m, or NONE
-        {
-            LineProbe l(L, x, y, z);
-            nb[4] = l.at(zp);
-            nb[5] = l.at(zm);
+        if (x == L.nx - 1) {
+            xp = L.px ? 0 : x;
+            if (!L.px) wall |= 1u << 0 | 1u << 6 | 1u << 7 | 1u << 8 | 1u << 9;  // c_x = +1
         }
+        const uint32_t nyw = (uint32_t)L.nw * L.ny, wz = (uint32_t)(z >> 5) * L.ny;
+        const uint4 *r0 = L.rec + (size_t)x * nyw + wz, *rm = L.rec + (size_t)xm * nyw + wz,
+                    *rp = L.rec + (size_t)xp * nyw + wz;
+        uint32_t off[Q - 1];  // compact index of x + c_m, then its population's offset
         {
-            LineProbe l(L, x, yp, z);
-            nb[2] = l.at(z);
-            nb[14] = l.at(zp);
-            nb[15] = l.at(zm);
+            const LineIndex l(__ldg(r0 + y), b, low, top);
+            off[4] = l.p;
+            off[5] = l.m;
         }
         {
-            LineProbe l(L, x, ym, z);
-            nb[3] = l.at(z);
-            nb[16] = l.at(zp);
-            nb[17] = l.at(zm);
+            const LineIndex l(__ldg(r0 + yp), b, low, top);
+            off[2] = l.c;
+            off[14] = l.p;
+            off[15] = l.m;
         }
-        if (hasp) {
-            {
-                LineProbe l(L, xp, y, z);
-                nb[0] = l.at(z);
-                nb[8] = l.at(zp);
-                nb[9] = l.at(zm);
-            }
-            nb[6] = LineProbe(L, xp, yp, z).at(z);
-            nb[7] = LineProbe(L, xp, ym, z).at(z);
-        } else {
-            nb[0] = nb[8] = nb[9] = nb[6] = nb[7] = NONE;
+        {
+            const LineIndex l(__ldg(r0 + ym), b, low, top);
+            off[3] = l.c;
+            off[16] = l.p;
+            off[17] = l.m;
         }
-        if (hasm) {
-            {
-                LineProbe l(L, xm, y, z);
-                nb[1] = l.at(z);
-                nb[12] = l.at(zp);
-                nb[13] = l.at(zm);
-            }
-            nb[10] = LineProbe(L, xm, yp, z).at(z);
-            nb[11] = LineProbe(L, xm, ym, z).at(z);
-        } else {
-            nb[1] = nb[12] = nb[13] = nb[10] = nb[11] = NONE;
+        {
+            const LineIndex l(__ldg(rp + y), b, low, top);
+            off[0] = l.c;
+            off[8] = l.p;
+            off[9] = l.m;
         }
+        {
+            const LineIndex l(__ldg(rm + y), b, low, top);
+            off[1] = l.c;
+            off[12] = l.p;
+            off[13] = l.m;
+        }
+        auto one = [&](const uint4* r) {
+            const uint2 v = __ldg(reinterpret_cast<const uint2*>(r));
+            return v.y + __popc(v.x & low);
+        };
+        off[6] = one(rp + yp);
+        off[7] = one(rp + ym);
+        off[10] = one(rm + yp);
+        off[11] = one(rm + ym);
         // 32-bit element offsets (19 nSpad < 2^32, checked at the layout)
         float g[Q];
 #pragma unroll
         for (int m = 0; m < Q - 1; ++m) {
-            uint32_t s = nb[opp(m)];
-            const uint32_t off = s != NONE ? (uint32_t)opp(m) * L.nSpad + s : (uint32_t)m * L.nSpad + i;
-            g[m] = to_f<ST>(f[off], L.fsi);
+            off[m] = (wall >> m) & 1u ? (uint32_t)opp(m) * L.nSpad + i : (uint32_t)m * L.nSpad + off[m];
+            g[opp(m)] = to_f<ST>(f[off[m]], L.fsi);
         }
         g[18] = to_f<ST>(f[18u * L.nSpad + i], L.fsi);
         if (SNAP) {
 #pragma unroll
-            for (int m = 0; m < Q; ++m) __stcs(snap + (uint32_t)m * L.nSpad + i, g[m]);
+            for (int m = 0; m < Q; ++m) __stcs(snap + (size_t)m * L.nSpad + i, g[m]);
         }
         float drho, jx, jy, jz;
         bgk(g, L.tau_inv, L.rho_f, drho, jx, jy, jz);
 #pragma unroll
-        for (int m = 0; m < Q - 1; ++m) {
-            uint32_t d = nb[m];
-            const uint32_t off = d != NONE ? (uint32_t)m * L.nSpad + d : (uint32_t)opp(m) * L.nSpad + i;
-            f[off] = from_f<ST>(g[m], L.fs);
-        }
+        for (int m = 0; m < Q - 1; ++m) f[off[m]] = from_f<ST>(g[m], L.fs);
         f[18u * L.nSpad + i] = from_f<ST>(g[18], L.fs);
         if (MON) mon_add(a, drho, jx, jy, jz, L.rho_f);
-        if ((i >= mon.pA0 && i < mon.pA1) || (i >= mon.pB0 && i < mon.pB1)) {
+        if (i >= mon.p0 && i < mon.p1) {
             a.pdrho += drho;
             a.pcnt += 1.f;
         }
-    }
+        }
     mon_flush<MON>(a, mon, true);
 }
 
 template <int ST>
-static void launch_collide_st(const Lat& L, const Mon& mon, bool odd, bool monitor, float* snap, int tile,
-                              cudaStream_t s) {
+static void launch_collide_st(const Lat& L, const Mon& mon, bool odd, bool monitor, const uint2* lw, float* snap,
+                              int tile, cudaStream_t s) {
     const uint32_t threads = odd ? L.nS : (L.nS + 3) / 4, blocks = (threads + tile - 1) / tile;
     if (odd) {
-        if (snap) launch_pdl(k_collide_odd<false, ST, true>, blocks, tile, s, L, mon, snap);
-        else if (monitor) launch_pdl(k_collide_odd<true, ST, false>, blocks, tile, s, L, mon, snap);
-        else launch_pdl(k_collide_odd<false, ST, false>, blocks, tile, s, L, mon, snap);
+        if (snap) launch_pdl(k_collide_odd<false, ST, true>, blocks, tile, s, L, mon, lw, snap);
+        else if (monitor) launch_pdl(k_collide_odd<true, ST, false>, blocks, tile, s, L, mon, lw, snap);
+        else launch_pdl(k_collide_odd<false, ST, false>, blocks, tile, s, L, mon, lw, snap);
     } else {
         if (snap) launch_pdl(k_collide_even<false, ST, true>, blocks, tile, s, L, mon, snap);
         else if (monitor) launch_pdl(k_collide_even<true, ST, false>, blocks, tile, s, L, mon, snap);
@@ -587,12 +580,13 @@ static void launch_collide_st(const Lat& L, const Mon& mon, bool odd, bool monit
 
 // tile: threads per block (64, 128 or 256; the kernels are bounded for 256);
 // snap: null, or where the state before the step goes (not with monitor)
-void launch_collide(const Lat& L, const Mon& mon, bool odd, bool monitor, float* snap, int tile, cudaStream_t s) {
+void launch_collide(const Lat& L, const Mon& mon, bool odd, bool monitor, const uint2* lw, float* snap, int tile,
+                    cudaStream_t s) {
     if (L.nS == 0) return;
     switch (L.st) {
-        case 0: launch_collide_st<0>(L, mon, odd, monitor, snap, tile, s); break;
-        case 1: launch_collide_st<1>(L, mon, odd, monitor, snap, tile, s); break;
-        default: launch_collide_st<2>(L, mon, odd, monitor, snap, tile, s); break;
+        case 0: launch_collide_st<0>(L, mon, odd, monitor, lw, snap, tile, s); break;
+        case 1: launch_collide_st<1>(L, mon, odd, monitor, lw, snap, tile, s); break;
+        default: launch_collide_st<2>(L, mon, odd, monitor, lw, snap, tile, s); break;
     }
 }
 
@@ -664,8 +658,8 @@ void launch_read_fields(const Lat& L, bool after_even, double* rho, double* u, u
 
 // Sums over the fluid nodes of every x plane of the current state: out[3 x]
 // += sum (rho - rho_f), out[3 x + 1] += sum rho u_x, out[3 x + 2] += count.
-// A plane's nodes are one range of each region of the compact order (its
-// first words' bases); PLANE_SPLIT blocks share a plane, every thread adds
+// A plane's nodes are one range of the compact order (from its first word's
+// base); PLANE_SPLIT blocks share a plane, every thread adds
 // its nodes' FP32 terms in FP64, and each block adds its sums to the plane's
 // with one atomic per quantity.  FP64 adds run at 2 lanes per clock and SM
 // here, so the count of them decides: one per node and quantity, against 64
@@ -679,27 +673,23 @@ template <bool AFTER_EVEN, int ST>
 __global__ void __launch_bounds__(PLANE_THREADS) k_plane_sums(Lat L, double* out) {
     const int px = blockIdx.x / PLANE_SPLIT, part = blockIdx.x % PLANE_SPLIT;
     const size_t w0 = (size_t)px * L.ny * L.nw;
-    const bool last = px + 1 == L.nx;
-    const uint4 r0 = L.rec[w0], r1 = last ? r0 : L.rec[w0 + (size_t)L.ny * L.nw];
+    const uint32_t lo = L.rec[w0].y, hi = px + 1 == L.nx ? L.nS : L.rec[w0 + (size_t)L.ny * L.nw].y;
     double sd = 0.0, sj = 0.0;
     uint32_t n = 0;
-    for (int region = 0; region < 2; ++region) {
-        const uint32_t lo = region ? r0.w : r0.z, hi = last ? (region ? L.nS : L.nA) : (region ? r1.w : r1.z);
-        for (uint32_t i = lo + part * PLANE_THREADS + threadIdx.x; i < hi; i += PLANE_SPLIT * PLANE_THREADS) {
-            if (!fluid_bit(L, i)) continue;
-            int x, y, z;
-            unpack_coord(L.coord[i], x, y, z);
-            float d = 0.f, jx = 0.f;
+    for (uint32_t i = lo + part * PLANE_THREADS + threadIdx.x; i < hi; i += PLANE_SPLIT * PLANE_THREADS) {
+        if (!fluid_bit(L, i)) continue;
+        int x, y, z;
+        unpack_coord(L.coord[i], x, y, z);
+        float d = 0.f, jx = 0.f;
 #pragma unroll
-            for (int m = 0; m < Q; ++m) {
-                const float g = to_f<ST>(*pop_loc<ST>(L, AFTER_EVEN, x, y, z, i, m), L.fsi);
-                d += g;
-                jx += cx(m) * g;
-            }
-            sd += (double)d;
-            sj += (double)jx;
-            ++n;
+        for (int m = 0; m < Q; ++m) {
+            const float g = to_f<ST>(*pop_loc<ST>(L, AFTER_EVEN, x, y, z, i, m), L.fsi);
+            d += g;
+            jx += cx(m) * g;
         }
+        sd += (double)d;
+        sj += (double)jx;
+        ++n;
     }
     const unsigned full = 0xffffffffu;
     n = __reduce_add_sync(full, n);

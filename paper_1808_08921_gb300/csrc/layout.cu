@@ -15,8 +15,8 @@
 //      Nodes deeper than `skin` inside a sphere are flagged "deep" (never
 //      stored); nodes within `skin` of a surface are flagged "band" (re-tested
 //      every step).  The inlet/outlet planes are never solid.
-//   2. word masks and counts per 32-node word; exclusive scans give the
-//      compact indices (region A = fluid now, region B = stored solid).
+//   2. word masks and counts per 32-node word; an exclusive scan gives the
+//      compact indices.
 //   3. compact coordinates, fluid bits, band list with candidate spheres,
 //      per-sphere surface lists for the link kernel (warp-padded; the box's
 //      lines visit only the shell where link nodes can be), and, on a
@@ -238,66 +238,75 @@ __global__ void __launch_bounds__(BOX_THREADS) k_paint(PaintArgs A) {
     });
 }
 
-// word masks: maskF = maskA = stored fluid, maskB = stored solid
+// the word of index w: plane x, word wz of its lines, line y
+__device__ __forceinline__ void word_at(const LayoutArgs& A, size_t w, int& x, int& y, int& wz) {
+    y = (int)(w % A.ny);
+    const size_t r = w / A.ny;
+    wz = (int)(r % A.nw);
+    x = (int)(r / A.nw);
+}
+
+// word masks: stored nodes and, of them, the fluid ones
 __global__ void k_words(LayoutArgs A) {
     size_t w = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     size_t W = (size_t)A.nx * A.ny * A.nw;
     if (w >= W) return;
-    int wz = (int)(w % A.nw);
-    size_t line = w / A.nw;
-    uint32_t mA = 0, mB = 0;
+    int x, y, wz;
+    word_at(A, w, x, y, wz);
+    const size_t line = (size_t)x * A.ny + y;
+    uint32_t mS = 0, mF = 0;
     for (int b = 0; b < 32; ++b) {
         int z = wz * 32 + b;
         if (z >= A.nz) break;
         size_t li = line * A.nz + z;
         bool fluid = A.owner[li] == OWNER_FLUID;
-        if (A.deep[li] && !fluid) continue;
-        if (fluid)
-            mA |= 1u << b;
-        else
-            mB |= 1u << b;
+        if (!fluid && (!A.deep || A.deep[li])) continue;
+        mS |= 1u << b;
+        if (fluid) mF |= 1u << b;
     }
-    A.rec[w] = make_uint4(mA, mA, 0u, 0u);
-    A.maskB[w] = mB;
-    A.cntA[w] = __popc(mA);
-    A.cntB[w] = __popc(mB);
+    A.rec[w] = make_uint4(mS, 0u, 0u, 0u);
+    A.fluid[w] = mF;
+    A.cnt[w] = __popc(mS);
 }
 
-__global__ void k_words_bases(LayoutArgs A, uint32_t nA) {
+// bases, and the indices of the nodes before and after the word (any value
+// where that node is not stored)
+__global__ void k_words_bases(LayoutArgs A) {
     size_t w = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     size_t W = (size_t)A.nx * A.ny * A.nw;
     if (w >= W) return;
-    A.rec[w].z = A.cntA[w];
-    A.rec[w].w = nA + A.cntB[w];
+    int x, y, wz;
+    word_at(A, w, x, y, wz);
+    auto index = [&](int z) {  // of node (x, y, z)
+        const size_t v = ((size_t)x * A.nw + (z >> 5)) * A.ny + y;
+        return A.cnt[v] + __popc(A.rec[v].x & ((1u << (z & 31)) - 1u));
+    };
+    const int z0 = 32 * wz, z1 = min(z0 + 32, A.nz);
+    A.rec[w].y = A.cnt[w];
+    A.rec[w].z = index(z0 == 0 ? A.nz - 1 : z0 - 1);
+    A.rec[w].w = index(z1 == A.nz ? 0 : z1);
 }
 
-__global__ void k_coords(LayoutArgs A) {
+// coordinates of the stored nodes and their fluid bits in compact order (the
+// word's fluid bits without its unstored places; fbits starts at zero)
+__global__ void k_coords(LayoutArgs A, uint32_t* fbits) {
     size_t w = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     size_t W = (size_t)A.nx * A.ny * A.nw;
     if (w >= W) return;
-    int wz = (int)(w % A.nw);
-    size_t line = w / A.nw;
-    int y = (int)(line % A.ny), x = (int)(line / A.ny);
-    uint4 r = A.rec[w];
-    uint32_t mB = A.maskB[w];
-    uint32_t ia = r.z, ib = r.w;
+    int x, y, wz;
+    word_at(A, w, x, y, wz);
+    const uint4 r = A.rec[w];
+    const uint32_t mF = A.fluid[w];
+    uint32_t n = 0, fl = 0;
     for (int b = 0; b < 32; ++b) {
-        uint32_t bit = 1u << b;
-        int z = wz * 32 + b;
-        if (r.y & bit) A.coord[ia++] = pack_coord(x, y, z);
-        if (mB & bit) A.coord[ib++] = pack_coord(x, y, z);
+        if (!((r.x >> b) & 1u)) continue;
+        A.coord[r.y + n] = pack_coord(x, y, wz * 32 + b);
+        fl |= ((mF >> b) & 1u) << n;
+        ++n;
     }
-}
-
-__global__ void k_fbits(uint32_t* fbits, uint32_t nA, uint32_t nwords) {
-    uint32_t k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= nwords) return;
-    uint32_t lo = k * 32;
-    uint32_t v;
-    if (lo + 32 <= nA) v = 0xffffffffu;
-    else if (lo >= nA) v = 0u;
-    else v = (1u << (nA - lo)) - 1u;
-    fbits[k] = v;
+    const unsigned long long bits = (unsigned long long)fl << (r.y & 31);
+    if ((uint32_t)bits) atomicOr(&fbits[r.y >> 5], (uint32_t)bits);
+    if ((uint32_t)(bits >> 32)) atomicOr(&fbits[(r.y >> 5) + 1], (uint32_t)(bits >> 32));
 }
 
 // re-layout: copy the natural populations (state between an odd and an even
@@ -307,7 +316,7 @@ __global__ void k_gather_old(Lat Lnew, Lat Lold) {
     T* fn = static_cast<T*>(Lnew.f);
     const T* fo = static_cast<const T*>(Lold.f);
     uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= Lnew.nA) return;
+    if (i >= Lnew.nS || !fluid_bit(Lnew, i)) return;
     int x, y, z;
     unpack_coord(Lnew.coord[i], x, y, z);
     bool fl;
@@ -552,21 +561,20 @@ void launch_words(const LayoutArgs& A, cudaStream_t s) {
     k_words<<<(unsigned)((W + 255) / 256), 256, 0, s>>>(A);
 }
 
-void launch_words_bases(const LayoutArgs& A, uint32_t nA, cudaStream_t s) {
+void launch_words_bases(const LayoutArgs& A, cudaStream_t s) {
     size_t W = (size_t)A.nx * A.ny * A.nw;
-    k_words_bases<<<(unsigned)((W + 255) / 256), 256, 0, s>>>(A, nA);
+    k_words_bases<<<(unsigned)((W + 255) / 256), 256, 0, s>>>(A);
 }
 
-void launch_coords(const LayoutArgs& A, uint32_t nA, uint32_t nSpad, uint32_t* fbits, cudaStream_t s) {
+void launch_coords(const LayoutArgs& A, uint32_t nSpad, uint32_t* fbits, cudaStream_t s) {
     size_t W = (size_t)A.nx * A.ny * A.nw;
-    k_coords<<<(unsigned)((W + 255) / 256), 256, 0, s>>>(A);
-    uint32_t nwords = nSpad / 32;
-    k_fbits<<<(nwords + 255) / 256, 256, 0, s>>>(fbits, nA, nwords);
+    cudaMemsetAsync(fbits, 0, nSpad / 8, s);
+    k_coords<<<(unsigned)((W + 255) / 256), 256, 0, s>>>(A, fbits);
 }
 
 void launch_gather_old(const Lat& Lnew, const Lat& Lold, cudaStream_t s) {
-    if (!Lnew.nA) return;
-    unsigned blocks = (Lnew.nA + 255) / 256;
+    if (!Lnew.nS) return;
+    unsigned blocks = (Lnew.nS + 255) / 256;
     if (Lnew.st == 0)  // the populations move as stored (no conversion)
         k_gather_old<float><<<blocks, 256, 0, s>>>(Lnew, Lold);
     else

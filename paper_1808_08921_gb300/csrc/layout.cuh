@@ -19,12 +19,11 @@ struct PaintArgs {
 struct LayoutArgs {
     int nx, ny, nz, nw;
     const int32_t* owner;
-    const uint8_t* deep;
+    const uint8_t* deep;    // null: no sphere moves, no solid node is stored
     const uint8_t* band;
     uint4* rec;
-    uint32_t* maskB;
-    uint32_t* cntA;
-    uint32_t* cntB;
+    uint32_t* fluid;
+    uint32_t* cnt;
     uint32_t* coord;
 };
 
@@ -94,8 +93,8 @@ void exclusive_scan(const uint32_t* in, uint32_t* out, size_t n, uint32_t* tmp, 
 size_t scan_tmp_size(size_t n);
 void launch_paint(const PaintArgs& A, int n, size_t N, cudaStream_t s);
 void launch_words(const LayoutArgs& A, cudaStream_t s);
-void launch_words_bases(const LayoutArgs& A, uint32_t nA, cudaStream_t s);
-void launch_coords(const LayoutArgs& A, uint32_t nA, uint32_t nSpad, uint32_t* fbits, cudaStream_t s);
+void launch_words_bases(const LayoutArgs& A, cudaStream_t s);
+void launch_coords(const LayoutArgs& A, uint32_t nSpad, uint32_t* fbits, cudaStream_t s);
 void launch_gather_old(const Lat& Lnew, const Lat& Lold, cudaStream_t s);
 void launch_band_collect(const LayoutArgs& A, uint32_t* band_coord, uint32_t* count, uint32_t cap,
                          cudaStream_t s);
