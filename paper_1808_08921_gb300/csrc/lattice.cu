@@ -466,17 +466,21 @@ struct LineIndex {
 // three neighbours each and four that give one.  Testing each neighbour's
 // fluid bit in its record, with two index regions per record and a second
 // record past a word's end, took 174 us on the 128 x 128 x 1024 column and 157
-// on 160^3 (all fluid), this form 160 and 138.  152 B per fluid node plus its
-// 8 B link word: 98 us and 97 us at the copy rate; it waits for its chain of
-// three dependent loads at 64 registers (80 leave fewer warps: 164 and 144;
-// 48 spill: 225 and 172).
+// on 160^3 (all fluid), this form 160 and 138 with the offsets in registers
+// (64; 80 leave fewer warps: 164 and 144; 48 spill: 225 and 172).  It waits
+// for its chain of three dependent loads, so the warps in flight count: the
+// offsets wait in shared memory from the loads to the stores, which leaves
+// 40 registers and 48 warps per SM, 139 and 120 us.  152 B per fluid node
+// plus its 8 B link word: 98 and 97 us at the copy rate.
 template <bool MON, int ST, bool SNAP>
-__global__ void __launch_bounds__(256, 4) k_collide_odd(Lat L, Mon mon, const uint2* __restrict__ lw, float* snap) {
+__global__ void __launch_bounds__(256, 6) k_collide_odd(Lat L, Mon mon, const uint2* __restrict__ lw, float* snap) {
     pdl_wait();
     pdl_trigger();
     auto* f = pops<ST>(L);
     uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
     MonAcc a = {0, 0, 0, 0, 0, 0, 0, 0, 0};
+    extern __shared__ uint32_t s_off[];  // [warp][Q - 1][lane]
+    uint32_t* off = s_off + (threadIdx.x >> 5) * ((Q - 1) * 32) + (threadIdx.x & 31);
     // three independent loads: then the word records, then the populations
     const bool in = i < L.nS;
     const uint32_t cw = in ? __ldcs(&L.coord[i]) : 0u, lwx = in ? __ldg(&lw[i].x) : 0u;
@@ -499,51 +503,51 @@ __global__ void __launch_bounds__(256, 4) k_collide_odd(Lat L, Mon mon, const ui
         const uint32_t nyw = (uint32_t)L.nw * L.ny, wz = (uint32_t)(z >> 5) * L.ny;
         const uint4 *r0 = L.rec + (size_t)x * nyw + wz, *rm = L.rec + (size_t)xm * nyw + wz,
                     *rp = L.rec + (size_t)xp * nyw + wz;
-        uint32_t off[Q - 1];  // compact index of x + c_m, then its population's offset
+        float g[Q];
+        // the place of the population between x and x + c_m, whose compact
+        // index is n: a 32-bit offset (19 nSpad < 2^32, checked at the layout)
+        auto take = [&](int m, uint32_t n) {
+            const uint32_t o = (wall >> m) & 1u ? (uint32_t)opp(m) * L.nSpad + i : (uint32_t)m * L.nSpad + n;
+            off[m * 32] = o;
+            g[opp(m)] = to_f<ST>(f[o], L.fsi);
+        };
         {
             const LineIndex l(__ldg(r0 + y), b, low, top);
-            off[4] = l.p;
-            off[5] = l.m;
+            take(4, l.p);
+            take(5, l.m);
         }
         {
             const LineIndex l(__ldg(r0 + yp), b, low, top);
-            off[2] = l.c;
-            off[14] = l.p;
-            off[15] = l.m;
+            take(2, l.c);
+            take(14, l.p);
+            take(15, l.m);
         }
         {
             const LineIndex l(__ldg(r0 + ym), b, low, top);
-            off[3] = l.c;
-            off[16] = l.p;
-            off[17] = l.m;
+            take(3, l.c);
+            take(16, l.p);
+            take(17, l.m);
         }
         {
             const LineIndex l(__ldg(rp + y), b, low, top);
-            off[0] = l.c;
-            off[8] = l.p;
-            off[9] = l.m;
+            take(0, l.c);
+            take(8, l.p);
+            take(9, l.m);
         }
         {
             const LineIndex l(__ldg(rm + y), b, low, top);
-            off[1] = l.c;
-            off[12] = l.p;
-            off[13] = l.m;
+            take(1, l.c);
+            take(12, l.p);
+            take(13, l.m);
         }
         auto one = [&](const uint4* r) {
             const uint2 v = __ldg(reinterpret_cast<const uint2*>(r));
             return v.y + __popc(v.x & low);
         };
-        off[6] = one(rp + yp);
-        off[7] = one(rp + ym);
-        off[10] = one(rm + yp);
-        off[11] = one(rm + ym);
-        // 32-bit element offsets (19 nSpad < 2^32, checked at the layout)
-        float g[Q];
-#pragma unroll
-        for (int m = 0; m < Q - 1; ++m) {
-            off[m] = (wall >> m) & 1u ? (uint32_t)opp(m) * L.nSpad + i : (uint32_t)m * L.nSpad + off[m];
-            g[opp(m)] = to_f<ST>(f[off[m]], L.fsi);
-        }
+        take(6, one(rp + yp));
+        take(7, one(rp + ym));
+        take(10, one(rm + yp));
+        take(11, one(rm + ym));
         g[18] = to_f<ST>(f[18u * L.nSpad + i], L.fsi);
         if (SNAP) {
 #pragma unroll
@@ -552,14 +556,14 @@ __global__ void __launch_bounds__(256, 4) k_collide_odd(Lat L, Mon mon, const ui
         float drho, jx, jy, jz;
         bgk(g, L.tau_inv, L.rho_f, drho, jx, jy, jz);
 #pragma unroll
-        for (int m = 0; m < Q - 1; ++m) f[off[m]] = from_f<ST>(g[m], L.fs);
+        for (int m = 0; m < Q - 1; ++m) f[off[m * 32]] = from_f<ST>(g[m], L.fs);
         f[18u * L.nSpad + i] = from_f<ST>(g[18], L.fs);
         if (MON) mon_add(a, drho, jx, jy, jz, L.rho_f);
         if (i >= mon.p0 && i < mon.p1) {
             a.pdrho += drho;
             a.pcnt += 1.f;
         }
-        }
+    }
     mon_flush<MON>(a, mon, true);
 }
 
@@ -567,10 +571,11 @@ template <int ST>
 static void launch_collide_st(const Lat& L, const Mon& mon, bool odd, bool monitor, const uint2* lw, float* snap,
                               int tile, cudaStream_t s) {
     const uint32_t threads = odd ? L.nS : (L.nS + 3) / 4, blocks = (threads + tile - 1) / tile;
+    const size_t smem = (size_t)(Q - 1) * tile * sizeof(uint32_t);  // 4.6 KB per 64 threads
     if (odd) {
-        if (snap) launch_pdl(k_collide_odd<false, ST, true>, blocks, tile, s, L, mon, lw, snap);
-        else if (monitor) launch_pdl(k_collide_odd<true, ST, false>, blocks, tile, s, L, mon, lw, snap);
-        else launch_pdl(k_collide_odd<false, ST, false>, blocks, tile, s, L, mon, lw, snap);
+        if (snap) launch_pdl_smem(k_collide_odd<false, ST, true>, blocks, tile, smem, s, L, mon, lw, snap);
+        else if (monitor) launch_pdl_smem(k_collide_odd<true, ST, false>, blocks, tile, smem, s, L, mon, lw, snap);
+        else launch_pdl_smem(k_collide_odd<false, ST, false>, blocks, tile, smem, s, L, mon, lw, snap);
     } else {
         if (snap) launch_pdl(k_collide_even<false, ST, true>, blocks, tile, s, L, mon, snap);
         else if (monitor) launch_pdl(k_collide_even<true, ST, false>, blocks, tile, s, L, mon, snap);
