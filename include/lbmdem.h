@@ -12,7 +12,7 @@
  *   2. BGK collide + stream of the D3Q19 fluid (Section 2.1, Eqs. 3-8);
  *   3. moving-wall half-way bounce-back on every fluid-solid link and the
  *      hydrodynamic force and torque on each sphere (Eqs. 14-15, 18-19);
- *      on even steps 2 and 3 can run as one kernel (link_mode below);
+ *      2 and 3 can run as one kernel (link_mode below);
  *   4. the pressure inlet with the oscillating density (Section 2.4, Zou-He
  *      form for D3Q19, Eq. 25, Table 2) and the outlet;
  *   5. K velocity-Verlet substeps of the spheres with Hertz normal and
@@ -100,8 +100,10 @@ typedef struct {
     int32_t max_flips;    /* node conversions per step the scratch holds; 0 = auto    */
     int32_t tile;         /* threads per block of collide+stream: 64 (0), 128 or 256  */
     int32_t device;       /* CUDA device ordinal                                      */
-    int32_t link_mode;    /* 2: an even step's links (Eqs. 14-15, 18-19) are taken inside
-                             its collide+stream kernel, an odd step's by the link kernel;
+    int32_t link_mode;    /* 2: a step's links (Eqs. 14-15, 18-19) are taken inside its
+                             collide+stream kernel, the odd steps' from 65536 stored
+                             nodes and two links per stored node up (below, by the
+                             link kernel);
                              1: the link kernel every step; 0 (default): 2 with FP32
                              storage and a largest sphere radius of 8 lattice units
                              or more, else 1.  Boxes narrower than 2 (R + skin + 2)
@@ -216,8 +218,7 @@ int lbm_dem_read_counters(lbmdem_ctx* c, int64_t out[10]);
  * milliseconds and the number of launches since the last read:
  * [0] collide+stream of the odd steps, [1] link kernel, [2] map update,
  * [3] inlet/outlet, [4] DEM substeps, [5] collide+stream of the even steps
- * (with the step's links where the even steps take them there: link_mode 2,
- * or 0 with FP32 storage). */
+ * ([0] and [5] with the step's links where link_mode takes them there). */
 int lbm_dem_set_timing(lbmdem_ctx* c, int32_t enable);
 int lbm_dem_read_timing(lbmdem_ctx* c, double ms[6], int64_t launches[6]);
 

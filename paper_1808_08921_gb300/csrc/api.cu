@@ -163,7 +163,7 @@ struct lbmdem_ctx {
     uint32_t nwarps = 0;
     uint32_t nlink_raw = 0;  // link records before padding
     DBuf<uint2> linkw;       // link word of every stored node
-    bool fused_links = false;
+    bool fused_links = false, dense_links = false;
     bool batched = false;  // steps being captured into a batch graph (columns share the GPU)
     DBuf<Flip> flip_rec;
     DBuf<float> flip_scratch;
@@ -603,7 +603,7 @@ static int build_layout(lbmdem_ctx* c, bool fresh) {
     launch_surf_fill(SA, np, s);
     CK(cudaGetLastError());
     c->nwarps = nlink / LINK_WARP;
-    // even steps take their links inside the collide kernel (link words from
+    // the steps take their links inside the collide kernel (link words from
     // the owner map) unless the sphere indices do not fit a link word, or a
     // periodic axis is narrow enough for a link node (within R + sqrt(3) of a
     // centre, R + skin after motion) to neighbour two images of one sphere:
@@ -611,13 +611,19 @@ static int build_layout(lbmdem_ctx* c, bool fresh) {
     const double reach = 2.0 * (c->Rmax + c->skin + 2.0);
     const bool wide = c->p.ny > reach && c->p.nz > reach && (!px || c->p.nx > reach);
     // (link_mode 0: with FP32 storage and spheres of radius 8 lu or more.
-    // With 16-bit storage the even collide kernel is bandwidth-light, and
-    // smaller spheres change along a 32-node run often enough that the
-    // per-warp sphere sums cost more than the link kernel: R 5.7 FCC, 0.106
-    // against 0.091 ms per step; R 11.4, 0.309 against 0.329 ms)
+    // R 11.4 FCC on 128 x 128 x 1024: 237 against 325 us per step with the
+    // link kernel every step.  Smaller spheres, R 5.7 on 64 x 64 x 512: 80
+    // against 83 us, but their stiffer contacts amplify the other order of
+    // the force sums, and results there stay what the link lists give; with
+    // 16-bit storage both kernels' populations are light and the link kernel
+    // rounds as the storage does)
     const bool want = c->p.link_mode == 2 ||
                       (c->p.link_mode == 0 && c->p.storage == LBMDEM_F32 && c->Rmax >= 8.0);
     c->fused_links = want && c->nwarps > 0 && np <= LW_MAX_SPHERES && wide;
+    // FCC media have 5 to 10 link records per stored node, a sphere alone in a
+    // box below one: there the link kernel is a few us of an odd step (160^3,
+    // R 9: 118 + 10 us against 127), and the even steps keep their sums' order
+    c->dense_links = nlink >= 2 * (uint64_t)nS;
     CK(c->linkw.ensure(nSpad));
     launch_link_words(make_lat(c), c->linkw.p, s);
     CK(cudaGetLastError());
@@ -691,7 +697,17 @@ static void record_pair_end(lbmdem_ctx* c, size_t idx, cudaStream_t st = nullptr
         cudaEventRecord(c->ev[2 * idx + 1], st);
 }
 
-static bool links_in_collide(const lbmdem_ctx* c, int parity) { return c->fused_links && parity == 0; }
+// Whether a step's links are taken inside its collide kernel: in lattices of
+// that kind (link_mode) every even step's, and the odd steps' where most
+// nodes have links, from ODD_LINKS_MIN stored nodes up.  R 11.4 FCC, the odd steps with the link
+// kernel against without, us per step: 159 k nodes 33.1 and 29.9, 629 k 54.4
+// and 46.3, 1.26 M 87.7 and 72.5, 4.46 M 283 and 238.  Smaller lattices
+// would gain too (41 k nodes 22.7 and 20.5) but keep the launches they are
+// documented with.
+constexpr uint32_t ODD_LINKS_MIN = 1u << 16;
+static bool links_in_collide(const lbmdem_ctx* c, int parity) {
+    return c->fused_links && (parity == 0 || (c->dense_links && c->nS >= ODD_LINKS_MIN));
+}
 
 static bool inlet_outlet_active(const lbmdem_ctx* c) {
     return c->p.inlet != LBMDEM_X_PERIODIC && !(c->p.inlet != 0 && c->p.outlet > 1);
@@ -773,7 +789,7 @@ static void enqueue_step(lbmdem_ctx* c, int parity, bool monitor, int inlet, boo
         }
         if (tm) record_pair_begin(c, parity == 1 ? 0 : 5, e);
         if (fused)
-            launch_collide_even_links(L, mon, P, c->linkw.p, monitor, c->p.tile > 0 ? c->p.tile : 64, s);
+            launch_collide_links(L, mon, P, parity == 1, monitor, !c->dense_links, c->linkw.p, c->p.tile > 0 ? c->p.tile : 64, s);
         else
             launch_collide(L, mon, parity == 1, monitor, c->linkw.p, snap, c->p.tile > 0 ? c->p.tile : 64, s);
         if (tm) record_pair_end(c, e);

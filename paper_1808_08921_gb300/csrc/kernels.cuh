@@ -146,8 +146,8 @@ struct LinkLists {
 };
 
 // Link word of a stored node (one 8-byte word per node), for the odd collide
-// kernel's fluid neighbours (.x) and the even steps' links inside the collide
-// kernel:
+// kernel's fluid neighbours (.x) and the links taken inside the collide
+// kernels:
 //   .x = link mask (bit m, m < 18: the neighbour x + c_m is solid) | sphere A << 18
 //   .y = B mask (bit m: that link's neighbour belongs to sphere B) | sphere B << 18
 // Sphere indices take 14 bits; LW_NONE stands for no sphere B, and as sphere
@@ -243,8 +243,8 @@ struct Dem {
 // lattice.cu
 void launch_collide(const Lat& L, const Mon& mon, bool odd, bool monitor, const uint2* lw, float* snap, int tile,
                     cudaStream_t s);
-void launch_collide_even_links(const Lat& L, const Mon& mon, const PartView& P, const uint2* lw, bool monitor,
-                               int tile, cudaStream_t s);
+void launch_collide_links(const Lat& L, const Mon& mon, const PartView& P, bool odd, bool monitor, bool few,
+                          const uint2* lw, int tile, cudaStream_t s);
 void launch_inlet_outlet(const Lat& L, const BC& bc, bool after_even, cudaStream_t s);
 void launch_plane_sums(const Lat& L, bool after_even, double* out, cudaStream_t s);
 void launch_read_fields(const Lat& L, bool after_even, double* rho, double* u, uint8_t* solid,

@@ -204,19 +204,291 @@ __global__ void __launch_bounds__(256) k_collide_even(Lat L, Mon mon, float* sna
     mon_flush<MON>(a, mon, true);
 }
 
-// ---- even step with the step's links (one node per lane and 32-node run)
+// ---- collide with the step's links (one node per lane)
 //
-// The even step is node-local, so the links of a node can be bounced where
-// its post-collision values are written.  For a link direction m of fluid
-// node x (x + c_m solid, owned by sphere p) the value leaving towards the
-// wall, g~_m, goes to slot opp(m) of x as g~_m - delta (Eq. 14, moving wall),
+// Where a node's post-collision values are written its links can be bounced.
+// For a link direction m of fluid node x (x + c_m solid, owned by sphere p)
+// the value leaving towards the wall, g~_m, goes to slot opp(m) of x, in an
+// even step as in an odd one, as g~_m - delta (Eq. 14, moving wall),
 //     delta = 6 w_m rho_f c_m . U,   U = V + W x r,   r = x - X,
 // the wall velocity at x (the half-link offset c_m / 2 drops out because
 // c_m . (W x c_m) = 0), and adds the link force c_m (2 g~_m - delta) of
 // Eq. 15 (counted about the rest state, as the link kernel does) and its
-// torque r x c_m (2 g~_m - delta) of Eq. 19 to the sphere.  Each thread keeps
-// two (sphere, force, torque) slots; at the end the warp sums the slots
-// sphere by sphere and adds each sum with one FP64 atomic per component.
+// torque r x c_m (2 g~_m - delta) of Eq. 19 to the sphere.  A node's links
+// belong to one sphere or two, each leaving its six sums in a column of
+// shared memory until the populations are stored; then the warp sums the
+// columns sphere by sphere and adds each sum with one FP64 atomic per
+// component.  The rare node of more than two spheres adds its own sums.
+
+// The links of node (x, y, z) to sphere p (bit m of msk: direction m): g
+// becomes what the slots take, out the sums.  u is 6 rho_f / 36 times the wall
+// velocity, so that delta is c.u, twice that on the axes, and a pair of
+// opposite directions shares it.
+__device__ __forceinline__ void node_links(const Lat& L, const PartView& P, int x, int y, int z, int p, uint32_t msk,
+                                           float g[Q], float out[6]) {
+    const float4 a = P.pk[3 * (size_t)p], b = P.pk[3 * (size_t)p + 1], c = P.pk[3 * (size_t)p + 2];
+    const int ox = __float_as_int(c.y), oy = __float_as_int(c.z), oz = __float_as_int(c.w);
+    const int ix = L.px ? imin_small(x - ox, L.nx) : x - ox;
+    const int iy = imin_small(y - oy, L.ny), iz = imin_small(z - oz, L.nz);
+    const float rx = (float)ix - a.x, ry = (float)iy - a.y, rz = (float)iz - a.z;
+    const float s = L.rho_f * (1.0f / 6.0f);
+    const float ux = s * (a.w + (b.w * rz - c.x * ry)), uy = s * (b.x + (c.x * rx - b.z * rz)),
+                uz = s * (b.y + (b.z * ry - b.w * rx));
+    float fx = 0.f, fy = 0.f, fz = 0.f;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        const int m = pair_m(k), o = opp(m);
+        float t = 0.f;
+        if (cx(m)) t += cx(m) > 0 ? ux : -ux;
+        if (cy(m)) t += cy(m) > 0 ? uy : -uy;
+        if (cz(m)) t += cz(m) > 0 ? uz : -uz;
+        const float d = k < 3 ? 2.0f * t : t;
+        const bool hm = (msk >> m) & 1u, ho = (msk >> o) & 1u;
+        float q = 0.f;
+        if (hm) {
+            q = 2.0f * g[m] - d;
+            g[m] -= d;
+        }
+        if (ho) {
+            q -= 2.0f * g[o] + d;
+            g[o] += d;
+        }
+        if (cx(m)) fx += cx(m) > 0 ? q : -q;
+        if (cy(m)) fy += cy(m) > 0 ? q : -q;
+        if (cz(m)) fz += cz(m) > 0 ? q : -q;
+    }
+    out[0] = fx;
+    out[1] = fy;
+    out[2] = fz;
+    out[3] = ry * fz - rz * fy;
+    out[4] = rz * fx - rx * fz;
+    out[5] = rx * fy - ry * fx;
+}
+
+// A lane's sums for two spheres (a and b, -1: none), in a column of shared
+// memory: force and torque of a, then of b.
+constexpr int LINK_COLS = 12;
+
+struct LinkSums {
+    float* col;
+    int a, b;
+};
+
+__device__ __forceinline__ void sums_put(float* c, const float v[6]) {
+#pragma unroll
+    for (int k = 0; k < 6; ++k) c[k * 32] = v[k];
+}
+
+// All links of a node with link word w.
+__device__ __forceinline__ void all_links(const Lat& L, const PartView& P, int x, int y, int z, uint2 w, uint32_t rep,
+                                          float g[Q], LinkSums& n) {
+    float v[6];
+    int pa = (int)(w.x >> 18), pb = (int)(w.y >> 18);
+    uint32_t mb = w.y & LW_MASK, ma = w.x & LW_MASK & ~mb;
+    if (pa == (int)LW_NONE) {
+        // neighbours of more than two spheres: their owners from the map, the
+        // third sphere's links (and a further one's) here, by this lane alone
+        int own[Q - 1];
+#pragma unroll
+        for (int m = 0; m < Q - 1; ++m) {
+            if (!((w.x >> m) & 1u)) continue;
+            int xs = x + cx(m);
+            if (L.px) xs = wrap1(xs, L.nx);
+            own[m] = __ldg(&L.owner[((size_t)xs * L.ny + wrap1(y + cy(m), L.ny)) * L.nz + wrap1(z + cz(m), L.nz)]);
+        }
+        uint32_t rem = w.x & LW_MASK;
+        auto next = [&](int& p) {  // the links of the first remaining direction's sphere
+            p = -1;
+            uint32_t sub = 0u;
+#pragma unroll
+            for (int m = 0; m < Q - 1; ++m) {
+                if (!((rem >> m) & 1u)) continue;
+                if (p < 0) p = own[m];
+                if (own[m] == p) sub |= 1u << m;
+            }
+            rem &= ~sub;
+            return sub;
+        };
+        ma = next(pa);
+        mb = next(pb);
+        while (rem) {
+            int p;
+            const uint32_t sub = next(p);
+            node_links(L, P, x, y, z, p, sub, g, v);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                atomicAdd(P.Fh + 3 * ((size_t)rep * P.n + p) + k, (double)v[k]);
+                atomicAdd(P.Th + 3 * ((size_t)rep * P.n + p) + k, (double)v[k + 3]);
+            }
+        }
+    }
+    n.a = pa;
+    node_links(L, P, x, y, z, pa, ma, g, v);
+    sums_put(n.col, v);
+    if (mb) {
+        n.b = pb;
+        node_links(L, P, x, y, z, pb, mb, g, v);
+        sums_put(n.col + 6 * 32, v);
+    }
+}
+
+// The warp's columns, sphere by sphere.
+__device__ __forceinline__ void columns_add(const PartView& P, uint32_t rep, LinkSums& n) {
+    const unsigned full = 0xffffffffu;
+    const uint32_t lane = threadIdx.x & 31;
+    const int comp = ((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1);
+    const bool adds = (lane & 3) == 0 && comp < 6;
+    double* dst = (comp < 3 ? P.Fh + comp : P.Th + (comp - 3)) + 3 * (size_t)rep * P.n;
+    for (;;) {
+        const int mine = n.a >= 0 ? n.a : n.b;
+        const unsigned act = __ballot_sync(full, mine >= 0);
+        if (!act) break;
+        const int p = __shfl_sync(full, mine, __ffs(act) - 1);
+        float s8[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        if (n.a == p || n.b == p) {  // not both
+            const float* v = n.a == p ? n.col : n.col + 6 * 32;
+#pragma unroll
+            for (int c = 0; c < 6; ++c) s8[c] = v[c * 32];
+            if (n.a == p) n.a = -1;
+            else n.b = -1;
+        }
+        // transposing butterfly (lane l ends with component 4 b4 + 2 b3 + b2)
+        {
+            const bool up = lane & 16;
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const float keep = up ? s8[c + 4] : s8[c], send = up ? s8[c] : s8[c + 4];
+                s8[c] = keep + __shfl_xor_sync(full, send, 16);
+            }
+        }
+        {
+            const bool up = lane & 8;
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                const float keep = up ? s8[c + 2] : s8[c], send = up ? s8[c] : s8[c + 2];
+                s8[c] = keep + __shfl_xor_sync(full, send, 8);
+            }
+        }
+        {
+            const bool up = lane & 4;
+            const float keep = up ? s8[1] : s8[0], send = up ? s8[0] : s8[1];
+            s8[0] = keep + __shfl_xor_sync(full, send, 4);
+        }
+        s8[0] += __shfl_xor_sync(full, s8[0], 2);
+        s8[0] += __shfl_xor_sync(full, s8[0], 1);
+        if (adds) atomicAdd(dst + 3 * (size_t)p, (double)s8[0]);
+    }
+}
+
+// Collision of a node whose links are taken with it: opposite directions share
+// their equilibrium terms, and the rest population takes what the moving
+// ones leave of the density, so that the FP32 weights conserve mass.
+__device__ __forceinline__ void bgk_pairs(float g[Q], float tau_inv, float rho_f, float& drho, float& jx, float& jy,
+                                          float& jz) {
+    float s[9], d[9];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        s[k] = g[pair_m(k)] + g[opp(pair_m(k))];
+        d[k] = g[pair_m(k)] - g[opp(pair_m(k))];
+    }
+    drho = (s[0] + s[1]) + (s[2] + s[3]) + ((s[4] + s[5]) + (s[6] + s[7])) + (s[8] + g[18]);
+    jx = jy = jz = 0.f;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        const int m = pair_m(k);
+        if (cx(m)) jx += cx(m) > 0 ? d[k] : -d[k];
+        if (cy(m)) jy += cy(m) > 0 ? d[k] : -d[k];
+        if (cz(m)) jz += cz(m) > 0 ? d[k] : -d[k];
+    }
+    const float rho = rho_f + drho, ir = 1.0f / rho;
+    const float ux = jx * ir, uy = jy * ir, uz = jz * ir;
+    // 36 t36 is 1 / tau but for rounding; what the relaxation keeps is taken
+    // from it, so that density and momentum are kept
+    const float t36 = tau_inv * (1.0f / 36.0f), om = fmaf(-36.0f, t36, 1.0f);
+    // weight 1/36 terms times 1 / tau: even part e + q cu^2, odd part l cu
+    const float e = t36 * (drho - 1.5f * rho * (ux * ux + uy * uy + uz * uz));
+    const float q = 4.5f * t36 * rho, l = 3.0f * t36 * rho;
+    float moving = 0.f;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        const int m = pair_m(k), o = opp(m);
+        float cu = 0.f;
+        if (cx(m)) cu += cx(m) > 0 ? ux : -ux;
+        if (cy(m)) cu += cy(m) > 0 ? uy : -uy;
+        if (cz(m)) cu += cz(m) > 0 ? uz : -uz;
+        float ev = e + (q * cu) * cu, od = l * cu;
+        if (k < 3) {
+            ev *= 2.0f;
+            od *= 2.0f;
+        }
+        moving += ev;
+        g[m] = om * g[m] + (ev + od);
+        g[o] = om * g[o] + (ev - od);
+    }
+    g[18] = om * g[18] + ((1.0f - om) * drho - 2.0f * moving);
+}
+
+template <int ST> __device__ __forceinline__ float ld1(const typename PopT<ST>::T* p, float fsi) {
+    return to_f<ST>(*p, fsi);
+}
+template <> __device__ __forceinline__ float ld1<0>(const float* p, float) { return __ldcs(p); }
+template <int ST> __device__ __forceinline__ void st1(typename PopT<ST>::T* p, float v, float fs) {
+    *p = from_f<ST>(v, fs);
+}
+template <> __device__ __forceinline__ void st1<0>(float* p, float v, float) { __stcs(p, v); }
+
+// Even step with the step's links.  152 B per node and its 12 B of words (104
+// us on the 128 x 128 x 1024 column) against about 880 instructions per warp: the
+// issue slots (65%) and the loads' latency bound it together, at 36 warps
+// per SM.  184 us with register slots per lane over two runs of nodes, 72
+// registers and every direction worked through alone; 181 so (64 and 48
+// registers are no faster).
+template <bool MON, int ST>
+__global__ void __maxnreg__(56)
+k_collide_even_links(Lat L, Mon mon, PartView P, const uint2* __restrict__ lwp) {
+    pdl_wait();
+    pdl_trigger();
+    auto* f = pops<ST>(L);
+    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x, rep = (i >> 5) % NREP;
+    MonAcc a = {0, 0, 0, 0, 0, 0, 0, 0, 0};
+    extern __shared__ float s_col[];  // [warp][LINK_COLS][lane]
+    LinkSums n = {s_col + (threadIdx.x >> 5) * (LINK_COLS * 32) + (threadIdx.x & 31), -1, -1};
+    if (i < L.nS && fluid_bit(L, i)) {
+        float g[Q];
+#pragma unroll
+        for (int m = 0; m < Q; ++m) g[m] = ld1<ST>(f + (size_t)m * L.nSpad + i, L.fsi);
+        const uint2 w = __ldg(&lwp[i]);
+        const uint32_t cw = __ldg(&L.coord[i]);
+        float drho, jx, jy, jz;
+        bgk_pairs(g, L.tau_inv, L.rho_f, drho, jx, jy, jz);
+        if (MON) mon_add(a, drho, jx, jy, jz, L.rho_f);
+        if (i >= mon.p0 && i < mon.p1) {
+            a.pdrho += drho;
+            a.pcnt += 1.f;
+        }
+        if (w.x & LW_MASK) {
+            int x, y, z;
+            unpack_coord(cw, x, y, z);
+            all_links(L, P, x, y, z, w, rep, g, n);
+        }
+#pragma unroll
+        for (int m = 0; m < Q; ++m) st1<ST>(f + (size_t)opp(m) * L.nSpad + i, g[m], L.fs);
+    }
+    columns_add(P, rep, n);
+    mon_flush<MON>(a, mon, true);
+}
+
+// ---- even step with few links
+//
+// The same for lattices where few nodes have links (a sphere alone in a box):
+// two slots per lane in registers carry the sums of two spheres over
+// EVEN_ROUNDS runs of nodes.  What such a flow has across its axis (plane
+// momenta, the torque on the sphere) is little more than the rounding of
+// these sums, and this order of them is kept: 48^3, R 8.9, 128 steps, those
+// momenta move by 1.7e-5 of themselves against 2.2e-5 with the columns and
+// 3.9e-5 with the odd steps' links in the collide kernel too.  Time per even
+// step: 60^3 10.5 us against 9.2 us with columns, 160^3 115 and 110 us; with
+// 5.3 links per node (128 x 128 x 1024 column) 184 and 181 us.
 
 struct LinkSlot {
     int p;
@@ -252,7 +524,7 @@ __device__ __forceinline__ void slot_add(LinkSlot& s0, LinkSlot& s1, const PartV
 }
 
 // The links of node (x, y, z) to sphere p (bit m of msk: direction m).
-__device__ __forceinline__ void node_links(const Lat& L, const PartView& P, int x, int y, int z, int p, uint32_t msk,
+__device__ __forceinline__ void slot_links(const Lat& L, const PartView& P, int x, int y, int z, int p, uint32_t msk,
                                            float g[Q], float out[6]) {
     const float4 a = P.pk[3 * (size_t)p], b = P.pk[3 * (size_t)p + 1], c = P.pk[3 * (size_t)p + 2];
     const int ox = __float_as_int(c.y), oy = __float_as_int(c.z), oz = __float_as_int(c.w);
@@ -290,15 +562,6 @@ __device__ __forceinline__ int neighbour_owner(const Lat& L, int x, int y, int z
     return L.owner[((size_t)xs * L.ny + ys) * L.nz + zs];
 }
 
-template <int ST> __device__ __forceinline__ float ld1(const typename PopT<ST>::T* p, float fsi) {
-    return to_f<ST>(*p, fsi);
-}
-template <> __device__ __forceinline__ float ld1<0>(const float* p, float) { return __ldcs(p); }
-template <int ST> __device__ __forceinline__ void st1(typename PopT<ST>::T* p, float v, float fs) {
-    *p = from_f<ST>(v, fs);
-}
-template <> __device__ __forceinline__ void st1<0>(float* p, float v, float) { __stcs(p, v); }
-
 // Each warp takes EVEN_ROUNDS consecutive runs of 32 nodes, one node per
 // lane and run (coalesced); the lanes' sphere slots carry over from run to
 // run (neighbouring runs mostly touch the same spheres), so the warp sums
@@ -306,11 +569,10 @@ template <> __device__ __forceinline__ void st1<0>(float* p, float v, float) { _
 constexpr int EVEN_ROUNDS = 2;
 
 // 72 registers (a few spills to L1): 28 resident warps per SM instead of 24
-// at the 80 the kernel would otherwise take, which hides more of the
-// population loads' latency (187 against 190 us on the 128 x 128 x 1024
-// column).  Launched with up to 256 threads per block.
+// at the 80 the kernel would otherwise take.  Launched with up to 256 threads
+// per block.
 template <bool MON, int ST>
-__global__ void __maxnreg__(72) k_collide_even_links(Lat L, Mon mon, PartView P, const uint2* __restrict__ lwp) {
+__global__ void __maxnreg__(72) k_collide_even_slots(Lat L, Mon mon, PartView P, const uint2* __restrict__ lwp) {
     pdl_wait();
     pdl_trigger();
     auto* f = pops<ST>(L);
@@ -343,10 +605,10 @@ __global__ void __maxnreg__(72) k_collide_even_links(Lat L, Mon mon, PartView P,
             const uint32_t pa = w.x >> 18, pb = w.y >> 18, sel = w.y & LW_MASK;
             float v[6];
             if (pa != LW_NONE) {
-                node_links(L, P, x, y, z, (int)pa, mask & ~sel, g, v);
+                slot_links(L, P, x, y, z, (int)pa, mask & ~sel, g, v);
                 slot_add(s0, s1, P, (int)pa, v, rep);
                 if (sel) {
-                    node_links(L, P, x, y, z, (int)pb, sel, g, v);
+                    slot_links(L, P, x, y, z, (int)pb, sel, g, v);
                     slot_add(s0, s1, P, (int)pb, v, rep);
                 }
             } else {
@@ -361,7 +623,7 @@ __global__ void __maxnreg__(72) k_collide_even_links(Lat L, Mon mon, PartView P,
 #pragma unroll
                     for (int m = 0; m < Q - 1; ++m)
                         if (((rem >> m) & 1u) && neighbour_owner(L, x, y, z, m) == p) sub |= 1u << m;
-                    node_links(L, P, x, y, z, p, sub, g, v);
+                    slot_links(L, P, x, y, z, p, sub, g, v);
                     slot_add(s0, s1, P, p, v, rep);
                     rem &= ~sub;
                 }
@@ -424,26 +686,6 @@ __global__ void __maxnreg__(72) k_collide_even_links(Lat L, Mon mon, PartView P,
     mon_flush<MON>(a, mon, true);
 }
 
-template <int ST>
-static void launch_even_links_st(const Lat& L, const Mon& mon, const PartView& P, const uint2* lw, bool monitor,
-                                 int tile, cudaStream_t s) {
-    const uint32_t blocks = (L.nS + tile * EVEN_ROUNDS - 1) / (tile * EVEN_ROUNDS);
-    if (monitor)
-        launch_pdl(k_collide_even_links<true, ST>, blocks, tile, s, L, mon, P, lw);
-    else
-        launch_pdl(k_collide_even_links<false, ST>, blocks, tile, s, L, mon, P, lw);
-}
-
-void launch_collide_even_links(const Lat& L, const Mon& mon, const PartView& P, const uint2* lw, bool monitor,
-                               int tile, cudaStream_t s) {
-    if (L.nS == 0) return;
-    switch (L.st) {
-        case 0: launch_even_links_st<0>(L, mon, P, lw, monitor, tile, s); break;
-        case 1: launch_even_links_st<1>(L, mon, P, lw, monitor, tile, s); break;
-        default: launch_even_links_st<2>(L, mon, P, lw, monitor, tile, s); break;
-    }
-}
-
 // Compact indices of the stored nodes at z, z + 1 and z - 1 of one z-line
 // from one population count: b = z & 31, low the bits below it; the word's
 // prev and next serve the line's neighbours outside the word.
@@ -472,8 +714,13 @@ struct LineIndex {
 // offsets wait in shared memory from the loads to the stores, which leaves
 // 40 registers and 48 warps per SM, 139 and 120 us.  152 B per fluid node
 // plus its 8 B link word: 98 and 97 us at the copy rate.
-template <bool MON, int ST, bool SNAP>
-__global__ void __launch_bounds__(256, 6) k_collide_odd(Lat L, Mon mon, const uint2* __restrict__ lw, float* snap) {
+//
+// With LINKS the step's links are taken here too (see above), at 56 registers:
+// 191 us on the same column (64: 196, 48 with spills: 196) against 138 and
+// 141 in a link kernel that loads and stores the links' populations again.
+template <bool MON, int ST, bool SNAP, bool LINKS>
+__global__ void __maxnreg__(LINKS ? 56 : 40)
+k_collide_odd(Lat L, Mon mon, const uint2* __restrict__ lw, float* snap, PartView P) {
     pdl_wait();
     pdl_trigger();
     auto* f = pops<ST>(L);
@@ -484,6 +731,9 @@ __global__ void __launch_bounds__(256, 6) k_collide_odd(Lat L, Mon mon, const ui
     // three independent loads: then the word records, then the populations
     const bool in = i < L.nS;
     const uint32_t cw = in ? __ldcs(&L.coord[i]) : 0u, lwx = in ? __ldg(&lw[i].x) : 0u;
+    LinkSums n = {reinterpret_cast<float*>(s_off + (blockDim.x >> 5) * ((Q - 1) * 32)) +
+                      (threadIdx.x >> 5) * (LINK_COLS * 32) + (threadIdx.x & 31),
+                  -1, -1};
     if (in && fluid_bit(L, i)) {
         uint32_t wall = lwx & LW_MASK;  // directions without a fluid neighbour
         int x, y, z;
@@ -554,7 +804,9 @@ __global__ void __launch_bounds__(256, 6) k_collide_odd(Lat L, Mon mon, const ui
             for (int m = 0; m < Q; ++m) __stcs(snap + (size_t)m * L.nSpad + i, g[m]);
         }
         float drho, jx, jy, jz;
-        bgk(g, L.tau_inv, L.rho_f, drho, jx, jy, jz);
+        if (LINKS) bgk_pairs(g, L.tau_inv, L.rho_f, drho, jx, jy, jz);
+        else bgk(g, L.tau_inv, L.rho_f, drho, jx, jy, jz);
+        if (LINKS && (lwx & LW_MASK)) all_links(L, P, x, y, z, __ldg(&lw[i]), (i >> 5) % NREP, g, n);
 #pragma unroll
         for (int m = 0; m < Q - 1; ++m) f[off[m * 32]] = from_f<ST>(g[m], L.fs);
         f[18u * L.nSpad + i] = from_f<ST>(g[18], L.fs);
@@ -564,7 +816,40 @@ __global__ void __launch_bounds__(256, 6) k_collide_odd(Lat L, Mon mon, const ui
             a.pcnt += 1.f;
         }
     }
+    if (LINKS) columns_add(P, (i >> 5) % NREP, n);
     mon_flush<MON>(a, mon, true);
+}
+
+template <int ST>
+static void launch_collide_links_st(const Lat& L, const Mon& mon, const PartView& P, bool odd, bool monitor,
+                                    bool few, const uint2* lw, int tile, cudaStream_t s) {
+    if (few && !odd) {
+        const uint32_t nodes = tile * EVEN_ROUNDS, blocks = (L.nS + nodes - 1) / nodes;
+        if (monitor) launch_pdl(k_collide_even_slots<true, ST>, blocks, tile, s, L, mon, P, lw);
+        else launch_pdl(k_collide_even_slots<false, ST>, blocks, tile, s, L, mon, P, lw);
+        return;
+    }
+    const uint32_t blocks = (L.nS + tile - 1) / tile;
+    const size_t smem = (size_t)(LINK_COLS + (odd ? Q - 1 : 0)) * tile * sizeof(float);
+    float* none = nullptr;
+    if (odd) {
+        if (monitor) launch_pdl_smem(k_collide_odd<true, ST, false, true>, blocks, tile, smem, s, L, mon, lw, none, P);
+        else launch_pdl_smem(k_collide_odd<false, ST, false, true>, blocks, tile, smem, s, L, mon, lw, none, P);
+    } else {
+        if (monitor) launch_pdl_smem(k_collide_even_links<true, ST>, blocks, tile, smem, s, L, mon, P, lw);
+        else launch_pdl_smem(k_collide_even_links<false, ST>, blocks, tile, smem, s, L, mon, P, lw);
+    }
+}
+
+// few: a lattice of few links per node (even steps only)
+void launch_collide_links(const Lat& L, const Mon& mon, const PartView& P, bool odd, bool monitor, bool few,
+                          const uint2* lw, int tile, cudaStream_t s) {
+    if (L.nS == 0) return;
+    switch (L.st) {
+        case 0: launch_collide_links_st<0>(L, mon, P, odd, monitor, few, lw, tile, s); break;
+        case 1: launch_collide_links_st<1>(L, mon, P, odd, monitor, few, lw, tile, s); break;
+        default: launch_collide_links_st<2>(L, mon, P, odd, monitor, few, lw, tile, s); break;
+    }
 }
 
 template <int ST>
@@ -573,9 +858,9 @@ static void launch_collide_st(const Lat& L, const Mon& mon, bool odd, bool monit
     const uint32_t threads = odd ? L.nS : (L.nS + 3) / 4, blocks = (threads + tile - 1) / tile;
     const size_t smem = (size_t)(Q - 1) * tile * sizeof(uint32_t);  // 4.6 KB per 64 threads
     if (odd) {
-        if (snap) launch_pdl_smem(k_collide_odd<false, ST, true>, blocks, tile, smem, s, L, mon, lw, snap);
-        else if (monitor) launch_pdl_smem(k_collide_odd<true, ST, false>, blocks, tile, smem, s, L, mon, lw, snap);
-        else launch_pdl_smem(k_collide_odd<false, ST, false>, blocks, tile, smem, s, L, mon, lw, snap);
+        if (snap) launch_pdl_smem(k_collide_odd<false, ST, true, false>, blocks, tile, smem, s, L, mon, lw, snap, PartView{});
+        else if (monitor) launch_pdl_smem(k_collide_odd<true, ST, false, false>, blocks, tile, smem, s, L, mon, lw, snap, PartView{});
+        else launch_pdl_smem(k_collide_odd<false, ST, false, false>, blocks, tile, smem, s, L, mon, lw, snap, PartView{});
     } else {
         if (snap) launch_pdl(k_collide_even<false, ST, true>, blocks, tile, s, L, mon, snap);
         else if (monitor) launch_pdl(k_collide_even<true, ST, false>, blocks, tile, s, L, mon, snap);
