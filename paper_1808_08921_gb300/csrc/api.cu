@@ -804,14 +804,14 @@ static void enqueue_step(lbmdem_ctx* c, int parity, bool monitor, int inlet, boo
         // side stream joined before the next step
         if (inlet_outlet_active(c) && inlet == INLET_NOW && !dem_active(c)) {
             if (tm) record_pair_begin(c, 3, e);
-            launch_inlet_outlet(L, bc, parity == 0, s);
+            launch_inlet_outlet(L, bc, c->linkw.p, parity == 0, s);
             if (tm) record_pair_end(c, e);
         } else if (inlet_outlet_active(c) && inlet == INLET_NOW) {
             cudaEventRecord(c->ev_fork, s);
             cudaStreamWaitEvent(c->side, c->ev_fork, 0);
             size_t e2 = 0;
             if (tm) record_pair_begin(c, 3, e2, c->side);
-            launch_inlet_outlet(L, bc, parity == 0, c->side);
+            launch_inlet_outlet(L, bc, c->linkw.p, parity == 0, c->side);
             if (tm) record_pair_end(c, e2, c->side);
             cudaEventRecord(c->ev_join, c->side);
             Dem D = make_dem(c);

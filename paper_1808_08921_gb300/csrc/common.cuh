@@ -277,9 +277,11 @@ constexpr int NREP = 4;
 
 // Exact "inside" test shared by painting and the map update: |y - X|^2 < R^2
 // in FP64 without contraction, X = Xref + dX (+ compensation).
+__device__ __forceinline__ double norm2_exact(double ax, double ay, double az) {
+    return __dadd_rn(__dadd_rn(__dmul_rn(ax, ax), __dmul_rn(ay, ay)), __dmul_rn(az, az));
+}
 __device__ __forceinline__ bool inside_exact(double ax, double ay, double az, double R) {
-    double s = __dadd_rn(__dadd_rn(__dmul_rn(ax, ax), __dmul_rn(ay, ay)), __dmul_rn(az, az));
-    return s < __dmul_rn(R, R);
+    return norm2_exact(ax, ay, az) < __dmul_rn(R, R);
 }
 
 // FP32 |a|^2 with a fixed rounding (no contraction), used identically by the
@@ -293,8 +295,7 @@ constexpr float FP32_MARGIN = 1e-5f;
 // |y - X|^2 / R^2 with the same operation order and rounding as the test
 // above; among the spheres that contain a node, the smallest ratio owns it.
 __device__ __forceinline__ double inside_ratio(double ax, double ay, double az, double R) {
-    double s = __dadd_rn(__dadd_rn(__dmul_rn(ax, ax), __dmul_rn(ay, ay)), __dmul_rn(az, az));
-    return __ddiv_rn(s, __dmul_rn(R, R));
+    return __ddiv_rn(norm2_exact(ax, ay, az), __dmul_rn(R, R));
 }
 
 __device__ __forceinline__ double minimg(double d, double L, int periodic) {

@@ -254,6 +254,8 @@ struct MapArgs {
     uint2* lw;      // link words, renewed around converted nodes
     BC bc;          // the previous step's inlet / outlet,
     int io_blocks;  // applied by the first io_blocks blocks of the band kernel
+    int sphere_blocks;  // its next ones prepare the spheres
+    bool ahead;         // the band kernel is launched behind the DEM
 };
 
 // Link word of the stored node (x, y, z) from the owner map (see LW_MASK):
@@ -321,71 +323,98 @@ __device__ __forceinline__ uint32_t* flip_masks(const Lat& L, int par) {
 // of the previous step (other parity) are cleared here from its queue.
 // Launched with a programmatic dependency on the DEM, which hides its launch
 // behind the substeps (2.2 us per step as an ordinary successor of the DEM and
-// of a boundary kernel on a second stream).
+// of a boundary kernel on a second stream).  After the DEM it is latency: the
+// boundary's places (3.7 us of dependent loads when found after the wait), the
+// spheres' tables (1.1 us, in blocks of their own) and the few nodes that take
+// the FP64 rule (4.7 us with one candidate after the other and a division
+// each) set its end, so all that can be read ahead is, and the candidates'
+// loads go together: 12 x 12 x 620 chain 31.3 -> 29.1 us per step, 64 x 64 x
+// 512 column 83.0 -> 82.0.
 template <bool AFTER_EVEN, int ST>
-__global__ void __launch_bounds__(256) k_map_band(MapArgs A) {
+__global__ void __launch_bounds__(256, 6) k_map_band(MapArgs A) {
     const Lat& L = A.L;
     if ((int)blockIdx.x < A.io_blocks) {
         __shared__ float s_drho;
         if (threadIdx.x == 0) s_drho = (float)source_drho(A.bc.src, *A.bc.t_dev);
+        const BoundaryNode<AFTER_EVEN, ST> node(L, A.bc, A.lw, blockIdx.x * blockDim.x + threadIdx.x);
         __syncthreads();
         pdl_wait();
         pdl_trigger();
-        inlet_outlet_node<AFTER_EVEN, ST>(L, A.bc, s_drho, blockIdx.x * blockDim.x + threadIdx.x);
+        node.apply(L, A.bc, s_drho);
         return;
     }
-    const uint32_t k = (blockIdx.x - A.io_blocks) * blockDim.x + threadIdx.x;
-    const float slack = k < A.band.n ? A.band.slack[k] : 0.f;
+    if ((int)blockIdx.x < A.io_blocks + A.sphere_blocks) {  // the spheres' sums and tables
+        const uint32_t k = (blockIdx.x - A.io_blocks) * blockDim.x + threadIdx.x;
+        pdl_wait();
+        pdl_trigger();
+        if (k >= (uint32_t)A.P.n) return;
+                for (int r = 0; r < NREP; ++r)
+                    for (int a = 0; a < 3; ++a) {
+                        A.P.Fh[3 * ((size_t)r * A.P.n + k) + a] = 0.0;
+                        A.P.Th[3 * ((size_t)r * A.P.n + k) + a] = 0.0;
+                    }
+                // moving-wall terms of this step's links of sphere k, per direction
+                // m: beta = 6 w rho_f (c x W) and alpha' = 6 w rho_f c.V - xf.beta,
+                // so that the term of Eq. 14 at a link node with offset rel from the
+                // sphere's lattice origin is alpha' + rel.beta
+                const float4 V = A.P.V[k], W = A.P.W[k], xf = A.P.xf[k];
+                const float s6 = 6.0f * A.L.rho_f;
+        #pragma unroll
+                for (int m = 0; m < Q - 1; ++m) {
+                    const float sw = s6 * wt(m);
+                    const float ex = (float)cx(m), ey = (float)cy(m), ez = (float)cz(m);
+                    const float bx = sw * (ey * W.z - ez * W.y), by = sw * (ez * W.x - ex * W.z),
+                                bz = sw * (ex * W.y - ey * W.x);
+                    const float alpha = sw * (ex * V.x + ey * V.y + ez * V.z);
+                    A.P.ab[(size_t)k * (Q - 1) + m] = make_float4(alpha - (xf.x * bx + xf.y * by + xf.z * bz), bx, by, bz);
+                }
+                // the same state for the even steps' links inside the collide kernel
+                const int4 o = A.P.orgw[k];
+                A.P.pk[3 * (size_t)k] = make_float4(xf.x, xf.y, xf.z, V.x);
+                A.P.pk[3 * (size_t)k + 1] = make_float4(V.y, V.z, W.x, W.y);
+                A.P.pk[3 * (size_t)k + 2] = make_float4(W.z, __int_as_float(o.x), __int_as_float(o.y), __int_as_float(o.z));
+        return;
+    }
+    // launched behind the DEM, what that does not write is read ahead of the
+    // wait for it: the band (fixed since the layout) and the owners (last written
+    // by the previous step's band kernel, which ended before the DEM began)
+    const uint32_t k = (blockIdx.x - A.io_blocks - A.sphere_blocks) * blockDim.x + threadIdx.x;
+    const bool in = k < A.band.n;
+    const float slack = in ? A.band.slack[k] : 0.f;
+    uint32_t cw = 0u;
+    int4 cand = make_int4(-1, -1, -1, -1);
+    int old = OWNER_FLUID;
+    auto load = [&] {
+        int cx_, cy_, cz_;
+        cw = A.band.coord[k];
+        cand = A.band.cand[k];
+        unpack_coord(cw, cx_, cy_, cz_);
+        old = L.owner[((size_t)cx_ * L.ny + cy_) * L.nz + cz_];
+    };
+    const bool ahead = in && A.ahead;
+    if (ahead) load();
     pdl_wait();
     pdl_trigger();
     if (k == 0) A.st->t_end[A.par] = A.st->t += 1ull;  // the step starts: t counts it from here on
     {
-        const uint32_t prev = min(A.st->nflip[A.par ^ 1], A.F.cap), stride = (gridDim.x - A.io_blocks) * blockDim.x;
+        const uint32_t prev = min(A.st->nflip[A.par ^ 1], A.F.cap),
+                       stride = (gridDim.x - A.io_blocks - A.sphere_blocks) * blockDim.x;
         for (uint32_t w = k; w < prev; w += stride) {
-            int x, y, z;
-            unpack_coord(A.F.rec[(size_t)(A.par ^ 1) * A.F.cap + w].coord, x, y, z);
-            flip_masks(L, A.par ^ 1)[word_of(L, x, y, z)] = 0u;
+            int fx, fy, fz;
+            unpack_coord(A.F.rec[(size_t)(A.par ^ 1) * A.F.cap + w].coord, fx, fy, fz);
+            flip_masks(L, A.par ^ 1)[word_of(L, fx, fy, fz)] = 0u;
         }
     }
-    if (k < (uint32_t)A.P.n) {
-        for (int r = 0; r < NREP; ++r)
-            for (int a = 0; a < 3; ++a) {
-                A.P.Fh[3 * ((size_t)r * A.P.n + k) + a] = 0.0;
-                A.P.Th[3 * ((size_t)r * A.P.n + k) + a] = 0.0;
-            }
-        // moving-wall terms of this step's links of sphere k, per direction
-        // m: beta = 6 w rho_f (c x W) and alpha' = 6 w rho_f c.V - xf.beta,
-        // so that the term of Eq. 14 at a link node with offset rel from the
-        // sphere's lattice origin is alpha' + rel.beta
-        const float4 V = A.P.V[k], W = A.P.W[k], xf = A.P.xf[k];
-        const float s6 = 6.0f * A.L.rho_f;
-#pragma unroll
-        for (int m = 0; m < Q - 1; ++m) {
-            const float sw = s6 * wt(m);
-            const float ex = (float)cx(m), ey = (float)cy(m), ez = (float)cz(m);
-            const float bx = sw * (ey * W.z - ez * W.y), by = sw * (ez * W.x - ex * W.z),
-                        bz = sw * (ex * W.y - ey * W.x);
-            const float alpha = sw * (ex * V.x + ey * V.y + ez * V.z);
-            A.P.ab[(size_t)k * (Q - 1) + m] = make_float4(alpha - (xf.x * bx + xf.y * by + xf.z * bz), bx, by, bz);
-        }
-        // the same state for the even steps' links inside the collide kernel
-        const int4 o = A.P.orgw[k];
-        A.P.pk[3 * (size_t)k] = make_float4(xf.x, xf.y, xf.z, V.x);
-        A.P.pk[3 * (size_t)k + 1] = make_float4(V.y, V.z, W.x, W.y);
-        A.P.pk[3 * (size_t)k + 2] = make_float4(W.z, __int_as_float(o.x), __int_as_float(o.y), __int_as_float(o.z));
-    }
-    if (k >= A.band.n) return;
+    if (!in) return;
     // a node farther from every candidate surface (at the layout) than any
     // sphere has moved since keeps its owner
     if (!A.st->layout_fresh) {
         const float moved = __uint_as_float(A.st->disp_layout_bits);
         if (slack > moved + 1e-5f * (1.f + moved)) return;
     }
+    if (!ahead) load();
     int x, y, z;
-    unpack_coord(A.band.coord[k], x, y, z);
-    const size_t li = ((size_t)x * L.ny + y) * L.nz + z;
-    const int old = L.owner[li];  // issued early: independent of the test
-    int4 cand = A.band.cand[k];
+    unpack_coord(cw, x, y, z);
     int c4[4] = {cand.x, cand.y, cand.z, cand.w};
     int best = OWNER_FLUID;
     if (L.px || (x > 0 && x < L.nx - 1)) {
@@ -394,50 +423,67 @@ __global__ void __launch_bounds__(256) k_map_band(MapArgs A) {
         // guarantees the FP64 answer, else the exact FP64 rule decides
         bool exact = false;
         float bestr = 0.f;
-        for (int a = 0; a < 4; ++a) {
-            int p = c4[a];
-            if (p < 0) break;
-            int4 o = A.P.orgw[p];  // origin wrapped into the box: |node - o| < L
-            float4 xf = A.P.xf[p];
-            int ix = L.px ? imin_small(x - o.x, L.nx) : x - o.x;
-            int iy = imin_small(y - o.y, L.ny), iz = imin_small(z - o.z, L.nz);
-            float ax = __fsub_rn((float)ix, xf.x), ay = __fsub_rn((float)iy, xf.y), az = __fsub_rn((float)iz, xf.z);
-            float d2 = norm2_rn(ax, ay, az);
-            float R2 = __fmul_rn(A.P.R[p], A.P.R[p]);
-            if (fabsf(d2 - R2) <= FP32_MARGIN * R2) {
-                exact = true;
-                break;
+        uint32_t near = 0u;  // the candidates that may hold the node
+#pragma unroll
+        for (int h = 0; h < 4; h += 2) {  // two at a time: their loads together
+            if (c4[h] < 0) break;
+            int4 o[2];  // origin wrapped into the box: |node - o| < L
+            float4 xf[2];
+            float R[2];
+#pragma unroll
+            for (int b = 0; b < 2; ++b) {
+                const int p = max(c4[h + b], 0);
+                o[b] = A.P.orgw[p];
+                xf[b] = A.P.xf[p];
+                R[b] = A.P.R[p];
             }
-            if (d2 < R2) {
-                float r = d2 / R2;
-                if (best != OWNER_FLUID && fabsf(r - bestr) <= 1e-5f) {
+#pragma unroll
+            for (int b = 0; b < 2; ++b) {
+                const int p = c4[h + b];
+                if (p < 0) break;
+                int ix = L.px ? imin_small(x - o[b].x, L.nx) : x - o[b].x;
+                int iy = imin_small(y - o[b].y, L.ny), iz = imin_small(z - o[b].z, L.nz);
+                float ax = __fsub_rn((float)ix, xf[b].x), ay = __fsub_rn((float)iy, xf[b].y),
+                      az = __fsub_rn((float)iz, xf[b].z);
+                float d2 = norm2_rn(ax, ay, az);
+                float R2 = __fmul_rn(R[b], R[b]);
+                if (fabsf(d2 - R2) <= FP32_MARGIN * R2) {
                     exact = true;
-                    break;
-                }
-                if (best == OWNER_FLUID || r < bestr) {
-                    best = p;
-                    bestr = r;
+                    near |= 1u << (h + b);
+                } else if (d2 < R2) {
+                    near |= 1u << (h + b);
+                    float r = d2 / R2;
+                    if (best != OWNER_FLUID && fabsf(r - bestr) <= 1e-5f) exact = true;
+                    if (best == OWNER_FLUID || r < bestr) {
+                        best = p;
+                        bestr = r;
+                    }
                 }
             }
         }
         if (exact) {
+            // the FP64 rule for the candidates that are not clearly outside.
+            // With equal radii the nearer centre has the smaller ratio; only
+            // distances that agree to 2^-50 take the division of the rule
             best = OWNER_FLUID;
-            double best_ratio = 0.0;
+            double bs = 0.0, br = 0.0;  // of the best: |y - X|^2 and R^2
+#pragma unroll
             for (int a = 0; a < 4; ++a) {  // candidates ascend: ties keep the lowest index
-                int p = c4[a];
-                if (p < 0) break;
+                if (!((near >> a) & 1u)) continue;
+                const int p = c4[a];
                 double X0, X1, X2;
                 centre(A.P, p, X0, X1, X2);
-                double ax = node_offset(x, X0, L.nx, L.px);
-                double ay = node_offset(y, X1, L.ny, 1);
-                double az = node_offset(z, X2, L.nz, 1);
-                double Rp = A.P.Rd[p];
-                if (inside_exact(ax, ay, az, Rp)) {
-                    double r = inside_ratio(ax, ay, az, Rp);
-                    if (best == OWNER_FLUID || r < best_ratio) {
-                        best = p;
-                        best_ratio = r;
-                    }
+                const double ax = node_offset(x, X0, L.nx, L.px), ay = node_offset(y, X1, L.ny, 1),
+                             az = node_offset(z, X2, L.nz, 1);
+                const double Rp = A.P.Rd[p], rr = __dmul_rn(Rp, Rp), ss = norm2_exact(ax, ay, az);
+                if (!(ss < rr)) continue;
+                bool closer = best == OWNER_FLUID;
+                if (!closer && rr == br && fabs(ss - bs) > 0x1p-50 * bs) closer = ss < bs;
+                else if (!closer) closer = __ddiv_rn(ss, rr) < __ddiv_rn(bs, br);
+                if (closer) {
+                    best = p;
+                    bs = ss;
+                    br = rr;
                 }
             }
         }
@@ -455,12 +501,12 @@ __global__ void __launch_bounds__(256) k_map_band(MapArgs A) {
             return;
         }
         Flip f;
-        f.coord = A.band.coord[k];
+        f.coord = cw;
         f.old_owner = old;
         f.new_owner = best;
         f.pad = 0;
         A.F.rec[(size_t)A.par * A.F.cap + slot] = f;
-        L.owner[li] = best;
+        L.owner[((size_t)x * L.ny + y) * L.nz + z] = best;
         if (old == OWNER_FLUID || best == OWNER_FLUID) {
             const uint32_t wi = word_of(L, x, y, z), bit = 1u << (z & 31);
             atomicXor(&L.fluid[wi], bit);
@@ -655,16 +701,15 @@ void launch_map_update(const Lat& L, const PartView& P, const Band& band, const 
                        cudaStream_t s) {
     const unsigned bb = shared_gpu ? 256 : 64;
     const unsigned io = inlet ? (unsigned)((2 * L.ny * L.nz + bb - 1) / bb) : 0u;
-    MapArgs A{L, P, band, F, st, step_parity, lw, inlet ? *inlet : BC{}, (int)io};
+    const unsigned sph = (unsigned)((P.n + bb - 1) / bb);
+    MapArgs A{L, P, band, F, st, step_parity, lw, inlet ? *inlet : BC{}, (int)io, (int)sph, early && !shared_gpu};
     const bool after_even = step_parity == 1;
-    uint32_t nb = band.n > (uint32_t)P.n ? band.n : (uint32_t)P.n;
-    if (nb == 0) nb = 1;
-    const unsigned blocks = io + (nb + bb - 1) / bb;
+    const unsigned blocks = io + sph + std::max(1u, (band.n + bb - 1) / bb);  // one counts the step in any case
     // the queued count is read on the device: fixed grids stride over it
     const unsigned grid = shared_gpu ? 152 : 4 * 152;
 #define LBMDEM_MB(AE, ST)                                                              \
     do {                                                                               \
-        if (early && !shared_gpu) launch_pdl(k_map_band<AE, ST>, blocks, bb, s, A);    \
+        if (A.ahead) launch_pdl(k_map_band<AE, ST>, blocks, bb, s, A);    \
         else k_map_band<AE, ST><<<blocks, bb, 0, s>>>(A);                              \
         if (band.n) launch_pdl(k_map_gather_convert<AE, ST>, grid, MAP_THREADS + LW_THREADS, s, A);    \
         if (band.n && AE) launch_pdl(k_map_scatter<ST>, grid, MAP_THREADS, s, A);      \

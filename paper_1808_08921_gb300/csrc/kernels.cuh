@@ -69,49 +69,96 @@ __device__ __forceinline__ void pressure_face(float g[Q], float drho_b, int side
     }
 }
 
+// Link word of a stored node (one 8-byte word per node), for the odd collide
+// kernel's fluid neighbours (.x) and the links taken inside the collide
+// kernels:
+//   .x = link mask (bit m, m < 18: the neighbour x + c_m is solid) | sphere A << 18
+//   .y = B mask (bit m: that link's neighbour belongs to sphere B) | sphere B << 18
+// Sphere indices take 14 bits; LW_NONE stands for no sphere B, and as sphere
+// A for a node whose solid neighbours belong to more than two spheres (its
+// links then read the owner map).  With more spheres than LW_MAX_SPHERES the
+// indices are cut off and only the mask is used.  Built at the layout from the owner map
+// and renewed for every converted node and its 18 neighbours.
+constexpr uint32_t LW_MASK = (1u << 18) - 1u;
+constexpr uint32_t LW_NONE = 0x3fffu;
+constexpr int LW_MAX_SPHERES = (int)LW_NONE;  // sphere indices 0 .. LW_NONE - 1
+
 // The inlet / outlet of the step that ended, one thread per boundary node:
-// k < ny nz the inlet plane, then the outlet plane.  drho: the source's
-// density deviation at the new time.
+// k < ny nz the inlet plane, then the outlet plane.  Where the populations it
+// reads are stored follows from the stored words, fixed since the layout, and
+// from the link words, which change only after every block of the band kernel
+// has ended: boundary blocks inside that kernel work by the map before its
+// conversions, and find the places before they wait for the previous kernel.
 template <bool AFTER_EVEN, int ST>
-__device__ __forceinline__ void inlet_outlet_node(const Lat& L, const BC& bc, float drho, int k) {
-    auto* f = pops<ST>(L);
-    const int plane = L.ny * L.nz;
-    if (k >= 2 * plane) return;
-    int side = k >= plane;
-    int yz = side ? k - plane : k;
-    int y = yz / L.nz, z = yz - y * L.nz;
-    int x = side ? L.nx - 1 : 0;
-    bool fl;
-    uint32_t i = stored_index(L, x, y, z, fl);
-    if (!fl || i == NONE) return;
-    if (side == 0) {
-        if (bc.inlet != 0) return;
-        float g[Q];
-#pragma unroll
-        for (int m = 0; m < Q; ++m)
-            if (cx(m) <= 0) g[m] = to_f<ST>(*pop_loc<ST>(L, AFTER_EVEN, x, y, z, i, m), L.fsi);
-        pressure_face(g, drho, 0);
-#pragma unroll
-        for (int m = 0; m < Q; ++m)
-            if (cx(m) > 0) f[(size_t)m * L.nSpad + i] = from_f<ST>(g[m], L.fs);  // source outside: own slot
-    } else if (bc.outlet == 0) {
-        bool ufl;
-        uint32_t u = stored_index(L, x - 1, y, z, ufl);
-        if (!ufl || u == NONE) return;
-#pragma unroll
-        for (int m = 0; m < Q; ++m)
-            if (cx(m) < 0) f[(size_t)m * L.nSpad + i] = *pop_loc<ST>(L, AFTER_EVEN, x - 1, y, z, u, m);
-    } else if (bc.outlet == 1) {
-        float g[Q];
-#pragma unroll
-        for (int m = 0; m < Q; ++m)
-            if (cx(m) >= 0) g[m] = to_f<ST>(*pop_loc<ST>(L, AFTER_EVEN, x, y, z, i, m), L.fsi);
-        pressure_face(g, 0.f, 1);
-#pragma unroll
-        for (int m = 0; m < Q; ++m)
-            if (cx(m) < 0) f[(size_t)m * L.nSpad + i] = from_f<ST>(g[m], L.fs);
+struct BoundaryNode {
+    uint32_t i;       // the node, NONE: nothing to do
+    int side;         // 0 inlet, 1 outlet
+    uint32_t src[Q];  // offsets of the populations read
+    uint32_t P;       // stride of a population
+
+    // natural population m of fluid node (x, y, z) = n with solid neighbours s;
+    // o: the direction against m, to the node (x, y, z) + d it comes from
+    __device__ __forceinline__ uint32_t place(const Lat& L, int x, int y, int z, uint32_t n, uint32_t s, int m, int o,
+                                              int dx, int dy, int dz) const {
+        const uint32_t own = (uint32_t)m * P + n;
+        if (!AFTER_EVEN) return own;
+        const int xs = x + dx, ys = wrap1(y + dy, L.ny), zs = wrap1(z + dz, L.nz);
+        const bool in = xs >= 0 && xs < L.nx;
+        const uint4 r = __ldg(&L.rec[word_of(L, in ? xs : x, ys, zs)]);
+        return !in || ((s >> o) & 1u) ? own : (uint32_t)o * P + rec_index(r, 1u << (zs & 31));
     }
-}
+
+    __device__ __forceinline__ BoundaryNode(const Lat& L, const BC& bc, const uint2* lw, int k) : i(NONE), P(L.nSpad) {
+        const int plane = L.ny * L.nz;
+        side = k >= plane;
+        if (k >= 2 * plane || (side == 0 && bc.inlet != 0) || (side == 1 && bc.outlet > 1)) return;
+        const int yz = side ? k - plane : k, y = yz / L.nz, z = yz - y * L.nz, x = side ? L.nx - 1 : 0;
+        // the boundary planes are never solid
+        const uint32_t bit = 1u << (z & 31), n = rec_index(L.rec[word_of(L, x, y, z)], bit);
+        const uint32_t s = lw[n].x;
+        if (side == 1 && bc.outlet == 0) {  // zero gradient: the neighbour's, if it is fluid
+            if (x == 0 || (s >> 1) & 1u) return;
+            const uint32_t u = rec_index(L.rec[word_of(L, x - 1, y, z)], bit), su = lw[u].x;
+#pragma unroll
+            for (int m = 0; m < Q; ++m)
+                if (cx(m) < 0) src[m] = place(L, x - 1, y, z, u, su, m, opp(m), -cx(m), -cy(m), -cz(m));
+        } else {
+#pragma unroll
+            for (int m = 0; m < Q - 1; ++m) {  // m at the outlet (cx >= 0), the opposite at the inlet
+                const int a = side ? -1 : 1;
+                if (cx(m) >= 0)
+                    src[m] = place(L, x, y, z, n, s, side ? m : opp(m), side ? opp(m) : m, a * cx(m), a * cy(m), a * cz(m));
+            }
+            src[18] = 18u * P + n;
+        }
+        i = n;
+    }
+
+    // drho: the source's density deviation at the new time
+    __device__ __forceinline__ void apply(const Lat& L, const BC& bc, float drho) const {
+        if (i == NONE) return;
+        auto* f = pops<ST>(L);
+        if (side == 1 && bc.outlet == 0) {
+#pragma unroll
+            for (int m = 0; m < Q; ++m)
+                if (cx(m) < 0) f[(size_t)m * P + i] = f[src[m]];
+            return;
+        }
+        float g[Q];
+#pragma unroll
+        for (int m = 0; m < Q - 1; ++m) {
+            if (cx(m) < 0) continue;
+            const float v = to_f<ST>(f[src[m]], L.fsi);
+            if (side) g[m] = v;
+            else g[opp(m)] = v;
+        }
+        g[18] = to_f<ST>(f[src[18]], L.fsi);
+        pressure_face(g, side ? 0.f : drho, side);
+#pragma unroll
+        for (int m = 0; m < Q; ++m)  // those that would come from outside: own slots
+            if (side ? cx(m) < 0 : cx(m) > 0) f[(size_t)m * P + i] = from_f<ST>(g[m], L.fs);
+    }
+};
 
 // Link lists for the link kernel.  Links are grouped by (sphere, direction
 // m, maybe), each group padded to whole chunks of 32 records, and each
@@ -144,20 +191,6 @@ struct LinkLists {
     const uint8_t* chunk_dir;  // LINK_CHUNKS bytes per warp
     uint32_t nwarps;
 };
-
-// Link word of a stored node (one 8-byte word per node), for the odd collide
-// kernel's fluid neighbours (.x) and the links taken inside the collide
-// kernels:
-//   .x = link mask (bit m, m < 18: the neighbour x + c_m is solid) | sphere A << 18
-//   .y = B mask (bit m: that link's neighbour belongs to sphere B) | sphere B << 18
-// Sphere indices take 14 bits; LW_NONE stands for no sphere B, and as sphere
-// A for a node whose solid neighbours belong to more than two spheres (its
-// links then read the owner map).  With more spheres than LW_MAX_SPHERES the
-// indices are cut off and only the mask is used.  Built at the layout from the owner map
-// and renewed for every converted node and its 18 neighbours.
-constexpr uint32_t LW_MASK = (1u << 18) - 1u;
-constexpr uint32_t LW_NONE = 0x3fffu;
-constexpr int LW_MAX_SPHERES = (int)LW_NONE;  // sphere indices 0 .. LW_NONE - 1
 
 // Nodes whose solid/fluid status can change before the next re-layout.
 struct Band {
@@ -245,7 +278,7 @@ void launch_collide(const Lat& L, const Mon& mon, bool odd, bool monitor, const 
                     cudaStream_t s);
 void launch_collide_links(const Lat& L, const Mon& mon, const PartView& P, bool odd, bool monitor, bool few,
                           const uint2* lw, int tile, cudaStream_t s);
-void launch_inlet_outlet(const Lat& L, const BC& bc, bool after_even, cudaStream_t s);
+void launch_inlet_outlet(const Lat& L, const BC& bc, const uint2* lw, bool after_even, cudaStream_t s);
 void launch_plane_sums(const Lat& L, bool after_even, double* out, cudaStream_t s);
 void launch_read_fields(const Lat& L, bool after_even, double* rho, double* u, uint8_t* solid,
                         cudaStream_t s);

@@ -883,19 +883,20 @@ void launch_collide(const Lat& L, const Mon& mon, bool odd, bool monitor, const 
 // ------------------------------------------------------------ inlet / outlet
 
 template <bool AFTER_EVEN, int ST>
-__global__ void k_inlet_outlet(Lat L, BC bc) {
+__global__ void k_inlet_outlet(Lat L, BC bc, const uint2* lw) {
     __shared__ float s_drho;
     if (threadIdx.x == 0) s_drho = (float)source_drho(bc.src, *bc.t_dev);
+    const BoundaryNode<AFTER_EVEN, ST> node(L, bc, lw, blockIdx.x * blockDim.x + threadIdx.x);
     __syncthreads();
-    inlet_outlet_node<AFTER_EVEN, ST>(L, bc, s_drho, blockIdx.x * blockDim.x + threadIdx.x);
+    node.apply(L, bc, s_drho);
 }
 
-void launch_inlet_outlet(const Lat& L, const BC& bc, bool after_even, cudaStream_t s) {
+void launch_inlet_outlet(const Lat& L, const BC& bc, const uint2* lw, bool after_even, cudaStream_t s) {
     if (L.px) return;
     if (bc.inlet != 0 && bc.outlet > 1) return;
     int n = 2 * L.ny * L.nz;
     int blocks = (n + 127) / 128;
-#define LBMDEM_IO(AE, ST) k_inlet_outlet<AE, ST><<<blocks, 128, 0, s>>>(L, bc)
+#define LBMDEM_IO(AE, ST) k_inlet_outlet<AE, ST><<<blocks, 128, 0, s>>>(L, bc, lw)
     LBMDEM_BY_STATE(LBMDEM_IO);
 #undef LBMDEM_IO
 }
