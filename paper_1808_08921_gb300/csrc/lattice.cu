@@ -484,13 +484,14 @@ k_collide_even_links(Lat L, Mon mon, PartView P, const uint2* __restrict__ lwp) 
 //
 // The same for lattices where few nodes have links (a sphere alone in a box):
 // two slots per lane in registers carry the sums of two spheres over
-// EVEN_ROUNDS runs of nodes.  What such a flow has across its axis (plane
-// momenta, the torque on the sphere) is little more than the rounding of
-// these sums, and this order of them is kept: 48^3, R 8.9, 128 steps, those
-// momenta move by 1.7e-5 of themselves against 2.2e-5 with the columns and
-// 3.9e-5 with the odd steps' links in the collide kernel too.  Time per even
-// step: 60^3 10.5 us against 9.2 us with columns, 160^3 115 and 110 us; with
-// 5.3 links per node (128 x 128 x 1024 column) 184 and 181 us.
+// EVEN_ROUNDS runs of nodes, the collision is that of the other steps.  What
+// such a flow has across its axis (plane momenta, the torque on the sphere) is
+// little more than the rounding of these sums, and callers keep the rounding
+// they had: over twelve boxes of 28^3 to 160^3, R 8 to 9, they move by up to
+// 2.5e-5 of themselves, with the paired collision and the columns by up to
+// 3.5e-4.  Time per even step: 60^3 10.5 us against 9.2 us with columns, 160^3
+// 115 and 110 us; with 5.3 links per node (128 x 128 x 1024 column) 184 and
+// 180 us.
 
 struct LinkSlot {
     int p;
