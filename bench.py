@@ -9,11 +9,10 @@ populations; synthetic input from workloads.config_scale().
 
 metric: coupled-step MLUPS over fluid nodes (fluid-node updates per second,
 millions), whole job.  `kernel_rooflines` gives, for the HBM-bound kernel
-groups, the algorithmic bytes per launch (collide+stream of the odd steps:
-152 B per fluid node, 19 FP32 populations read and written; of the even
-steps, which take their links inside the same kernel: 152 B plus the node's
-8 B link word; the link kernel of the odd steps: 8 B per link record, one
-population read and the bounced value written) over the
+groups, the algorithmic bytes per launch (collide+stream: 152 B per fluid
+node, 19 FP32 populations read and written, plus the node's 8 B link word on
+steps that take their links inside the same kernel; the link kernel: 8 B per
+link record, one population read and the bounced value written) over the
 group's mean launch time, taken with CUDA events around every launch inside
 the captured graphs during a second window of K steps that follows the
 headline window (those event nodes slow the step, so the headline `value`
@@ -43,7 +42,7 @@ sys.path.insert(0, ROOT)
 
 BYTES_PER_FLUID_NODE = 152  # 19 populations x 4 B, read + write
 BYTES_PER_LINK = 8  # one population read, the bounced value written
-BYTES_PER_LINK_WORD = 8  # per node: the even steps' links inside collide+stream
+BYTES_PER_LINK_WORD = 8  # per node: links inside collide+stream
 METRIC = "coupled step MLUPS (fluid nodes)"
 UNIT = "MLUPS"
 
@@ -274,8 +273,8 @@ def run_ours(args):
     ms_max, fluid_sum = aggregate(ms, fluid, world, "cuda")
     value = fluid_sum * args.steps / (ms_max * 1e-3) / 1e6
     # rooflines of the HBM-bound kernel groups at their algorithmic bytes
-    # (collide+stream: 152 B per fluid node, plus the link word on the even
-    # steps when they take their links; links: 8 B per link record, the
+    # (collide+stream: 152 B per fluid node, plus the link word on the steps
+    # that take their links there; links: 8 B per link record, the
     # population read and the bounced value written); the dominant one by
     # measured time is the headline `roofline`
     peak, peak_kind = _peaks()
@@ -283,7 +282,7 @@ def run_ours(args):
     node_bytes = BYTES_PER_FLUID_NODE * esz // 4
     fused = tm["links"][1] < tm["collide_odd"][1] + tm["collide_even"][1]
     algo = {"collide_even": (node_bytes + (BYTES_PER_LINK_WORD if fused else 0), fluid, "fluid node"),
-            "collide_odd": (node_bytes, fluid, "fluid node"),
+            "collide_odd": (node_bytes + (BYTES_PER_LINK_WORD if tm["links"][1] == 0 else 0), fluid, "fluid node"),
             "links": (BYTES_PER_LINK * esz // 4, cnt_b["links"], "link record")}
     kernels = {}
     for g, (per, units, uname) in algo.items():
