@@ -29,20 +29,6 @@
 
 namespace lbmdem {
 
-// neighbour table: nbr[m][i] = compact index of x_i + c_m if fluid, else NONE
-__global__ void k_adj_nbr(Lat L, uint32_t* nbr) {
-    uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= L.nS) return;
-    int x, y, z;
-    unpack_coord(L.coord[i], x, y, z);
-#pragma unroll
-    for (int m = 0; m < Q - 1; ++m) nbr[(size_t)m * L.nSpad + i] = fluid_index(L, x, y, z, cx(m), cy(m), cz(m));
-}
-
-void launch_adj_nbr(const Lat& L, uint32_t* nbr, cudaStream_t s) {
-    if (L.nS) k_adj_nbr<<<(L.nS + 255) / 256, 256, 0, s>>>(L, nbr);
-}
-
 // B^T in place on the adjoint of n_{t+1}: one thread per boundary node pair
 // (inlet node of a (y, z) line, outlet node and its upstream node).
 __global__ void k_adj_boundary(AdjArgs A, double shape, double* d_amp) {
@@ -86,8 +72,10 @@ void launch_adj_boundary(const AdjArgs& A, double shape, double* d_amp, cudaStre
     k_adj_boundary<<<(n + 127) / 128, 128, 0, s>>>(A, shape, d_amp);
 }
 
-// a_t = J_C(n_t)^T S^T b + dl_t/dn_t, and the omega derivative.  300 B per node
-// with the neighbour table: 34 us on 0.52 M fluid nodes, 0.68 of the copy rate.
+// a_t = J_C(n_t)^T S^T b + dl_t/dn_t, and the omega derivative.  240 B per node,
+// 18.4 us at the copy rate on 0.52 M fluid nodes; the neighbours from word
+// records and link words, as in the odd collide kernel: 25.2 us against 33.4 us
+// with a table of 18 indices per node.
 __global__ void __launch_bounds__(256) k_adj_step(AdjArgs A, const float* nat, float* out, float dl,
                                                   double* d_omega) {
     const Lat& L = A.L;
@@ -100,11 +88,12 @@ __global__ void __launch_bounds__(256) k_adj_step(AdjArgs A, const float* nat, f
 #pragma unroll
         for (int m = 0; m < Q; ++m) g[m] = __ldcs(nat + (size_t)m * P + i);
         float s[Q];
-#pragma unroll
-        for (int j = 0; j < Q - 1; ++j) {
-            uint32_t d = A.nbr[(size_t)j * P + i];
-            s[j] = d != NONE ? A.adj[(size_t)j * P + d] : A.adj[(size_t)opp(j) * P + i];
-        }
+        int x, y, z;
+        unpack_coord(__ldg(&L.coord[i]), x, y, z);
+        uint32_t wall = __ldg(&A.lw[i].x) & LW_MASK;
+        for_neighbours(L, x, y, z, wall, [&](int j, uint32_t n) {
+            s[j] = (wall >> j) & 1u ? A.adj[(size_t)opp(j) * P + i] : A.adj[(size_t)j * P + n];
+        });
         s[18] = A.adj[(size_t)18 * P + i];
         const RevMoments M = rev_moments(g, L.rho_f);
         RevSums R;
@@ -119,7 +108,7 @@ __global__ void __launch_bounds__(256) k_adj_step(AdjArgs A, const float* nat, f
         }
         R.finish(M, s[18]);
         const float om = L.tau_inv;
-        const float add = (int)(L.coord[i] >> 20) == A.probe_x ? dl : 0.f;
+        const float add = x == A.probe_x ? dl : 0.f;
 #pragma unroll
         for (int j = 0; j < Q; ++j)
             out[(size_t)j * P + i] = (1.0f - om) * s[j] + om * (R.A + R.dot(j)) + add;

@@ -1670,12 +1670,10 @@ int lbm_dem_adjoint(lbmdem_ctx* c, int64_t steps, int32_t every, const double* t
     // the reverse sweep's memory, mapped while the forward run is on the GPU
     const size_t nbytes = (size_t)Q * c->nSpad * sizeof(float);
     DBuf<float> nat, adj, adj2;
-    DBuf<uint32_t> nbr;
     DBuf<double> grads;
     CK(nat.alloc((size_t)Q * c->nSpad * (size_t)every));
     CK(adj.alloc((size_t)Q * c->nSpad));
     CK(adj2.alloc((size_t)Q * c->nSpad));
-    CK(nbr.alloc((size_t)(Q - 1) * c->nSpad));
     CK(grads.alloc(GRAD_COPIES + 1));  // omega derivative copies, then the amplitude's
     std::vector<double> trace((size_t)(t0 + steps));
     int64_t len = 0;
@@ -1699,7 +1697,6 @@ int lbm_dem_adjoint(lbmdem_ctx* c, int64_t steps, int32_t every, const double* t
     // natural populations of every step, then walk the adjoint back
     CK(cudaMemsetAsync(adj.p, 0, nbytes, s));
     CK(cudaMemsetAsync(grads.p, 0, (GRAD_COPIES + 1) * sizeof(double), s));
-    launch_adj_nbr(make_lat(c), nbr.p, s);
     CK(cudaGetLastError());
     const int64_t t_end = c->t;
     for (int64_t g = nseg - 1; g >= 0; --g) {
@@ -1721,7 +1718,7 @@ int lbm_dem_adjoint(lbmdem_ctx* c, int64_t steps, int32_t every, const double* t
         }
         c->suppress_probe = false;
         CK(cudaGetLastError());
-        AdjArgs A{L, nbr.p, adj.p, c->p.inlet, c->p.outlet, c->p.probe_x};
+        AdjArgs A{L, c->linkw.p, adj.p, c->p.inlet, c->p.outlet, c->p.probe_x};
         for (int64_t k = n - 1; k >= 0; --k) {
             int64_t t = tg + k;  // step t -> t + 1
             A.adj = adj.p;

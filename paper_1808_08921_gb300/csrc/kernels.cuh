@@ -83,6 +83,77 @@ constexpr uint32_t LW_MASK = (1u << 18) - 1u;
 constexpr uint32_t LW_NONE = 0x3fffu;
 constexpr int LW_MAX_SPHERES = (int)LW_NONE;  // sphere indices 0 .. LW_NONE - 1
 
+// Compact indices of the stored nodes at z, z + 1 and z - 1 of one z-line
+// from one population count: b = z & 31, low the bits below it; the word's
+// prev and next serve the line's neighbours outside the word.
+struct LineIndex {
+    uint32_t c, p, m;
+    __device__ __forceinline__ LineIndex(const uint4& r, uint32_t b, uint32_t low, bool top) {
+        c = r.y + __popc(r.x & low);
+        p = top ? r.w : c + ((r.x >> b) & 1u);
+        m = b == 0u ? r.z : c - ((r.x >> ((b - 1u) & 31u)) & 1u);
+    }
+};
+
+// take(m, n) for the 18 neighbours x + c_m, n the compact index where the
+// neighbour is stored (any value where it is not), from nine word records;
+// the directions that leave the x range join `wall` before the first call.
+template <class Take>
+__device__ __forceinline__ void for_neighbours(const Lat& L, int x, int y, int z, uint32_t& wall, Take take) {
+    const uint32_t b = z & 31, low = (1u << b) - 1u;
+    const bool top = b == 31u || z == L.nz - 1;
+    const int ym = y == 0 ? L.ny - 1 : y - 1, yp = y == L.ny - 1 ? 0 : y + 1;
+    int xm = x - 1, xp = x + 1;
+    if (x == 0) {
+        xm = L.px ? L.nx - 1 : 0;
+        if (!L.px) wall |= 1u << 1 | 1u << 10 | 1u << 11 | 1u << 12 | 1u << 13;  // c_x = -1
+    }
+    if (x == L.nx - 1) {
+        xp = L.px ? 0 : x;
+        if (!L.px) wall |= 1u << 0 | 1u << 6 | 1u << 7 | 1u << 8 | 1u << 9;  // c_x = +1
+    }
+    const uint32_t nyw = (uint32_t)L.nw * L.ny, wz = (uint32_t)(z >> 5) * L.ny;
+    const uint4 *r0 = L.rec + (size_t)x * nyw + wz, *rm = L.rec + (size_t)xm * nyw + wz,
+                *rp = L.rec + (size_t)xp * nyw + wz;
+    {
+        const LineIndex l(__ldg(r0 + y), b, low, top);
+        take(4, l.p);
+        take(5, l.m);
+    }
+    {
+        const LineIndex l(__ldg(r0 + yp), b, low, top);
+        take(2, l.c);
+        take(14, l.p);
+        take(15, l.m);
+    }
+    {
+        const LineIndex l(__ldg(r0 + ym), b, low, top);
+        take(3, l.c);
+        take(16, l.p);
+        take(17, l.m);
+    }
+    {
+        const LineIndex l(__ldg(rp + y), b, low, top);
+        take(0, l.c);
+        take(8, l.p);
+        take(9, l.m);
+    }
+    {
+        const LineIndex l(__ldg(rm + y), b, low, top);
+        take(1, l.c);
+        take(12, l.p);
+        take(13, l.m);
+    }
+    auto one = [&](const uint4* r) {
+        const uint2 v = __ldg(reinterpret_cast<const uint2*>(r));
+        return v.y + __popc(v.x & low);
+    };
+    take(6, one(rp + yp));
+    take(7, one(rp + ym));
+    take(10, one(rm + yp));
+    take(11, one(rm + ym));
+}
+
 // The inlet / outlet of the step that ended, one thread per boundary node:
 // k < ny nz the inlet plane, then the outlet plane.  Where the populations it
 // reads are stored follows from the stored words, fixed since the layout, and
@@ -301,11 +372,10 @@ int dem_launches(int n, int K);  // kernels of one launch_dem_step
 // adjoint.cu: reverse-mode kernels of the lattice step for a fixed packing
 struct AdjArgs {
     Lat L;
-    const uint32_t* nbr;  // [18][nSpad] compact index of x + c_m if fluid, else NONE
+    const uint2* lw;  // link words (a fixed packing's never change)
     float* adj;           // [19][nSpad] adjoint of the natural populations
     int inlet, outlet, probe_x;
 };
-void launch_adj_nbr(const Lat& L, uint32_t* nbr, cudaStream_t s);
 void launch_adj_boundary(const AdjArgs& A, double shape, double* d_amp, cudaStream_t s);
 void launch_adj_step(const AdjArgs& A, const float* nat, float* out, float dl, double* d_omega, cudaStream_t s);
 

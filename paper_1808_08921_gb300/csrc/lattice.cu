@@ -689,18 +689,6 @@ __global__ void __maxnreg__(72) k_collide_even_slots(Lat L, Mon mon, PartView P,
     mon_flush<MON>(a, mon, true);
 }
 
-// Compact indices of the stored nodes at z, z + 1 and z - 1 of one z-line
-// from one population count: b = z & 31, low the bits below it; the word's
-// prev and next serve the line's neighbours outside the word.
-struct LineIndex {
-    uint32_t c, p, m;
-    __device__ __forceinline__ LineIndex(const uint4& r, uint32_t b, uint32_t low, bool top) {
-        c = r.y + __popc(r.x & low);
-        p = top ? r.w : c + ((r.x >> b) & 1u);
-        m = b == 0u ? r.z : c - ((r.x >> ((b - 1u) & 31u)) & 1u);
-    }
-};
-
 // Odd step: node x gathers direction m from slot opp(m) of x - c_m (or from
 // its own slot m when x - c_m is solid or outside), collides, and scatters
 // direction m to slot m of x + c_m (or its own slot opp(m)): the population
@@ -741,21 +729,6 @@ k_collide_odd(Lat L, Mon mon, const uint2* __restrict__ lw, float* snap, PartVie
         uint32_t wall = lwx & LW_MASK;  // directions without a fluid neighbour
         int x, y, z;
         unpack_coord(cw, x, y, z);
-        const uint32_t b = z & 31, low = (1u << b) - 1u;
-        const bool top = b == 31u || z == L.nz - 1;
-        const int ym = y == 0 ? L.ny - 1 : y - 1, yp = y == L.ny - 1 ? 0 : y + 1;
-        int xm = x - 1, xp = x + 1;
-        if (x == 0) {
-            xm = L.px ? L.nx - 1 : 0;
-            if (!L.px) wall |= 1u << 1 | 1u << 10 | 1u << 11 | 1u << 12 | 1u << 13;  // c_x = -1
-        }
-        if (x == L.nx - 1) {
-            xp = L.px ? 0 : x;
-            if (!L.px) wall |= 1u << 0 | 1u << 6 | 1u << 7 | 1u << 8 | 1u << 9;  // c_x = +1
-        }
-        const uint32_t nyw = (uint32_t)L.nw * L.ny, wz = (uint32_t)(z >> 5) * L.ny;
-        const uint4 *r0 = L.rec + (size_t)x * nyw + wz, *rm = L.rec + (size_t)xm * nyw + wz,
-                    *rp = L.rec + (size_t)xp * nyw + wz;
         float g[Q];
         // the place of the population between x and x + c_m, whose compact
         // index is n: a 32-bit offset (19 nSpad < 2^32, checked at the layout)
@@ -764,43 +737,7 @@ k_collide_odd(Lat L, Mon mon, const uint2* __restrict__ lw, float* snap, PartVie
             off[m * 32] = o;
             g[opp(m)] = to_f<ST>(f[o], L.fsi);
         };
-        {
-            const LineIndex l(__ldg(r0 + y), b, low, top);
-            take(4, l.p);
-            take(5, l.m);
-        }
-        {
-            const LineIndex l(__ldg(r0 + yp), b, low, top);
-            take(2, l.c);
-            take(14, l.p);
-            take(15, l.m);
-        }
-        {
-            const LineIndex l(__ldg(r0 + ym), b, low, top);
-            take(3, l.c);
-            take(16, l.p);
-            take(17, l.m);
-        }
-        {
-            const LineIndex l(__ldg(rp + y), b, low, top);
-            take(0, l.c);
-            take(8, l.p);
-            take(9, l.m);
-        }
-        {
-            const LineIndex l(__ldg(rm + y), b, low, top);
-            take(1, l.c);
-            take(12, l.p);
-            take(13, l.m);
-        }
-        auto one = [&](const uint4* r) {
-            const uint2 v = __ldg(reinterpret_cast<const uint2*>(r));
-            return v.y + __popc(v.x & low);
-        };
-        take(6, one(rp + yp));
-        take(7, one(rp + ym));
-        take(10, one(rm + yp));
-        take(11, one(rm + ym));
+        for_neighbours(L, x, y, z, wall, take);
         g[18] = to_f<ST>(f[18u * L.nSpad + i], L.fsi);
         if (SNAP) {
 #pragma unroll
