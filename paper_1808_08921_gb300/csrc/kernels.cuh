@@ -215,19 +215,28 @@ struct BoundaryNode {
                 if (cx(m) < 0) f[(size_t)m * P + i] = f[src[m]];
             return;
         }
+        // the two faces apart: with the face as a value the compiler contracts
+        // the formulas differently and FP16 populations round differently
         float g[Q];
+        if (side == 0) {
 #pragma unroll
-        for (int m = 0; m < Q - 1; ++m) {
-            if (cx(m) < 0) continue;
-            const float v = to_f<ST>(f[src[m]], L.fsi);
-            if (side) g[m] = v;
-            else g[opp(m)] = v;
+            for (int m = 0; m < Q - 1; ++m)
+                if (cx(m) >= 0) g[opp(m)] = to_f<ST>(f[src[m]], L.fsi);
+            g[18] = to_f<ST>(f[src[18]], L.fsi);
+            pressure_face(g, drho, 0);
+#pragma unroll
+            for (int m = 0; m < Q; ++m)
+                if (cx(m) > 0) f[(size_t)m * P + i] = from_f<ST>(g[m], L.fs);  // source outside: own slot
+        } else {
+#pragma unroll
+            for (int m = 0; m < Q - 1; ++m)
+                if (cx(m) >= 0) g[m] = to_f<ST>(f[src[m]], L.fsi);
+            g[18] = to_f<ST>(f[src[18]], L.fsi);
+            pressure_face(g, 0.f, 1);
+#pragma unroll
+            for (int m = 0; m < Q; ++m)
+                if (cx(m) < 0) f[(size_t)m * P + i] = from_f<ST>(g[m], L.fs);
         }
-        g[18] = to_f<ST>(f[src[18]], L.fsi);
-        pressure_face(g, side ? 0.f : drho, side);
-#pragma unroll
-        for (int m = 0; m < Q; ++m)  // those that would come from outside: own slots
-            if (side ? cx(m) < 0 : cx(m) > 0) f[(size_t)m * P + i] = from_f<ST>(g[m], L.fs);
     }
 };
 
