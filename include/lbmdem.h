@@ -294,7 +294,8 @@ int lbm_dem_batch_set_time_limit(lbmdem_batch* b, double seconds);
 /* Advance column i by steps[i] >= 0 coupled steps in one graph launch
  * (asynchronous like lbm_dem_step; the graph is built for the call, after a
  * re-layout check and, for a column at an odd step, one single step).
- * Errors: INVALID_ARG, a column's latched status, CUDA. */
+ * Errors: INVALID_ARG, a column's latched status, STATE (a column whose
+ * last set_packing failed), CUDA. */
 int lbm_dem_batch_step(lbmdem_batch* b, const int64_t* steps);
 
 /* Wait for the batch and every column; returns the first column status

@@ -24,6 +24,7 @@
 
 #include "../../include/lbmdem.h"
 #include "common.cuh"
+#include "devmem.cuh"
 #include "kernels.cuh"
 #include "layout.cuh"
 
@@ -31,100 +32,9 @@ using namespace lbmdem;
 
 namespace {
 
-template <class T>
-struct DBuf {
-    T* p = nullptr;
-    size_t n = 0;
-    bool own = true;  // false: a part of a Slab
-    DBuf() = default;
-    DBuf(const DBuf&) = delete;
-    DBuf& operator=(const DBuf&) = delete;
-    ~DBuf() { release(); }
-    cudaError_t alloc(size_t count) {
-        release();
-        if (count == 0) count = 1;
-        cudaError_t e = cudaMalloc((void**)&p, sizeof(T) * count);
-        if (e != cudaSuccess) {
-            p = nullptr;
-            n = 0;
-            return e;
-        }
-        n = count;
-        return cudaSuccess;
-    }
-    cudaError_t ensure(size_t count) { return count <= n && p ? cudaSuccess : alloc(count + count / 8); }
-    void release() {
-        if (p && own) cudaFree(p);
-        p = nullptr;
-        n = 0;
-        own = true;
-    }
-    void view(T* q, size_t count) {
-        release();
-        p = q;
-        n = count;
-        own = false;
-    }
-    void swap(DBuf& o) {
-        std::swap(p, o.p);
-        std::swap(n, o.n);
-        std::swap(own, o.own);
-    }
-};
-
-// Several arrays in one device allocation: an allocation and its release take
-// 65 us here whatever its size up to some 100 MB, and a context holds some
-// sixty arrays.  take() is called in two passes over the same arrays: a first
-// one that measures, then, after reserve(), one that hands the parts out.
-struct Slab {
-    DBuf<uint8_t> mem;
-    size_t off = 0;
-    bool measuring = true;
-    void measure() {
-        off = 0;
-        measuring = true;
-    }
-    // keeps a block that is large enough; the parts of an earlier one are gone
-    cudaError_t reserve() {
-        cudaError_t e = off <= mem.n ? cudaSuccess : mem.alloc(off);
-        off = 0;
-        measuring = false;
-        return e;
-    }
-    template <class T>
-    void take(DBuf<T>& b, size_t count) {
-        count = std::max<size_t>(count, 1);
-        off = (off + 255) / 256 * 256;
-        if (!measuring) b.view(reinterpret_cast<T*>(mem.p + off), count);
-        off += sizeof(T) * count;
-    }
-};
-
 constexpr int NGROUP = 6;  // collide odd, links, map update, inlet/outlet, DEM, collide even
 
 }  // namespace
-
-// cell-list buffers (per-sphere cell, per-cell counts, starts, fill cursors
-// and the spheres in cell order)
-struct CellBufs {
-    Slab slab;
-    DBuf<int> of, count, start, fill, order;
-    cudaError_t ensure(size_t np, size_t ncell) {
-        if (of.n >= np && fill.n >= ncell && of.p) return cudaSuccess;
-        auto parts = [&] {
-            slab.take(of, np);
-            slab.take(order, np);
-            slab.take(count, ncell + 1);
-            slab.take(start, ncell + 1);
-            slab.take(fill, ncell);
-        };
-        slab.measure();
-        parts();
-        cudaError_t e = slab.reserve();
-        if (e == cudaSuccess) parts();
-        return e;
-    }
-};
 
 struct lbmdem_ctx {
     lbmdem_params p{};
@@ -1544,6 +1454,7 @@ int lbm_dem_batch_step(lbmdem_batch* b, const int64_t* steps) {
         if (rem[i] < 0) return bfail(b, LBMDEM_ERR_INVALID_ARG, "steps[%d] < 0", i);
         if (c->status_latched)
             return bfail(b, c->status_latched, "column %d: %s", i, status_text(c->status_latched));
+        if (!c->have_packing) return bfail(b, LBMDEM_ERR_STATE, "column %d: no packing", i);  // its last one failed
         if (int r = ensure_probe(c, c->t + rem[i] + 1)) return bfail(b, r, "column %d: %s", i, c->err.c_str());
         if (rem[i] == 0) continue;
         // host-side work before the launch: the re-layout decision, and a
