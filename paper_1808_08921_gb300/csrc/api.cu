@@ -75,10 +75,7 @@ struct lbmdem_ctx {
     DBuf<uint2> linkw;       // link word of every stored node
     bool fused_links = false, dense_links = false;
     bool batched = false;  // steps being captured into a batch graph (columns share the GPU)
-    DBuf<Flip> flip_rec;
-    DBuf<float> flip_scratch;
-    DBuf<uint8_t> flip_valid;
-    uint32_t flip_cap = 0;
+    ConversionBufs<Flip> flips;
     uint32_t probe0 = 0, probe1 = 0;
     // particles
     Slab part_slab;
@@ -540,12 +537,7 @@ static int build_layout(lbmdem_ctx* c, bool fresh) {
     // conversion scratch
     uint32_t cap = c->p.max_flips > 0 ? (uint32_t)c->p.max_flips
                                       : std::min<uint32_t>(1u << 20, std::max<uint32_t>(4096u, nband / 8));
-    if (cap != c->flip_cap) {
-        CK(c->flip_rec.alloc(2 * (size_t)cap));
-        CK(c->flip_scratch.alloc((size_t)cap * Q * Q));
-        CK(c->flip_valid.alloc((size_t)cap * Q));
-        c->flip_cap = cap;
-    }
+    CK(c->flips.ensure(cap, Q));
     // probe plane's range in compact order
     c->probe0 = c->probe1 = 0;
     int xp = c->p.probe_x;
@@ -670,7 +662,7 @@ static void enqueue_step(lbmdem_ctx* c, int parity, bool monitor, int inlet, boo
         Lat L = make_lat(c);
         PartView P = make_part(c);
         Band B{c->band_coord.p, c->band_cand.p, c->band_slack.p, tested_band(c)};
-        FlipBuf F{c->flip_rec.p, c->flip_scratch.p, c->flip_valid.p, c->flip_cap};
+        FlipBuf F{c->flips.rec.p, c->flips.scratch.p, c->flips.valid.p, c->flips.cap};
         DevStats* sd = c->st.p;
         const BC bc{c->p.inlet, c->p.outlet, c->src, &sd->t_end[parity]};
         const BC bc_prev{c->p.inlet, c->p.outlet, c->src, &sd->t_end[parity ^ 1]};

@@ -122,4 +122,23 @@ struct CellBufs {
     }
 };
 
+// scratch of the node conversions: `cap` conversions per step, queued by step
+// parity, each with q x q gathered populations
+template <class Rec>
+struct ConversionBufs {
+    DBuf<Rec> rec;
+    DBuf<float> scratch;
+    DBuf<uint8_t> valid;
+    uint32_t cap = 0;  // 0 until all three are there
+    cudaError_t ensure(uint32_t want, size_t q) {
+        if (want == cap) return cudaSuccess;
+        cap = 0;
+        cudaError_t e = rec.alloc(2 * (size_t)want);
+        if (e == cudaSuccess) e = scratch.alloc(want * q * q);
+        if (e == cudaSuccess) e = valid.alloc(want * q);
+        if (e == cudaSuccess) cap = want;
+        return e;
+    }
+};
+
 }  // namespace lbmdem

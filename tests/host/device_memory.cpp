@@ -100,6 +100,21 @@ int main() {
         check("lists", l.b, 500);
         largest = SIZE_MAX;
     }
+    {
+        lbmdem::ConversionBufs<int> f;
+        auto whole = [&](const char* what, size_t n) {
+            check(what, f.rec, 2 * n);
+            check(what, f.scratch, 9 * n);
+            check(what, f.valid, 3 * n);
+        };
+        if (f.ensure(100, 3)) bad = 1;
+        whole("conversions", 100);
+        largest = 20000;  // the queue fits, the populations do not
+        if (f.ensure(1000, 3) != cudaErrorMemoryAllocation) bad = 1;
+        if (f.ensure(100, 3)) bad = 1;
+        whole("conversions after a refusal", 100);
+        largest = SIZE_MAX;
+    }
     if (!live.empty()) {
         std::printf("%zu blocks not given back\n", live.size());
         bad = 1;
