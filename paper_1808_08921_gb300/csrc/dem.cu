@@ -601,11 +601,28 @@ __global__ void __launch_bounds__(SUB_THREADS) k_dem_begin(Dem D) {
     if (t == 0) *D.layout_fresh = 0u;  // this step's map update is done
     float3 fa, ta;
     hydro_drive(D, i, tl, have, (threadIdx.x & 31) & ~(TEAM - 1), fa, ta);
+    // the team's lanes all read what two of them replace
+    float3 dx = make_float3(0.f, 0.f, 0.f), c = dx, fc = dx, tc = dx, v = dx, w = dx;
+    float4 q = make_float4(1.f, 0.f, 0.f, 0.f);
+    bool fixed = true;
+    float im = 0.f, iI = 0.f;
+    if (have) {
+        dx = f3(D.dX[i]);
+        c = f3(D.dXc[i]);
+        q = D.q[i];
+        fc = f3(D.Fc[i]);
+        tc = f3(D.Tc[i]);
+        v = f3(D.V[i]);
+        w = f3(D.W[i]);
+        fixed = D.fixed[i] != 0;
+        im = D.invm[i];
+        iI = D.invI[i];
+    }
+    __syncwarp();
     if (!have) return;
     if (tl == 0) D.Fa[i] = make_float4(fa.x, fa.y, fa.z, 0.f);
     if (tl == 1) D.Ta[i] = make_float4(ta.x, ta.y, ta.z, 0.f);
-    open_substep(D, i, tl, 0, f3(D.dX[i]), f3(D.dXc[i]), D.q[i], f3(D.Fc[i]), f3(D.Tc[i]), fa, ta, f3(D.V[i]), f3(D.W[i]), D.fixed[i] != 0, D.invm[i],
-                 D.invI[i]);
+    open_substep(D, i, tl, 0, dx, c, q, fc, tc, fa, ta, v, w, fixed, im, iI);
 }
 
 __global__ void __launch_bounds__(SUB_THREADS) k_dem_substep(Dem D, int s) {
