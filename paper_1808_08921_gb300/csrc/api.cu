@@ -98,6 +98,7 @@ struct lbmdem_ctx {
     DBuf<int> nb_slot, dem_foreign, dem_slots;  // exchange slots of the one-launch DEM
     DBuf<float> nb_R;
     DBuf<uint16_t> dem_push;
+    DemShape dem;                   // the packing's
     int* dem_slots_host = nullptr;  // pinned, valid once the stream is synchronised after build_neighbours
     CellGrid grid{};
     CellBufs cells;       // the DEM's cell list (cells 2 R + dem_skin wide)
@@ -215,6 +216,7 @@ static PartView make_part(lbmdem_ctx* c) {
 static Dem make_dem(lbmdem_ctx* c) {
     Dem D{};
     D.n = c->np;
+    D.shape = c->dem;
     D.K = c->p.dem_substeps;
     D.dt = 1.0f / (float)c->p.dem_substeps;
     D.kn = (float)(2.0 * c->p.E_p / (3.0 * (1.0 - c->p.nu_p * c->p.nu_p)));
@@ -359,6 +361,7 @@ static int build_neighbours(lbmdem_ctx* c, bool carry) {
     c->nb_sh.swap(c->nb_sh2);
     c->nb_dref.swap(c->nb_dref2);
     c->nb_ft.swap(c->nb_ft2);
+    c->dem = dem_shape(np);
     // exchange slots; every caller synchronises the stream before it launches a step
     launch_dem_ghosts(make_dem(c), c->nb_slot.p, c->dem_push.p, c->dem_foreign.p, c->dem_slots.p, c->stream);
     CK(cudaGetLastError());
@@ -638,7 +641,7 @@ enum { INLET_NOW = 0, INLET_NEXT = 1 };
 // and the step's links are not in the collide kernel), inlet/outlet (if any
 // and not left to the next step), DEM
 static int64_t kernels_per_step(const lbmdem_ctx* c, int parity, int inlet = INLET_NOW, bool last = true) {
-    int64_t k = dem_active(c) ? dem_launches(c->np, c->p.dem_substeps) : 0;
+    int64_t k = dem_active(c) ? dem_launches(c->dem, c->p.dem_substeps) : 0;
     if (c->lbm) {
         k += map_update_launches(tested_band(c), parity);
         k += c->nS ? 1 : 0;

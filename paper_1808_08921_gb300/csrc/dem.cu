@@ -30,6 +30,7 @@
 #include "common.cuh"
 #include "kernels.cuh"
 #include "layout.cuh"
+#include "per_device.cuh"
 
 namespace lbmdem {
 
@@ -749,23 +750,17 @@ __global__ void __launch_bounds__(SUB_THREADS) k_dem_init(Dem D) {
 
 // ------------------------------------------------------------ launches
 
-// Largest cluster (CTAs of DSM_THREADS threads) k_dem_step_dsm can run with
-// on each device, found on the first initialisation launch (outside any
-// stream capture); 0 = not found (the launches per substep serve).
-static int g_dsm_cluster[64];
-static bool g_dsm_probed[64];
 constexpr size_t dsm_smem(int slots) { return (size_t)slots * DSM_BUFS * RECORD_BYTES; }
 
-static void probe_dsm(int dev) {
-    if (dev < 0 || dev >= 64 || g_dsm_probed[dev]) return;
-    g_dsm_probed[dev] = true;
-    g_dsm_cluster[dev] = 0;
+// Largest cluster (CTAs of DSM_THREADS threads) k_dem_step_dsm can run with on
+// the current device, 0 where it cannot run.
+static int find_dsm_cluster() {
     const size_t most = dsm_smem(DEM_MAX_CTAS * DSM_THREADS / TEAM);  // every sphere in every CTA
     if (cudaFuncSetAttribute(k_dem_step_dsm<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
         cudaFuncSetAttribute(k_dem_step_dsm<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most) !=
             cudaSuccess) {
         cudaGetLastError();
-        return;
+        return 0;
     }
     for (int C : {DEM_MAX_CTAS, 8}) {
         cudaLaunchConfig_t cfg = {};
@@ -780,44 +775,36 @@ static void probe_dsm(int dev) {
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         int ncl = 0;
-        if (cudaOccupancyMaxActiveClusters(&ncl, k_dem_step_dsm<true>, &cfg) == cudaSuccess && ncl > 0) {
-            g_dsm_cluster[dev] = C;
-            break;
-        }
+        if (cudaOccupancyMaxActiveClusters(&ncl, k_dem_step_dsm<true>, &cfg) == cudaSuccess && ncl > 0) return C;
         cudaGetLastError();
     }
+    return 0;
 }
 
-// CTAs and threads per CTA of the one-launch form for n spheres; false where
-// they do not fit one cluster.  The smallest CTAs that fit: a CTA holds half
-// an SM's registers at 256 threads, so DEM clusters of concurrent columns
-// (batches) find room next to the lattice kernels.
-static bool dsm_shape(int n, int& C, int& T) {
+// The smallest CTAs that fit: a CTA holds half an SM's registers at 256
+// threads, so DEM clusters of concurrent columns (batches) find room next to
+// the lattice kernels.
+DemShape dem_shape(int n) {
+    static PerDevice<int> cluster;
     int dev = 0;
     cudaGetDevice(&dev);
-    const int cmax = dev >= 0 && dev < 64 ? g_dsm_cluster[dev] : 0;
+    const int cmax = cluster.get(dev, find_dsm_cluster);
     const long long need = (long long)TEAM * (n > 0 ? n : 1);
-    if (cmax <= 0 || need > (long long)cmax * DSM_THREADS) return false;
-    T = need <= (long long)cmax * (DSM_THREADS / 2) ? DSM_THREADS / 2 : DSM_THREADS;
-    C = (int)((need + T - 1) / T);
-    if (C == 1) T = (int)(((need + 31) / 32) * 32);
-    return true;
+    if (cmax <= 0 || need > (long long)cmax * DSM_THREADS) return {};
+    const int T = need <= (long long)cmax * (DSM_THREADS / 2) ? DSM_THREADS / 2 : DSM_THREADS;
+    const int C = (int)((need + T - 1) / T);
+    return {C, C == 1 ? (int)(((need + 31) / 32) * 32) : T};
 }
 
 void launch_dem_ghosts(const Dem& D, int* nb_slot, uint16_t* push, int* foreign, int* slots, cudaStream_t s) {
-    int dev = 0, C, T;
-    cudaGetDevice(&dev);
-    probe_dsm(dev);
+    const DemShape h = D.shape;
     cudaMemsetAsync(slots, 0, sizeof(int), s);
-    if (D.n <= 0 || !dsm_shape(D.n, C, T)) return;
-    if (C < DEM_MAX_CTAS) cudaMemsetAsync(push, 0xff, sizeof(uint16_t) * (size_t)D.n * DEM_MAX_CTAS, s);
-    k_dem_ghosts<<<C, 256, D.n, s>>>(D, T / TEAM, nb_slot, push, foreign, slots);
+    if (D.n <= 0 || !h.ctas) return;
+    if (h.ctas < DEM_MAX_CTAS) cudaMemsetAsync(push, 0xff, sizeof(uint16_t) * (size_t)D.n * DEM_MAX_CTAS, s);
+    k_dem_ghosts<<<h.ctas, 256, D.n, s>>>(D, h.threads / TEAM, nb_slot, push, foreign, slots);
 }
 
-int dem_launches(int n, int K) {
-    int C, T;
-    return dsm_shape(n, C, T) ? 1 : K + 1;
-}
+int dem_launches(DemShape h, int K) { return h.ctas ? 1 : K + 1; }
 
 void launch_dem_init(const Dem& D, cudaStream_t s) {
     const unsigned blocks = (unsigned)(((long long)TEAM * D.n + SUB_THREADS - 1) / SUB_THREADS);
@@ -825,8 +812,8 @@ void launch_dem_init(const Dem& D, cudaStream_t s) {
 }
 
 void launch_dem_step(const Dem& D, cudaStream_t s) {
-    int C, T;
-    if (!dsm_shape(D.n, C, T)) {
+    const int C = D.shape.ctas;
+    if (!C) {
         const unsigned blocks = (unsigned)(((long long)TEAM * D.n + SUB_THREADS - 1) / SUB_THREADS);
         launch_pdl(k_dem_begin, blocks, SUB_THREADS, s, D);
         for (int k = 0; k < D.K; ++k) launch_pdl(k_dem_substep, blocks, SUB_THREADS, s, D, k);
@@ -844,7 +831,7 @@ void launch_dem_step(const Dem& D, cudaStream_t s) {
     cfg.attrs = attr;
     cfg.numAttrs = C > 1 ? 2 : 1;
     cfg.gridDim = dim3(C, 1, 1);
-    cfg.blockDim = dim3(T, 1, 1);
+    cfg.blockDim = dim3(D.shape.threads, 1, 1);
     cfg.dynamicSmemBytes = dsm_smem(D.slots);
     if (C > 1) cudaLaunchKernelEx(&cfg, k_dem_step_dsm<true>, D);
     else cudaLaunchKernelEx(&cfg, k_dem_step_dsm<false>, D);

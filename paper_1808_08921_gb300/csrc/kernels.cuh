@@ -296,9 +296,17 @@ struct FlipBuf {
 // CTAs of the largest cluster the one-launch DEM takes.
 constexpr int DEM_MAX_CTAS = 16;
 
+// Launch of the one-launch DEM: CTAs of its cluster (0: a launch per substep
+// serves instead) and threads per CTA.  Chosen once for a packing: the exchange
+// slots are laid out for it.
+struct DemShape {
+    int ctas = 0, threads = 0;
+};
+
 // DEM state (Section 2.2).
 struct Dem {
     int n, K;
+    DemShape shape;
     float dt;                // 1 / K
     float kn, kt, mu;        // Eqs. 11-12 prefactors
     float3 g;                // body force
@@ -377,7 +385,8 @@ void launch_link_words(const Lat& L, uint2* lw, cudaStream_t s);
 void launch_dem_ghosts(const Dem& D, int* nb_slot, uint16_t* push, int* foreign, int* slots, cudaStream_t s);
 void launch_dem_init(const Dem& D, cudaStream_t s);
 void launch_dem_step(const Dem& D, cudaStream_t s);
-int dem_launches(int n, int K);  // kernels of one launch_dem_step
+DemShape dem_shape(int n);              // for n spheres on the current device
+int dem_launches(DemShape h, int K);  // kernels of one launch_dem_step
 // adjoint.cu: reverse-mode kernels of the lattice step for a fixed packing
 struct AdjArgs {
     Lat L;

@@ -25,3 +25,7 @@ def _run(name, tmp_path):
 
 def test_arrays_after_a_refused_allocation(tmp_path):
     _run("device_memory", tmp_path)
+
+
+def test_threads_agree_on_a_device(tmp_path):
+    _run("per_device", tmp_path)
