@@ -1565,14 +1565,16 @@ int lbm_dem_adjoint(lbmdem_ctx* c, int64_t steps, int32_t every, const double* t
     const size_t esz = c->p.storage == LBMDEM_F32 ? 4 : 2;
     const size_t fbytes = (size_t)Q * c->nSpad * esz;
     const int64_t nseg = (steps + every - 1) / every;
-    // forward with a checkpoint of the populations at the start of every segment
+    // forward with a checkpoint of the populations at the start of every
+    // segment; the last one is the end of the run, put back at the end
     DBuf<uint8_t> ck;
-    CK(ck.alloc(fbytes * (size_t)nseg));
+    CK(ck.alloc(fbytes * (size_t)(nseg + 1)));
     for (int64_t g = 0; g < nseg; ++g) {
         CK(cudaMemcpyAsync(ck.p + fbytes * g, c->f.p, fbytes, cudaMemcpyDeviceToDevice, s));
         int64_t n = std::min<int64_t>(every, steps - g * every);
         if (int r = lbm_dem_step(c, n)) return r;
     }
+    CK(cudaMemcpyAsync(ck.p + fbytes * nseg, c->f.p, fbytes, cudaMemcpyDeviceToDevice, s));
     // the reverse sweep's memory, mapped while the forward run is on the GPU
     const size_t nbytes = (size_t)Q * c->nSpad * sizeof(float);
     DBuf<float> nat, adj, adj2;
@@ -1613,12 +1615,11 @@ int lbm_dem_adjoint(lbmdem_ctx* c, int64_t steps, int32_t every, const double* t
         CK(cudaMemcpyAsync(&c->st.p->t, &tdev, sizeof(tdev), cudaMemcpyHostToDevice, s));
         c->t = tg;
         Lat L = make_lat(c);
-        // the trace is already complete; the forces are those of the last step
-        // recomputed
+        // the trace is complete, and the forces are the last forward step's:
+        // no recomputed step takes its links
         c->suppress_probe = true;
         for (int64_t k = 0; k < n; ++k) {
-            const bool last = k == n - 1;
-            enqueue_step(c, (int)(c->t & 1), false, last ? INLET_NOW : INLET_NEXT, k > 0, last && g == 0,
+            enqueue_step(c, (int)(c->t & 1), false, k == n - 1 ? INLET_NOW : INLET_NEXT, k > 0, false,
                          nat.p + (size_t)Q * c->nSpad * k);
             c->t += 1;
         }
@@ -1637,11 +1638,9 @@ int lbm_dem_adjoint(lbmdem_ctx* c, int64_t steps, int32_t every, const double* t
     }
     // leave the context where the forward run ended
     c->t = t_end;
-    {
-        // the last segment's recomputation ended at t_end with the same state
-        unsigned long long tdev = (unsigned long long)t_end;
-        CK(cudaMemcpyAsync(&c->st.p->t, &tdev, sizeof(tdev), cudaMemcpyHostToDevice, s));
-    }
+    const unsigned long long tdev = (unsigned long long)t_end;
+    CK(cudaMemcpyAsync(&c->st.p->t, &tdev, sizeof(tdev), cudaMemcpyHostToDevice, s));
+    CK(cudaMemcpyAsync(c->f.p, ck.p + fbytes * nseg, fbytes, cudaMemcpyDeviceToDevice, s));
     double gh[GRAD_COPIES + 1];
     CK(cudaMemcpyAsync(gh, grads.p, sizeof(gh), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
