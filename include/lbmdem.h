@@ -107,9 +107,9 @@ typedef struct {
                              1: the link kernel every step; 0 (default): 2 with FP32
                              storage and a largest sphere radius of 8 lattice units
                              or more, else 1.  Boxes narrower than 2 (R + skin + 2)
-                             on a periodic axis, and packings of more than 16383
-                             spheres, always take 1.  Same results up to FP32
-                             summation order.                                          */
+                             on a periodic axis, packings of more than 16383
+                             spheres and packings of fixed spheres always take 1.
+                             Same results up to FP32 summation order.                  */
     void* cuda_stream;    /* cudaStream_t to issue on; NULL = a stream of the context */
 } lbmdem_params;
 

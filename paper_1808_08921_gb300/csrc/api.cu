@@ -529,7 +529,10 @@ static int build_layout(lbmdem_ctx* c, bool fresh) {
     // rounds as the storage does)
     const bool want = c->p.link_mode == 2 ||
                       (c->p.link_mode == 0 && c->p.storage == LBMDEM_F32 && c->Rmax >= 8.0);
-    c->fused_links = want && c->nwarps > 0 && np <= LW_MAX_SPHERES && wide;
+    // Not where every sphere is fixed: there only the last step of a call takes
+    // its links, and the collision must not round otherwise in that step than
+    // in the others, or the fluid would depend on how a run is split into calls
+    c->fused_links = want && c->any_mobile && c->nwarps > 0 && np <= LW_MAX_SPHERES && wide;
     // FCC media have 5 to 10 link records per stored node, a sphere alone in a
     // box below one: there the link kernel is a few us of an odd step (160^3,
     // R 9: 118 + 10 us against 127), and the even steps keep their sums' order
@@ -670,11 +673,7 @@ static void enqueue_step(lbmdem_ctx* c, int parity, bool monitor, int inlet, boo
         const BC bc{c->p.inlet, c->p.outlet, c->src, &sd->t_end[parity]};
         const BC bc_prev{c->p.inlet, c->p.outlet, c->src, &sd->t_end[parity ^ 1]};
         const bool links = links_taken(c, last);
-        bool fused = links && links_in_collide(c, parity);
-        if (fused && snap) {  // the kernel with links writes no snapshot
-            fused = false;
-            c->launches += 1;
-        }
+        const bool fused = links && links_in_collide(c, parity);  // free spheres: never with a snapshot
         if (!links) P.n = 0;  // nor the spheres' tables
         if (tm) record_pair_begin(c, 2, e);
         launch_map_update(L, P, B, F, sd, parity, c->linkw.p,
