@@ -533,10 +533,12 @@ static int build_layout(lbmdem_ctx* c, bool fresh) {
     // its links, and the collision must not round otherwise in that step than
     // in the others, or the fluid would depend on how a run is split into calls
     c->fused_links = want && c->any_mobile && c->nwarps > 0 && np <= LW_MAX_SPHERES && wide;
-    // FCC media have 5 to 10 link records per stored node, a sphere alone in a
-    // box below one: there the link kernel is a few us of an odd step (160^3,
-    // R 9: 118 + 10 us against 127), and the even steps keep their sums' order
-    c->dense_links = nlink >= 2 * (uint64_t)nS;
+    // FCC media have 7 (R 11.4) to 11 (R 5.7) link records per stored node,
+    // those of band nodes among them, a sphere alone in a box at most a half:
+    // there the link kernel is a few us of an odd step (160^3, R 9: 118 + 10 us
+    // against 127), and the even steps keep their sums' order.  The records
+    // are counted without the lists' padding, which small spheres' are half of
+    c->dense_links = c->nlink_raw >= 2 * (uint64_t)nS;
     CK(c->linkw.ensure(nSpad));
     launch_link_words(make_lat(c), c->linkw.p, s);
     CK(cudaGetLastError());

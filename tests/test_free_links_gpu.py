@@ -1,10 +1,12 @@
 """Links in the collide kernels where a sphere is free (with fixed spheres
 alone the link kernel takes them): a fluid node between three overlapping
-spheres, in a lattice of few links per node."""
+spheres, in a lattice of few links per node; and which lattices count as ones
+of few links."""
 import numpy as np
 import pytest
 
 import oracle
+import workloads
 from paper_1808_08921_gb300 import lbmdem
 from test_links_fused_gpu import _close, _launches, _run, _three_spheres
 from test_parity_gpu import compare_fields, compare_particles
@@ -26,3 +28,14 @@ def test_three_spheres_one_of_them_free(steps):
     compare_particles(g, o, R=w.R)
     g.close()
     o.close()
+
+
+@pytest.mark.parametrize("a,R,cx,odd", [(13, 2.5, 10, False), (12, 2.5, 12, False), (16, 3.5, 6, True)])
+def test_two_links_per_stored_node(a, R, cx, odd):
+    """Small spheres' link records are padded to three and four times their
+    number; the odd steps take their links by the number without padding."""
+    w = workloads.fcc_column(a * cx, 2 * a, 2 * a, 0.8, float(a), R, jitter=0.01, seed=4, period=60, substeps=2)
+    c = _run(w, 4, 2)[2]
+    assert c["stored"] >= 65536 and (c["links"] >= 2 * c["stored"]) == odd
+    assert 0.75 < c["links"] / (2 * c["stored"]) < 1.25
+    assert _launches(w, 4, 1) - _launches(w, 4, 2) == (4 if odd else 2)
