@@ -2,11 +2,17 @@
 // coupled step loop (CUDA graphs of several steps), re-layouts and read-outs.
 //
 // One coupled step t -> t+1 on the context stream (Sections 2.1-2.4):
-//   map update (re-test band nodes, convert covered/uncovered nodes)
-//   collide + stream (even or odd AA kernel)
-//   link bounce-back + hydrodynamic force and torque
-//   inlet / outlet
-//   K DEM substeps (one cluster launch; also advances the device step counter)
+//   map update: counts the step, applies the previous step's inlet / outlet
+//     where it left them, re-tests band nodes and converts covered and
+//     uncovered ones
+//   collide + stream (even or odd AA kernel), with the links where link_mode
+//     takes them there
+//   else link bounce-back + hydrodynamic force and torque
+//   inlet / outlet of a run's last step (the others': next step's map update)
+//   K DEM substeps (one launch of one cluster, or beyond what a cluster holds
+//     a launch per substep)
+// A packing of fixed spheres has neither conversions nor DEM, and links only in
+// a run's last step.
 // Steps are captured in CUDA graphs of `graph_steps` steps starting at even t.
 // With mobile spheres the host reads back the largest displacement since the
 // last re-layout every few graphs and rebuilds the compact lattice and the
@@ -609,11 +615,10 @@ static void record_pair_end(lbmdem_ctx* c, size_t idx, cudaStream_t st = nullptr
 
 // Whether a step's links are taken inside its collide kernel: in lattices of
 // that kind (link_mode) every even step's, and the odd steps' where most
-// nodes have links, from ODD_LINKS_MIN stored nodes up.  R 11.4 FCC, the odd steps with the link
-// kernel against without, us per step: 159 k nodes 33.1 and 29.9, 629 k 54.4
-// and 46.3, 1.26 M 87.7 and 72.5, 4.46 M 283 and 238.  Smaller lattices
-// would gain too (41 k nodes 22.7 and 20.5) but keep the launches they are
-// documented with.
+// nodes have links, from ODD_LINKS_MIN stored nodes up (the bound link_mode is
+// documented with).  R 11.4 FCC, the odd steps with the link kernel against
+// without, us per step: 159 k nodes 33.1 and 29.9, 629 k 54.4 and 46.3, 1.26 M
+// 87.7 and 72.5, 4.46 M 283 and 238; below the bound, 41 k nodes, 22.7 and 20.5.
 constexpr uint32_t ODD_LINKS_MIN = 1u << 16;
 static bool links_in_collide(const lbmdem_ctx* c, int parity) {
     return c->fused_links && (parity == 0 || (c->dense_links && c->nS >= ODD_LINKS_MIN));
@@ -1480,8 +1485,7 @@ int lbm_dem_batch_step(lbmdem_batch* b, const int64_t* steps) {
         lbmdem_ctx* c = b->cols[i];
         BCK(cudaStreamWaitEvent(c->stream, b->done, 0));
         if (rem[i] <= 0) continue;
-        for (int64_t k = 0; k < rem[i]; ++k)  // a pair's even step leaves its inlet to the odd one
-        {
+        for (int64_t k = 0; k < rem[i]; ++k) {  // a pair's even step leaves its inlet to the odd one
             const bool last = k % 2 == 1 || k + 1 == rem[i];
             c->launches += kernels_per_step(c, (int)(k & 1), last ? INLET_NOW : INLET_NEXT, last);
         }

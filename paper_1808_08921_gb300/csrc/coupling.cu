@@ -33,8 +33,6 @@
 
 namespace lbmdem {
 
-
-
 // Directions of Eq. 3 as a constant table, read with a warp-uniform index.
 struct DirC {
     float cx, cy, cz, w;
@@ -348,31 +346,31 @@ __global__ void __launch_bounds__(256, 6) k_map_band(MapArgs A) {
         pdl_wait();
         pdl_trigger();
         if (k >= (uint32_t)A.P.n) return;
-                for (int r = 0; r < NREP; ++r)
-                    for (int a = 0; a < 3; ++a) {
-                        A.P.Fh[3 * ((size_t)r * A.P.n + k) + a] = 0.0;
-                        A.P.Th[3 * ((size_t)r * A.P.n + k) + a] = 0.0;
-                    }
-                // moving-wall terms of this step's links of sphere k, per direction
-                // m: beta = 6 w rho_f (c x W) and alpha' = 6 w rho_f c.V - xf.beta,
-                // so that the term of Eq. 14 at a link node with offset rel from the
-                // sphere's lattice origin is alpha' + rel.beta
-                const float4 V = A.P.V[k], W = A.P.W[k], xf = A.P.xf[k];
-                const float s6 = 6.0f * A.L.rho_f;
-        #pragma unroll
-                for (int m = 0; m < Q - 1; ++m) {
-                    const float sw = s6 * wt(m);
-                    const float ex = (float)cx(m), ey = (float)cy(m), ez = (float)cz(m);
-                    const float bx = sw * (ey * W.z - ez * W.y), by = sw * (ez * W.x - ex * W.z),
-                                bz = sw * (ex * W.y - ey * W.x);
-                    const float alpha = sw * (ex * V.x + ey * V.y + ez * V.z);
-                    A.P.ab[(size_t)k * (Q - 1) + m] = make_float4(alpha - (xf.x * bx + xf.y * by + xf.z * bz), bx, by, bz);
-                }
-                // the same state for the even steps' links inside the collide kernel
-                const int4 o = A.P.orgw[k];
-                A.P.pk[3 * (size_t)k] = make_float4(xf.x, xf.y, xf.z, V.x);
-                A.P.pk[3 * (size_t)k + 1] = make_float4(V.y, V.z, W.x, W.y);
-                A.P.pk[3 * (size_t)k + 2] = make_float4(W.z, __int_as_float(o.x), __int_as_float(o.y), __int_as_float(o.z));
+        for (int r = 0; r < NREP; ++r)
+            for (int a = 0; a < 3; ++a) {
+                A.P.Fh[3 * ((size_t)r * A.P.n + k) + a] = 0.0;
+                A.P.Th[3 * ((size_t)r * A.P.n + k) + a] = 0.0;
+            }
+        // moving-wall terms of this step's links of sphere k, per direction
+        // m: beta = 6 w rho_f (c x W) and alpha' = 6 w rho_f c.V - xf.beta,
+        // so that the term of Eq. 14 at a link node with offset rel from the
+        // sphere's lattice origin is alpha' + rel.beta
+        const float4 V = A.P.V[k], W = A.P.W[k], xf = A.P.xf[k];
+        const float s6 = 6.0f * A.L.rho_f;
+#pragma unroll
+        for (int m = 0; m < Q - 1; ++m) {
+            const float sw = s6 * wt(m);
+            const float ex = (float)cx(m), ey = (float)cy(m), ez = (float)cz(m);
+            const float bx = sw * (ey * W.z - ez * W.y), by = sw * (ez * W.x - ex * W.z),
+                        bz = sw * (ex * W.y - ey * W.x);
+            const float alpha = sw * (ex * V.x + ey * V.y + ez * V.z);
+            A.P.ab[(size_t)k * (Q - 1) + m] = make_float4(alpha - (xf.x * bx + xf.y * by + xf.z * bz), bx, by, bz);
+        }
+        // the same state for links taken inside the collide kernels
+        const int4 o = A.P.orgw[k];
+        A.P.pk[3 * (size_t)k] = make_float4(xf.x, xf.y, xf.z, V.x);
+        A.P.pk[3 * (size_t)k + 1] = make_float4(V.y, V.z, W.x, W.y);
+        A.P.pk[3 * (size_t)k + 2] = make_float4(W.z, __int_as_float(o.x), __int_as_float(o.y), __int_as_float(o.z));
         return;
     }
     // launched behind the DEM, what that does not write is read ahead of the

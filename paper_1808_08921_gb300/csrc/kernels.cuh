@@ -77,8 +77,8 @@ __device__ __forceinline__ void pressure_face(float g[Q], float drho_b, int side
 // Sphere indices take 14 bits; LW_NONE stands for no sphere B, and as sphere
 // A for a node whose solid neighbours belong to more than two spheres (its
 // links then read the owner map).  With more spheres than LW_MAX_SPHERES the
-// indices are cut off and only the mask is used.  Built at the layout from the owner map
-// and renewed for every converted node and its 18 neighbours.
+// indices are cut off and only the mask is used.  Built at the layout from the
+// owner map and renewed for every converted node and its 18 neighbours.
 constexpr uint32_t LW_MASK = (1u << 18) - 1u;
 constexpr uint32_t LW_NONE = 0x3fffu;
 constexpr int LW_MAX_SPHERES = (int)LW_NONE;  // sphere indices 0 .. LW_NONE - 1
@@ -329,8 +329,8 @@ struct Dem {
     const double* Th;
     double* Fh_prev;         // the sums of the previous step
     double* Th_prev;
-    float4* Fa;              // applied: mean of this and the previous step
-    float4* Ta;
+    float4* Fa;              // applied: mean of this and the previous step (launches per
+    float4* Ta;              // substep only: one launch keeps it in registers)
     const float* R;
     const float* invm;
     const float* invI;
