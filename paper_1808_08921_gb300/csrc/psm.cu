@@ -67,10 +67,11 @@ __device__ __forceinline__ double image(double d, double L, double iL, bool peri
 // order, the spheres that can reach the segment (their distance in the x, y
 // plane and to the z interval, with a margin of 0.01 lu over the exact test
 // below, far above the FP32 rounding of offsets within the box); its nodes then
-// evaluate only those.  Evaluating every sphere at every node is FP64 arithmetic at 2 lanes per clock and SM: 7.77 ms for
-// 128 spheres on 64 x 64 x 256, against 0.31 ms.  The kept spheres go through
-// the same test and product in the same order, so eps is the same bit for
-// bit.  A segment reached by more than EPS_LIST spheres walks them all.
+// evaluate only those.  Evaluating every sphere at every node is FP64
+// arithmetic at 2 lanes per clock and SM: 7.77 ms for 128 spheres on 64 x 64 x
+// 256, against 0.31 ms.  The kept spheres go through the same test and product
+// in the same order, so eps is the same bit for bit.  A segment reached by more
+// than EPS_LIST spheres walks them all.
 constexpr int EPS_LIST = 256;
 __global__ void k_psm_eps(PsmArgs A, const double* X, const double* R, int n, float* eps) {
     __shared__ int s_list[EPS_LIST];
