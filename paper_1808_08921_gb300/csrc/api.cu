@@ -527,12 +527,12 @@ static int build_layout(lbmdem_ctx* c, bool fresh) {
     const double reach = 2.0 * (c->Rmax + c->skin + 2.0);
     const bool wide = c->p.ny > reach && c->p.nz > reach && (!px || c->p.nx > reach);
     // (link_mode 0: with FP32 storage and spheres of radius 8 lu or more.
-    // R 11.4 FCC on 128 x 128 x 1024: 237 against 325 us per step with the
+    // R 11.4 FCC on 128 x 128 x 1024: 226 against 299 us per step with the
     // link kernel every step.  Smaller spheres, R 5.7 on 64 x 64 x 512: 80
     // against 83 us, but their stiffer contacts amplify the other order of
-    // the force sums, and results there stay what the link lists give; with
-    // 16-bit storage both kernels' populations are light and the link kernel
-    // rounds as the storage does)
+    // the force sums, and results there stay what the link lists give; 16-bit
+    // storage keeps the rounding of the link kernel, 253 us per step on the R
+    // 11.4 column against 207 in the collide kernels)
     const bool want = c->p.link_mode == 2 ||
                       (c->p.link_mode == 0 && c->p.storage == LBMDEM_F32 && c->Rmax >= 8.0);
     // Not where every sphere is fixed: there only the last step of a call takes
@@ -617,8 +617,8 @@ static void record_pair_end(lbmdem_ctx* c, size_t idx, cudaStream_t st = nullptr
 // that kind (link_mode) every even step's, and the odd steps' where most
 // nodes have links, from ODD_LINKS_MIN stored nodes up (the bound link_mode is
 // documented with).  R 11.4 FCC, the odd steps with the link kernel against
-// without, us per step: 159 k nodes 33.1 and 29.9, 629 k 54.4 and 46.3, 1.26 M
-// 87.7 and 72.5, 4.46 M 283 and 238; below the bound, 41 k nodes, 22.7 and 20.5.
+// without, us per step: 158 k nodes 37.4 and 34.5, 631 k 60.5 and 55.5, 1.25 M
+// 92.5 and 81.7, 4.46 M 266 and 226; below the bound, 45 k nodes, 27.3 and 25.4.
 constexpr uint32_t ODD_LINKS_MIN = 1u << 16;
 static bool links_in_collide(const lbmdem_ctx* c, int parity) {
     return c->fused_links && (parity == 0 || (c->dense_links && c->nS >= ODD_LINKS_MIN));
