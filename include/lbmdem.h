@@ -232,7 +232,7 @@ int lbm_dem_read_timing(lbmdem_ctx* c, double ms[6], int64_t launches[6]);
  * the populations checkpointed every `every` (even) steps and each segment
  * recomputed once.  Writes *loss, *dL_dtau, *dL_damp and, if not NULL,
  * trace_out[steps] = p(k).  Leaves the context at t0 + steps, as lbm_dem_step
- * would.  Device memory: the checkpoints (steps / every + 1 population copies)
+ * would.  Device memory: the checkpoints (steps / every population copies)
  * and `every` FP32 snapshots.  Errors: INVALID_ARG, STATE (mobile spheres, no
  * probe, odd t), OOM, CUDA. */
 int lbm_dem_adjoint(lbmdem_ctx* c, int64_t steps, int32_t every, const double* target, double* loss,

@@ -1570,16 +1570,14 @@ int lbm_dem_adjoint(lbmdem_ctx* c, int64_t steps, int32_t every, const double* t
     const size_t esz = c->p.storage == LBMDEM_F32 ? 4 : 2;
     const size_t fbytes = (size_t)Q * c->nSpad * esz;
     const int64_t nseg = (steps + every - 1) / every;
-    // forward with a checkpoint of the populations at the start of every
-    // segment; the last one is the end of the run, put back at the end
+    // forward with a checkpoint of the populations at the start of every segment
     DBuf<uint8_t> ck;
-    CK(ck.alloc(fbytes * (size_t)(nseg + 1)));
+    CK(ck.alloc(fbytes * (size_t)nseg));
     for (int64_t g = 0; g < nseg; ++g) {
         CK(cudaMemcpyAsync(ck.p + fbytes * g, c->f.p, fbytes, cudaMemcpyDeviceToDevice, s));
         int64_t n = std::min<int64_t>(every, steps - g * every);
         if (int r = lbm_dem_step(c, n)) return r;
     }
-    CK(cudaMemcpyAsync(ck.p + fbytes * nseg, c->f.p, fbytes, cudaMemcpyDeviceToDevice, s));
     // the reverse sweep's memory, mapped while the forward run is on the GPU
     const size_t nbytes = (size_t)Q * c->nSpad * sizeof(float);
     DBuf<float> nat, adj, adj2;
@@ -1615,7 +1613,11 @@ int lbm_dem_adjoint(lbmdem_ctx* c, int64_t steps, int32_t every, const double* t
     for (int64_t g = nseg - 1; g >= 0; --g) {
         int64_t n = std::min<int64_t>(every, steps - g * every);
         int64_t tg = t0 + g * every;
+        // the end of the run, wanted again below, takes the place of the last
+        // checkpoint, by way of the snapshots' memory
+        if (g == nseg - 1) CK(cudaMemcpyAsync(nat.p, c->f.p, fbytes, cudaMemcpyDeviceToDevice, s));
         CK(cudaMemcpyAsync(c->f.p, ck.p + fbytes * g, fbytes, cudaMemcpyDeviceToDevice, s));
+        if (g == nseg - 1) CK(cudaMemcpyAsync(ck.p + fbytes * g, nat.p, fbytes, cudaMemcpyDeviceToDevice, s));
         unsigned long long tdev = (unsigned long long)tg;
         CK(cudaMemcpyAsync(&c->st.p->t, &tdev, sizeof(tdev), cudaMemcpyHostToDevice, s));
         c->t = tg;
@@ -1645,7 +1647,7 @@ int lbm_dem_adjoint(lbmdem_ctx* c, int64_t steps, int32_t every, const double* t
     c->t = t_end;
     const unsigned long long tdev = (unsigned long long)t_end;
     CK(cudaMemcpyAsync(&c->st.p->t, &tdev, sizeof(tdev), cudaMemcpyHostToDevice, s));
-    CK(cudaMemcpyAsync(c->f.p, ck.p + fbytes * nseg, fbytes, cudaMemcpyDeviceToDevice, s));
+    CK(cudaMemcpyAsync(c->f.p, ck.p + fbytes * (nseg - 1), fbytes, cudaMemcpyDeviceToDevice, s));
     double gh[GRAD_COPIES + 1];
     CK(cudaMemcpyAsync(gh, grads.p, sizeof(gh), cudaMemcpyDeviceToHost, s));
     CK(cudaStreamSynchronize(s));
