@@ -30,6 +30,7 @@ struct DBuf {
         if (count == 0) count = 1;
         cudaError_t e = cudaMalloc((void**)&p, sizeof(T) * count);
         if (e != cudaSuccess) {
+            cudaGetLastError();  // reported here: not again after a later launch
             p = nullptr;
             n = 0;
             return e;

@@ -10,9 +10,15 @@
 static std::map<char*, size_t> live;  // blocks given out and not given back
 static size_t largest = SIZE_MAX;     // requests above this are refused
 
+static cudaError_t last_error = cudaSuccess;
+extern "C" cudaError_t cudaGetLastError() {
+    const cudaError_t e = last_error;
+    last_error = cudaSuccess;
+    return e;
+}
 extern "C" cudaError_t cudaMalloc(void** p, size_t bytes) {
     *p = nullptr;
-    if (bytes > largest) return cudaErrorMemoryAllocation;
+    if (bytes > largest) return last_error = cudaErrorMemoryAllocation;
     char* q = static_cast<char*>(std::malloc(bytes));
     live[q] = bytes;
     *p = q;
@@ -114,6 +120,10 @@ int main() {
         if (f.ensure(100, 3)) bad = 1;
         whole("conversions after a refusal", 100);
         largest = SIZE_MAX;
+    }
+    if (last_error != cudaSuccess) {
+        std::printf("a refusal is left for a later check to find\n");
+        bad = 1;
     }
     if (!live.empty()) {
         std::printf("%zu blocks not given back\n", live.size());
