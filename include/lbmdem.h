@@ -141,13 +141,15 @@ int lbm_dem_set_pressure_source(lbmdem_ctx* c, int32_t waveform, double amplitud
                                 double omega, int64_t t_n, double t0);
 
 /* Advance n >= 0 coupled steps.  Errors: STATE (no packing), CUDA, and the
- * latched device status (UNSTABLE, SKIN, CAPACITY) when it is read back. */
+ * latched device status (UNSTABLE, SKIN, CAPACITY) when it is read back; OOM
+ * or CUDA from a re-layout, after which the context needs a new packing. */
 int lbm_dem_step(lbmdem_ctx* c, int64_t n);
 
 /* Rebuild the compact lattice, the surface and link lists and the neighbour
  * lists around the current sphere positions.  lbm_dem_step does this by
  * itself when a sphere has moved half its skin; the state must sit between
- * an odd and an even step (t even).  Errors: STATE (t odd or no packing). */
+ * an odd and an even step (t even).  Errors: STATE (t odd or no packing); OOM,
+ * CUDA: the context needs a new packing. */
 int lbm_dem_relayout(lbmdem_ctx* c);
 
 /* Synchronise the stream and return the latched device status (0 or an

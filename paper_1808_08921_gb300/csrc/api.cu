@@ -842,8 +842,12 @@ static int check_and_relayout(lbmdem_ctx* c, bool& did) {
 
 // ------------------------------------------------------------ public API
 
+// A re-layout that fails half-way (no memory) leaves arrays of two layouts: the
+// context then has no packing until the next set_packing.
 static int relayout(lbmdem_ctx* c) {
     cudaStream_t s = c->stream;
+    c->have_packing = false;
+    destroy_graph(c);
     launch_rebase(c->Xref.p, c->dX.p, c->dXc.p, c->np, s);
     CK(cudaGetLastError());
     if (int r = build_cells(c)) return r;
@@ -855,7 +859,7 @@ static int relayout(lbmdem_ctx* c) {
     CK(cudaGetLastError());
     if (!c->lbm) CK(cudaStreamSynchronize(s));  // the exchange slots' count (build_layout synchronises)
     c->relayouts++;
-    destroy_graph(c);
+    c->have_packing = true;
     return 0;
 }
 

@@ -76,7 +76,7 @@ def attempt(k, call):
     assert np.abs(out[3] - ref[3]).max() <= 1e-9
     return got
 
-call = dict(set_packing=lambda s: pack(s, large))[sys.argv[2]]
+call = dict(set_packing=lambda s: pack(s, large), relayout=lambda s: s.relayout())[sys.argv[2]]
 k = 0
 while attempt(k, call) == OOM:
     k += 1
@@ -87,7 +87,7 @@ print("usable")
 """
 
 
-@pytest.mark.parametrize("call", ["set_packing"])
+@pytest.mark.parametrize("call", ["set_packing", "relayout"])
 def test_every_allocation_refused_in_turn(call, tmp_path):
     cc, shim = shutil.which("gcc"), str(tmp_path / "refuse_alloc.so")
     subprocess.run([cc, "-shared", "-fPIC", "-O1", os.path.join(ROOT, "tests", "host", "refuse_alloc.c"), "-o", shim,
